@@ -19,7 +19,8 @@ struct PushThreads {
 };
 
 // Per-warp double-buffered stage: [stage][slot][lane][4] for the particle arrays (slots ox oz dux
-// duy duz w in 2D; ox oy oz dux duy duz w in 3D), then [stage][lane][4] ids.
+// duy duz w in 2D; ox oy oz dux duy duz w in 3D), then [stage][lane][4] ids. Lane l copies a pack of 4
+// slots; a cell's lanes then take the particles of all its packs in turn, U at a time (PushPlan).
 template <typename T, int NDIM>
 struct PushStage {
   static constexpr int NSLOT = NDIM == 3 ? 7 : 6;
@@ -515,9 +516,30 @@ __device__ __forceinline__ void deposit3_reg(T (&acc)[NVP], const EsirDir<T>& X,
     }
 }
 
+// FP32 2D: each lane takes two neighbouring particles at a time, with the arithmetic of the pair
+// in packed FP32x2 instructions (one instruction advances both particles) and the two rebins
+// interleaved, so one dependent chain carries two particles.
+template <typename T, int NDIM>
+struct PushPaired {
+  static constexpr bool value = sizeof(T) == 4 && NDIM == 2;
+};
+
+// Rounds of a full item: 4 particles a lane, one or (paired) two per round.
+template <typename T, int NDIM>
+struct PushRounds {
+  static constexpr int value = PushPaired<T, NDIM>::value ? 2 : 4;
+};
+
 // Work assignment of the push kernel: a warp takes CPW = 32/LPC cells of its tile at a time,
 // LPC lanes per cell. The cell's particles are split into packs of 4 consecutive slots of one
-// species (electron packs first); lane l of the cell takes packs l, l + LPC, ... . Each lane sums
+// species (electron packs first); an item is LPC packs of every cell of the group, copied by one lane
+// each (16-byte copies: 8-byte ones cost the 3D push 40 %). Within an item the cell's lanes take its
+// 4 LPC slots in turn, lane l the slots U l .. U l + U - 1 of every round of U LPC slots, and the warp
+// runs only the rounds that its fullest cell needs. A cell of 17 + 16 particles costs its warp 9 rounds
+// of single particles (12 when every lane walked its own pack), and with 4 + 4 particles all four
+// lanes work (two of them before). Measured on 512x1024 FP32 cells, push per step: 16 per species at
+// c dt/dz = 0.5 (even cells) 330 -> 311 us and 0.3 523 -> 507 us, 8 per species 319 -> 231 us, 4 per
+// species 241 -> 174 us; 256x512 FP64 at 0.3 1.99 -> 1.76 ms; 3D 64x64x256 0.87 -> 0.84 ms. Each lane sums
 // the Esirkepov contributions of its particles in registers (the window of RegLayout: every
 // particle that neither steps back across a face nor crosses a transverse face); at the end one
 // segmented butterfly transpose-reduction over the cell's LPC lanes leaves PER = NVP/LPC of the
@@ -529,20 +551,20 @@ struct PushPlan {
   static constexpr int PER = (NV + LPC - 1) / LPC;
   static constexpr int NVP = PER * LPC;
   static constexpr int CPW = 32 / LPC;
+  // Round a cell (c-th of the group) starts a full item with: a round reads U LPC neighbouring values
+  // of every cell, and cells whose values lie in the same banks start with different rounds.
+  template <typename T>
+  static __device__ __forceinline__ int first_round(int c) {
+    constexpr int NR = PushRounds<T, NDIM>::value;
+    constexpr int M = (sizeof(T) == 8 || NR == 2 ? 16 : 32) / LPC;  // cells read in one pass of the banks
+    return (M > NR ? c / (M / NR) : c) & (NR - 1);
+  }
 };
 
 // Resident blocks per SM the push kernel is compiled for (register budget): FP32 2D fits two.
 template <typename T, int NDIM>
 struct PushMinBlocks {
   static constexpr int value = (sizeof(T) == 4 && NDIM == 2) ? 2 : 1;
-};
-
-// FP32 2D: each lane takes the particles of its pack two at a time, with the arithmetic of the pair
-// in packed FP32x2 instructions (one instruction advances both particles) and the two rebins
-// interleaved, so one dependent chain carries two particles.
-template <typename T, int NDIM>
-struct PushPaired {
-  static constexpr bool value = sizeof(T) == 4 && NDIM == 2;
 };
 
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -745,27 +767,32 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
 #pragma unroll
       for (int i = 0; i < NVP; ++i) acc[i] = T(0);
     }
-    {
-      const int q = sl + it * LPC;
+    // rounds of this item: up to the last slot in use of the fullest cell
+    constexpr int NR = PushRounds<T, NDIM>::value, U = 4 / NR;
+    int nk = 4 * (nq - it * LPC);  // slots of the cell's packs from this item on, then the last pack's empty ones
+    if (nk > 0 && nk <= 4 * LPC) nk -= 4 * (nq > nq0 ? nq - nq0 : nq0) - (nq > nq0 ? n1 : n0);
+    const int nrnd = min(NR, (__reduce_max_sync(0xffffffffu, nk) + U * LPC - 1) / (U * LPC));
+    const int rnd0 = nrnd == NR ? PL::template first_round<T>(lane / LPC) : 0;
+#pragma unroll 1
+    for (int rnd = 0; rnd < nrnd; ++rnd) {
+      // the lane's slots k .. k + U - 1 of the cell's 4 LPC slots in this item
+      const int k = U * (sl + LPC * ((rnd + rnd0) & (NR - 1)));
+      const int q = it * LPC + (k >> 2);
       const bool has = q < nq;
       const int s = (has && q >= nq0) ? 1 : 0;
-      const int q4 = 4 * (s ? q - nq0 : q);
-      const int cnt = has ? min(4, (s ? n1 : n0) - q4) : 0;
+      const int cnt = has ? (s ? n1 + 4 * nq0 : n0) - 4 * q - (k & 3) : 0;  // particles from slot k on
       const SpeciesBuf<T> pout = s ? r.out[1] : r.out[0];
       const T qs = s ? T(1) : T(-1);
-      const T* st_x = SG::at(stg, stage, 0, lane);  // array a of the lane's pack at st_x + slot(a) * 128
-      const unsigned* st_id = SG::id_at(stg, stage, lane);
+      const T* st_x = SG::at(stg, stage, 0, lane - sl) + k;  // array a of slot k at st_x + slot(a) * 128
+      const unsigned* st_id = SG::id_at(stg, stage, lane - sl) + k;
       if constexpr (PushPaired<T, NDIM>::value) {
         const float2 hh = make_float2(qs * r.hq, qs * r.hq);
         const float2 u02 = make_float2(r.u0, r.u0), one2 = make_float2(1.f, 1.f);
         const float2 dtdx2 = make_float2(r.dtdx, r.dtdx), dtdz2 = make_float2(r.dtdz, r.dtdz);
         const unsigned lt = (1u << lane) - 1u;
-#pragma unroll 1
-        for (int rp = 0; rp < 4; rp += 2) {
-          // the pack elements (ja, ja + 1) of this pair, one 8-byte load per array; lanes 8-15 and
-          // 24-31 take the other pair first, so a half-warp's loads cover all 32 banks
-          const int ja = 2 * (((rp >> 1) + (lane >> 3)) & 1), jb = ja + 1;
-          const bool va = ja < cnt, vb = jb < cnt;
+        {
+          constexpr int ja = 0, jb = 1;  // the pair: one 8-byte load per array
+          const bool va = cnt > 0, vb = cnt > 1;
           const float2 pox = *reinterpret_cast<const float2*>(st_x + ja);
           const float2 poz = *reinterpret_cast<const float2*>(st_x + SG::slot(2) * 128 + ja);
           const float2 pux = *reinterpret_cast<const float2*>(st_x + SG::slot(3) * 128 + ja);
@@ -950,12 +977,9 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
                   exb.shift, ezb.shift);
         }
       } else {
-#pragma unroll 1
-      for (int rnd = 0; rnd < 4; ++rnd) {
-        // pack element of this round, rotated by lane / 8 so the 32 lanes' shared-memory reads of
-        // one array fall in distinct banks
-        const int jj = (rnd + (lane >> 3)) & 3;
-        const bool valid = jj < cnt;
+      {
+        constexpr int jj = 0;
+        const bool valid = cnt > 0;
         int dkey = -1 - lane;  // unique per lane when there is no particle
         bool leave = false;
         T nox = T(0), noy = T(0), noz = T(0), ux = T(0), uy = T(0), uz = T(0);
