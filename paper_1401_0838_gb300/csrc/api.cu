@@ -299,7 +299,7 @@ void rebuild_taps(pic_handle* h) {
 // Particle tiles of the run's grid (push_tiles), spread over up to `spread` blocks.
 static void set_tiles(pic_handle* h, int spread) {
   int nt[3], te[3];
-  const bool ho = h->cfg.shape_order != 1 || h->cfg.scheme == PIC_MOMENTUM;  // the run's push is k_push_ho
+  const bool ho = h->cfg.shape_order != 1;  // cubic shapes have tiles of their own
   push_tiles(h->cfg.ndim, h->es, ho, h->cfg.nx, h->cfg.ny, h->cfg.nz, spread, nt, te);
   h->ntx = nt[0];
   h->nty = nt[1];

@@ -103,17 +103,22 @@ struct PTile<double, 3> {
   static constexpr int TX = 8, TY = 8, TZ = 8;
 };
 
-// Particle tile of the cubic and momentum-conserving push (k_push_ho): tall along the drift in 2D
-// too (the momentum-conserving push measured 14 % faster than on 16x16 tiles, the cubic the same).
+// Particle tile of the cubic push (k_push_ho): as PTile in 2D; in 3D the two-node halo makes narrow
+// tiles mostly halo (a 2x2x128 tile would stage 9 nodes a cell), so 4x4 columns, as tall as shared memory
+// allows.
 template <typename T, int NDIM>
 struct HoTile;
 template <typename T>
 struct HoTile<T, 2> {
   static constexpr int TX = 4, TY = 1, TZ = 64;
 };
-template <typename T>
-struct HoTile<T, 3> {
-  static constexpr int TX = 8, TY = 8, TZ = 8;
+template <>
+struct HoTile<float, 3> {
+  static constexpr int TX = 4, TY = 4, TZ = 32;
+};
+template <>
+struct HoTile<double, 3> {
+  static constexpr int TX = 4, TY = 4, TZ = 16;
 };
 
 // Everything a kernel needs about one simulation (passed by value as a kernel parameter).

@@ -84,8 +84,7 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// Particle tiles of a grid: the push kernel's tile (PTile, or HoTile for the cubic and momentum-
-// conserving push) for the precision (es bytes per value), halved (down to 4 cells, the longest
+// Particle tiles of a grid: the push kernel's tile (PTile, or HoTile for cubic shapes) for the precision (es bytes per value), halved (down to 4 cells, the longest
 // extent first) while twice the tiles still fit in `spread` blocks, so that a small grid spreads over
 // the SMs. spread = 0 keeps the full tile. te: cells per tile and direction.
 void push_tiles(int ndim, int es, bool ho, int nx, int ny, int nz, int spread, int nt[3], int te[3]);

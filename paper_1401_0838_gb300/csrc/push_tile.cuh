@@ -1,0 +1,1754 @@
+// One particle tile of the push: gather + Boris + move + Esirkepov deposition + rebin, shared by the
+// linear push (k_particles.cu) and the cubic and momentum-conserving push (k_push_ho.cu). See
+// k_particles.cu for the particle storage.
+#pragma once
+#include "common.cuh"
+#include "fastmath.cuh"
+
+namespace picgb {
+
+// Threads per push block: 8 warps; the 3D FP32 kernel, one block per SM, takes 12 warps. Cubic shapes
+// (ORDER 3): the 51 register sums of the 2D window leave 168 registers a thread, two blocks of 6 warps
+// in FP32; 3D FP64 6 warps (their stages have to fit in shared memory).
+template <typename T, int NDIM, int ORDER = 1>
+struct PushThreads {
+  static constexpr int value = ORDER == 3 ? (NDIM == 3 ? (sizeof(T) == 4 ? 384 : 192) : (sizeof(T) == 4 ? 192 : 256))
+                                          : (NDIM == 3 && sizeof(T) == 4) ? 384 : 256;
+};
+
+// The tile's compile-time extents by shape order.
+template <typename T, int NDIM, int ORDER>
+struct PushTileOf {
+  using type = PTile<T, NDIM>;
+};
+template <typename T, int NDIM>
+struct PushTileOf<T, NDIM, 3> {
+  using type = HoTile<T, NDIM>;
+};
+
+// Per-warp double-buffered stage: [stage][slot][lane][4] for the particle arrays (slots ox oz dux
+// duy duz w in 2D; ox oy oz dux duy duz w in 3D), then [stage][lane][4] ids. Lane l copies a pack of 4
+// slots; a cell's lanes then take the particles of all its packs in turn, U at a time (PushPlan).
+template <typename T, int NDIM>
+struct PushStage {
+  static constexpr int NSLOT = NDIM == 3 ? 7 : 6;
+  // slot of array a (0 ox, 1 oy, 2 oz, 3 dux, 4 duy, 5 duz, 6 w); 2D stages no oy
+  static constexpr __host__ __device__ int slot(int a) { return NDIM == 3 ? a : (a > 1 ? a - 1 : a); }
+  static constexpr __host__ __device__ size_t per_warp_elems() {
+    return 2 * NSLOT * 32 * 4 + (2 * 32 * 4 * sizeof(unsigned) + sizeof(T) - 1) / sizeof(T);
+  }
+  static __device__ __forceinline__ T* at(T* base, int stage, int arr, int lane) {
+    return base + ((stage * NSLOT + slot(arr)) * 32 + lane) * 4;
+  }
+  static __device__ __forceinline__ unsigned* id_at(T* base, int stage, int lane) {
+    return reinterpret_cast<unsigned*>(base + 2 * NSLOT * 32 * 4) + (stage * 32 + lane) * 4;
+  }
+};
+
+
+// FP32 2D: each lane takes two neighbouring particles at a time, with the arithmetic of the pair
+// in packed FP32x2 instructions (one instruction advances both particles) and the two rebins
+// interleaved, so one dependent chain carries two particles.
+template <typename T, int NDIM>
+struct PushPaired {
+  static constexpr bool value = sizeof(T) == 4 && NDIM == 2;
+};
+
+// WIN: the gather reads every particle's nodes from one window of its cell (gather_window), as the
+// cubic and the momentum-conserving gathers do; a paired push then keeps every node twice, so that one
+// 8-byte load yields the packed operand for both particles.
+template <typename T, int NDIM, int ORDER = 1, bool WIN = false>
+struct PushSmem {
+  using TL = typename PushTileOf<T, NDIM, ORDER>::type;
+  static constexpr int TX = TL::TX, TY = TL::TY, TZ = TL::TZ;
+  static constexpr int NCL = TX * TY * TZ;
+  static constexpr int H = (ORDER + 1) / 2;
+  // gather tile: nodes [X0-H, X0+TX+H) per direction (y only in 3D)
+  static constexpr int GX = TX + 2 * H, GY = (NDIM == 3 ? TY + 2 * H : 1), GZ = TZ + 2 * H, GN = GX * GY * GZ;
+  static constexpr int GCOPY = WIN && PushPaired<T, NDIM>::value ? 2 : 1;  // stored values per node
+  // current tile: nodes [X0-H, X0+TX+H]
+  static constexpr int JX = TX + 2 * H + 1, JY = (NDIM == 3 ? TY + 2 * H + 1 : 1), JZ = TZ + 2 * H + 1;
+  static constexpr int JN = JX * JY * JZ;
+  // particles leaving the tile, buffered per block: [7][LVB] values (ox oy oz dux duy duz w), LVB
+  // keys, LVB ids and the buffer's counter; written to the global leaver list once per tile
+  static constexpr int LVB = (NDIM == 3 && sizeof(T) == 8) ? 128 : 512;  // 3D FP64: within 227 KB
+  static constexpr size_t lv_bytes() { return (size_t)LVB * (7 * sizeof(T) + 2 * sizeof(int)) + 16; }
+  static constexpr size_t bytes() {
+    return sizeof(T) * (6 * GN * GCOPY + 3 * JN) + sizeof(int) * (4 * NCL) + 16 +
+           sizeof(T) * PushStage<T, NDIM>::per_warp_elems() * (PushThreads<T, NDIM, ORDER>::value / 32) + 16 + lv_bytes();
+  }
+};
+
+// Per-direction interpolation weights of a particle at cell-relative offset o:
+// integer-node S1 (base 0: nodes 0, 1), half-node S1 (Uniform: base -1 or 0), half-node S0
+// (Galerkin: node 0). Bases are relative to the particle's cell.
+template <typename T>
+struct DirW {
+  T i0, i1;     // integer nodes 0 and 1
+  int hb;       // half-node base (-1 or 0)
+  T h0, h1;     // half nodes hb, hb+1
+};
+
+template <typename T>
+__device__ __forceinline__ DirW<T> dir_weights(T o) {
+  DirW<T> d;
+  d.i0 = T(1) - o;
+  d.i1 = o;
+  if (o < T(0.5)) {
+    d.hb = -1;
+    T g = o + T(0.5);
+    d.h0 = T(1) - g;
+    d.h1 = g;
+  } else {
+    d.hb = 0;
+    T g = o - T(0.5);
+    d.h0 = T(1) - g;
+    d.h1 = g;
+  }
+  return d;
+}
+
+// One direction of the gather: returns (base, w0, w1, two) for stagger st and scheme.
+template <typename T, int SCHEME>
+__device__ __forceinline__ void pick(const DirW<T>& d, int st, int& base, T& w0, T& w1, bool& two) {
+  if (!st) {
+    base = 0; w0 = d.i0; w1 = d.i1; two = true;
+  } else if (SCHEME == 0) {  // Galerkin: S0 along a half-staggered direction
+    base = 0; w0 = T(1); w1 = T(0); two = false;
+  } else {                   // Uniform: S1 at the half-integer nodes
+    base = d.hb; w0 = d.h0; w1 = d.h1; two = true;
+  }
+}
+
+// Stagger of Ex Ey Ez Bx By Bz along x, y, z.
+__device__ __constant__ int c_stag[6][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {0, 1, 1}, {1, 0, 1}, {1, 1, 0}};
+
+template <typename T, int NDIM, int SCHEME>
+__device__ __forceinline__ T gather_comp(const T* __restrict__ sgc, int c, int lx, int ly, int lz, const DirW<T>& dx,
+                                         const DirW<T>& dy, const DirW<T>& dz) {
+  using S = PushSmem<T, NDIM>;
+  int bx, by = 0, bz;
+  T x0, x1, y0 = T(1), y1 = T(0), z0, z1;
+  bool tx, ty = false, tz;
+  pick<T, SCHEME>(dx, c_stag[c][0], bx, x0, x1, tx);
+  if (NDIM == 3) pick<T, SCHEME>(dy, c_stag[c][1], by, y0, y1, ty);
+  pick<T, SCHEME>(dz, c_stag[c][2], bz, z0, z1, tz);
+  // smem index of node (lx+bx, ly+by, lz+bz), +1 halo offset per direction
+  const int ix = lx + bx + 1, iy = (NDIM == 3 ? ly + by + 1 : 0), iz = lz + bz + 1;
+  const T* p = sgc + (iz * S::GY + iy) * S::GX + ix;
+  T acc;
+  {
+    T r0 = x0 * p[0] + (tx ? x1 * p[1] : T(0));
+    T r1 = T(0);
+    if (ty) {
+      const T* q = p + S::GX;
+      r1 = x0 * q[0] + (tx ? x1 * q[1] : T(0));
+    }
+    acc = z0 * (y0 * r0 + y1 * r1);
+  }
+  if (tz) {
+    const T* p2 = p + S::GX * S::GY;
+    T r0 = x0 * p2[0] + (tx ? x1 * p2[1] : T(0));
+    T r1 = T(0);
+    if (ty) {
+      const T* q = p2 + S::GX;
+      r1 = x0 * q[0] + (tx ? x1 * q[1] : T(0));
+    }
+    acc += z1 * (y0 * r0 + y1 * r1);
+  }
+  return acc;
+}
+
+// One direction of an Esirkepov move of displacement d (|d| < 1 cell) from offset o in [0,1):
+// the 3-node window (origin a = -1 or 0 relative to the cell), the start shapes S0 and the shape
+// changes dS on it, and the new cell shift and offset. dS is formed from d itself (slope times
+// the move on the linear piece of the spline), not as S(o + d) - S(o), so that moves far below one
+// ulp of the offset (the transverse drift of a cold relativistic beam) keep full relative
+// precision; the three dS always sum to zero (charge conservation).
+template <typename T>
+struct EsirDir {
+  int a, shift;
+  T off;
+  T S0[3], dS[3];
+};
+
+// Comparisons of the push's values. FP64: integer tests on the IEEE bit patterns, exact for every
+// value that is not a NaN (the offsets and displacements compared here are finite), which keeps
+// them off the narrow FP64 pipe that bounds the FP64 push. FP32: plain comparisons.
+template <typename T>
+__device__ __forceinline__ bool is_neg(T x) {  // x < 0 (-0 is not)
+  if constexpr (sizeof(T) == 8) return (unsigned long long)__double_as_longlong(x) > 0x8000000000000000ull;
+  else return x < T(0);
+}
+template <typename T>
+__device__ __forceinline__ bool is_pos(T x) {  // x > 0
+  if constexpr (sizeof(T) == 8) return __double_as_longlong(x) > 0;
+  else return x > T(0);
+}
+template <typename T>
+__device__ __forceinline__ bool ge_one(T x) {  // x >= 1
+  if constexpr (sizeof(T) == 8) return __double_as_longlong(x) >= 0x3FF0000000000000ll;
+  else return x >= T(1);
+}
+template <typename T>
+__device__ __forceinline__ bool is_zero(T x) {  // x == 0 (either sign)
+  if constexpr (sizeof(T) == 8) return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) == 0;
+  else return x == T(0);
+}
+template <typename T>
+__device__ __forceinline__ bool abs_lt_one(T x) {  // -1 < x < 1; false for a NaN or an infinity
+  if constexpr (sizeof(T) == 8) return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) < 0x3FF0000000000000ll;
+  else return x > T(-1) && x < T(1);
+}
+
+template <typename T>
+__device__ __forceinline__ EsirDir<T> esir_dir(T o, T d) {
+  EsirDir<T> e;
+  const T x1 = o + d;
+  if (is_neg(x1)) {  // into the cell below: window nodes -1, 0, 1
+    e.a = -1;
+    e.S0[0] = T(0); e.S0[1] = T(1) - o; e.S0[2] = o;
+    e.dS[0] = -x1; e.dS[2] = -o; e.dS[1] = -(e.dS[0] + e.dS[2]);
+    e.off = T(1) + x1;
+    e.shift = -1;
+    if (ge_one(e.off)) { e.off = T(0); e.shift = 0; }
+  } else {
+    e.a = 0;
+    e.S0[0] = T(1) - o; e.S0[1] = o; e.S0[2] = T(0);
+    const T am = T(1) - o;  // distance to the upper face
+    const T c = d - am;     // x1 - 1, without the rounding of x1
+    if (ge_one(x1) && is_pos(c)) {  // into the cell above: nodes 0, 1, 2
+      e.dS[0] = -am; e.dS[2] = c; e.dS[1] = -(e.dS[0] + e.dS[2]);
+      e.off = c;
+      e.shift = 1;
+    } else {  // same cell (or onto the upper face within rounding)
+      e.dS[0] = -d; e.dS[1] = d; e.dS[2] = T(0);
+      if (ge_one(x1)) { e.off = T(0); e.shift = 1; }
+      else { e.off = x1; e.shift = 0; }
+    }
+  }
+  return e;
+}
+
+// Layout of one particle's current contributions: index i -> (component, node offset in the
+// 3-node window). 2D: 6 Jx (b*2+a), 6 Jz (6+a*2+b), 9 Jy (12+b*3+a). 3D: 18 Jx ((c*3+b)*2+a),
+// 18 Jy (18+(c*3+a)*2+b), 18 Jz (36+(b*3+a)*2+c); a, b, c are the x, y, z node offsets.
+template <int NDIM>
+struct DepLayout;
+template <>
+struct DepLayout<2> {
+  static constexpr int NV = 21;
+  static __device__ __forceinline__ void at(int i, int& comp, int& a, int& b, int& c) {
+    b = 0;
+    if (i < 6) { comp = 0; c = i >> 1; a = i & 1; }
+    else if (i < 12) { comp = 2; a = (i - 6) >> 1; c = (i - 6) & 1; }
+    else { comp = 1; c = (i - 12) / 3; a = (i - 12) % 3; }
+  }
+};
+template <>
+struct DepLayout<3> {
+  static constexpr int NV = 54;
+  static __device__ __forceinline__ void at(int i, int& comp, int& a, int& b, int& c) {
+    if (i < 18) { comp = 0; a = i & 1; b = (i >> 1) % 3; c = (i >> 1) / 3; }
+    else if (i < 36) { const int m = i - 18; comp = 1; b = m & 1; a = (m >> 1) % 3; c = (m >> 1) / 3; }
+    else { const int m = i - 36; comp = 2; c = m & 1; a = (m >> 1) % 3; b = (m >> 1) / 3; }
+  }
+};
+
+// Periodic index of g in [-n, 2n) without a modulo (callers guarantee the range: near_ok, or a
+// neighbour cell index in [-1, n]).
+__device__ __forceinline__ int wrap_near_p(int g, int n) { return g < 0 ? g + n : (g >= n ? g - n : g); }
+
+// FP32 uses the hardware reciprocal square root and fast division (relative error ~1e-7, inside
+// the 1e-5 per-step bar); FP64 keeps IEEE division and square root.
+
+// Galerkin gather (order 0 along each half-staggered direction, order 1 elsewhere): the nodes are
+// the same for every particle of a cell, so they are read once per lane and each component is an
+// affine or bilinear function of the cell offsets. Node (a, b, c) of a component is its value at
+// offsets (a, b, c) from the cell's own node in the shared-memory tile.
+template <typename T, int NDIM>
+struct GalCache;
+
+template <typename T>
+struct GalCache<T, 2> {
+  // Ex: x half -> S0; z -> S1. Ey: S1 x, S1 z. Ez: S1 x; z half -> S0. Bx: S1 x; S0 z.
+  // By: S0 x, S0 z. Bz: S0 x; S1 z.
+  T ex0, ex1, ey00, ey10, ey01, ey11, ez0, ez1, bx0, bx1, by0, bz0, bz1;
+  __device__ __forceinline__ void load(const T* sg, int lx, int ly, int lz) {
+    using S = PushSmem<T, 2>;
+    const int p = (lz + 1) * S::GX + lx + 1;
+    const T* e = sg;
+    ex0 = e[p]; ex1 = e[p + S::GX] - ex0;
+    e = sg + S::GN;
+    ey00 = e[p]; ey10 = e[p + 1] - ey00; ey01 = e[p + S::GX] - ey00; ey11 = e[p + S::GX + 1] - e[p + S::GX] - ey10;
+    e = sg + 2 * S::GN;
+    ez0 = e[p]; ez1 = e[p + 1] - ez0;
+    e = sg + 3 * S::GN;
+    bx0 = e[p]; bx1 = e[p + 1] - bx0;
+    by0 = sg[4 * S::GN + p];
+    e = sg + 5 * S::GN;
+    bz0 = e[p]; bz1 = e[p + S::GX] - bz0;
+  }
+  __device__ __forceinline__ void interp(T ox, T, T oz, T (&F)[6]) const {
+    F[0] = ex0 + oz * ex1;
+    F[1] = ey00 + ox * ey10 + oz * (ey01 + ox * ey11);
+    F[2] = ez0 + ox * ez1;
+    F[3] = bx0 + ox * bx1;
+    F[4] = by0;
+    F[5] = bz0 + oz * bz1;
+  }
+};
+
+template <typename T>
+struct GalCache<T, 3> {
+  // Ex: S0 x, bilinear (y, z). Ey: S0 y, bilinear (x, z). Ez: S0 z, bilinear (x, y).
+  // Bx: S0 y, z, linear x. By: S0 x, z, linear y. Bz: S0 x, y, linear z.
+  T e[3][4], b[3][2];
+  __device__ __forceinline__ void bil(const T* f, int p, int s1, int s2, T (&o)[4]) {
+    o[0] = f[p];
+    o[1] = f[p + s1] - o[0];
+    o[2] = f[p + s2] - o[0];
+    o[3] = f[p + s1 + s2] - f[p + s2] - o[1];
+  }
+  __device__ __forceinline__ void load(const T* sg, int lx, int ly, int lz) {
+    using S = PushSmem<T, 3>;
+    const int p = ((lz + 1) * S::GY + ly + 1) * S::GX + lx + 1;
+    const int sx = 1, sy = S::GX, sz = S::GX * S::GY;
+    bil(sg, p, sy, sz, e[0]);
+    bil(sg + S::GN, p, sx, sz, e[1]);
+    bil(sg + 2 * S::GN, p, sx, sy, e[2]);
+    b[0][0] = sg[3 * S::GN + p]; b[0][1] = sg[3 * S::GN + p + sx] - b[0][0];
+    b[1][0] = sg[4 * S::GN + p]; b[1][1] = sg[4 * S::GN + p + sy] - b[1][0];
+    b[2][0] = sg[5 * S::GN + p]; b[2][1] = sg[5 * S::GN + p + sz] - b[2][0];
+  }
+  __device__ __forceinline__ void interp(T ox, T oy, T oz, T (&F)[6]) const {
+    F[0] = e[0][0] + oy * e[0][1] + oz * (e[0][2] + oy * e[0][3]);
+    F[1] = e[1][0] + ox * e[1][1] + oz * (e[1][2] + ox * e[1][3]);
+    F[2] = e[2][0] + ox * e[2][1] + oy * (e[2][2] + ox * e[2][3]);
+    F[3] = b[0][0] + ox * b[0][1];
+    F[4] = b[1][0] + oy * b[1][1];
+    F[5] = b[2][0] + oz * b[2][1];
+  }
+};
+
+// Esirkepov contributions of one particle, written as sums into the 3-node window of its own
+// cell (layout of DepLayout). With f = S0 + dS/2 per direction, the 2D out-of-plane weight
+// S0x S0z + dSx S0z/2 + S0x dSz/2 + dSx dSz/3 equals fx fz + dSx dSz / 12, and the running sums
+// of the in-plane weights at the two half-nodes are dS[0] and -dS[2] times the transverse factor.
+template <typename T, int NVP>
+__device__ __forceinline__ void deposit2(T (&acc)[NVP], const EsirDir<T>& X, const EsirDir<T>& Z, T cx, T cy, T cz) {
+  T fx[3], fz[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    fx[a] = X.S0[a] + T(0.5) * X.dS[a];
+    fz[a] = Z.S0[a] + T(0.5) * Z.dS[a];
+  }
+  const T gx0 = cx * X.dS[0], gx1 = -cx * X.dS[2];
+  const T gz0 = cz * Z.dS[0], gz1 = -cz * Z.dS[2];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    acc[b * 2 + 0] += gx0 * fz[b];
+    acc[b * 2 + 1] += gx1 * fz[b];
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    acc[6 + a * 2 + 0] += gz0 * fx[a];
+    acc[6 + a * 2 + 1] += gz1 * fx[a];
+  }
+  T hx[3], kx[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    hx[a] = cy * fx[a];
+    kx[a] = cy * X.dS[a] * T(1.0 / 12.0);
+  }
+#pragma unroll
+  for (int b = 0; b < 3; ++b)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) acc[12 + b * 3 + a] += hx[a] * fz[b] + kx[a] * Z.dS[b];
+}
+
+// Same contributions added to shared memory at the window origin (wx, wz) (tile indices).
+template <typename T, int NDIM>
+__device__ __noinline__ void deposit2_smem(T* sj, int wx, int wz, EsirDir<T> X, EsirDir<T> Z, T cx, T cy, T cz) {
+  using S = PushSmem<T, NDIM>;
+  T v[DepLayout<2>::NV];
+#pragma unroll
+  for (int i = 0; i < DepLayout<2>::NV; ++i) v[i] = T(0);
+  deposit2<T, DepLayout<2>::NV>(v, X, Z, cx, cy, cz);
+  const int key = wz * S::JX + wx;
+#pragma unroll
+  for (int i = 0; i < DepLayout<2>::NV; ++i) {
+    int comp, a, b, c;
+    DepLayout<2>::at(i, comp, a, b, c);
+    atomicAdd(sj + comp * S::JN + key + c * S::JX + a, v[i]);
+  }
+}
+
+// 3D: W_a = dS_a T(b1, b2) with T = f f + dS dS / 12 over the two transverse directions.
+template <typename T, int NVP>
+__device__ __forceinline__ void deposit3(T (&acc)[NVP], const EsirDir<T>& X, const EsirDir<T>& Y, const EsirDir<T>& Z,
+                                         T cx, T cy, T cz) {
+  T fx[3], fy[3], fz[3], kx[3], ky[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    fx[a] = X.S0[a] + T(0.5) * X.dS[a];
+    fy[a] = Y.S0[a] + T(0.5) * Y.dS[a];
+    fz[a] = Z.S0[a] + T(0.5) * Z.dS[a];
+    kx[a] = X.dS[a] * T(1.0 / 12.0);
+    ky[a] = Y.dS[a] * T(1.0 / 12.0);
+  }
+  const T gx0 = cx * X.dS[0], gx1 = -cx * X.dS[2];
+  const T gy0 = cy * Y.dS[0], gy1 = -cy * Y.dS[2];
+  const T gz0 = cz * Z.dS[0], gz1 = -cz * Z.dS[2];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {  // Jx(a+1/2, b, c)
+      const T t = fy[b] * fz[c] + ky[b] * Z.dS[c];
+      acc[(c * 3 + b) * 2 + 0] += gx0 * t;
+      acc[(c * 3 + b) * 2 + 1] += gx1 * t;
+    }
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {  // Jy(a, b+1/2, c)
+      const T t = fx[a] * fz[c] + kx[a] * Z.dS[c];
+      acc[18 + (c * 3 + a) * 2 + 0] += gy0 * t;
+      acc[18 + (c * 3 + a) * 2 + 1] += gy1 * t;
+    }
+#pragma unroll
+  for (int b = 0; b < 3; ++b)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {  // Jz(a, b, c+1/2)
+      const T t = fx[a] * fy[b] + kx[a] * Y.dS[b];
+      acc[36 + (b * 3 + a) * 2 + 0] += gz0 * t;
+      acc[36 + (b * 3 + a) * 2 + 1] += gz1 * t;
+    }
+}
+
+template <typename T, int NDIM>
+__device__ __noinline__ void deposit3_smem(T* sj, int wx, int wy, int wz, EsirDir<T> X, EsirDir<T> Y, EsirDir<T> Z,
+                                           T cx, T cy, T cz) {
+  using S = PushSmem<T, NDIM>;
+  T v[DepLayout<3>::NV];
+#pragma unroll
+  for (int i = 0; i < DepLayout<3>::NV; ++i) v[i] = T(0);
+  deposit3<T, DepLayout<3>::NV>(v, X, Y, Z, cx, cy, cz);
+  const int key = (wz * S::JY + wy) * S::JX + wx;
+#pragma unroll
+  for (int i = 0; i < DepLayout<3>::NV; ++i) {
+    int comp, a, b, c;
+    DepLayout<3>::at(i, comp, a, b, c);
+    atomicAdd(sj + comp * S::JN + key + (c * S::JY + b) * S::JX + a, v[i]);
+  }
+}
+
+// The sums each lane keeps in registers: the Esirkepov window of a particle that starts in its own
+// cell, does not step back across a face, and does not cross its cell's upper face in x (nor, in
+// 3D, in y). Such a particle's shape changes vanish at the window's third transverse node (S0 and
+// dS are zero there), so its contributions there are exactly zero: of the 3-node window only
+// x nodes 0-1 (2D: 13 of the 21 sums; 3D: y nodes 0-1 too, 20 of the 54) carry it. Every other
+// particle (a transverse face crossed, or a step back) adds its full window to shared memory.
+// 2D layout: 3 Jx (node a = 0, z node c = i), 4 Jz (3 + a*2 + c), 6 Jy (7 + c*2 + a).
+// 3D layout: 6 Jx (a = 0; c*2 + b), 6 Jy (b = 0; 6 + c*2 + a), 8 Jz (12 + (b*2 + a)*2 + c).
+// Cubic, 2D (ORDER 3; nodes from one below the cell: x 0-3, z 0-4): 15 Jx (c*3 + a), 16 Jz
+// (15 + a*4 + c), 20 Jy (31 + c*4 + a). Cubic in 3D deposits after the push (deposit3_cubic).
+template <int NDIM, int ORDER = 1>
+struct RegLayout;
+template <>
+struct RegLayout<2, 3> {
+  static constexpr int NV = 51;
+  static __device__ __forceinline__ void at(int i, int& comp, int& a, int& b, int& c) {
+    b = 0;
+    if (i < 15) { comp = 0; c = i / 3; a = i - 3 * c; }
+    else if (i < 31) { comp = 2; a = (i - 15) >> 2; c = (i - 15) & 3; }
+    else { comp = 1; c = (i - 31) >> 2; a = (i - 31) & 3; }
+  }
+};
+template <>
+struct RegLayout<3, 3> {
+  static constexpr int NV = 1;  // no sums are kept across rounds
+  static __device__ __forceinline__ void at(int, int&, int&, int&, int&) {}
+};
+template <>
+struct RegLayout<2, 1> {
+  static constexpr int NV = 13;
+  static __device__ __forceinline__ void at(int i, int& comp, int& a, int& b, int& c) {
+    b = 0;
+    if (i < 3) { comp = 0; a = 0; c = i; }
+    else if (i < 7) { comp = 2; a = (i - 3) >> 1; c = (i - 3) & 1; }
+    else { comp = 1; c = (i - 7) >> 1; a = (i - 7) & 1; }
+  }
+};
+template <>
+struct RegLayout<3, 1> {
+  static constexpr int NV = 20;
+  static __device__ __forceinline__ void at(int i, int& comp, int& a, int& b, int& c) {
+    if (i < 6) { comp = 0; a = 0; b = i & 1; c = i >> 1; }
+    else if (i < 12) { const int k = i - 6; comp = 1; b = 0; a = k & 1; c = k >> 1; }
+    else { const int k = i - 12; comp = 2; c = k & 1; a = (k >> 1) & 1; b = k >> 2; }
+  }
+};
+
+// Whether a particle's window fits the register sums (see RegLayout).
+template <typename T, int NDIM>
+__device__ __forceinline__ bool reg_window(const EsirDir<T>& X, const EsirDir<T>& Y, const EsirDir<T>& Z) {
+  if (NDIM == 3) return (X.a | Y.a | Z.a) == 0 && is_zero(X.dS[2]) && is_zero(Y.dS[2]);
+  return (X.a | Z.a) == 0 && is_zero(X.dS[2]);
+}
+
+// The contributions of deposit2 / deposit3 that can be nonzero for such a particle, into the
+// register layout (the same products and sums as the full window).
+template <typename T, int NVP>
+__device__ __forceinline__ void deposit2_reg(T (&acc)[NVP], const EsirDir<T>& X, const EsirDir<T>& Z, T cx, T cy,
+                                             T cz) {
+  const T fx0 = X.S0[0] + T(0.5) * X.dS[0], fx1 = X.S0[1] + T(0.5) * X.dS[1];
+  T fz[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) fz[b] = Z.S0[b] + T(0.5) * Z.dS[b];
+  const T gx0 = cx * X.dS[0];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) acc[b] += gx0 * fz[b];
+  const T gz0 = cz * Z.dS[0], gz1 = -cz * Z.dS[2];
+  acc[3] += gz0 * fx0;
+  acc[4] += gz1 * fx0;
+  acc[5] += gz0 * fx1;
+  acc[6] += gz1 * fx1;
+  const T hx0 = cy * fx0, hx1 = cy * fx1;
+  const T kx0 = cy * X.dS[0] * T(1.0 / 12.0), kx1 = cy * X.dS[1] * T(1.0 / 12.0);
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    acc[7 + 2 * b] += hx0 * fz[b] + kx0 * Z.dS[b];
+    acc[8 + 2 * b] += hx1 * fz[b] + kx1 * Z.dS[b];
+  }
+}
+
+template <typename T, int NVP>
+__device__ __forceinline__ void deposit3_reg(T (&acc)[NVP], const EsirDir<T>& X, const EsirDir<T>& Y,
+                                             const EsirDir<T>& Z, T cx, T cy, T cz) {
+  T fx[2], fy[2], fz[3], kx[2], ky[2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    fx[a] = X.S0[a] + T(0.5) * X.dS[a];
+    fy[a] = Y.S0[a] + T(0.5) * Y.dS[a];
+    kx[a] = X.dS[a] * T(1.0 / 12.0);
+    ky[a] = Y.dS[a] * T(1.0 / 12.0);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) fz[c] = Z.S0[c] + T(0.5) * Z.dS[c];
+  const T gx0 = cx * X.dS[0], gy0 = cy * Y.dS[0];
+  const T gz0 = cz * Z.dS[0], gz1 = -cz * Z.dS[2];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) acc[c * 2 + b] += gx0 * (fy[b] * fz[c] + ky[b] * Z.dS[c]);  // Jx(1/2, b, c)
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int a = 0; a < 2; ++a) acc[6 + c * 2 + a] += gy0 * (fx[a] * fz[c] + kx[a] * Z.dS[c]);  // Jy(a, 1/2, c)
+#pragma unroll
+  for (int b = 0; b < 2; ++b)
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {  // Jz(a, b, c + 1/2)
+      const T t = fx[a] * fy[b] + kx[a] * Y.dS[b];
+      acc[12 + (b * 2 + a) * 2 + 0] += gz0 * t;
+      acc[12 + (b * 2 + a) * 2 + 1] += gz1 * t;
+    }
+}
+
+// Rounds of a full item: 4 particles a lane, one or (paired) two per round.
+template <typename T, int NDIM>
+struct PushRounds {
+  static constexpr int value = PushPaired<T, NDIM>::value ? 2 : 4;
+};
+
+// Work assignment of the push kernel: a warp takes CPW = 32/LPC cells of its tile at a time,
+// LPC lanes per cell. The cell's particles are split into packs of 4 consecutive slots of one
+// species (electron packs first); an item is LPC packs of every cell of the group, copied by one lane
+// each (16-byte copies: 8-byte ones cost the 3D push 40 %). Within an item the cell's lanes take its
+// 4 LPC slots in turn, lane l the slots U l .. U l + U - 1 of every round of U LPC slots, and the warp
+// runs only the rounds that its fullest cell needs. A cell of 17 + 16 particles costs its warp 9 rounds
+// of single particles (12 when every lane walked its own pack), and with 4 + 4 particles all four
+// lanes work (two of them before). Measured on 512x1024 FP32 cells, push per step: 16 per species at
+// c dt/dz = 0.5 (even cells) 330 -> 311 us and 0.3 523 -> 507 us, 8 per species 319 -> 231 us, 4 per
+// species 241 -> 174 us; 256x512 FP64 at 0.3 1.99 -> 1.76 ms; 3D 64x64x256 0.87 -> 0.84 ms. Each lane sums
+// the Esirkepov contributions of its particles in registers (the window of RegLayout: every
+// particle that neither steps back across a face nor crosses a transverse face); at the end one
+// segmented butterfly transpose-reduction over the cell's LPC lanes leaves PER = NVP/LPC of the
+// cell's NVP (padded) sums in each lane, added to shared memory with distinct addresses. The other
+// particles add their full 3-node window to shared memory directly.
+template <int NDIM, int LPC, int ORDER = 1>
+struct PushPlan {
+  static constexpr int NV = RegLayout<NDIM, ORDER>::NV;
+  static constexpr int PER = (NV + LPC - 1) / LPC;
+  static constexpr int NVP = PER * LPC;
+  static constexpr int CPW = 32 / LPC;
+  // Round a cell (c-th of the group) starts a full item with: a round reads U LPC neighbouring values
+  // of every cell, and cells whose values lie in the same banks start with different rounds.
+  template <typename T>
+  static __device__ __forceinline__ int first_round(int c) {
+    constexpr int NR = PushRounds<T, NDIM>::value;
+    constexpr int M = (sizeof(T) == 8 || NR == 2 ? 16 : 32) / LPC;  // cells read in one pass of the banks
+    return (M > NR ? c / (M / NR) : c) & (NR - 1);
+  }
+};
+
+// Resident blocks per SM the push kernel is compiled for (register budget): FP32 2D fits two.
+template <typename T, int NDIM>
+struct PushMinBlocks {
+  static constexpr int value = (sizeof(T) == 4 && NDIM == 2) ? 2 : 1;
+};
+
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// ---------------------------------------------------------------------------------------------
+// Cubic shapes and the momentum-conserving gather.
+// ---------------------------------------------------------------------------------------------
+// Centred B-splines.
+template <typename T>
+__device__ __forceinline__ T bspl(int n, T t) {
+  const T a = t < T(0) ? -t : t;
+  if (n == 0) return (t >= T(-0.5) && t < T(0.5)) ? T(1) : T(0);
+  if (n == 1) return a < T(1) ? T(1) - a : T(0);
+  if (n == 2) {
+    if (a <= T(0.5)) return T(0.75) - a * a;
+    if (a < T(1.5)) return T(0.5) * (T(1.5) - a) * (T(1.5) - a);
+    return T(0);
+  }
+  if (a <= T(1)) return T(2.0 / 3.0) - a * a + T(0.5) * a * a * a;
+  if (a < T(2)) return (T(2) - a) * (T(2) - a) * (T(2) - a) * T(1.0 / 6.0);
+  return T(0);
+}
+
+// S_n(a0 - d) - S_n(a0) for the particle shape (n = 1 or 3): on one polynomial piece from the
+// displacement (linear: slope times -d; cubic: the terminating Taylor series), else the difference.
+template <typename T>
+__device__ __forceinline__ T shape_change(int n, T a0, T d) {
+  const T a1 = a0 - d;
+  if (n == 1) {
+    const int p0 = (a0 > T(-1)) + (a0 > T(0)) + (a0 >= T(1)), p1 = (a1 > T(-1)) + (a1 > T(0)) + (a1 >= T(1));
+    if (p0 == p1) return p0 == 1 ? -d : (p0 == 2 ? d : T(0));
+    return bspl(1, a1) - bspl(1, a0);
+  }
+  const int p0 = (a0 > T(-2)) + (a0 > T(-1)) + (a0 > T(0)) + (a0 > T(1)) + (a0 >= T(2));
+  const int p1 = (a1 > T(-2)) + (a1 > T(-1)) + (a1 > T(0)) + (a1 > T(1)) + (a1 >= T(2));
+  if (p0 != p1) return bspl(3, a1) - bspl(3, a0);
+  T d1, d2, d3;  // P', P'', P''' of the piece at a0
+  switch (p0) {
+    case 1: d1 = T(0.5) * (T(2) + a0) * (T(2) + a0); d2 = T(2) + a0; d3 = T(1); break;
+    case 2: d1 = -T(2) * a0 - T(1.5) * a0 * a0; d2 = -T(2) - T(3) * a0; d3 = T(-3); break;
+    case 3: d1 = -T(2) * a0 + T(1.5) * a0 * a0; d2 = -T(2) + T(3) * a0; d3 = T(3); break;
+    case 4: d1 = -T(0.5) * (T(2) - a0) * (T(2) - a0); d2 = T(2) - a0; d3 = T(-1); break;
+    default: return T(0);
+  }
+  return -d * (d1 - d * (T(0.5) * d2 - d * d3 * T(1.0 / 6.0)));
+}
+
+// Stagger of Ex Ey Ez Bx By Bz along x, y, z (compile-time, so that the gather's orders and loop
+// bounds fold for each unrolled component).
+__host__ __device__ constexpr int stag_ho(int c, int axis) {
+  return axis == 0 ? (c == 0 || c == 4 || c == 5) : (axis == 1 ? (c == 1 || c == 3 || c == 5) : (c == 2 || c == 3 || c == 4));
+}
+
+// One value, or the values of a particle pair in one packed FP32x2 operand.
+template <typename T>
+struct Lanes1 {
+  using V = T;
+  static __device__ __forceinline__ V set(T a) { return a; }
+  static __device__ __forceinline__ V node(const T* p) { return *p; }
+  static __device__ __forceinline__ V fma(V a, V b, V c) { return a * b + c; }
+  static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+  static __device__ __forceinline__ V neg(V a) { return -a; }
+  static __device__ __forceinline__ V pick_low(V a, V lo, V hi) { return a < T(0.5) ? lo : hi; }
+};
+struct Lanes2 {
+  using V = float2;
+  static __device__ __forceinline__ V set(float a) { return make_float2(a, a); }
+  static __device__ __forceinline__ V node(const float* p) { return *reinterpret_cast<const float2*>(p); }
+  static __device__ __forceinline__ V fma(V a, V b, V c) { return __ffma2_rn(a, b, c); }
+  static __device__ __forceinline__ V mul(V a, V b) { return __fmul2_rn(a, b); }
+  static __device__ __forceinline__ V add(V a, V b) { return __fadd2_rn(a, b); }
+  static __device__ __forceinline__ V neg(V a) { return make_float2(-a.x, -a.y); }
+  static __device__ __forceinline__ V pick_low(V a, V lo, V hi) {
+    return make_float2(a.x < 0.5f ? lo.x : hi.x, a.y < 0.5f ? lo.y : hi.y);
+  }
+};
+
+// Weights of the cubic spline on the nodes -1, 0, 1, 2 of the cell for an offset o in [0, 1].
+template <class L, typename T, typename V>
+__device__ __forceinline__ void cubic_weights(V o, V (&w)[4]) {
+  const V p = L::add(L::set(T(1)), L::neg(o));
+  const V o2 = L::mul(o, o), p2 = L::mul(p, p);
+  const V six = L::set(T(1.0 / 6.0)), half = L::set(T(0.5)), two3 = L::set(T(2.0 / 3.0));
+  w[0] = L::mul(L::mul(p2, p), six);
+  w[3] = L::mul(L::mul(o2, o), six);
+  w[1] = L::fma(o2, L::fma(half, o, L::set(T(-1))), two3);  // 2/3 - o^2 + o^3 / 2
+  w[2] = L::fma(p2, L::fma(half, p, L::set(T(-1))), two3);
+}
+
+// Nodes of one direction of the gather: NI integer nodes from FI on, NS half-staggered ones from FS
+// on, relative to the cell. Every particle of a cell reads the same nodes: the Uniform cubic gather on
+// half-staggered nodes takes five, with a zero weight at one end (the range of its four depends on the
+// half of the cell the particle is in).
+template <int ORDER, int SCHEME>
+struct WinNodes {
+  static constexpr int NI = ORDER + 1, FI = -(ORDER - 1) / 2;
+  static constexpr int NS = SCHEME == 0 ? ORDER : ORDER + 2, FS = ORDER == 3 ? (SCHEME == 0 ? -1 : -2) : 0;
+};
+template <class L, typename T, typename V, int ORDER, int SCHEME>
+__device__ __forceinline__ void win_weights(V o, V (&wi)[4], V (&ws)[5]) {
+  if constexpr (ORDER == 1) {
+    wi[0] = L::add(L::set(T(1)), L::neg(o));
+    wi[1] = o;
+  } else {
+    cubic_weights<L, T, V>(o, wi);
+    if constexpr (SCHEME == 0) {  // quadratic spline about the half node: t = o - 1/2
+      const V t = L::add(o, L::set(T(-0.5))), half = L::set(T(0.5));
+      const V q = L::add(half, L::neg(t)), r = L::add(half, t);
+      ws[0] = L::mul(half, L::mul(q, q));
+      ws[1] = L::fma(L::neg(t), t, L::set(T(0.75)));
+      ws[2] = L::mul(half, L::mul(r, r));
+    } else if constexpr (SCHEME == 1) {
+      const V f = L::pick_low(o, L::add(o, L::set(T(0.5))), L::add(o, L::set(T(-0.5))));
+      V c[4];
+      cubic_weights<L, T, V>(f, c);
+      const V z = L::set(T(0));
+      ws[0] = L::pick_low(o, c[0], z);
+      ws[1] = L::pick_low(o, c[1], c[0]);
+      ws[2] = L::pick_low(o, c[2], c[1]);
+      ws[3] = L::pick_low(o, c[3], c[2]);
+      ws[4] = L::pick_low(o, z, c[3]);
+    }
+  }
+}
+
+// Component C of the gather from the window of cell (lx, ly, lz). The momentum-conserving scheme
+// (2) reads integer nodes only: its tile holds the node averages.
+template <class L, typename T, typename V, int NDIM, int ORDER, int SCHEME, int C>
+__device__ __forceinline__ V window_comp(const T* sg, int lx, int ly, int lz, const V (&xi)[4], const V (&xs)[5],
+                                         const V (&yi)[4], const V (&ys)[5], const V (&zi)[4], const V (&zs)[5]) {
+  using S = PushSmem<T, NDIM, ORDER, true>;
+  using W = WinNodes<ORDER, SCHEME>;
+  constexpr bool SX = SCHEME != 2 && stag_ho(C, 0), SY = SCHEME != 2 && stag_ho(C, 1), SZ = SCHEME != 2 && stag_ho(C, 2);
+  constexpr int NX = SX ? W::NS : W::NI, NY = NDIM == 3 ? (SY ? W::NS : W::NI) : 1, NZ = SZ ? W::NS : W::NI;
+  const int ix = lx + S::H + (SX ? W::FS : W::FI), iz = lz + S::H + (SZ ? W::FS : W::FI);
+  const int iy = NDIM == 3 ? ly + S::H + (SY ? W::FS : W::FI) : 0;
+  const T* p = sg + (C * S::GN + (iz * S::GY + iy) * S::GX + ix) * S::GCOPY;
+  V acc = L::set(T(0));
+#pragma unroll
+  for (int c = 0; c < NZ; ++c) {
+    V plane = L::set(T(0));
+#pragma unroll
+    for (int b = 0; b < NY; ++b) {
+      const T* q = p + (c * S::GY + b) * S::GX * S::GCOPY;
+      V row = L::mul(SX ? xs[0] : xi[0], L::node(q));
+#pragma unroll
+      for (int a = 1; a < NX; ++a) row = L::fma(SX ? xs[a] : xi[a < 4 ? a : 3], L::node(q + a * S::GCOPY), row);
+      if (NDIM == 3) plane = L::fma(SY ? ys[b] : yi[b < 4 ? b : 3], row, plane);
+      else plane = row;
+    }
+    acc = L::fma(SZ ? zs[c] : zi[c < 4 ? c : 3], plane, acc);
+  }
+  return acc;
+}
+
+template <class L, typename T, typename V, int NDIM, int ORDER, int SCHEME>
+__device__ __forceinline__ void gather_window(const T* sg, int lx, int ly, int lz, V ox, V oy, V oz, V (&F)[6]) {
+  V xi[4], xs[5], yi[4], ys[5], zi[4], zs[5];
+  win_weights<L, T, V, ORDER, SCHEME>(ox, xi, xs);
+  if (NDIM == 3) win_weights<L, T, V, ORDER, SCHEME>(oy, yi, ys);
+  win_weights<L, T, V, ORDER, SCHEME>(oz, zi, zs);
+  F[0] = window_comp<L, T, V, NDIM, ORDER, SCHEME, 0>(sg, lx, ly, lz, xi, xs, yi, ys, zi, zs);
+  F[1] = window_comp<L, T, V, NDIM, ORDER, SCHEME, 1>(sg, lx, ly, lz, xi, xs, yi, ys, zi, zs);
+  F[2] = window_comp<L, T, V, NDIM, ORDER, SCHEME, 2>(sg, lx, ly, lz, xi, xs, yi, ys, zi, zs);
+  F[3] = window_comp<L, T, V, NDIM, ORDER, SCHEME, 3>(sg, lx, ly, lz, xi, xs, yi, ys, zi, zs);
+  F[4] = window_comp<L, T, V, NDIM, ORDER, SCHEME, 4>(sg, lx, ly, lz, xi, xs, yi, ys, zi, zs);
+  F[5] = window_comp<L, T, V, NDIM, ORDER, SCHEME, 5>(sg, lx, ly, lz, xi, xs, yi, ys, zi, zs);
+}
+
+// The staged copies made ready for gather_window: averaged from the Yee locations to the nodes for
+// the momentum-conserving scheme (node i gets (v[i-1] + v[i]) / 2 along each half-staggered direction, x
+// then y then z), and every node stored twice for a paired push. Each thread holds its results in
+// registers across a barrier, so the tile is rewritten in place. The lowest node along a staggered
+// direction has no neighbour in the tile and keeps its value; no particle of the tile reads it.
+template <typename T, int NDIM, int ORDER, int SCHEME>
+__device__ __forceinline__ void window_nodes(T* sg) {
+  using S = PushSmem<T, NDIM, ORDER, true>;
+  constexpr int NT = PushThreads<T, NDIM, ORDER>::value, NE = (6 * S::GN + NT - 1) / NT;
+  if (SCHEME != 2 && S::GCOPY == 1) return;
+  const int tid = threadIdx.x;
+  T v[NE];
+#pragma unroll
+  for (int m = 0; m < NE; ++m) {
+    const int e = tid + m * NT;
+    v[m] = T(0);
+    if (e >= 6 * S::GN) continue;
+    if (SCHEME != 2) {
+      v[m] = sg[e];
+      continue;
+    }
+    const int c = e / S::GN, rem = e - c * S::GN;
+    const int lz = rem / (S::GX * S::GY), ly = (rem / S::GX) % S::GY, lx = rem % S::GX;
+    const int sx = stag_ho(c, 0) && lx > 0 ? 1 : 0;
+    const int sy = NDIM == 3 && stag_ho(c, 1) && ly > 0 ? S::GX : 0;
+    const int sz = stag_ho(c, 2) && lz > 0 ? S::GX * S::GY : 0;
+    const T* p = sg + e;
+    auto ax = [&](const T* q) { return sx ? T(0.5) * (q[0] + q[-sx]) : q[0]; };
+    auto ay = [&](const T* q) { return sy ? T(0.5) * (ax(q) + ax(q - sy)) : ax(q); };
+    v[m] = sz ? T(0.5) * (ay(p) + ay(p - sz)) : ay(p);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < NE; ++m) {
+    const int e = tid + m * NT;
+    if (e >= 6 * S::GN) continue;
+    sg[e * S::GCOPY] = v[m];
+    if (S::GCOPY == 2) sg[e * 2 + 1] = v[m];
+  }
+  __syncthreads();
+}
+
+// One direction of a cubic Esirkepov move: S0 + dS / 2 and the shape change dS on the nodes -1 .. 3 of
+// the start cell for a move d that stays in the cell or enters the next one up (`up`, at offset c
+// there), formed from the displacement itself on one polynomial piece (full relative precision for small
+// moves) and as the difference across the face.
+template <typename T>
+struct CubicDir {
+  T m[5], dS[5];
+};
+template <typename T>
+__device__ __forceinline__ CubicDir<T> cubic_dir(T o, T d, bool up, T c) {
+  CubicDir<T> r;
+  T s[4];
+  cubic_weights<Lanes1<T>, T, T>(o, s);
+  const T p = T(1) - o, d2 = d * d, d6 = d * T(1.0 / 6.0);
+  T e0 = -d6 * (T(3) * p * (p - d) + d2);
+  T e3 = d6 * (T(3) * o * (o + d) + d2);
+  T e1 = d * (T(1.5) * o * (o + d) - T(2) * o - d + T(0.5) * d2);
+  T e2 = -(e0 + e1 + e3), e4 = T(0);
+  if (up) {
+    T n[4];
+    cubic_weights<Lanes1<T>, T, T>(c, n);
+    e0 = -s[0];
+    e1 = n[0] - s[1];
+    e2 = n[1] - s[2];
+    e3 = n[2] - s[3];
+    e4 = n[3];
+  }
+  r.dS[0] = e0; r.dS[1] = e1; r.dS[2] = e2; r.dS[3] = e3; r.dS[4] = e4;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) r.m[a] = s[a] + T(0.5) * r.dS[a];
+  r.m[4] = T(0.5) * e4;
+  return r;
+}
+// running sums of dS, the weights of the current on the four edges (all five dS sum to zero)
+template <typename T>
+__device__ __forceinline__ void cubic_run(const CubicDir<T>& r, T (&P)[4]) {
+  P[0] = r.dS[0];
+  P[1] = r.dS[0] + r.dS[1];
+  P[2] = -(r.dS[3] + r.dS[4]);
+  P[3] = -r.dS[4];
+}
+
+// 2D cubic deposit into the register layout: x stays in its cell, z stays or steps up.
+template <typename T, int NVP>
+__device__ __forceinline__ void deposit2_cubic(T (&acc)[NVP], const CubicDir<T>& X, const CubicDir<T>& Z, T cx, T cy,
+                                               T cz) {
+  T PX[4], PZ[4];
+  cubic_run(X, PX);
+  cubic_run(Z, PZ);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const T g = cx * PX[a];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) acc[c * 3 + a] += g * Z.m[c];
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const T g = cz * PZ[c];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) acc[15 + a * 4 + c] += g * X.m[a];
+  }
+  const T k = cy * T(1.0 / 12.0);
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const T h = cy * X.m[a], q = k * X.dS[a];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) acc[31 + c * 4 + a] += h * Z.m[c] + q * Z.dS[c];
+  }
+}
+
+// Any cubic move of less than a cell, straight into the tile's current: the window nodes -2 .. 3 of
+// the start cell. The rare particles that step back or cross a transverse face take this path.
+template <typename T, int NDIM>
+__device__ __noinline__ void deposit_general(T* sj, int lx, int ly, int lz, T ox, T oy, T oz, T dx, T dy, T dz, T cx,
+                                             T cy, T cz) {
+  using S = PushSmem<T, NDIM, 3, true>;
+  constexpr int NW = 6;
+  T Tx[NW], Ty[NW], Tz[NW], ex[NW], ey[NW], ez[NW];
+#pragma unroll 1
+  for (int a = 0; a < NW; ++a) {
+    const T node = T(a - 2);
+    ex[a] = shape_change(3, node - ox, dx);
+    Tx[a] = bspl(3, node - ox) + T(0.5) * ex[a];
+    ez[a] = shape_change(3, node - oz, dz);
+    Tz[a] = bspl(3, node - oz) + T(0.5) * ez[a];
+    ey[a] = NDIM == 3 ? shape_change(3, node - oy, dy) : T(0);
+    Ty[a] = NDIM == 3 ? bspl(3, node - oy) + T(0.5) * ey[a] : T(0);
+  }
+  // window node 0 (two below the cell) is current-tile index (lx, ly, lz)
+  T* w0 = sj + (lz * S::JY + (NDIM == 3 ? ly : 0)) * S::JX + lx;
+  if (NDIM == 2) {
+#pragma unroll 1
+    for (int b = 0; b < NW; ++b) {
+      T px = T(0), pz = T(0);
+#pragma unroll 1
+      for (int a = 0; a < NW; ++a) {
+        px += ex[a];  // the last running sum closes to zero
+        pz += ez[a];
+        if (a < NW - 1) {
+          const T vx = cx * px * Tz[b], vz = cz * pz * Tx[b];
+          if (vx != T(0)) atomicAdd(w0 + b * S::JX + a, vx);
+          if (vz != T(0)) atomicAdd(w0 + 2 * S::JN + a * S::JX + b, vz);
+        }
+        const T vy = cy * (Tx[a] * Tz[b] + ex[a] * ez[b] * T(1.0 / 12.0));
+        if (vy != T(0)) atomicAdd(w0 + S::JN + b * S::JX + a, vy);
+      }
+    }
+    return;
+  }
+#pragma unroll 1
+  for (int t2 = 0; t2 < NW; ++t2)
+#pragma unroll 1
+    for (int t1 = 0; t1 < NW; ++t1) {
+      const T gx = Ty[t1] * Tz[t2] + ey[t1] * ez[t2] * T(1.0 / 12.0);  // Jx: (y, z) = (t1, t2)
+      const T gy = Tx[t1] * Tz[t2] + ex[t1] * ez[t2] * T(1.0 / 12.0);  // Jy: (x, z) = (t1, t2)
+      const T gz = Tx[t1] * Ty[t2] + ex[t1] * ey[t2] * T(1.0 / 12.0);  // Jz: (x, y) = (t1, t2)
+      T px = T(0), py = T(0), pz = T(0);
+#pragma unroll 1
+      for (int a = 0; a < NW - 1; ++a) {
+        px += ex[a];
+        py += ey[a];
+        pz += ez[a];
+        const T vx = cx * px * gx, vy = cy * py * gy, vz = cz * pz * gz;
+        if (vx != T(0)) atomicAdd(w0 + (t2 * S::JY + t1) * S::JX + a, vx);
+        if (vy != T(0)) atomicAdd(w0 + S::JN + (t2 * S::JY + a) * S::JX + t1, vy);
+        if (vz != T(0)) atomicAdd(w0 + 2 * S::JN + (a * S::JY + t2) * S::JX + t1, vz);
+      }
+    }
+}
+
+// 3D cubic deposit of one item and one component (0 Jx, 1 Jy, 2 Jz). The window of all components has 184
+// sums, more than a thread can hold beside the push, so the push leaves each particle's offsets,
+// displacements and charge (zero: nothing to add) in its stage slot and the three components are summed
+// one after another, 60 to 64 sums at a time, over the lane's particles of the item, then over the
+// cell's lanes. Positions: x and y stay in their cell, z stays or steps up. Layouts: Jx (c*4 + b)*3 + a,
+// Jy (c*4 + a)*3 + b, Jz (b*4 + a)*4 + c, on nodes from one below the cell (origin `j`).
+template <typename T, int LPC, int COMP>
+__device__ __forceinline__ void deposit3_cubic(const T* st, int sl, int nrnd, int rnd0, T coef, T* j) {
+  using S = PushSmem<T, 3, 3, true>;
+  constexpr int NV = COMP == 2 ? 64 : 60, PER = (NV + LPC - 1) / LPC, NVP = PER * LPC;
+  const int lane = threadIdx.x & 31;
+  T acc[NVP];
+#pragma unroll
+  for (int i = 0; i < NVP; ++i) acc[i] = T(0);
+#pragma unroll 1
+  for (int rnd = 0; rnd < nrnd; ++rnd) {
+    const T* q = st + sl + LPC * ((rnd + rnd0) & 3);
+    const T ox = q[0], oy = q[128], oz = q[256], dx = q[384], dy = q[512], dz = q[640], qw = coef * q[768];
+    const T c = dz - (T(1) - oz);
+    const CubicDir<T> X = cubic_dir(ox, dx, false, T(0)), Y = cubic_dir(oy, dy, false, T(0));
+    const CubicDir<T> Z = cubic_dir(oz, dz, ge_one(oz + dz) && is_pos(c), c);
+    const CubicDir<T>& A = COMP == 0 ? X : (COMP == 1 ? Y : Z);  // along the component
+    const CubicDir<T>& B = COMP == 0 ? Y : X;                    // the fast transverse direction
+    const CubicDir<T>& C = COMP == 2 ? Y : Z;                    // the slow one (Z: five nodes)
+    constexpr int NA = COMP == 2 ? 4 : 3, NC = COMP == 2 ? 4 : 5;
+    T P[4];
+    cubic_run(A, P);
+#pragma unroll
+    for (int a = 0; a < NA; ++a) P[a] *= qw;
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const T t = B.m[b] * C.m[k] + B.dS[b] * T(1.0 / 12.0) * C.dS[k];
+#pragma unroll
+        for (int a = 0; a < NA; ++a) acc[(k * 4 + b) * NA + a] += P[a] * t;
+      }
+  }
+#pragma unroll
+  for (int sh = LPC / 2; sh >= 1; sh >>= 1) {
+    const bool up = (lane & sh) != 0;
+#pragma unroll
+    for (int i = 0; i < PER * sh; ++i) {
+      const T send = up ? acc[i] : acc[i + PER * sh];
+      const T keep = up ? acc[i + PER * sh] : acc[i];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, sh);
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < PER; ++m) {
+    const int i = sl * PER + m;
+    if (i >= NV || acc[m] == T(0)) continue;
+    int a, b, c;
+    if (COMP == 2) { c = i & 3; a = (i >> 2) & 3; b = i >> 4; }
+    else if (COMP == 1) { const int k = i / 3; b = i - 3 * k; a = k & 3; c = k >> 2; }
+    else { const int k = i / 3; a = i - 3 * k; b = k & 3; c = k >> 2; }
+    atomicAdd(j + COMP * S::JN + (c * S::JY + b) * S::JX + a, acc[m]);
+  }
+}
+
+// Reciprocal square root of the window gathers' push: FP32 refined by one Newton step (as accurate as
+// the quotient 1 / sqrt), FP64 as fast_rsqrt.
+__device__ __forceinline__ double fine_rsqrt(double x) { return fast_rsqrt(x); }
+__device__ __forceinline__ float fine_rsqrt(float x) {
+  const float y = rsqrtf(x);
+  return fmaf(fmaf(-0.5f * x * y, y, 0.5f), y, y);
+}
+
+template <typename T, int NDIM, int SCHEME, int LPC, int ORDER = 1>
+__device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
+  constexpr bool WIN = ORDER == 3 || SCHEME == 2;    // the gather reads the cell's window of nodes
+  constexpr bool LATE = NDIM == 3 && ORDER == 3;     // the deposit follows the push of each item
+  using S = PushSmem<T, NDIM, ORDER, WIN>;
+  using PL = PushPlan<NDIM, LPC, ORDER>;
+  constexpr int TX = S::TX, TY = S::TY, NCL = S::NCL;
+  constexpr int NV = PL::NV, PER = PL::PER, NVP = PL::NVP, CPW = PL::CPW;
+  constexpr int PUSH_THREADS = PushThreads<T, NDIM, ORDER>::value, NWARP = PUSH_THREADS / 32;
+  static_assert(NCL % CPW == 0, "cells per tile must be a multiple of the cells per warp");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* sg = reinterpret_cast<T*>(smem_raw);
+  T* sj = sg + 6 * S::GN * S::GCOPY;
+  int* sn = reinterpret_cast<int*>(sj + 3 * S::JN);  // [species][cell] particle counts (input)
+  int* scnt = sn + 2 * NCL;                          // [species][cell] output counts of this tile
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // per-warp stages start on a 16-byte boundary after the counts (cp.async destinations)
+  const size_t stage_off = ((size_t)(reinterpret_cast<unsigned char*>(scnt + 2 * NCL) - smem_raw) + 15) & ~(size_t)15;
+  using SG = PushStage<T, NDIM>;
+  T* stg = reinterpret_cast<T*>(smem_raw + stage_off) + (size_t)warp * SG::per_warp_elems();
+  // the tile's leaver buffer follows every warp's stage
+  const size_t lv_off = (stage_off + sizeof(T) * SG::per_warp_elems() * NWARP + 15) & ~(size_t)15;
+  T* lvv = reinterpret_cast<T*>(smem_raw + lv_off);
+  int* lvk = reinterpret_cast<int*>(lvv + 7 * S::LVB);
+  unsigned* lvi = reinterpret_cast<unsigned*>(lvk + S::LVB);
+  int* lvn = reinterpret_cast<int*>(lvi + S::LVB);
+  const int tix = tile % r.ntx;
+  const int tiy = (tile / r.ntx) % r.nty;
+  const int tiz = tile / (r.ntx * r.nty);
+  // the run's tile extents (r.tex <= TX ...): cells past them stay empty, as at the grid's edge
+  const int X0 = tix * r.tex, Y0 = tiy * r.tey, Z0 = tiz * r.tez;
+  const int wx = min(r.tex, r.nx - X0), wy = min(r.tey, r.ny - Y0), wz = min(r.tez, r.nz - Z0);
+  const long long nxy = (long long)r.nx * r.ny;
+
+  const bool has_w = r.in[0].w != nullptr;
+  const bool has_id = r.in[0].id != nullptr;
+  const int sl = lane % LPC;  // lane within its cell group
+
+  // 1. field copies of the tile and its halo into shared memory (periodic wrap); zero the current
+  const bool near_ok = r.nx >= S::GX && r.nz >= S::GZ && (NDIM == 2 || r.ny >= S::GY);
+  for (int e = tid; e < 6 * S::GN; e += PUSH_THREADS) {
+    int c = e / S::GN, rem = e - c * S::GN;
+    int lz = rem / (S::GX * S::GY);
+    int ly = (rem / S::GX) % S::GY;
+    int lx = rem % S::GX;
+    // tile + halo lies within one period of the grid when the grid is at least as wide
+    int gx = near_ok ? wrap_near_p(X0 - S::H + lx, r.nx) : wrapi(X0 - S::H + lx, r.nx);
+    int gy = NDIM == 3 ? (near_ok ? wrap_near_p(Y0 - S::H + ly, r.ny) : wrapi(Y0 - S::H + ly, r.ny)) : 0;
+    int gz = near_ok ? wrap_near_p(Z0 - S::H + lz, r.nz) : wrapi(Z0 - S::H + lz, r.nz);
+    const T* src = r.g[0];
+    switch (c) {  // constant-indexed parameter reads (no local copy of r.g)
+      case 1: src = r.g[1]; break;
+      case 2: src = r.g[2]; break;
+      case 3: src = r.g[3]; break;
+      case 4: src = r.g[4]; break;
+      case 5: src = r.g[5]; break;
+      default: break;
+    }
+    copy1_async(sg + e, src + (long long)gz * nxy + (long long)gy * r.nx + gx);
+  }
+  for (int e = tid; e < 3 * S::JN; e += PUSH_THREADS) sj[e] = T(0);
+  // 2. particle counts of the tile's cells, copied in the same asynchronous batch as the fields (one
+  // global round trip for both); then clamped, and the input counts zeroed (they are the next
+  // step's output counts). Each thread reads back only the counts it copied itself.
+  for (int cl = tid; cl < NCL; cl += PUSH_THREADS) {
+    const int lx = cl % TX, ly = (cl / TX) % TY, lz = cl / (TX * TY);
+    if (lx < wx && ly < wy && lz < wz) {
+      const long long cell = (long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx;
+      copy1_async(sn + cl, r.in[0].cnt + cell);
+      copy1_async(sn + NCL + cl, r.in[1].cnt + cell);
+    } else {
+      sn[cl] = 0;
+      sn[NCL + cl] = 0;
+    }
+    scnt[cl] = 0;
+    scnt[NCL + cl] = 0;
+  }
+  // The first item of the warp's first cell group, in the same batch although the counts are not in
+  // yet: lane sl takes pack sl of species 0, as it does whenever its cell holds more than 4 sl
+  // particles of species 0 (slots below cap: inside the cell's own bin). A lane whose first pack is
+  // of species 1 copies it again once the counts are known.
+  {
+    const int c = warp * CPW + lane / LPC;  // every warp has a first group (NCL / CPW >= NWARP)
+    const int lx = c % TX, ly = (c / TX) % TY, lz = c / (TX * TY);
+    if (lx < wx && ly < wy && lz < wz && 4 * sl + 4 <= r.cap) {
+      const long long slot0 =
+          ((long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx) * r.cap + 4 * sl;
+      const SpeciesBuf<T>& pin = r.in[0];
+      const T* src[7] = {pin.ox, pin.oy, pin.oz, pin.dux, pin.duy, pin.duz, pin.w};
+#pragma unroll
+      for (int arr = 0; arr < 7; ++arr) {
+        if (arr == 1 && NDIM == 2) continue;
+        if (arr == 6 && !has_w) continue;
+        copy4_async(SG::at(stg, 0, arr, lane), src[arr] + slot0);
+      }
+      if (has_id) copy4_async(SG::id_at(stg, 0, lane), pin.id + slot0);
+    }
+  }
+  static_assert(NCL / CPW >= NWARP, "every warp needs a first cell group");
+  cp_async_commit();
+  cp_async_wait_all();
+  for (int cl = tid; cl < NCL; cl += PUSH_THREADS) {
+    const int lx = cl % TX, ly = (cl / TX) % TY, lz = cl / (TX * TY);
+    if (lx < wx && ly < wy && lz < wz) {
+      const long long cell = (long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx;
+      sn[cl] = min(sn[cl], r.cap);  // the excess of a full bin waits in the spill list
+      sn[NCL + cl] = min(sn[NCL + cl], r.cap);
+      r.in[0].cnt[cell] = 0;
+      r.in[1].cnt[cell] = 0;
+    }
+  }
+  // cell groups after each warp's first one are handed out in the order warps ask for them, so
+  // warps whose groups hold more packs do fewer groups
+  __shared__ int s_next_group;
+  if (tid == 0) {
+    *lvn = 0;
+    s_next_group = PUSH_THREADS / 32;
+  }
+  __syncthreads();
+  if constexpr (WIN) window_nodes<T, NDIM, ORDER, SCHEME>(sg);
+
+  T kin = T(0);
+  int npush = 0;
+
+  // Items of this warp: (cell group, pack round). The packs of the next item are copied into the
+  // warp's shared-memory stage with cp.async while the current item is computed.
+  constexpr int NGRP = NCL / CPW;
+  auto group_iters = [&](int g) -> int {
+    const int c = g * CPW + lane / LPC;
+    const int nq = ((sn[c] + 3) >> 2) + ((sn[NCL + c] + 3) >> 2);
+    return __reduce_max_sync(0xffffffffu, (nq + LPC - 1) / LPC);
+  };
+  // fix: only the packs the speculative first copy did not cover (species 1, or slots past cap)
+  auto issue = [&](int g, int it, int stage, bool fix) {
+    const int c = g * CPW + lane / LPC;
+    const int n0 = sn[c], n1 = sn[NCL + c];
+    const int nq0 = (n0 + 3) >> 2, nq = nq0 + ((n1 + 3) >> 2);
+    const int q = sl + it * LPC;
+    if (q >= nq) return;
+    const int s = q >= nq0 ? 1 : 0;
+    const int q4 = 4 * (s ? q - nq0 : q);
+    if (fix && s == 0 && q4 + 4 <= r.cap) return;
+    const int lx = c % TX, ly = (c / TX) % TY, lz = c / (TX * TY);
+    const long long slot0 = ((long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx) * r.cap + q4;
+    const SpeciesBuf<T> pin = s ? r.in[1] : r.in[0];
+    const T* src[7] = {pin.ox, pin.oy, pin.oz, pin.dux, pin.duy, pin.duz, pin.w};
+#pragma unroll
+    for (int arr = 0; arr < 7; ++arr) {
+      if (arr == 1 && NDIM == 2) continue;
+      if (arr == 6 && !has_w) continue;
+      copy4_async(SG::at(stg, stage, arr, lane), src[arr] + slot0);
+    }
+    if (has_id) copy4_async(SG::id_at(stg, stage, lane), pin.id + slot0);
+  };
+
+  auto take_group = [&]() -> int {
+    int v = 0;
+    if (lane == 0) v = atomicAdd(&s_next_group, 1);
+    return __shfl_sync(0xffffffffu, v, 0);
+  };
+  int g = warp, it = 0;
+  int giters = g < NGRP ? group_iters(g) : 0;
+  while (g < NGRP && giters == 0) {
+    g = take_group();
+    giters = g < NGRP ? group_iters(g) : 0;
+  }
+  int stage = 0;
+  if (g < NGRP) issue(g, 0, 0, g == warp);  // the first group's first item was copied speculatively
+  cp_async_commit();
+  T acc[NVP];
+  GalCache<T, NDIM> gc;  // Galerkin nodes of the lane's cell, loaded once per cell group
+  while (g < NGRP) {
+    // prefetch the next item
+    int ng = g, nit = it + 1, niters = giters;
+    if (nit >= giters) {
+      nit = 0;
+      do {
+        ng = take_group();
+        niters = ng < NGRP ? group_iters(ng) : 0;
+      } while (ng < NGRP && niters == 0);
+    }
+    if (ng < NGRP) issue(ng, nit, stage ^ 1, false);
+    cp_async_commit();
+    cp_async_wait_1();
+    __syncwarp();
+
+    const int cl = g * CPW + lane / LPC;
+    const int lx = cl % TX, ly = (cl / TX) % TY, lz = cl / (TX * TY);
+    const int gi = X0 + lx, gj = Y0 + ly, gk = Z0 + lz;
+    const int n0 = sn[cl], n1 = sn[NCL + cl];
+    const int nq0 = (n0 + 3) >> 2, nq = nq0 + ((n1 + 3) >> 2);
+    const int okey = ((lz + 1) * S::JY + (NDIM == 3 ? ly + 1 : 0)) * S::JX + lx + 1;  // cell-origin window
+    if (it == 0) {
+      if (SCHEME == 0 && !WIN) gc.load(sg, lx, ly, lz);
+#pragma unroll
+      for (int i = 0; i < NVP; ++i) acc[i] = T(0);
+    }
+    // rounds of this item: up to the last slot in use of the fullest cell
+    constexpr int NR = PushRounds<T, NDIM>::value, U = 4 / NR;
+    int nk = 4 * (nq - it * LPC);  // slots of the cell's packs from this item on, then the last pack's empty ones
+    if (nk > 0 && nk <= 4 * LPC) nk -= 4 * (nq > nq0 ? nq - nq0 : nq0) - (nq > nq0 ? n1 : n0);
+    const int nrnd = min(NR, (__reduce_max_sync(0xffffffffu, nk) + U * LPC - 1) / (U * LPC));
+    const int rnd0 = nrnd == NR ? PL::template first_round<T>(lane / LPC) : 0;
+#pragma unroll 1
+    for (int rnd = 0; rnd < nrnd; ++rnd) {
+      // the lane's slots k .. k + U - 1 of the cell's 4 LPC slots in this item
+      const int k = U * (sl + LPC * ((rnd + rnd0) & (NR - 1)));
+      const int q = it * LPC + (k >> 2);
+      const bool has = q < nq;
+      const int s = (has && q >= nq0) ? 1 : 0;
+      const int cnt = has ? (s ? n1 + 4 * nq0 : n0) - 4 * q - (k & 3) : 0;  // particles from slot k on
+      const SpeciesBuf<T> pout = s ? r.out[1] : r.out[0];
+      const T qs = s ? T(1) : T(-1);
+      const T* st_x = SG::at(stg, stage, 0, lane - sl) + k;  // array a of slot k at st_x + slot(a) * 128
+      const unsigned* st_id = SG::id_at(stg, stage, lane - sl) + k;
+      if constexpr (PushPaired<T, NDIM>::value) {
+        const float2 hh = make_float2(qs * r.hq, qs * r.hq);
+        const float2 u02 = make_float2(r.u0, r.u0), one2 = make_float2(1.f, 1.f);
+        const float2 dtdx2 = make_float2(r.dtdx, r.dtdx), dtdz2 = make_float2(r.dtdz, r.dtdz);
+        const unsigned lt = (1u << lane) - 1u;
+        {
+          constexpr int ja = 0, jb = 1;  // the pair: one 8-byte load per array
+          const bool va = cnt > 0, vb = cnt > 1;
+          const float2 pox = *reinterpret_cast<const float2*>(st_x + ja);
+          const float2 poz = *reinterpret_cast<const float2*>(st_x + SG::slot(2) * 128 + ja);
+          const float2 pux = *reinterpret_cast<const float2*>(st_x + SG::slot(3) * 128 + ja);
+          const float2 puy = *reinterpret_cast<const float2*>(st_x + SG::slot(4) * 128 + ja);
+          const float2 puz = *reinterpret_cast<const float2*>(st_x + SG::slot(5) * 128 + ja);
+          // an empty slot stands in as a particle at rest with no weight (finite, deposits nothing)
+          const float oxa = va ? pox.x : 0.5f, oza = va ? poz.x : 0.5f;
+          const float uxa = va ? pux.x : 0.f, uya = va ? puy.x : 0.f, uza = va ? puz.x : 0.f;
+          const float oxb = vb ? pox.y : 0.5f, ozb = vb ? poz.y : 0.5f;
+          const float uxb = vb ? pux.y : 0.f, uyb = vb ? puy.y : 0.f, uzb = vb ? puz.y : 0.f;
+          float wa = 0.f, wb = 0.f;
+          if (has_w) {
+            const float2 pw = *reinterpret_cast<const float2*>(st_x + SG::slot(6) * 128 + ja);
+            wa = va ? pw.x : 0.f;
+            wb = vb ? pw.y : 0.f;
+          } else {
+            wa = va ? r.wconst : 0.f;
+            wb = vb ? r.wconst : 0.f;
+          }
+          // gather
+          float2 F2[6];
+          float Fa[6], Fb[6];
+          if constexpr (WIN) {
+            gather_window<Lanes2, float, float2, 2, ORDER, SCHEME>(sg, lx, 0, lz, make_float2(oxa, oxb), make_float2(0.f, 0.f),
+                                                                   make_float2(oza, ozb), F2);
+          } else if (SCHEME == 0) {
+            gc.interp(oxa, 0.f, oza, Fa);
+            gc.interp(oxb, 0.f, ozb, Fb);
+          } else {
+            const DirW<float> xa = dir_weights(oxa), za = dir_weights(oza), xb = dir_weights(oxb),
+                              zb = dir_weights(ozb), y0 = dir_weights(0.f);
+#pragma unroll
+            for (int c = 0; c < 6; ++c) {
+              Fa[c] = gather_comp<float, 2, SCHEME>(sg + c * S::GN, c, lx, 0, lz, xa, y0, za);
+              Fb[c] = gather_comp<float, 2, SCHEME>(sg + c * S::GN, c, lx, 0, lz, xb, y0, zb);
+            }
+          }
+          if constexpr (!WIN) {
+#pragma unroll
+            for (int c = 0; c < 6; ++c) F2[c] = make_float2(Fa[c], Fb[c]);
+          }
+          const float2 Ex = F2[0], Ey = F2[1], Ez = F2[2], Bx = F2[3], By = F2[4], Bz = F2[5];
+          // relativistic Boris of the pair, momenta relative to the drift u0 z_hat
+          const float2 mx = fma2(hh, Ex, make_float2(uxa, uxb));
+          const float2 my = fma2(hh, Ey, make_float2(uya, uyb));
+          const float2 mz = fma2(hh, Ez, make_float2(uza, uzb));
+          const float2 Mz = add2(u02, mz);
+          float2 m2 = fma2(mx, mx, one2);
+          m2 = fma2(my, my, m2);
+          m2 = fma2(Mz, Mz, m2);
+          const float2 hig = mul2(hh, WIN ? make_float2(fine_rsqrt(m2.x), fine_rsqrt(m2.y))
+                                       : make_float2(fast_rsqrt(m2.x), fast_rsqrt(m2.y)));
+          const float2 tx = mul2(hig, Bx), ty = mul2(hig, By), tz = mul2(hig, Bz);
+          float2 t2 = fma2(tx, tx, one2);
+          t2 = fma2(ty, ty, t2);
+          t2 = fma2(tz, tz, t2);
+          const float2 sf = make_float2(fast_div(2.f, t2.x), fast_div(2.f, t2.y));
+          const float2 sx = mul2(sf, tx), sy = mul2(sf, ty), sz = mul2(sf, tz);
+          const float2 qx = fma2(my, tz, fma2(neg2(Mz), ty, mx));
+          const float2 qy = fma2(Mz, tx, fma2(neg2(mx), tz, my));
+          const float2 qz = fma2(mx, ty, fma2(neg2(my), tx, Mz));
+          const float2 ux2 = fma2(qy, sz, fma2(neg2(qz), sy, fma2(hh, Ex, mx)));
+          const float2 uy2 = fma2(qz, sx, fma2(neg2(qx), sz, fma2(hh, Ey, my)));
+          const float2 uz2 = fma2(qx, sy, fma2(neg2(qy), sx, fma2(hh, Ez, mz)));
+          const float2 Uz = add2(u02, uz2);
+          float2 u2 = mul2(ux2, ux2);
+          u2 = fma2(uy2, uy2, u2);
+          u2 = fma2(Uz, Uz, u2);
+          const float2 gp = add2(one2, u2);
+          const float2 ign = WIN ? make_float2(fine_rsqrt(gp.x), fine_rsqrt(gp.y))
+                                 : make_float2(fast_rsqrt(gp.x), fast_rsqrt(gp.y));
+          const float2 g1 = fma2(gp, ign, one2);  // gamma + 1; gamma - 1 = u^2 / (gamma + 1)
+          kin = fmaf(wa, fast_div(u2.x, g1.x), kin);
+          kin = fmaf(wb, fast_div(u2.y, g1.y), kin);
+          npush += (va ? 1 : 0) + (vb ? 1 : 0);
+          const float2 vy2 = mul2(uy2, ign);
+          const float2 ddx2 = mul2(dtdx2, mul2(ux2, ign)), ddz2 = mul2(dtdz2, mul2(Uz, ign));
+          float dxa = ddx2.x, dza = ddz2.x, dxb = ddx2.y, dzb = ddz2.y;
+          float nuxa = ux2.x, nuya = uy2.x, nuza = uz2.x, vya = vy2.x;
+          float nuxb = ux2.y, nuyb = uy2.y, nuzb = uz2.y, vyb = vy2.y;
+          if (!(dxa > -1.f && dxa < 1.f && dza > -1.f && dza < 1.f)) {
+            flag_error(r.err, ERR_NONFINITE);
+            dxa = dza = nuxa = nuya = nuza = vya = 0.f;
+          }
+          if (!(dxb > -1.f && dxb < 1.f && dzb > -1.f && dzb < 1.f)) {
+            flag_error(r.err, ERR_NONFINITE);
+            dxb = dzb = nuxb = nuyb = nuzb = vyb = 0.f;
+          }
+          // Esirkepov deposits
+          const EsirDir<float> exa = esir_dir(oxa, dxa), eza = esir_dir(oza, dza);
+          const EsirDir<float> exb = esir_dir(oxb, dxb), ezb = esir_dir(ozb, dzb);
+          if (va) {
+            const float qw = qs * wa;
+            const float cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vya * r.jfy2d;
+            if constexpr (ORDER == 3) {
+              if (reg_window<float, 2>(exa, exa, eza))
+                deposit2_cubic<float, NVP>(acc, cubic_dir(oxa, dxa, false, 0.f),
+                                           cubic_dir(oza, dza, eza.dS[2] != 0.f, eza.off), cx, cy, cz);
+              else deposit_general<float, 2>(sj, lx, 0, lz, oxa, 0.f, oza, dxa, 0.f, dza, cx, cy, cz);
+            } else if (reg_window<float, 2>(exa, exa, eza)) deposit2_reg<float, NVP>(acc, exa, eza, cx, cy, cz);
+            else deposit2_smem<float, NDIM>(sj, lx + exa.a + 1, lz + eza.a + 1, exa, eza, cx, cy, cz);
+          }
+          if (vb) {
+            const float qw = qs * wb;
+            const float cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vyb * r.jfy2d;
+            if constexpr (ORDER == 3) {
+              if (reg_window<float, 2>(exb, exb, ezb))
+                deposit2_cubic<float, NVP>(acc, cubic_dir(oxb, dxb, false, 0.f),
+                                           cubic_dir(ozb, dzb, ezb.dS[2] != 0.f, ezb.off), cx, cy, cz);
+              else deposit_general<float, 2>(sj, lx, 0, lz, oxb, 0.f, ozb, dxb, 0.f, dzb, cx, cy, cz);
+            } else if (reg_window<float, 2>(exb, exb, ezb)) deposit2_reg<float, NVP>(acc, exb, ezb, cx, cy, cz);
+            else deposit2_smem<float, NDIM>(sj, lx + exb.a + 1, lz + ezb.a + 1, exb, ezb, cx, cy, cz);
+          }
+          // destinations: a cell of this tile (key (cell * 2 + species) in the tile) or, leaving
+          // the tile, the global cell (key global cell * 2 + species)
+          int dka = -1 - lane, dkb = -1 - lane;
+          bool lva = false, lvb = false;
+          if (va) {
+            const int nlx = lx + exa.shift, nlz = lz + eza.shift;
+            if (nlx >= 0 && nlx < wx && nlz >= 0 && nlz < wz) {
+              dka = (nlz * TX + nlx) * 2 + s;
+            } else {
+              lva = true;
+              dka = (wrap_near_p(gk + eza.shift, r.nz) * r.nx + wrap_near_p(gi + exa.shift, r.nx)) * 2 + s;
+            }
+          }
+          if (vb) {
+            const int nlx = lx + exb.shift, nlz = lz + ezb.shift;
+            if (nlx >= 0 && nlx < wx && nlz >= 0 && nlz < wz) {
+              dkb = (nlz * TX + nlx) * 2 + s;
+            } else {
+              lvb = true;
+              dkb = (wrap_near_p(gk + ezb.shift, r.nz) * r.nx + wrap_near_p(gi + exb.shift, r.nx)) * 2 + s;
+            }
+          }
+          // rebin of the pair: consecutive slots per (destination, species) for each particle of the
+          // pair, the two reservations interleaved
+          const bool sta = va && !lva, stb = vb && !lvb;
+          const unsigned pa = __match_any_sync(0xffffffffu, sta ? dka : -1 - lane);
+          const unsigned pb = __match_any_sync(0xffffffffu, stb ? dkb : -1 - lane);
+          const int lda = __ffs(pa) - 1, ldb = __ffs(pb) - 1;
+          int ba = 0, bb = 0;
+          if (sta && lane == lda) ba = atomicAdd(scnt + (dka & 1) * NCL + (dka >> 1), __popc(pa));
+          if (stb && lane == ldb) bb = atomicAdd(scnt + (dkb & 1) * NCL + (dkb >> 1), __popc(pb));
+          ba = __shfl_sync(0xffffffffu, ba, lda) + __popc(pa & lt);
+          bb = __shfl_sync(0xffffffffu, bb, ldb) + __popc(pb & lt);
+          const bool fa = sta && ba >= r.cap, fb = stb && bb >= r.cap;  // full bins: on to k_migrate
+          // leavers: the tile's shared buffer (one reservation for the pair), then the global list
+          // for full bins and once the shared buffer is full
+          const unsigned lma = __ballot_sync(0xffffffffu, lva), lmb = __ballot_sync(0xffffffffu, lvb);
+          int lsa = 0, lsb = 0;
+          if (lma | lmb) {
+            int b0 = 0;
+            if (lane == 0) b0 = atomicAdd(lvn, __popc(lma) + __popc(lmb));
+            b0 = __shfl_sync(0xffffffffu, b0, 0);
+            lsa = b0 + __popc(lma & lt);
+            lsb = b0 + __popc(lma) + __popc(lmb & lt);
+          }
+          const bool ga = fa || (lva && lsa >= S::LVB), gb = fb || (lvb && lsb >= S::LVB);
+          const unsigned gma = __ballot_sync(0xffffffffu, ga), gmb = __ballot_sync(0xffffffffu, gb);
+          long long goa = 0, gob = 0;
+          if (gma | gmb) {
+            int b0 = 0;
+            if (lane == 0) b0 = atomicAdd(r.lv_count, __popc(gma) + __popc(gmb));
+            b0 = __shfl_sync(0xffffffffu, b0, 0);
+            goa = (long long)b0 + __popc(gma & lt);
+            gob = (long long)b0 + __popc(gma) + __popc(gmb & lt);
+          }
+          const int gcell = gk * r.nx + gi;  // cells < 2^30
+          auto place = [&](bool st, bool full, bool lv, bool g, int dk, int jo, int ls, long long go, float nox,
+                           float noz, float ux, float uy, float uz, float w, unsigned id, int shx, int shz) {
+            const int dcell = gcell + shz * r.nx + shx;  // a cell of this tile when st
+            if (st && !full) {
+              const long long o = (long long)dcell * r.cap + jo;
+              pout.ox[o] = nox;
+              pout.oz[o] = noz;
+              pout.dux[o] = ux;
+              pout.duy[o] = uy;
+              pout.duz[o] = uz;
+              if (has_w) pout.w[o] = w;
+              if (has_id) pout.id[o] = id;
+            } else if (g) {
+              if (go < r.lv_cap) list_put(r.lv, go, full ? dcell * 2 + (dk & 1) : dk, nox, 0.f, noz, ux, uy, uz, w, id);
+              else flag_error(r.err, ERR_OVERFLOW);
+            } else if (lv) {
+              lvk[ls] = dk;
+              lvv[ls] = nox;
+              lvv[2 * S::LVB + ls] = noz;
+              lvv[3 * S::LVB + ls] = ux;
+              lvv[4 * S::LVB + ls] = uy;
+              lvv[5 * S::LVB + ls] = uz;
+              if (has_w) lvv[6 * S::LVB + ls] = w;
+              if (has_id) lvi[ls] = id;
+            }
+          };
+          if (va)
+            place(sta, fa, lva, ga, dka, ba, lsa, goa, exa.off, eza.off, nuxa, nuya, nuza, wa, has_id ? st_id[ja] : 0u,
+                  exa.shift, eza.shift);
+          if (vb)
+            place(stb, fb, lvb, gb, dkb, bb, lsb, gob, exb.off, ezb.off, nuxb, nuyb, nuzb, wb, has_id ? st_id[jb] : 0u,
+                  exb.shift, ezb.shift);
+        }
+      } else {
+      {
+        constexpr int jj = 0;
+        const bool valid = cnt > 0;
+        int dkey = -1 - lane;  // unique per lane when there is no particle
+        bool leave = false;
+        T nox = T(0), noy = T(0), noz = T(0), ux = T(0), uy = T(0), uz = T(0);
+        const T w = (has_w && valid) ? st_x[SG::slot(6) * 128 + jj] : r.wconst;
+        if (valid) {
+          const T o_x = st_x[jj], o_y = NDIM == 3 ? st_x[SG::slot(1) * 128 + jj] : T(0), o_z = st_x[SG::slot(2) * 128 + jj];
+          ux = st_x[SG::slot(3) * 128 + jj];
+          uy = st_x[SG::slot(4) * 128 + jj];
+          uz = st_x[SG::slot(5) * 128 + jj];
+          // gather
+          T F[6];
+          if constexpr (WIN) {
+            gather_window<Lanes1<T>, T, T, NDIM, ORDER, SCHEME>(sg, lx, ly, lz, o_x, o_y, o_z, F);
+          } else if (SCHEME == 0) {
+            gc.interp(o_x, o_y, o_z, F);
+          } else {
+            const DirW<T> dwx = dir_weights(o_x), dwy = dir_weights(o_y), dwz = dir_weights(o_z);
+#pragma unroll
+            for (int c = 0; c < 6; ++c)
+              F[c] = gather_comp<T, NDIM, SCHEME>(sg + c * S::GN, c, lx, ly, lz, dwx, dwy, dwz);
+          }
+          // relativistic Boris, momenta relative to the drift u0 z_hat
+          const T h = qs * r.hq;
+          const T mx = ux + h * F[0], my = uy + h * F[1], mz = uz + h * F[2];
+          const T Mz = r.u0 + mz;
+          const T mm = T(1) + mx * mx + my * my + Mz * Mz;
+          const T ig = WIN ? fine_rsqrt(mm) : fast_rsqrt(mm);
+          const T tx = h * F[3] * ig, ty = h * F[4] * ig, tz = h * F[5] * ig;
+          const T sf = fast_div(T(2), T(1) + tx * tx + ty * ty + tz * tz);
+          const T sx = sf * tx, sy = sf * ty, sz = sf * tz;
+          const T qx = mx + (my * tz - Mz * ty);
+          const T qy = my + (Mz * tx - mx * tz);
+          const T qz = Mz + (mx * ty - my * tx);
+          ux = mx + (qy * sz - qz * sy) + h * F[0];
+          uy = my + (qz * sx - qx * sz) + h * F[1];
+          uz = mz + (qx * sy - qy * sx) + h * F[2];
+          const T Uz = r.u0 + uz;
+          const T u2 = ux * ux + uy * uy + Uz * Uz;
+          const T ign = WIN ? fine_rsqrt(T(1) + u2) : fast_rsqrt(T(1) + u2);
+          T vx = ux * ign, vy = uy * ign;
+          const T vz = Uz * ign;
+          kin += w * fast_div(u2, (T(1) + u2) * ign + T(1));  // gamma - 1 = u^2 / (gamma + 1)
+          ++npush;
+          // move (cell-relative displacement in grid units)
+          T ddx = r.dtdx * vx, ddy = NDIM == 3 ? r.dtdy * vy : T(0), ddz = r.dtdz * vz;
+          if (!(abs_lt_one(ddx) && abs_lt_one(ddy) && abs_lt_one(ddz))) {
+            flag_error(r.err, ERR_NONFINITE);
+            ddx = ddy = ddz = T(0);
+            ux = uy = uz = T(0);
+            vy = T(0);
+          }
+          const EsirDir<T> ex_ = esir_dir(o_x, ddx);
+          const EsirDir<T> ez_ = esir_dir(o_z, ddz);
+          EsirDir<T> ey_;
+          if (NDIM == 3) ey_ = esir_dir(o_y, ddy);
+          else { ey_.a = 0; ey_.shift = 0; ey_.off = T(0); }
+          // Esirkepov deposit: summed in registers when the window fits RegLayout (no step back across
+          // a face and no transverse crossing), else straight to shared memory
+          const T qw = qs * w;
+          const bool own = reg_window<T, NDIM>(ex_, NDIM == 3 ? ey_ : ex_, ez_);
+          if constexpr (LATE) {  // summed after the item's push, from the particle's stage slot
+            T* q = const_cast<T*>(st_x) + jj;
+            q[3 * 128] = ddx;
+            q[4 * 128] = ddy;
+            q[5 * 128] = ddz;
+            q[6 * 128] = own ? qw : T(0);
+            if (!own)
+              deposit_general<T, 3>(sj, lx, ly, lz, o_x, o_y, o_z, ddx, ddy, ddz, qw * r.jfx, qw * r.jfy, qw * r.jfz);
+          } else if constexpr (ORDER == 3) {
+            const T cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vy * r.jfy2d;
+            if (own)
+              deposit2_cubic<T, NVP>(acc, cubic_dir(o_x, ddx, false, T(0)),
+                                     cubic_dir(o_z, ddz, !is_zero(ez_.dS[2]), ez_.off), cx, cy, cz);
+            else deposit_general<T, 2>(sj, lx, 0, lz, o_x, T(0), o_z, ddx, T(0), ddz, cx, cy, cz);
+          } else if (NDIM == 2) {
+            const T cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vy * r.jfy2d;
+            if (own) deposit2_reg<T, NVP>(acc, ex_, ez_, cx, cy, cz);
+            else deposit2_smem<T, NDIM>(sj, lx + ex_.a + 1, lz + ez_.a + 1, ex_, ez_, cx, cy, cz);
+          } else {
+            const T cx = qw * r.jfx, cy = qw * r.jfy, cz = qw * r.jfz;
+            if (own) deposit3_reg<T, NVP>(acc, ex_, ey_, ez_, cx, cy, cz);
+            else deposit3_smem<T, NDIM>(sj, lx + ex_.a + 1, ly + ey_.a + 1, lz + ez_.a + 1, ex_, ey_, ez_, cx, cy, cz);
+          }
+          // new cell and offsets
+          nox = ex_.off;
+          noy = NDIM == 3 ? ey_.off : T(0);
+          noz = ez_.off;
+          const int nlx = lx + ex_.shift, nly = NDIM == 3 ? ly + ey_.shift : 0, nlz = lz + ez_.shift;
+          if (nlx >= 0 && nlx < wx && nly >= 0 && nly < wy && nlz >= 0 && nlz < wz) {
+            dkey = ((nlz * TY + nly) * TX + nlx) * 2 + s;  // stays in this tile
+          } else {
+            leave = true;  // global destination, as cell * 2 + species
+            // one cell across a face: the index stays within [-1, n] (cells < 2^30: int keys)
+            const int ni = wrap_near_p(gi + ex_.shift, r.nx);
+            const int nj = NDIM == 3 ? wrap_near_p(gj + ey_.shift, r.ny) : 0;
+            const int nk = wrap_near_p(gk + ez_.shift, r.nz);
+            dkey = ((nk * r.ny + nj) * r.nx + ni) * 2 + s;
+          }
+        }
+        if (LATE && !valid) {  // an empty slot: finite values and no charge for the deposit
+#pragma unroll
+          for (int a = 0; a < 7; ++a) const_cast<T*>(st_x)[jj + a * 128] = T(0);
+        }
+        // rebin. Destination in this tile: lanes with the same (cell, species) reserve consecutive
+        // slots with one shared-memory atomic on the tile's output counts. Destination in another
+        // tile: the particle is appended to the leaver list (one global atomic per warp), which
+        // k_migrate inserts after this kernel.
+        const bool stay = valid && !leave;
+        const unsigned peers = __match_any_sync(0xffffffffu, stay ? dkey : -1 - lane);
+        const int leader = __ffs(peers) - 1;
+        const int rank = __popc(peers & ((1u << lane) - 1u));
+        int base = 0;
+        if (stay && lane == leader) base = atomicAdd(scnt + (dkey & 1) * NCL + (dkey >> 1), __popc(peers));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        // a full destination bin: the particle goes through the global leaver list instead, and
+        // k_migrate spills it when the bin is still full there (nothing is dropped)
+        const bool full = stay && base + rank >= r.cap;
+        const unsigned fmask = __ballot_sync(0xffffffffu, full);
+        long long fglob = 0;
+        if (fmask) {
+          const int fl = __ffs(fmask) - 1;
+          int fb = 0;
+          if (lane == fl) fb = atomicAdd(r.lv_count, __popc(fmask));
+          fb = __shfl_sync(0xffffffffu, fb, fl);
+          fglob = (long long)fb + __popc(fmask & ((1u << lane) - 1u));
+        }
+        // leavers: a slot in the tile's shared-memory buffer (one shared atomic per warp), or, once
+        // the buffer is full, straight in the global list
+        const unsigned lmask = __ballot_sync(0xffffffffu, valid && leave);
+        int lslot = 0;
+        long long lglob = 0;
+        if (lmask) {
+          const int lleader = __ffs(lmask) - 1;
+          int b = 0;
+          if (lane == lleader) b = atomicAdd(lvn, __popc(lmask));
+          b = __shfl_sync(0xffffffffu, b, lleader);
+          lslot = b + __popc(lmask & ((1u << lane) - 1u));
+          const unsigned gmask = __ballot_sync(0xffffffffu, valid && leave && lslot >= S::LVB);
+          if (gmask) {
+            const int gl = __ffs(gmask) - 1;
+            int gb = 0;
+            if (lane == gl) gb = atomicAdd(r.lv_count, __popc(gmask));
+            gb = __shfl_sync(0xffffffffu, gb, gl);
+            lglob = (long long)gb + __popc(gmask & ((1u << lane) - 1u));
+          }
+        }
+        if (stay) {
+          const int j = base + rank;
+          const int dl = dkey >> 1;
+          const int dx = dl % TX, dy = (dl / TX) % TY, dz = dl / (TX * TY);
+          const int dcell = ((Z0 + dz) * r.ny + Y0 + dy) * r.nx + X0 + dx;  // cells < 2^30
+          if (!full) {
+            const long long o = (long long)dcell * r.cap + j;
+            pout.ox[o] = nox;
+            if (NDIM == 3) pout.oy[o] = noy;
+            pout.oz[o] = noz;
+            pout.dux[o] = ux;
+            pout.duy[o] = uy;
+            pout.duz[o] = uz;
+            if (has_w) pout.w[o] = w;
+            if (has_id) pout.id[o] = st_id[jj];
+          } else if (fglob < r.lv_cap) {
+            list_put(r.lv, fglob, dcell * 2 + (dkey & 1), nox, noy, noz, ux, uy, uz, w, has_id ? st_id[jj] : 0u);
+          } else {
+            flag_error(r.err, ERR_OVERFLOW);
+          }
+        } else if (valid && lslot < S::LVB) {
+          lvk[lslot] = dkey;
+          lvv[lslot] = nox;
+          if (NDIM == 3) lvv[S::LVB + lslot] = noy;
+          lvv[2 * S::LVB + lslot] = noz;
+          lvv[3 * S::LVB + lslot] = ux;
+          lvv[4 * S::LVB + lslot] = uy;
+          lvv[5 * S::LVB + lslot] = uz;
+          if (has_w) lvv[6 * S::LVB + lslot] = w;
+          if (has_id) lvi[lslot] = st_id[jj];
+        } else if (valid) {
+          const long long o = lglob;
+          if (o < r.lv_cap) {
+            r.lv.key[o] = dkey;
+            r.lv.ox[o] = nox;
+            if (NDIM == 3) r.lv.oy[o] = noy;
+            r.lv.oz[o] = noz;
+            r.lv.dux[o] = ux;
+            r.lv.duy[o] = uy;
+            r.lv.duz[o] = uz;
+            if (has_w) r.lv.w[o] = w;
+            if (has_id) r.lv.id[o] = st_id[jj];
+          } else {
+            flag_error(r.err, ERR_OVERFLOW);
+          }
+        }
+      }
+      }
+    }
+    if constexpr (LATE) {
+      __syncwarp();
+      const T* st = SG::at(stg, stage, 0, lane - sl);
+      T* j = sj + okey;
+      deposit3_cubic<T, LPC, 0>(st, sl, nrnd, rnd0, r.jfx, j);
+      deposit3_cubic<T, LPC, 1>(st, sl, nrnd, rnd0, r.jfy, j);
+      deposit3_cubic<T, LPC, 2>(st, sl, nrnd, rnd0, r.jfz, j);
+    }
+    if (!LATE && it == giters - 1) {
+      // 3. segmented transpose-reduction of the cell's register sums over its LPC lanes
+#pragma unroll
+      for (int sh = LPC / 2; sh >= 1; sh >>= 1) {
+        const bool up = (lane & sh) != 0;
+#pragma unroll
+        for (int j = 0; j < PER * sh; ++j) {
+          const T send = up ? acc[j] : acc[j + PER * sh];
+          const T keep = up ? acc[j + PER * sh] : acc[j];
+          acc[j] = keep + __shfl_xor_sync(0xffffffffu, send, sh);
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < PER; ++m) {
+        const int i = sl * PER + m;
+        if (i < NV && acc[m] != T(0)) {
+          int comp, a, b, c;
+          RegLayout<NDIM, ORDER>::at(i, comp, a, b, c);
+          atomicAdd(sj + comp * S::JN + okey + (c * S::JY + b) * S::JX + a, acc[m]);
+        }
+      }
+    }
+    __syncwarp();  // the stage just read is refilled by the next iteration's prefetch
+    g = ng;
+    it = nit;
+    giters = niters;
+    stage ^= 1;
+  }
+  cp_async_wait_all();
+  __syncthreads();
+
+  // 4. the tile's buffered leavers: one reservation in the global list, then a coalesced copy
+  __shared__ int lv_base;
+  const int nlv = min(*lvn, S::LVB);
+  if (tid == 0) lv_base = nlv > 0 ? atomicAdd(r.lv_count, nlv) : 0;
+  __syncthreads();
+  for (int e = tid; e < nlv; e += PUSH_THREADS) {
+    const long long o = (long long)lv_base + e;
+    if (o < r.lv_cap) {
+      r.lv.key[o] = lvk[e];
+      r.lv.ox[o] = lvv[e];
+      if (NDIM == 3) r.lv.oy[o] = lvv[S::LVB + e];
+      r.lv.oz[o] = lvv[2 * S::LVB + e];
+      r.lv.dux[o] = lvv[3 * S::LVB + e];
+      r.lv.duy[o] = lvv[4 * S::LVB + e];
+      r.lv.duz[o] = lvv[5 * S::LVB + e];
+      if (has_w) r.lv.w[o] = lvv[6 * S::LVB + e];
+      if (has_id) r.lv.id[o] = lvi[e];
+    } else {
+      flag_error(r.err, ERR_OVERFLOW);
+    }
+  }
+
+  // 5. output counts of the tile's cells (leavers from other tiles are added by k_migrate); a count
+  // past the capacity (particles sent on through the leaver list) is stored as the capacity
+  for (int cl = tid; cl < NCL; cl += PUSH_THREADS) {
+    const int lx = cl % TX, ly = (cl / TX) % TY, lz = cl / (TX * TY);
+    if (lx < wx && ly < wy && lz < wz) {
+      const long long cell = (long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx;
+      r.out[0].cnt[cell] = min(scnt[cl], r.cap);
+      r.out[1].cnt[cell] = min(scnt[NCL + cl], r.cap);
+    }
+  }
+
+  // 6. flush the tile's current to global memory
+  for (int e = tid; e < 3 * S::JN; e += PUSH_THREADS) {
+    T v = sj[e];
+    if (v == T(0)) continue;
+    int c = e / S::JN, rem = e - c * S::JN;
+    int lz = rem / (S::JX * S::JY);
+    int ly = (rem / S::JX) % S::JY;
+    int lx = rem % S::JX;
+    int gx = near_ok ? wrap_near_p(X0 - S::H + lx, r.nx) : wrapi(X0 - S::H + lx, r.nx);
+    int gy = NDIM == 3 ? (near_ok ? wrap_near_p(Y0 - S::H + ly, r.ny) : wrapi(Y0 - S::H + ly, r.ny)) : 0;
+    int gz = near_ok ? wrap_near_p(Z0 - S::H + lz, r.nz) : wrapi(Z0 - S::H + lz, r.nz);
+    atomicAdd(r.j[c] + (long long)gz * nxy + (long long)gy * r.nx + gx, v);
+  }
+
+  // 7. kinetic energy and particle count of this step: per-thread partial sums in the working
+  // precision, FP64 across the block and the grid
+  if (r.kin) {
+    double kd = (double)kin;
+    int nd = npush;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      kd += __shfl_xor_sync(0xffffffffu, kd, o);
+      nd += __shfl_xor_sync(0xffffffffu, nd, o);
+    }
+    __shared__ double skin[NWARP];
+    __shared__ int swcnt[NWARP];
+    if (lane == 0) {
+      skin[warp] = kd;
+      swcnt[warp] = nd;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      double t = 0;
+      long long c = 0;
+      for (int w2 = 0; w2 < NWARP; ++w2) {
+        t += skin[w2];
+        c += swcnt[w2];
+      }
+      atomicAdd(r.kin, t);
+      atomicAdd(r.kin + 1, (double)c);
+    }
+  }
+}
+
+}  // namespace picgb

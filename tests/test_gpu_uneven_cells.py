@@ -38,7 +38,8 @@ def _uneven(ndim, nx, ny, nz, seed, gamma=130.0):
 # to 8, then 8, then 16)
 @pytest.mark.parametrize("precision", [1, 0])
 @pytest.mark.parametrize("ndim,ppc,scheme,order", [(2, 4, 0, 1), (2, 20, 0, 1), (2, 4, 1, 1), (3, 8, 0, 1), (3, 12, 0, 1),
-                                                   (3, 20, 1, 1)])
+                                                   (3, 20, 1, 1), (2, 4, 0, 3), (2, 4, 1, 3), (2, 4, 2, 3), (2, 4, 2, 1),
+                                                   (3, 8, 0, 3), (3, 8, 1, 3), (3, 8, 2, 3), (3, 8, 2, 1)])
 def test_step_uneven_cells(ndim, ppc, scheme, order, precision):
     nx, ny, nz = (19, 1, 45) if ndim == 2 else (11, 7, 13)
     cfg = make_cfg(ndim=ndim, nx=nx, ny=ny, nz=nz, dt=0.5, scheme=scheme, precision=precision, ppc=ppc, order=order,
