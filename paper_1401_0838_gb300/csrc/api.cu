@@ -34,7 +34,7 @@ struct pic_handle {
   void* fb[6] = {};  // the other E, B buffers: the fused Yee update writes there, then the two swap
   void* g[6] = {};   // gather copies
   void* jf[3] = {};  // filtered current (aliases f[6..8] when J is not filtered)
-  void* parr[2][2][8] = {};  // [species][buffer][ox oy oz dux duy duz w id]
+  void* parr[2][2][4] = {};  // [species][buffer][q r w id] (SpeciesBuf)
   int* cnt[2][2] = {};
   int parity = 0;
   int* d_err = nullptr;
@@ -222,6 +222,12 @@ void dfree(pic_handle* h, void*& p) {
   p = nullptr;
 }
 
+// Bytes per slot of array a of the particle bins (SpeciesBuf: q, r, w, id).
+size_t slot_bytes(const pic_handle* h, int a) {
+  if (a == 3) return 4;
+  return h->es * (a == 0 ? 4 : a == 1 && h->cfg.ndim == 3 ? 2 : 1);
+}
+
 // Leaver and spill lists with room for n particles each (every particle of the run fits, so a
 // step can hand all of them on, and nothing is dropped however many bins are full).
 int alloc_lists(pic_handle* h, long long n) {
@@ -344,14 +350,10 @@ RunDev<T> make_run(pic_handle* h, int parity) {
     for (int io = 0; io < 2; ++io) {
       int b = io == 0 ? parity : 1 - parity;
       SpeciesBuf<T> sb;
-      sb.ox = (T*)h->parr[s][b][0];
-      sb.oy = (T*)h->parr[s][b][1];
-      sb.oz = (T*)h->parr[s][b][2];
-      sb.dux = (T*)h->parr[s][b][3];
-      sb.duy = (T*)h->parr[s][b][4];
-      sb.duz = (T*)h->parr[s][b][5];
-      sb.w = (T*)h->parr[s][b][6];
-      sb.id = (unsigned*)h->parr[s][b][7];
+      sb.q = (T*)h->parr[s][b][0];
+      sb.r = (T*)h->parr[s][b][1];
+      sb.w = (T*)h->parr[s][b][2];
+      sb.id = (unsigned*)h->parr[s][b][3];
       sb.cnt = h->cnt[s][b];
       if (io == 0) r.in[s] = sb; else r.out[s] = sb;
     }
@@ -726,23 +728,23 @@ int settle(pic_handle* h) {
   // new bins for both buffers and species; the old ones are freed only once all are in place
   const pic_config& c = h->cfg;
   const size_t slots = (size_t)h->ncell * (size_t)nc;
-  void* np_[2][2][8] = {};
+  void* np_[2][2][4] = {};
   bool ok = true;
   for (int sp = 0; sp < 2 && ok; ++sp)
     for (int b = 0; b < 2 && ok; ++b)
-      for (int a = 0; a < 8 && ok; ++a) {
+      for (int a = 0; a < 4 && ok; ++a) {
         if (!h->parr[sp][b][a]) continue;  // arrays the run does not carry
-        ok = (np_[sp][b][a] = dalloc(h, slots * (a == 7 ? 4 : h->es))) != nullptr;
+        ok = (np_[sp][b][a] = dalloc(h, slots * slot_bytes(h, a))) != nullptr;
       }
   if (!ok) {
     for (int sp = 0; sp < 2; ++sp)
       for (int b = 0; b < 2; ++b)
-        for (int a = 0; a < 8; ++a) dfree(h, np_[sp][b][a]);
+        for (int a = 0; a < 4; ++a) dfree(h, np_[sp][b][a]);
     return fail(h, PIC_E_OOM, "particle bin growth: allocation failed");
   }
   for (int sp = 0; sp < 2; ++sp)
     for (int b = 0; b < 2; ++b)
-      for (int a = 0; a < 8; ++a)
+      for (int a = 0; a < 4; ++a)
         if (h->parr[sp][b][a]) {
           dfree(h, h->parr[sp][b][a]);
           h->parr[sp][b][a] = np_[sp][b][a];
@@ -1011,11 +1013,10 @@ int pic_create(const pic_config* cfg_in, pic_handle** out) {
   const size_t slots = (size_t)h->ncell * cap;
   for (int s = 0; s < 2 && ok; ++s)
     for (int b = 0; b < 2 && ok; ++b) {
-      for (int a = 0; a < 8 && ok; ++a) {
-        if (a == 1 && c.ndim == 2) continue;
-        if (a == 6 && !h->has_w) continue;
-        if (a == 7 && !h->has_id) continue;
-        ok = (h->parr[s][b][a] = dalloc(h, slots * (a == 7 ? 4 : h->es))) != nullptr;
+      for (int a = 0; a < 4 && ok; ++a) {
+        if (a == 2 && !h->has_w) continue;
+        if (a == 3 && !h->has_id) continue;
+        ok = (h->parr[s][b][a] = dalloc(h, slots * slot_bytes(h, a))) != nullptr;
       }
       if (ok) ok = (h->cnt[s][b] = (int*)dalloc(h, sizeof(int) * h->ncell)) != nullptr;
     }

@@ -19,15 +19,73 @@ constexpr int MAX_ZTAPS = 33;  // combined z stencil: Psi (9 taps) convolved wit
 constexpr int MAX_XTAPS = 25;  // filter stencil along x or y
 
 // One species' particle storage in one of the two ping-pong buffers. Slot s of the arrays
-// belongs to cell s / cap; cell c holds cnt[c] particles in slots [c*cap, c*cap + cnt[c]).
+// belongs to cell s / cap; cell c holds cnt[c] particles in slots [c*cap, c*cap + cnt[c]). A particle's
+// values lie side by side in two arrays, so the push writes a particle with two vector stores instead of
+// one store per value: its particles scatter to the bins of two or more cells, and what that costs is
+// the stores' separate cache lines.
 template <typename T>
 struct SpeciesBuf {
-  T *ox, *oy, *oz;     // offsets in [0,1) inside the cell (oy unused in 2D)
-  T *dux, *duy, *duz;  // u - u0 z_hat
-  T* w;                // per-particle weight or nullptr
-  unsigned* id;        // particle id or nullptr
-  int* cnt;            // particles per cell
+  T* q;          // four values per slot: ox oz dux duy (2D), ox oy oz dux (3D); offsets in [0,1)
+  T* r;          // duz (2D), duy duz (3D) per slot; u - u0 z_hat
+  T* w;          // per-particle weight or nullptr
+  unsigned* id;  // particle id or nullptr
+  int* cnt;      // particles per cell
 };
+
+// Four (two) consecutive values, aligned to 4 (2) values.
+__device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void ld4(const double* p, double (&v)[4]) {
+  const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
+  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+__device__ __forceinline__ void ld2(const float* p, float (&v)[2]) {
+  const float2 t = *reinterpret_cast<const float2*>(p);
+  v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void ld2(const double* p, double (&v)[2]) {
+  const double2 t = *reinterpret_cast<const double2*>(p);
+  v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void st4(float* p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ void st4(double* p, double a, double b, double c, double d) {
+  *reinterpret_cast<double2*>(p) = make_double2(a, b);
+  *reinterpret_cast<double2*>(p + 2) = make_double2(c, d);
+}
+__device__ __forceinline__ void st2(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
+__device__ __forceinline__ void st2(double* p, double a, double b) {
+  *reinterpret_cast<double2*>(p) = make_double2(a, b);
+}
+
+// Offsets and momenta of slot o.
+template <typename T>
+struct PartVals {
+  T ox, oy, oz, ux, uy, uz;
+};
+template <typename T>
+__device__ __forceinline__ PartVals<T> part_get(const SpeciesBuf<T>& b, int ndim, long long o) {
+  T v[4];
+  ld4(b.q + 4 * o, v);
+  if (ndim == 2) return PartVals<T>{v[0], T(0), v[1], v[2], v[3], b.r[o]};
+  T u[2];
+  ld2(b.r + 2 * o, u);
+  return PartVals<T>{v[0], v[1], v[2], v[3], u[0], u[1]};
+}
+template <typename T>
+__device__ __forceinline__ void part_put(const SpeciesBuf<T>& b, int ndim, long long o, T ox, T oy, T oz, T ux, T uy,
+                                         T uz) {
+  if (ndim == 2) {
+    st4(b.q + 4 * o, ox, oz, ux, uy);
+    b.r[o] = uz;
+  } else {
+    st4(b.q + 4 * o, ox, oy, oz, ux);
+    st2(b.r + 2 * o, uy, uz);
+  }
+}
 
 // Particles that left their tile in a push (appended by the push kernel, inserted into their
 // destination bins by the migrate kernel). key = destination cell * 2 + species. The same layout
@@ -229,12 +287,13 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-__device__ __forceinline__ void copy4_async(float* dst, const float* src) { cp_async16(dst, src); }
-__device__ __forceinline__ void copy4_async(double* dst, const double* src) {
-  cp_async16(dst, src);
-  cp_async16(dst + 2, src + 2);
+// BYTES (a multiple of 16) from and to 16-byte aligned addresses
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  static_assert(BYTES % 16 == 0, "16-byte pieces");
+#pragma unroll
+  for (int i = 0; i < BYTES; i += 16) cp_async16((char*)dst + i, (const char*)src + i);
 }
-__device__ __forceinline__ void copy4_async(unsigned* dst, const unsigned* src) { cp_async16(dst, src); }
 __device__ __forceinline__ void copy1_async(float* dst, const float* src) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(src) : "memory");

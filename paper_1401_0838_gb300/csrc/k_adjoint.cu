@@ -45,12 +45,13 @@ __global__ void __launch_bounds__(256) k_tape(const __grid_constant__ RunDev<T> 
   }
   f.cell[id] = (int)cell;
   f.species[id] = s;
-  f.ox[id] = b.ox[src];
-  if (f.oy) f.oy[id] = r.ndim == 3 ? b.oy[src] : T(0);
-  f.oz[id] = b.oz[src];
-  f.dux[id] = b.dux[src];
-  f.duy[id] = b.duy[src];
-  f.duz[id] = b.duz[src];
+  const PartVals<T> v = part_get(b, r.ndim, src);
+  f.ox[id] = v.ox;
+  if (f.oy) f.oy[id] = v.oy;
+  f.oz[id] = v.oz;
+  f.dux[id] = v.ux;
+  f.duy[id] = v.uy;
+  f.duz[id] = v.uz;
   if (f.w) f.w[id] = b.w ? b.w[src] : r.wconst;
   }
 }

@@ -1207,7 +1207,8 @@ __global__ void k_kinetic(const __grid_constant__ RunDev<T> r, double* out) {
       n = n > r.cap ? r.cap : n;
       for (int j = threadIdx.x; j < n; j += 32) {
         long long o = c * r.cap + j;
-        double ux = b.dux[o], uy = b.duy[o], uz = (double)r.u0 + (double)b.duz[o];
+        const PartVals<T> v = part_get(b, r.ndim, o);
+        double ux = v.ux, uy = v.uy, uz = (double)r.u0 + (double)v.uz;
         double u2 = ux * ux + uy * uy + uz * uz;
         double w = b.w ? (double)b.w[o] : (double)r.wconst;
         acc += w * u2 / (sqrt(1.0 + u2) + 1.0);

@@ -56,9 +56,10 @@ __global__ void __launch_bounds__(RHO_THREADS) k_rho(const __grid_constant__ Run
         const long long o = cell * r.cap + slot;
         const double qw = q * (b.w ? (double)b.w[o] : (double)r.wconst) * inv_dv;
         double wx[4], wy[4] = {1.0, 0.0, 0.0, 0.0}, wz[4];
-        node_weights(order, (double)b.ox[o], wx);
-        if (r.ndim == 3) node_weights(order, (double)b.oy[o], wy);
-        node_weights(order, (double)b.oz[o], wz);
+        const PartVals<T> v = part_get(b, r.ndim, o);
+        node_weights(order, (double)v.ox, wx);
+        if (r.ndim == 3) node_weights(order, (double)v.oy, wy);
+        node_weights(order, (double)v.oz, wz);
         const int ny_n = r.ndim == 3 ? nn : 1;
         for (int c = 0; c < nn; ++c) {
           const long long kz = wrap_any(k + lo + c, r.nz);

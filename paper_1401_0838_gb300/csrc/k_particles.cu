@@ -248,12 +248,7 @@ __device__ __forceinline__ void migrate_body(const RunDev<T>& r, int* other_coun
     }
     const int j = j0 + rank;
     const long long o = cell * r.cap + j;
-    b.ox[o] = ox;
-    if (r.ndim == 3) b.oy[o] = oy;
-    b.oz[o] = oz;
-    b.dux[o] = ux;
-    b.duy[o] = uy;
-    b.duz[o] = uz;
+    part_put(b, r.ndim, o, ox, oy, oz, ux, uy, uz);
     if (b.w) b.w[o] = w;
     if (b.id) b.id[o] = id;
   }
@@ -306,12 +301,7 @@ __device__ __forceinline__ void insert_particle(const RunDev<T>& r, int s, long 
     return;
   }
   long long o = cell * cap + j;
-  b.ox[o] = ox;
-  if (b.oy) b.oy[o] = oy;
-  b.oz[o] = oz;
-  b.dux[o] = ux;
-  b.duy[o] = uy;
-  b.duz[o] = uz;
+  part_put(b, r.ndim, o, ox, oy, oz, ux, uy, uz);
   if (b.w) b.w[o] = w;
   if (b.id) b.id[o] = id;
 }
@@ -472,12 +462,13 @@ __global__ void k_export(const __grid_constant__ RunDev<T> r, int s, const long 
     if (d >= f.np) return;
     f.cell[d] = (int)cell;
     f.species[d] = s;
-    f.ox[d] = b.ox[src];
-    if (f.oy) f.oy[d] = r.ndim == 3 ? b.oy[src] : T(0);
-    f.oz[d] = b.oz[src];
-    f.dux[d] = b.dux[src];
-    f.duy[d] = b.duy[src];
-    f.duz[d] = b.duz[src];
+    const PartVals<T> v = part_get(b, r.ndim, src);
+    f.ox[d] = v.ox;
+    if (f.oy) f.oy[d] = v.oy;
+    f.oz[d] = v.oz;
+    f.dux[d] = v.ux;
+    f.duy[d] = v.uy;
+    f.duz[d] = v.uz;
     if (f.w) f.w[d] = b.w ? b.w[src] : r.wconst;
     if (f.id) f.id[d] = b.id ? b.id[src] : 0u;
   }

@@ -26,27 +26,30 @@ struct PushTileOf<T, NDIM, 3> {
   using type = HoTile<T, NDIM>;
 };
 
-// Per-warp double-buffered stage: [stage][slot][lane][4] for the particle arrays (slots ox oz dux
-// duy duz w in 2D; ox oy oz dux duy duz w in 3D), then [stage][lane][4] ids. Lane l copies a pack of 4
-// slots; a cell's lanes then take the particles of all its packs in turn, U at a time (PushPlan).
+// Per-warp double-buffered stage of an item (32 packs of 4 slots, cell by cell): [32][4][4] values q,
+// [32][4][RW] values r, [32][4] weights per stage (SpeciesBuf's arrays), then [stage][32][4] ids. The
+// four slots of pack p of a cell follow those of pack p - 1, so slot k of the cell's 4 LPC is element k
+// from the cell's first lane.
 template <typename T, int NDIM>
 struct PushStage {
-  static constexpr int NSLOT = NDIM == 3 ? 7 : 6;
-  // slot of array a (0 ox, 1 oy, 2 oz, 3 dux, 4 duy, 5 duz, 6 w); 2D stages no oy
-  static constexpr __host__ __device__ int slot(int a) { return NDIM == 3 ? a : (a > 1 ? a - 1 : a); }
+  static constexpr int RW = NDIM == 3 ? 2 : 1;
+  static constexpr int ELEMS = 32 * (16 + 4 * RW + 4);  // per stage
   static constexpr __host__ __device__ size_t per_warp_elems() {
-    return 2 * NSLOT * 32 * 4 + (2 * 32 * 4 * sizeof(unsigned) + sizeof(T) - 1) / sizeof(T);
+    return 2 * ELEMS + (2 * 32 * 4 * sizeof(unsigned) + sizeof(T) - 1) / sizeof(T);
   }
-  static __device__ __forceinline__ T* at(T* base, int stage, int arr, int lane) {
-    return base + ((stage * NSLOT + slot(arr)) * 32 + lane) * 4;
+  static __device__ __forceinline__ T* q(T* base, int stage, int lane) { return base + stage * ELEMS + lane * 16; }
+  static __device__ __forceinline__ T* r(T* base, int stage, int lane) {
+    return base + stage * ELEMS + 32 * 16 + lane * 4 * RW;
   }
-  static __device__ __forceinline__ unsigned* id_at(T* base, int stage, int lane) {
-    return reinterpret_cast<unsigned*>(base + 2 * NSLOT * 32 * 4) + (stage * 32 + lane) * 4;
+  static __device__ __forceinline__ T* w(T* base, int stage, int lane) {
+    return base + stage * ELEMS + 32 * (16 + 4 * RW) + lane * 4;
+  }
+  static __device__ __forceinline__ unsigned* id(T* base, int stage, int lane) {
+    return reinterpret_cast<unsigned*>(base + 2 * ELEMS) + (stage * 32 + lane) * 4;
   }
 };
 
-
-// FP32 2D: each lane takes two neighbouring particles at a time, with the arithmetic of the pair
+// FP32 2D: each lane takes two particles of its cell at a time, with the arithmetic of the pair
 // in packed FP32x2 instructions (one instruction advances both particles) and the two rebins
 // interleaved, so one dependent chain carries two particles.
 template <typename T, int NDIM>
@@ -566,7 +569,7 @@ struct PushRounds {
 // LPC lanes per cell. The cell's particles are split into packs of 4 consecutive slots of one
 // species (electron packs first); an item is LPC packs of every cell of the group, copied by one lane
 // each (16-byte copies: 8-byte ones cost the 3D push 40 %). Within an item the cell's lanes take its
-// 4 LPC slots in turn, lane l the slots U l .. U l + U - 1 of every round of U LPC slots, and the warp
+// 4 LPC slots in turn, one window of LPC slots (a paired push: two windows) per round, and the warp
 // runs only the rounds that its fullest cell needs. A cell of 17 + 16 particles costs its warp 9 rounds
 // of single particles (12 when every lane walked its own pack), and with 4 + 4 particles all four
 // lanes work (two of them before). Measured on 512x1024 FP32 cells, push per step: 16 per species at
@@ -583,14 +586,10 @@ struct PushPlan {
   static constexpr int PER = (NV + LPC - 1) / LPC;
   static constexpr int NVP = PER * LPC;
   static constexpr int CPW = 32 / LPC;
-  // Round a cell (c-th of the group) starts a full item with: a round reads U LPC neighbouring values
-  // of every cell, and cells whose values lie in the same banks start with different rounds.
-  template <typename T>
-  static __device__ __forceinline__ int first_round(int c) {
-    constexpr int NR = PushRounds<T, NDIM>::value;
-    constexpr int M = (sizeof(T) == 8 || NR == 2 ? 16 : 32) / LPC;  // cells read in one pass of the banks
-    return (M > NR ? c / (M / NR) : c) & (NR - 1);
-  }
+  // An item's 4 LPC slots of a cell form four windows of LPC slots, one per lane each. Which window the
+  // cell (c-th of the group) starts a full item with: neighbouring cells start with different ones,
+  // because the same window of neighbouring cells lies in the same shared-memory banks.
+  static __device__ __forceinline__ int first_window(int c) { return LPC == 4 ? (c >> 1) + (c & 1) : c; }
 };
 
 // Resident blocks per SM the push kernel is compiled for (register budget): FP32 2D fits two.
@@ -949,7 +948,8 @@ __device__ __noinline__ void deposit_general(T* sj, int lx, int ly, int lz, T ox
 // cell's lanes. Positions: x and y stay in their cell, z stays or steps up. Layouts: Jx (c*4 + b)*3 + a,
 // Jy (c*4 + a)*3 + b, Jz (b*4 + a)*4 + c, on nodes from one below the cell (origin `j`).
 template <typename T, int LPC, int COMP>
-__device__ __forceinline__ void deposit3_cubic(const T* st, int sl, int nrnd, int rnd0, T coef, T* j) {
+__device__ __forceinline__ void deposit3_cubic(const T* stq, const T* str, const T* stw, int sl, int nrnd, int rnd0,
+                                               T coef, T* j) {
   using S = PushSmem<T, 3, 3, true>;
   constexpr int NV = COMP == 2 ? 64 : 60, PER = (NV + LPC - 1) / LPC, NVP = PER * LPC;
   const int lane = threadIdx.x & 31;
@@ -958,8 +958,11 @@ __device__ __forceinline__ void deposit3_cubic(const T* st, int sl, int nrnd, in
   for (int i = 0; i < NVP; ++i) acc[i] = T(0);
 #pragma unroll 1
   for (int rnd = 0; rnd < nrnd; ++rnd) {
-    const T* q = st + sl + LPC * ((rnd + rnd0) & 3);
-    const T ox = q[0], oy = q[128], oz = q[256], dx = q[384], dy = q[512], dz = q[640], qw = coef * q[768];
+    const int k = sl + LPC * ((rnd + rnd0) & 3);
+    T q[4], e[2];
+    ld4(stq + 4 * k, q);
+    ld2(str + 2 * k, e);
+    const T ox = q[0], oy = q[1], oz = q[2], dx = q[3], dy = e[0], dz = e[1], qw = coef * stw[k];
     const T c = dz - (T(1) - oz);
     const CubicDir<T> X = cubic_dir(ox, dx, false, T(0)), Y = cubic_dir(oy, dy, false, T(0));
     const CubicDir<T> Z = cubic_dir(oz, dz, ge_one(oz + dz) && is_pos(c), c);
@@ -1088,26 +1091,36 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     scnt[cl] = 0;
     scnt[NCL + cl] = 0;
   }
+  // One item into a stage: slots [4 it LPC, 4 (it + 1) LPC) of the packs of the lane's cell, whose bin
+  // starts at slot bin0 and holds nq0 packs of species 0 of nq in all. The q values go slot by slot over
+  // the cell's lanes (neighbouring lanes copy neighbouring slots), the rest one pack per lane. fix: only
+  // the packs of species 1.
+  auto copy_item = [&](long long bin0, int it, int nq0, int nq, int stage, bool fix) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int k = j * LPC + sl, pk = it * LPC + (k >> 2);
+      if (pk >= nq || (fix && pk < nq0)) continue;
+      const bool s1 = pk >= nq0;
+      const long long slot = bin0 + 4 * (s1 ? pk - nq0 : pk) + (k & 3);
+      copy_async<4 * sizeof(T)>(SG::q(stg, stage, lane - sl) + 4 * k, (s1 ? r.in[1].q : r.in[0].q) + 4 * slot);
+    }
+    const int pk = it * LPC + sl;
+    if (pk >= nq || (fix && pk < nq0)) return;
+    const bool s1 = pk >= nq0;
+    const long long slot = bin0 + 4 * (s1 ? pk - nq0 : pk);
+    copy_async<4 * SG::RW * sizeof(T)>(SG::r(stg, stage, lane), (s1 ? r.in[1].r : r.in[0].r) + SG::RW * slot);
+    if (has_w) copy_async<4 * sizeof(T)>(SG::w(stg, stage, lane), (s1 ? r.in[1].w : r.in[0].w) + slot);
+    if (has_id) copy_async<16>(SG::id(stg, stage, lane), (s1 ? r.in[1].id : r.in[0].id) + slot);
+  };
   // The first item of the warp's first cell group, in the same batch although the counts are not in
-  // yet: lane sl takes pack sl of species 0, as it does whenever its cell holds more than 4 sl
-  // particles of species 0 (slots below cap: inside the cell's own bin). A lane whose first pack is
-  // of species 1 copies it again once the counts are known.
+  // yet: packs of species 0 only, as the item holds whenever its cell has that many (slots below cap, a
+  // multiple of 4: inside the cell's own bin). Its packs of species 1 are copied once the counts are known.
   {
     const int c = warp * CPW + lane / LPC;  // every warp has a first group (NCL / CPW >= NWARP)
     const int lx = c % TX, ly = (c / TX) % TY, lz = c / (TX * TY);
-    if (lx < wx && ly < wy && lz < wz && 4 * sl + 4 <= r.cap) {
-      const long long slot0 =
-          ((long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx) * r.cap + 4 * sl;
-      const SpeciesBuf<T>& pin = r.in[0];
-      const T* src[7] = {pin.ox, pin.oy, pin.oz, pin.dux, pin.duy, pin.duz, pin.w};
-#pragma unroll
-      for (int arr = 0; arr < 7; ++arr) {
-        if (arr == 1 && NDIM == 2) continue;
-        if (arr == 6 && !has_w) continue;
-        copy4_async(SG::at(stg, 0, arr, lane), src[arr] + slot0);
-      }
-      if (has_id) copy4_async(SG::id_at(stg, 0, lane), pin.id + slot0);
-    }
+    if (lx < wx && ly < wy && lz < wz)
+      copy_item(((long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx) * r.cap, 0, r.cap >> 2, r.cap >> 2, 0,
+                false);
   }
   static_assert(NCL / CPW >= NWARP, "every warp needs a first cell group");
   cp_async_commit();
@@ -1143,27 +1156,12 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     const int nq = ((sn[c] + 3) >> 2) + ((sn[NCL + c] + 3) >> 2);
     return __reduce_max_sync(0xffffffffu, (nq + LPC - 1) / LPC);
   };
-  // fix: only the packs the speculative first copy did not cover (species 1, or slots past cap)
   auto issue = [&](int g, int it, int stage, bool fix) {
     const int c = g * CPW + lane / LPC;
     const int n0 = sn[c], n1 = sn[NCL + c];
     const int nq0 = (n0 + 3) >> 2, nq = nq0 + ((n1 + 3) >> 2);
-    const int q = sl + it * LPC;
-    if (q >= nq) return;
-    const int s = q >= nq0 ? 1 : 0;
-    const int q4 = 4 * (s ? q - nq0 : q);
-    if (fix && s == 0 && q4 + 4 <= r.cap) return;
     const int lx = c % TX, ly = (c / TX) % TY, lz = c / (TX * TY);
-    const long long slot0 = ((long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx) * r.cap + q4;
-    const SpeciesBuf<T> pin = s ? r.in[1] : r.in[0];
-    const T* src[7] = {pin.ox, pin.oy, pin.oz, pin.dux, pin.duy, pin.duz, pin.w};
-#pragma unroll
-    for (int arr = 0; arr < 7; ++arr) {
-      if (arr == 1 && NDIM == 2) continue;
-      if (arr == 6 && !has_w) continue;
-      copy4_async(SG::at(stg, stage, arr, lane), src[arr] + slot0);
-    }
-    if (has_id) copy4_async(SG::id_at(stg, stage, lane), pin.id + slot0);
+    copy_item(((long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx) * r.cap, it, nq0, nq, stage, fix);
   };
 
   auto take_group = [&]() -> int {
@@ -1213,46 +1211,39 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     int nk = 4 * (nq - it * LPC);  // slots of the cell's packs from this item on, then the last pack's empty ones
     if (nk > 0 && nk <= 4 * LPC) nk -= 4 * (nq > nq0 ? nq - nq0 : nq0) - (nq > nq0 ? n1 : n0);
     const int nrnd = min(NR, (__reduce_max_sync(0xffffffffu, nk) + U * LPC - 1) / (U * LPC));
-    const int rnd0 = nrnd == NR ? PL::template first_round<T>(lane / LPC) : 0;
+    const int win0 = U == 2 || nrnd == NR ? PL::first_window(lane / LPC) : 0;
+    const T* stq = SG::q(stg, stage, lane - sl);  // slot k of the cell: stq[4 k], str[RW k], stw[k], sti[k]
+    const T* str = SG::r(stg, stage, lane - sl);
+    const T* stw = SG::w(stg, stage, lane - sl);
+    const unsigned* sti = SG::id(stg, stage, lane - sl);
+    // whether slot k of the cell's 4 LPC holds a particle, and its species
+    auto slot_of = [&](int k, int& s) -> bool {
+      const int q = it * LPC + (k >> 2);
+      s = q >= nq0 ? 1 : 0;
+      return q < nq && (s ? n1 + 4 * nq0 : n0) > 4 * q + (k & 3);
+    };
 #pragma unroll 1
     for (int rnd = 0; rnd < nrnd; ++rnd) {
-      // the lane's slots k .. k + U - 1 of the cell's 4 LPC slots in this item
-      const int k = U * (sl + LPC * ((rnd + rnd0) & (NR - 1)));
-      const int q = it * LPC + (k >> 2);
-      const bool has = q < nq;
-      const int s = (has && q >= nq0) ? 1 : 0;
-      const int cnt = has ? (s ? n1 + 4 * nq0 : n0) - 4 * q - (k & 3) : 0;  // particles from slot k on
-      const SpeciesBuf<T> pout = s ? r.out[1] : r.out[0];
-      const T qs = s ? T(1) : T(-1);
-      const T* st_x = SG::at(stg, stage, 0, lane - sl) + k;  // array a of slot k at st_x + slot(a) * 128
-      const unsigned* st_id = SG::id_at(stg, stage, lane - sl) + k;
       if constexpr (PushPaired<T, NDIM>::value) {
-        const float2 hh = make_float2(qs * r.hq, qs * r.hq);
         const float2 u02 = make_float2(r.u0, r.u0), one2 = make_float2(1.f, 1.f);
         const float2 dtdx2 = make_float2(r.dtdx, r.dtdx), dtdz2 = make_float2(r.dtdz, r.dtdz);
         const unsigned lt = (1u << lane) - 1u;
         {
-          constexpr int ja = 0, jb = 1;  // the pair: one 8-byte load per array
-          const bool va = cnt > 0, vb = cnt > 1;
-          const float2 pox = *reinterpret_cast<const float2*>(st_x + ja);
-          const float2 poz = *reinterpret_cast<const float2*>(st_x + SG::slot(2) * 128 + ja);
-          const float2 pux = *reinterpret_cast<const float2*>(st_x + SG::slot(3) * 128 + ja);
-          const float2 puy = *reinterpret_cast<const float2*>(st_x + SG::slot(4) * 128 + ja);
-          const float2 puz = *reinterpret_cast<const float2*>(st_x + SG::slot(5) * 128 + ja);
+          // the pair: the lane's slots in two windows
+          const int ka = sl + LPC * ((win0 + 2 * rnd) & (2 * nrnd - 1));
+          const int kb = sl + LPC * ((win0 + 2 * rnd + 1) & (2 * nrnd - 1));
+          int s_a, s_b;
+          const bool va = slot_of(ka, s_a), vb = slot_of(kb, s_b);
+          const float2 hh = make_float2(s_a ? r.hq : -r.hq, s_b ? r.hq : -r.hq);
+          float qa[4], qb[4];
+          ld4(stq + 4 * ka, qa);
+          ld4(stq + 4 * kb, qb);
           // an empty slot stands in as a particle at rest with no weight (finite, deposits nothing)
-          const float oxa = va ? pox.x : 0.5f, oza = va ? poz.x : 0.5f;
-          const float uxa = va ? pux.x : 0.f, uya = va ? puy.x : 0.f, uza = va ? puz.x : 0.f;
-          const float oxb = vb ? pox.y : 0.5f, ozb = vb ? poz.y : 0.5f;
-          const float uxb = vb ? pux.y : 0.f, uyb = vb ? puy.y : 0.f, uzb = vb ? puz.y : 0.f;
-          float wa = 0.f, wb = 0.f;
-          if (has_w) {
-            const float2 pw = *reinterpret_cast<const float2*>(st_x + SG::slot(6) * 128 + ja);
-            wa = va ? pw.x : 0.f;
-            wb = vb ? pw.y : 0.f;
-          } else {
-            wa = va ? r.wconst : 0.f;
-            wb = vb ? r.wconst : 0.f;
-          }
+          const float oxa = va ? qa[0] : 0.5f, oza = va ? qa[1] : 0.5f;
+          const float uxa = va ? qa[2] : 0.f, uya = va ? qa[3] : 0.f, uza = va ? str[ka] : 0.f;
+          const float oxb = vb ? qb[0] : 0.5f, ozb = vb ? qb[1] : 0.5f;
+          const float uxb = vb ? qb[2] : 0.f, uyb = vb ? qb[3] : 0.f, uzb = vb ? str[kb] : 0.f;
+          const float wa = va ? (has_w ? stw[ka] : r.wconst) : 0.f, wb = vb ? (has_w ? stw[kb] : r.wconst) : 0.f;
           // gather
           float2 F2[6];
           float Fa[6], Fb[6];
@@ -1326,7 +1317,7 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           const EsirDir<float> exa = esir_dir(oxa, dxa), eza = esir_dir(oza, dza);
           const EsirDir<float> exb = esir_dir(oxb, dxb), ezb = esir_dir(ozb, dzb);
           if (va) {
-            const float qw = qs * wa;
+            const float qw = s_a ? wa : -wa;
             const float cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vya * r.jfy2d;
             if constexpr (ORDER == 3) {
               if (reg_window<float, 2>(exa, exa, eza))
@@ -1337,7 +1328,7 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
             else deposit2_smem<float, NDIM>(sj, lx + exa.a + 1, lz + eza.a + 1, exa, eza, cx, cy, cz);
           }
           if (vb) {
-            const float qw = qs * wb;
+            const float qw = s_b ? wb : -wb;
             const float cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vyb * r.jfy2d;
             if constexpr (ORDER == 3) {
               if (reg_window<float, 2>(exb, exb, ezb))
@@ -1354,19 +1345,19 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           if (va) {
             const int nlx = lx + exa.shift, nlz = lz + eza.shift;
             if (nlx >= 0 && nlx < wx && nlz >= 0 && nlz < wz) {
-              dka = (nlz * TX + nlx) * 2 + s;
+              dka = (nlz * TX + nlx) * 2 + s_a;
             } else {
               lva = true;
-              dka = (wrap_near_p(gk + eza.shift, r.nz) * r.nx + wrap_near_p(gi + exa.shift, r.nx)) * 2 + s;
+              dka = (wrap_near_p(gk + eza.shift, r.nz) * r.nx + wrap_near_p(gi + exa.shift, r.nx)) * 2 + s_a;
             }
           }
           if (vb) {
             const int nlx = lx + exb.shift, nlz = lz + ezb.shift;
             if (nlx >= 0 && nlx < wx && nlz >= 0 && nlz < wz) {
-              dkb = (nlz * TX + nlx) * 2 + s;
+              dkb = (nlz * TX + nlx) * 2 + s_b;
             } else {
               lvb = true;
-              dkb = (wrap_near_p(gk + ezb.shift, r.nz) * r.nx + wrap_near_p(gi + exb.shift, r.nx)) * 2 + s;
+              dkb = (wrap_near_p(gk + ezb.shift, r.nz) * r.nx + wrap_near_p(gi + exb.shift, r.nx)) * 2 + s_b;
             }
           }
           // rebin of the pair: consecutive slots per (destination, species) for each particle of the
@@ -1408,13 +1399,11 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
             const int dcell = gcell + shz * r.nx + shx;  // a cell of this tile when st
             if (st && !full) {
               const long long o = (long long)dcell * r.cap + jo;
-              pout.ox[o] = nox;
-              pout.oz[o] = noz;
-              pout.dux[o] = ux;
-              pout.duy[o] = uy;
-              pout.duz[o] = uz;
-              if (has_w) pout.w[o] = w;
-              if (has_id) pout.id[o] = id;
+              const bool s1 = (dk & 1) != 0;
+              st4((s1 ? r.out[1].q : r.out[0].q) + 4 * o, nox, noz, ux, uy);
+              (s1 ? r.out[1].r : r.out[0].r)[o] = uz;
+              if (has_w) (s1 ? r.out[1].w : r.out[0].w)[o] = w;
+              if (has_id) (s1 ? r.out[1].id : r.out[0].id)[o] = id;
             } else if (g) {
               if (go < r.lv_cap) list_put(r.lv, go, full ? dcell * 2 + (dk & 1) : dk, nox, 0.f, noz, ux, uy, uz, w, id);
               else flag_error(r.err, ERR_OVERFLOW);
@@ -1430,25 +1419,38 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
             }
           };
           if (va)
-            place(sta, fa, lva, ga, dka, ba, lsa, goa, exa.off, eza.off, nuxa, nuya, nuza, wa, has_id ? st_id[ja] : 0u,
+            place(sta, fa, lva, ga, dka, ba, lsa, goa, exa.off, eza.off, nuxa, nuya, nuza, wa, has_id ? sti[ka] : 0u,
                   exa.shift, eza.shift);
           if (vb)
-            place(stb, fb, lvb, gb, dkb, bb, lsb, gob, exb.off, ezb.off, nuxb, nuyb, nuzb, wb, has_id ? st_id[jb] : 0u,
+            place(stb, fb, lvb, gb, dkb, bb, lsb, gob, exb.off, ezb.off, nuxb, nuyb, nuzb, wb, has_id ? sti[kb] : 0u,
                   exb.shift, ezb.shift);
         }
       } else {
       {
-        constexpr int jj = 0;
-        const bool valid = cnt > 0;
+        const int k = sl + LPC * ((rnd + win0) & 3);
+        int s;
+        const bool valid = slot_of(k, s);
+        const SpeciesBuf<T> pout = s ? r.out[1] : r.out[0];
+        const T qs = s ? T(1) : T(-1);
         int dkey = -1 - lane;  // unique per lane when there is no particle
         bool leave = false;
         T nox = T(0), noy = T(0), noz = T(0), ux = T(0), uy = T(0), uz = T(0);
-        const T w = (has_w && valid) ? st_x[SG::slot(6) * 128 + jj] : r.wconst;
+        const T w = (has_w && valid) ? stw[k] : r.wconst;
         if (valid) {
-          const T o_x = st_x[jj], o_y = NDIM == 3 ? st_x[SG::slot(1) * 128 + jj] : T(0), o_z = st_x[SG::slot(2) * 128 + jj];
-          ux = st_x[SG::slot(3) * 128 + jj];
-          uy = st_x[SG::slot(4) * 128 + jj];
-          uz = st_x[SG::slot(5) * 128 + jj];
+          T p4[4];
+          ld4(stq + 4 * k, p4);
+          const T o_x = p4[0], o_y = NDIM == 3 ? p4[1] : T(0), o_z = NDIM == 3 ? p4[2] : p4[1];
+          if constexpr (NDIM == 3) {
+            T p2[2];
+            ld2(str + 2 * k, p2);
+            ux = p4[3];
+            uy = p2[0];
+            uz = p2[1];
+          } else {
+            ux = p4[2];
+            uy = p4[3];
+            uz = str[k];
+          }
           // gather
           T F[6];
           if constexpr (WIN) {
@@ -1501,11 +1503,9 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           const T qw = qs * w;
           const bool own = reg_window<T, NDIM>(ex_, NDIM == 3 ? ey_ : ex_, ez_);
           if constexpr (LATE) {  // summed after the item's push, from the particle's stage slot
-            T* q = const_cast<T*>(st_x) + jj;
-            q[3 * 128] = ddx;
-            q[4 * 128] = ddy;
-            q[5 * 128] = ddz;
-            q[6 * 128] = own ? qw : T(0);
+            const_cast<T*>(stq)[4 * k + 3] = ddx;
+            st2(const_cast<T*>(str) + 2 * k, ddy, ddz);
+            const_cast<T*>(stw)[k] = own ? qw : T(0);
             if (!own)
               deposit_general<T, 3>(sj, lx, ly, lz, o_x, o_y, o_z, ddx, ddy, ddz, qw * r.jfx, qw * r.jfy, qw * r.jfz);
           } else if constexpr (ORDER == 3) {
@@ -1540,8 +1540,9 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           }
         }
         if (LATE && !valid) {  // an empty slot: finite values and no charge for the deposit
-#pragma unroll
-          for (int a = 0; a < 7; ++a) const_cast<T*>(st_x)[jj + a * 128] = T(0);
+          st4(const_cast<T*>(stq) + 4 * k, T(0), T(0), T(0), T(0));
+          st2(const_cast<T*>(str) + 2 * k, T(0), T(0));
+          const_cast<T*>(stw)[k] = T(0);
         }
         // rebin. Destination in this tile: lanes with the same (cell, species) reserve consecutive
         // slots with one shared-memory atomic on the tile's output counts. Destination in another
@@ -1593,16 +1594,11 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           const int dcell = ((Z0 + dz) * r.ny + Y0 + dy) * r.nx + X0 + dx;  // cells < 2^30
           if (!full) {
             const long long o = (long long)dcell * r.cap + j;
-            pout.ox[o] = nox;
-            if (NDIM == 3) pout.oy[o] = noy;
-            pout.oz[o] = noz;
-            pout.dux[o] = ux;
-            pout.duy[o] = uy;
-            pout.duz[o] = uz;
+            part_put(pout, NDIM, o, nox, noy, noz, ux, uy, uz);
             if (has_w) pout.w[o] = w;
-            if (has_id) pout.id[o] = st_id[jj];
+            if (has_id) pout.id[o] = sti[k];
           } else if (fglob < r.lv_cap) {
-            list_put(r.lv, fglob, dcell * 2 + (dkey & 1), nox, noy, noz, ux, uy, uz, w, has_id ? st_id[jj] : 0u);
+            list_put(r.lv, fglob, dcell * 2 + (dkey & 1), nox, noy, noz, ux, uy, uz, w, has_id ? sti[k] : 0u);
           } else {
             flag_error(r.err, ERR_OVERFLOW);
           }
@@ -1615,7 +1611,7 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           lvv[4 * S::LVB + lslot] = uy;
           lvv[5 * S::LVB + lslot] = uz;
           if (has_w) lvv[6 * S::LVB + lslot] = w;
-          if (has_id) lvi[lslot] = st_id[jj];
+          if (has_id) lvi[lslot] = sti[k];
         } else if (valid) {
           const long long o = lglob;
           if (o < r.lv_cap) {
@@ -1627,7 +1623,7 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
             r.lv.duy[o] = uy;
             r.lv.duz[o] = uz;
             if (has_w) r.lv.w[o] = w;
-            if (has_id) r.lv.id[o] = st_id[jj];
+            if (has_id) r.lv.id[o] = sti[k];
           } else {
             flag_error(r.err, ERR_OVERFLOW);
           }
@@ -1637,11 +1633,10 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     }
     if constexpr (LATE) {
       __syncwarp();
-      const T* st = SG::at(stg, stage, 0, lane - sl);
       T* j = sj + okey;
-      deposit3_cubic<T, LPC, 0>(st, sl, nrnd, rnd0, r.jfx, j);
-      deposit3_cubic<T, LPC, 1>(st, sl, nrnd, rnd0, r.jfy, j);
-      deposit3_cubic<T, LPC, 2>(st, sl, nrnd, rnd0, r.jfz, j);
+      deposit3_cubic<T, LPC, 0>(stq, str, stw, sl, nrnd, win0, r.jfx, j);
+      deposit3_cubic<T, LPC, 1>(stq, str, stw, sl, nrnd, win0, r.jfy, j);
+      deposit3_cubic<T, LPC, 2>(stq, str, stw, sl, nrnd, win0, r.jfz, j);
     }
     if (!LATE && it == giters - 1) {
       // 3. segmented transpose-reduction of the cell's register sums over its LPC lanes
