@@ -663,6 +663,11 @@ struct Lanes1 {
   static __device__ __forceinline__ V add(V a, V b) { return a + b; }
   static __device__ __forceinline__ V neg(V a) { return -a; }
   static __device__ __forceinline__ V pick_low(V a, V lo, V hi) { return a < T(0.5) ? lo : hi; }
+  using B = bool;
+  static __device__ __forceinline__ V sel(B m, V a, V b) { return m ? a : b; }
+};
+struct Bool2 {
+  bool x, y;
 };
 struct Lanes2 {
   using V = float2;
@@ -675,6 +680,8 @@ struct Lanes2 {
   static __device__ __forceinline__ V pick_low(V a, V lo, V hi) {
     return make_float2(a.x < 0.5f ? lo.x : hi.x, a.y < 0.5f ? lo.y : hi.y);
   }
+  using B = Bool2;
+  static __device__ __forceinline__ V sel(B m, V a, V b) { return make_float2(m.x ? a.x : b.x, m.y ? a.y : b.y); }
 };
 
 // Weights of the cubic spline on the nodes -1, 0, 1, 2 of the cell for an offset o in [0, 1].
@@ -778,7 +785,6 @@ template <typename T, int NDIM, int ORDER, int SCHEME>
 __device__ __forceinline__ void window_nodes(T* sg) {
   using S = PushSmem<T, NDIM, ORDER, true>;
   constexpr int NT = PushThreads<T, NDIM, ORDER>::value, NE = (6 * S::GN + NT - 1) / NT;
-  if (SCHEME != 2 && S::GCOPY == 1) return;
   const int tid = threadIdx.x;
   T v[NE];
 #pragma unroll
@@ -811,73 +817,158 @@ __device__ __forceinline__ void window_nodes(T* sg) {
   __syncthreads();
 }
 
+// One direction of a pair's move d from offsets o: the distance am to the upper face and the offset c
+// past it (d - am, without the rounding of o + d), whether each particle steps back (`down`) or into the
+// next cell (`up`), and the new cell shifts and offsets; the cases and rounding of esir_dir.
+struct PairMove {
+  float2 am, c;
+  Bool2 down, up;
+  int sha, shb;
+  float offa, offb;
+};
+__device__ __forceinline__ void move_one(float x1, float c, bool& down, bool& up, int& sh, float& off) {
+  down = x1 < 0.f;
+  const bool top = x1 >= 1.f;
+  up = top && c > 0.f;
+  const float below = 1.f + x1;
+  off = down ? below : (top ? (up ? c : 0.f) : x1);
+  sh = down ? -1 : (top ? 1 : 0);
+  if (down && below >= 1.f) {
+    off = 0.f;
+    sh = 0;
+  }
+}
+__device__ __forceinline__ PairMove pair_move(float2 o, float2 d) {
+  PairMove m;
+  const float2 x1 = __fadd2_rn(o, d);
+  m.am = __fadd2_rn(make_float2(1.f, 1.f), make_float2(-o.x, -o.y));
+  m.c = __fadd2_rn(d, make_float2(-m.am.x, -m.am.y));
+  move_one(x1.x, m.c.x, m.down.x, m.up.x, m.sha, m.offa);
+  move_one(x1.y, m.c.y, m.down.y, m.up.y, m.shb, m.offb);
+  return m;
+}
+
+// The contributions of deposit2_reg for a pair, in packed arithmetic, one accumulator half per particle:
+// with e0 = am or d (into the next cell or not) and e2 = c or 0, the shape changes are -e0, e0 - e2, e2.
+// The coefficients of a particle that does not fit the register window are zero.
+template <int NVP>
+__device__ __forceinline__ void deposit2_pair(float2 (&acc)[NVP], float2 ox, float2 dx, const PairMove& X, float2 oz,
+                                              float2 dz, const PairMove& Z, float2 cx, float2 cy, float2 cz) {
+  const float2 half = make_float2(0.5f, 0.5f), mhalf = make_float2(-0.5f, -0.5f);
+  const float2 e0 = Lanes2::sel(Z.up, Z.am, dz), e2 = Lanes2::sel(Z.up, Z.c, make_float2(0.f, 0.f));
+  const float2 e1 = __fadd2_rn(e0, Lanes2::neg(e2));
+  const float2 fx0 = __ffma2_rn(mhalf, dx, X.am), fx1 = __ffma2_rn(half, dx, ox);
+  const float2 fz[3] = {__ffma2_rn(mhalf, e0, Z.am), __ffma2_rn(half, e1, oz), __fmul2_rn(half, e2)};
+  const float2 dS[3] = {Lanes2::neg(e0), e1, e2};
+  const float2 gx0 = Lanes2::neg(__fmul2_rn(cx, dx));
+#pragma unroll
+  for (int b = 0; b < 3; ++b) acc[b] = __ffma2_rn(gx0, fz[b], acc[b]);
+  const float2 gz0 = Lanes2::neg(__fmul2_rn(cz, e0)), gz1 = Lanes2::neg(__fmul2_rn(cz, e2));
+  acc[3] = __ffma2_rn(gz0, fx0, acc[3]);
+  acc[4] = __ffma2_rn(gz1, fx0, acc[4]);
+  acc[5] = __ffma2_rn(gz0, fx1, acc[5]);
+  acc[6] = __ffma2_rn(gz1, fx1, acc[6]);
+  const float2 hx0 = __fmul2_rn(cy, fx0), hx1 = __fmul2_rn(cy, fx1);
+  const float2 kx1 = __fmul2_rn(__fmul2_rn(cy, dx), make_float2(1.f / 12.f, 1.f / 12.f)), kx0 = Lanes2::neg(kx1);
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    acc[7 + 2 * b] = __ffma2_rn(hx0, fz[b], __ffma2_rn(kx0, dS[b], acc[7 + 2 * b]));
+    acc[8 + 2 * b] = __ffma2_rn(hx1, fz[b], __ffma2_rn(kx1, dS[b], acc[8 + 2 * b]));
+  }
+}
+// A particle of a pair outside the register window: its full window, into shared memory.
+template <typename T>
+__device__ __noinline__ void deposit2_far(T* sj, int lx, int lz, T ox, T oz, T dx, T dz, T cx, T cy, T cz) {
+  const EsirDir<T> X = esir_dir(ox, dx), Z = esir_dir(oz, dz);
+  deposit2_smem<T, 2>(sj, lx + X.a + 1, lz + Z.a + 1, X, Z, cx, cy, cz);
+}
+
 // One direction of a cubic Esirkepov move: S0 + dS / 2 and the shape change dS on the nodes -1 .. 3 of
 // the start cell for a move d that stays in the cell or enters the next one up (`up`, at offset c
 // there), formed from the displacement itself on one polynomial piece (full relative precision for small
-// moves) and as the difference across the face.
-template <typename T>
+// moves) and as the difference across the face. One particle or (Lanes2) a pair.
+template <typename V>
 struct CubicDir {
-  T m[5], dS[5];
+  V m[5], dS[5];
 };
-template <typename T>
-__device__ __forceinline__ CubicDir<T> cubic_dir(T o, T d, bool up, T c) {
-  CubicDir<T> r;
-  T s[4];
-  cubic_weights<Lanes1<T>, T, T>(o, s);
-  const T p = T(1) - o, d2 = d * d, d6 = d * T(1.0 / 6.0);
-  T e0 = -d6 * (T(3) * p * (p - d) + d2);
-  T e3 = d6 * (T(3) * o * (o + d) + d2);
-  T e1 = d * (T(1.5) * o * (o + d) - T(2) * o - d + T(0.5) * d2);
-  T e2 = -(e0 + e1 + e3), e4 = T(0);
-  if (up) {
-    T n[4];
-    cubic_weights<Lanes1<T>, T, T>(c, n);
-    e0 = -s[0];
-    e1 = n[0] - s[1];
-    e2 = n[1] - s[2];
-    e3 = n[2] - s[3];
-    e4 = n[3];
-  }
-  r.dS[0] = e0; r.dS[1] = e1; r.dS[2] = e2; r.dS[3] = e3; r.dS[4] = e4;
+template <class L, typename T, bool UP>
+__device__ __forceinline__ CubicDir<typename L::V> cubic_dir(typename L::V o, typename L::V d, typename L::B up,
+                                                             typename L::V c) {
+  using V = typename L::V;
+  CubicDir<V> r;
+  V s[4], e[5];
+  cubic_weights<L, T, V>(o, s);
+  const V p = L::add(L::set(T(1)), L::neg(o)), d2 = L::mul(d, d), d6 = L::mul(d, L::set(T(1.0 / 6.0)));
+  const V three = L::set(T(3));
+  const V pd = L::mul(p, L::add(p, L::neg(d))), od = L::mul(o, L::add(o, d));
+  e[0] = L::neg(L::mul(d6, L::fma(three, pd, d2)));
+  e[3] = L::mul(d6, L::fma(three, od, d2));
+  e[1] = L::mul(d, L::fma(L::set(T(1.5)), od, L::fma(L::set(T(-2)), o, L::fma(L::set(T(0.5)), d2, L::neg(d)))));
+  e[2] = L::neg(L::add(L::add(e[0], e[1]), e[3]));
+  e[4] = L::set(T(0));
+  if constexpr (UP) {
+    V n[4];
+    cubic_weights<L, T, V>(c, n);
+    e[0] = L::sel(up, L::neg(s[0]), e[0]);
 #pragma unroll
-  for (int a = 0; a < 4; ++a) r.m[a] = s[a] + T(0.5) * r.dS[a];
-  r.m[4] = T(0.5) * e4;
+    for (int a = 1; a < 4; ++a) e[a] = L::sel(up, L::add(n[a - 1], L::neg(s[a])), e[a]);
+    e[4] = L::sel(up, n[3], e[4]);
+  }
+#pragma unroll
+  for (int a = 0; a < 5; ++a) r.dS[a] = e[a];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) r.m[a] = L::fma(L::set(T(0.5)), e[a], s[a]);
+  r.m[4] = L::mul(L::set(T(0.5)), e[4]);
   return r;
 }
 // running sums of dS, the weights of the current on the four edges (all five dS sum to zero)
-template <typename T>
-__device__ __forceinline__ void cubic_run(const CubicDir<T>& r, T (&P)[4]) {
+template <class L, typename V>
+__device__ __forceinline__ void cubic_run(const CubicDir<V>& r, V (&P)[4]) {
   P[0] = r.dS[0];
-  P[1] = r.dS[0] + r.dS[1];
-  P[2] = -(r.dS[3] + r.dS[4]);
-  P[3] = -r.dS[4];
+  P[1] = L::add(r.dS[0], r.dS[1]);
+  P[2] = L::neg(L::add(r.dS[3], r.dS[4]));
+  P[3] = L::neg(r.dS[4]);
 }
 
-// 2D cubic deposit into the register layout: x stays in its cell, z stays or steps up.
-template <typename T, int NVP>
-__device__ __forceinline__ void deposit2_cubic(T (&acc)[NVP], const CubicDir<T>& X, const CubicDir<T>& Z, T cx, T cy,
-                                               T cz) {
-  T PX[4], PZ[4];
-  cubic_run(X, PX);
-  cubic_run(Z, PZ);
+// acc += a b for one particle, or for both of a pair
+template <typename T>
+__device__ __forceinline__ void add_prod(T& acc, T a, T b) {
+  acc += a * b;
+}
+__device__ __forceinline__ void add_prod(float& acc, float2 a, float2 b) {
+  acc = fmaf(a.x, b.x, acc);
+  acc = fmaf(a.y, b.y, acc);
+}
+
+// 2D cubic deposit into the register layout: x stays in its cell, z stays or steps up (a particle that
+// does otherwise comes with zero coefficients).
+template <class L, typename T, int NVP, typename V>
+__device__ __forceinline__ void deposit2_cubic(T (&acc)[NVP], const CubicDir<V>& X, const CubicDir<V>& Z, V cx, V cy,
+                                               V cz) {
+  V PX[4], PZ[4];
+  cubic_run<L>(X, PX);
+  cubic_run<L>(Z, PZ);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const T g = cx * PX[a];
+    const V g = L::mul(cx, PX[a]);
 #pragma unroll
-    for (int c = 0; c < 5; ++c) acc[c * 3 + a] += g * Z.m[c];
+    for (int c = 0; c < 5; ++c) add_prod(acc[c * 3 + a], g, Z.m[c]);
   }
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    const T g = cz * PZ[c];
+    const V g = L::mul(cz, PZ[c]);
 #pragma unroll
-    for (int a = 0; a < 4; ++a) acc[15 + a * 4 + c] += g * X.m[a];
+    for (int a = 0; a < 4; ++a) add_prod(acc[15 + a * 4 + c], g, X.m[a]);
   }
-  const T k = cy * T(1.0 / 12.0);
+  const V k = L::mul(cy, L::set(T(1.0 / 12.0)));
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
-    const T h = cy * X.m[a], q = k * X.dS[a];
+    const V h = L::mul(cy, X.m[a]), q = L::mul(k, X.dS[a]);
 #pragma unroll
-    for (int c = 0; c < 5; ++c) acc[31 + c * 4 + a] += h * Z.m[c] + q * Z.dS[c];
+    for (int c = 0; c < 5; ++c) {
+      add_prod(acc[31 + c * 4 + a], h, Z.m[c]);
+      add_prod(acc[31 + c * 4 + a], q, Z.dS[c]);
+    }
   }
 }
 
@@ -964,14 +1055,15 @@ __device__ __forceinline__ void deposit3_cubic(const T* stq, const T* str, const
     ld2(str + 2 * k, e);
     const T ox = q[0], oy = q[1], oz = q[2], dx = q[3], dy = e[0], dz = e[1], qw = coef * stw[k];
     const T c = dz - (T(1) - oz);
-    const CubicDir<T> X = cubic_dir(ox, dx, false, T(0)), Y = cubic_dir(oy, dy, false, T(0));
-    const CubicDir<T> Z = cubic_dir(oz, dz, ge_one(oz + dz) && is_pos(c), c);
+    using L1 = Lanes1<T>;
+    const CubicDir<T> X = cubic_dir<L1, T, false>(ox, dx, false, T(0)), Y = cubic_dir<L1, T, false>(oy, dy, false, T(0));
+    const CubicDir<T> Z = cubic_dir<L1, T, true>(oz, dz, ge_one(oz + dz) && is_pos(c), c);
     const CubicDir<T>& A = COMP == 0 ? X : (COMP == 1 ? Y : Z);  // along the component
     const CubicDir<T>& B = COMP == 0 ? Y : X;                    // the fast transverse direction
     const CubicDir<T>& C = COMP == 2 ? Y : Z;                    // the slow one (Z: five nodes)
     constexpr int NA = COMP == 2 ? 4 : 3, NC = COMP == 2 ? 4 : 5;
     T P[4];
-    cubic_run(A, P);
+    cubic_run<L1>(A, P);
 #pragma unroll
     for (int a = 0; a < NA; ++a) P[a] *= qw;
 #pragma unroll
@@ -1143,7 +1235,7 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     s_next_group = PUSH_THREADS / 32;
   }
   __syncthreads();
-  if constexpr (WIN) window_nodes<T, NDIM, ORDER, SCHEME>(sg);
+  if constexpr (SCHEME == 2 || S::GCOPY == 2) window_nodes<T, NDIM, ORDER, SCHEME>(sg);
 
   T kin = T(0);
   int npush = 0;
@@ -1178,7 +1270,10 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   int stage = 0;
   if (g < NGRP) issue(g, 0, 0, g == warp);  // the first group's first item was copied speculatively
   cp_async_commit();
+  // the register sums; a linear paired push keeps one half per particle of the pair until the group's end
+  constexpr bool ACC2 = PushPaired<T, NDIM>::value && ORDER == 1;
   T acc[NVP];
+  float2 acc2[ACC2 ? NVP : 1];
   GalCache<T, NDIM> gc;  // Galerkin nodes of the lane's cell, loaded once per cell group
   while (g < NGRP) {
     // prefetch the next item
@@ -1205,6 +1300,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
       if (SCHEME == 0 && !WIN) gc.load(sg, lx, ly, lz);
 #pragma unroll
       for (int i = 0; i < NVP; ++i) acc[i] = T(0);
+#pragma unroll
+      for (int i = 0; i < (ACC2 ? NVP : 1); ++i) acc2[i] = make_float2(0.f, 0.f);
     }
     // rounds of this item: up to the last slot in use of the fullest cell
     constexpr int NR = PushRounds<T, NDIM>::value, U = 4 / NR;
@@ -1313,51 +1410,54 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
             flag_error(r.err, ERR_NONFINITE);
             dxb = dzb = nuxb = nuyb = nuzb = vyb = 0.f;
           }
-          // Esirkepov deposits
-          const EsirDir<float> exa = esir_dir(oxa, dxa), eza = esir_dir(oza, dza);
-          const EsirDir<float> exb = esir_dir(oxb, dxb), ezb = esir_dir(ozb, dzb);
-          if (va) {
-            const float qw = s_a ? wa : -wa;
-            const float cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vya * r.jfy2d;
-            if constexpr (ORDER == 3) {
-              if (reg_window<float, 2>(exa, exa, eza))
-                deposit2_cubic<float, NVP>(acc, cubic_dir(oxa, dxa, false, 0.f),
-                                           cubic_dir(oza, dza, eza.dS[2] != 0.f, eza.off), cx, cy, cz);
-              else deposit_general<float, 2>(sj, lx, 0, lz, oxa, 0.f, oza, dxa, 0.f, dza, cx, cy, cz);
-            } else if (reg_window<float, 2>(exa, exa, eza)) deposit2_reg<float, NVP>(acc, exa, eza, cx, cy, cz);
-            else deposit2_smem<float, NDIM>(sj, lx + exa.a + 1, lz + eza.a + 1, exa, eza, cx, cy, cz);
+          // Esirkepov deposits: in registers where the window fits (RegLayout), the coefficients zero
+          // otherwise, and the rest (a step back or across an x face) to shared memory
+          const float2 o_x = make_float2(oxa, oxb), o_z = make_float2(oza, ozb);
+          const float2 d_x = make_float2(dxa, dxb), d_z = make_float2(dza, dzb);
+          const PairMove X = pair_move(o_x, d_x), Z = pair_move(o_z, d_z);
+          const bool rega = !(X.down.x || X.up.x || Z.down.x), regb = !(X.down.y || X.up.y || Z.down.y);
+          const float2 qw = make_float2(s_a ? wa : -wa, s_b ? wb : -wb);
+          const float2 qr = make_float2(rega ? qw.x : 0.f, regb ? qw.y : 0.f);
+          const float2 jx2 = make_float2(r.jfx, r.jfx), jy2 = make_float2(r.jfy2d, r.jfy2d), jz2 = make_float2(r.jfz, r.jfz);
+          const float2 vyp = make_float2(vya, vyb);
+          if constexpr (ORDER == 3)
+            deposit2_cubic<Lanes2, float, NVP, float2>(acc, cubic_dir<Lanes2, float, false>(o_x, d_x, Bool2{}, o_x),
+                                                       cubic_dir<Lanes2, float, true>(o_z, d_z, Z.up, Z.c), mul2(qr, jx2),
+                                                       mul2(mul2(qr, vyp), jy2), mul2(qr, jz2));
+          else
+            deposit2_pair<NVP>(acc2, o_x, d_x, X, o_z, d_z, Z, mul2(qr, jx2), mul2(mul2(qr, vyp), jy2), mul2(qr, jz2));
+          if (!rega && va) {
+            if constexpr (ORDER == 3)
+              deposit_general<float, 2>(sj, lx, 0, lz, oxa, 0.f, oza, dxa, 0.f, dza, qw.x * r.jfx, qw.x * vya * r.jfy2d,
+                                        qw.x * r.jfz);
+            else deposit2_far(sj, lx, lz, oxa, oza, dxa, dza, qw.x * r.jfx, qw.x * vya * r.jfy2d, qw.x * r.jfz);
           }
-          if (vb) {
-            const float qw = s_b ? wb : -wb;
-            const float cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vyb * r.jfy2d;
-            if constexpr (ORDER == 3) {
-              if (reg_window<float, 2>(exb, exb, ezb))
-                deposit2_cubic<float, NVP>(acc, cubic_dir(oxb, dxb, false, 0.f),
-                                           cubic_dir(ozb, dzb, ezb.dS[2] != 0.f, ezb.off), cx, cy, cz);
-              else deposit_general<float, 2>(sj, lx, 0, lz, oxb, 0.f, ozb, dxb, 0.f, dzb, cx, cy, cz);
-            } else if (reg_window<float, 2>(exb, exb, ezb)) deposit2_reg<float, NVP>(acc, exb, ezb, cx, cy, cz);
-            else deposit2_smem<float, NDIM>(sj, lx + exb.a + 1, lz + ezb.a + 1, exb, ezb, cx, cy, cz);
+          if (!regb && vb) {
+            if constexpr (ORDER == 3)
+              deposit_general<float, 2>(sj, lx, 0, lz, oxb, 0.f, ozb, dxb, 0.f, dzb, qw.y * r.jfx, qw.y * vyb * r.jfy2d,
+                                        qw.y * r.jfz);
+            else deposit2_far(sj, lx, lz, oxb, ozb, dxb, dzb, qw.y * r.jfx, qw.y * vyb * r.jfy2d, qw.y * r.jfz);
           }
           // destinations: a cell of this tile (key (cell * 2 + species) in the tile) or, leaving
           // the tile, the global cell (key global cell * 2 + species)
           int dka = -1 - lane, dkb = -1 - lane;
           bool lva = false, lvb = false;
           if (va) {
-            const int nlx = lx + exa.shift, nlz = lz + eza.shift;
+            const int nlx = lx + X.sha, nlz = lz + Z.sha;
             if (nlx >= 0 && nlx < wx && nlz >= 0 && nlz < wz) {
               dka = (nlz * TX + nlx) * 2 + s_a;
             } else {
               lva = true;
-              dka = (wrap_near_p(gk + eza.shift, r.nz) * r.nx + wrap_near_p(gi + exa.shift, r.nx)) * 2 + s_a;
+              dka = (wrap_near_p(gk + Z.sha, r.nz) * r.nx + wrap_near_p(gi + X.sha, r.nx)) * 2 + s_a;
             }
           }
           if (vb) {
-            const int nlx = lx + exb.shift, nlz = lz + ezb.shift;
+            const int nlx = lx + X.shb, nlz = lz + Z.shb;
             if (nlx >= 0 && nlx < wx && nlz >= 0 && nlz < wz) {
               dkb = (nlz * TX + nlx) * 2 + s_b;
             } else {
               lvb = true;
-              dkb = (wrap_near_p(gk + ezb.shift, r.nz) * r.nx + wrap_near_p(gi + exb.shift, r.nx)) * 2 + s_b;
+              dkb = (wrap_near_p(gk + Z.shb, r.nz) * r.nx + wrap_near_p(gi + X.shb, r.nx)) * 2 + s_b;
             }
           }
           // rebin of the pair: consecutive slots per (destination, species) for each particle of the
@@ -1419,11 +1519,11 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
             }
           };
           if (va)
-            place(sta, fa, lva, ga, dka, ba, lsa, goa, exa.off, eza.off, nuxa, nuya, nuza, wa, has_id ? sti[ka] : 0u,
-                  exa.shift, eza.shift);
+            place(sta, fa, lva, ga, dka, ba, lsa, goa, X.offa, Z.offa, nuxa, nuya, nuza, wa, has_id ? sti[ka] : 0u,
+                  X.sha, Z.sha);
           if (vb)
-            place(stb, fb, lvb, gb, dkb, bb, lsb, gob, exb.off, ezb.off, nuxb, nuyb, nuzb, wb, has_id ? sti[kb] : 0u,
-                  exb.shift, ezb.shift);
+            place(stb, fb, lvb, gb, dkb, bb, lsb, gob, X.offb, Z.offb, nuxb, nuyb, nuzb, wb, has_id ? sti[kb] : 0u,
+                  X.shb, Z.shb);
         }
       } else {
       {
@@ -1511,8 +1611,9 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           } else if constexpr (ORDER == 3) {
             const T cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vy * r.jfy2d;
             if (own)
-              deposit2_cubic<T, NVP>(acc, cubic_dir(o_x, ddx, false, T(0)),
-                                     cubic_dir(o_z, ddz, !is_zero(ez_.dS[2]), ez_.off), cx, cy, cz);
+              deposit2_cubic<Lanes1<T>, T, NVP, T>(acc, cubic_dir<Lanes1<T>, T, false>(o_x, ddx, false, T(0)),
+                                                   cubic_dir<Lanes1<T>, T, true>(o_z, ddz, !is_zero(ez_.dS[2]), ez_.off),
+                                                   cx, cy, cz);
             else deposit_general<T, 2>(sj, lx, 0, lz, o_x, T(0), o_z, ddx, T(0), ddz, cx, cy, cz);
           } else if (NDIM == 2) {
             const T cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vy * r.jfy2d;
@@ -1640,6 +1741,10 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     }
     if (!LATE && it == giters - 1) {
       // 3. segmented transpose-reduction of the cell's register sums over its LPC lanes
+      if constexpr (ACC2) {
+#pragma unroll
+        for (int i = 0; i < NVP; ++i) acc[i] = acc2[i].x + acc2[i].y;
+      }
 #pragma unroll
       for (int sh = LPC / 2; sh >= 1; sh >>= 1) {
         const bool up = (lane & sh) != 0;
