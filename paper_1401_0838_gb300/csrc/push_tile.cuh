@@ -372,7 +372,7 @@ __device__ __forceinline__ void deposit2(T (&acc)[NVP], const EsirDir<T>& X, con
 
 // Same contributions added to shared memory at the window origin (wx, wz) (tile indices).
 template <typename T, int NDIM>
-__device__ __noinline__ void deposit2_smem(T* sj, int wx, int wz, EsirDir<T> X, EsirDir<T> Z, T cx, T cy, T cz) {
+__device__ __forceinline__ void deposit2_smem(T* sj, int wx, int wz, EsirDir<T> X, EsirDir<T> Z, T cx, T cy, T cz) {
   using S = PushSmem<T, NDIM>;
   T v[DepLayout<2>::NV];
 #pragma unroll
@@ -430,7 +430,7 @@ __device__ __forceinline__ void deposit3(T (&acc)[NVP], const EsirDir<T>& X, con
 }
 
 template <typename T, int NDIM>
-__device__ __noinline__ void deposit3_smem(T* sj, int wx, int wy, int wz, EsirDir<T> X, EsirDir<T> Y, EsirDir<T> Z,
+__device__ __forceinline__ void deposit3_smem(T* sj, int wx, int wy, int wz, EsirDir<T> X, EsirDir<T> Y, EsirDir<T> Z,
                                            T cx, T cy, T cz) {
   using S = PushSmem<T, NDIM>;
   T v[DepLayout<3>::NV];
@@ -492,72 +492,6 @@ struct RegLayout<3, 1> {
     else { const int k = i - 12; comp = 2; c = k & 1; a = (k >> 1) & 1; b = k >> 2; }
   }
 };
-
-// Whether a particle's window fits the register sums (see RegLayout).
-template <typename T, int NDIM>
-__device__ __forceinline__ bool reg_window(const EsirDir<T>& X, const EsirDir<T>& Y, const EsirDir<T>& Z) {
-  if (NDIM == 3) return (X.a | Y.a | Z.a) == 0 && is_zero(X.dS[2]) && is_zero(Y.dS[2]);
-  return (X.a | Z.a) == 0 && is_zero(X.dS[2]);
-}
-
-// The contributions of deposit2 / deposit3 that can be nonzero for such a particle, into the
-// register layout (the same products and sums as the full window).
-template <typename T, int NVP>
-__device__ __forceinline__ void deposit2_reg(T (&acc)[NVP], const EsirDir<T>& X, const EsirDir<T>& Z, T cx, T cy,
-                                             T cz) {
-  const T fx0 = X.S0[0] + T(0.5) * X.dS[0], fx1 = X.S0[1] + T(0.5) * X.dS[1];
-  T fz[3];
-#pragma unroll
-  for (int b = 0; b < 3; ++b) fz[b] = Z.S0[b] + T(0.5) * Z.dS[b];
-  const T gx0 = cx * X.dS[0];
-#pragma unroll
-  for (int b = 0; b < 3; ++b) acc[b] += gx0 * fz[b];
-  const T gz0 = cz * Z.dS[0], gz1 = -cz * Z.dS[2];
-  acc[3] += gz0 * fx0;
-  acc[4] += gz1 * fx0;
-  acc[5] += gz0 * fx1;
-  acc[6] += gz1 * fx1;
-  const T hx0 = cy * fx0, hx1 = cy * fx1;
-  const T kx0 = cy * X.dS[0] * T(1.0 / 12.0), kx1 = cy * X.dS[1] * T(1.0 / 12.0);
-#pragma unroll
-  for (int b = 0; b < 3; ++b) {
-    acc[7 + 2 * b] += hx0 * fz[b] + kx0 * Z.dS[b];
-    acc[8 + 2 * b] += hx1 * fz[b] + kx1 * Z.dS[b];
-  }
-}
-
-template <typename T, int NVP>
-__device__ __forceinline__ void deposit3_reg(T (&acc)[NVP], const EsirDir<T>& X, const EsirDir<T>& Y,
-                                             const EsirDir<T>& Z, T cx, T cy, T cz) {
-  T fx[2], fy[2], fz[3], kx[2], ky[2];
-#pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    fx[a] = X.S0[a] + T(0.5) * X.dS[a];
-    fy[a] = Y.S0[a] + T(0.5) * Y.dS[a];
-    kx[a] = X.dS[a] * T(1.0 / 12.0);
-    ky[a] = Y.dS[a] * T(1.0 / 12.0);
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) fz[c] = Z.S0[c] + T(0.5) * Z.dS[c];
-  const T gx0 = cx * X.dS[0], gy0 = cy * Y.dS[0];
-  const T gz0 = cz * Z.dS[0], gz1 = -cz * Z.dS[2];
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int b = 0; b < 2; ++b) acc[c * 2 + b] += gx0 * (fy[b] * fz[c] + ky[b] * Z.dS[c]);  // Jx(1/2, b, c)
-#pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int a = 0; a < 2; ++a) acc[6 + c * 2 + a] += gy0 * (fx[a] * fz[c] + kx[a] * Z.dS[c]);  // Jy(a, 1/2, c)
-#pragma unroll
-  for (int b = 0; b < 2; ++b)
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {  // Jz(a, b, c + 1/2)
-      const T t = fx[a] * fy[b] + kx[a] * Y.dS[b];
-      acc[12 + (b * 2 + a) * 2 + 0] += gz0 * t;
-      acc[12 + (b * 2 + a) * 2 + 1] += gz1 * t;
-    }
-}
 
 // Rounds of a full item: 4 particles a lane, one or (paired) two per round.
 template <typename T, int NDIM>
@@ -658,7 +592,7 @@ struct Lanes1 {
   using V = T;
   static __device__ __forceinline__ V set(T a) { return a; }
   static __device__ __forceinline__ V node(const T* p) { return *p; }
-  static __device__ __forceinline__ V fma(V a, V b, V c) { return a * b + c; }
+  static __device__ __forceinline__ V fma(V a, V b, V c) { return ::fma(a, b, c); }
   static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
   static __device__ __forceinline__ V add(V a, V b) { return a + b; }
   static __device__ __forceinline__ V neg(V a) { return -a; }
@@ -817,27 +751,38 @@ __device__ __forceinline__ void window_nodes(T* sg) {
   __syncthreads();
 }
 
-// One direction of a pair's move d from offsets o: the distance am to the upper face and the offset c
-// past it (d - am, without the rounding of o + d), whether each particle steps back (`down`) or into the
-// next cell (`up`), and the new cell shifts and offsets; the cases and rounding of esir_dir.
+// One direction of a move d from offset o: the distance am to the upper face and the offset c past it
+// (d - am, without the rounding of o + d), whether the particle steps back (`down`) or into the next cell
+// (`up`), and its new cell shift and offset; the cases and rounding of esir_dir, without branches (a
+// divergent branch costs the FP64 pipe both sides).
+template <typename T>
+__device__ __forceinline__ void move_one(T x1, T c, bool& down, bool& up, int& sh, T& off) {
+  down = is_neg(x1);
+  const bool top = !down && ge_one(x1);
+  up = top && is_pos(c);
+  const T below = T(1) + x1;
+  const bool back = down && ge_one(below);  // rounding put it back on this cell's lower face
+  off = down ? (back ? T(0) : below) : (top ? (up ? c : T(0)) : x1);
+  sh = down ? (back ? 0 : -1) : (top ? 1 : 0);
+}
+template <typename T>
+struct Move1 {
+  T am, c, off;
+  bool down, up;
+  int sh;
+  __device__ __forceinline__ Move1(T o, T d) {
+    am = T(1) - o;
+    c = d - am;
+    move_one(o + d, c, down, up, sh, off);
+  }
+};
+// The same for a pair.
 struct PairMove {
   float2 am, c;
   Bool2 down, up;
   int sha, shb;
   float offa, offb;
 };
-__device__ __forceinline__ void move_one(float x1, float c, bool& down, bool& up, int& sh, float& off) {
-  down = x1 < 0.f;
-  const bool top = x1 >= 1.f;
-  up = top && c > 0.f;
-  const float below = 1.f + x1;
-  off = down ? below : (top ? (up ? c : 0.f) : x1);
-  sh = down ? -1 : (top ? 1 : 0);
-  if (down && below >= 1.f) {
-    off = 0.f;
-    sh = 0;
-  }
-}
 __device__ __forceinline__ PairMove pair_move(float2 o, float2 d) {
   PairMove m;
   const float2 x1 = __fadd2_rn(o, d);
@@ -848,39 +793,87 @@ __device__ __forceinline__ PairMove pair_move(float2 o, float2 d) {
   return m;
 }
 
-// The contributions of deposit2_reg for a pair, in packed arithmetic, one accumulator half per particle:
-// with e0 = am or d (into the next cell or not) and e2 = c or 0, the shape changes are -e0, e0 - e2, e2.
-// The coefficients of a particle that does not fit the register window are zero.
-template <int NVP>
-__device__ __forceinline__ void deposit2_pair(float2 (&acc)[NVP], float2 ox, float2 dx, const PairMove& X, float2 oz,
-                                              float2 dz, const PairMove& Z, float2 cx, float2 cy, float2 cz) {
-  const float2 half = make_float2(0.5f, 0.5f), mhalf = make_float2(-0.5f, -0.5f);
-  const float2 e0 = Lanes2::sel(Z.up, Z.am, dz), e2 = Lanes2::sel(Z.up, Z.c, make_float2(0.f, 0.f));
-  const float2 e1 = __fadd2_rn(e0, Lanes2::neg(e2));
-  const float2 fx0 = __ffma2_rn(mhalf, dx, X.am), fx1 = __ffma2_rn(half, dx, ox);
-  const float2 fz[3] = {__ffma2_rn(mhalf, e0, Z.am), __ffma2_rn(half, e1, oz), __fmul2_rn(half, e2)};
-  const float2 dS[3] = {Lanes2::neg(e0), e1, e2};
-  const float2 gx0 = Lanes2::neg(__fmul2_rn(cx, dx));
+// The shapes of a linear move that fits the register window: f = S0 + dS / 2 on the cell's nodes. A
+// transverse direction stays in its cell (dS = -d, d); along z, with e0 = am or d (into the next cell or
+// not) and e2 = c or 0, the shape changes are -e0, e0 - e2, e2.
+template <class L, typename T>
+struct LinearZ {
+  using V = typename L::V;
+  V e0, e1, e2, f0, f1, f2;
+  __device__ __forceinline__ LinearZ(V o, V d, V am, V c, typename L::B up) {
+    e0 = L::sel(up, am, d);
+    e2 = L::sel(up, c, L::set(T(0)));
+    e1 = L::add(e0, L::neg(e2));
+    f0 = L::fma(L::set(T(-0.5)), e0, am);
+    f1 = L::fma(L::set(T(0.5)), e1, o);
+    f2 = L::mul(L::set(T(0.5)), e2);
+  }
+};
+
+// 2D linear deposit into the register layout, one particle or a pair (one accumulator half each). The
+// weights are the Esirkepov ones in the form of deposit2; the coefficients of a particle that does not
+// fit the register window are zero.
+template <class L, typename T, int NVP>
+__device__ __forceinline__ void deposit2_lin(typename L::V (&acc)[NVP], typename L::V ox, typename L::V dx,
+                                             typename L::V amx, const LinearZ<L, T>& Z, typename L::V cx,
+                                             typename L::V cy, typename L::V cz) {
+  using V = typename L::V;
+  const V fx0 = L::fma(L::set(T(-0.5)), dx, amx), fx1 = L::fma(L::set(T(0.5)), dx, ox);
+  const V gx0 = L::neg(L::mul(cx, dx));
+  acc[0] = L::fma(gx0, Z.f0, acc[0]);
+  acc[1] = L::fma(gx0, Z.f1, acc[1]);
+  acc[2] = L::fma(gx0, Z.f2, acc[2]);
+  const V gz0 = L::neg(L::mul(cz, Z.e0)), gz1 = L::neg(L::mul(cz, Z.e2));
+  acc[3] = L::fma(gz0, fx0, acc[3]);
+  acc[4] = L::fma(gz1, fx0, acc[4]);
+  acc[5] = L::fma(gz0, fx1, acc[5]);
+  acc[6] = L::fma(gz1, fx1, acc[6]);
+  const V h0 = L::mul(cy, fx0), h1 = L::mul(cy, fx1);
+  const V k1 = L::mul(L::mul(cy, dx), L::set(T(1.0 / 12.0))), k0 = L::neg(k1);
+  acc[7] = L::fma(h0, Z.f0, L::fma(k1, Z.e0, acc[7]));  // k0 dS0 = -k1 (-e0)
+  acc[8] = L::fma(h1, Z.f0, L::fma(k0, Z.e0, acc[8]));
+  acc[9] = L::fma(h0, Z.f1, L::fma(k0, Z.e1, acc[9]));
+  acc[10] = L::fma(h1, Z.f1, L::fma(k1, Z.e1, acc[10]));
+  acc[11] = L::fma(h0, Z.f2, L::fma(k0, Z.e2, acc[11]));
+  acc[12] = L::fma(h1, Z.f2, L::fma(k1, Z.e2, acc[12]));
+}
+
+// 3D linear deposit into the register layout (the weights of deposit3): x and y stay in their cell.
+template <typename T, int NVP>
+__device__ __forceinline__ void deposit3_lin(T (&acc)[NVP], T ox, T dx, T oy, T dy, const LinearZ<Lanes1<T>, T>& Z,
+                                             T cx, T cy, T cz) {
+  const T fx0 = fma(T(-0.5), dx, T(1) - ox), fx1 = fma(T(0.5), dx, ox);
+  const T fy0 = fma(T(-0.5), dy, T(1) - oy), fy1 = fma(T(0.5), dy, oy);
+  const T kx = dx * T(1.0 / 12.0), ky = dy * T(1.0 / 12.0);
+  const T fz[3] = {Z.f0, Z.f1, Z.f2}, ez[3] = {-Z.e0, Z.e1, Z.e2};
+  const T gx = -(cx * dx), gy = -(cy * dy), g0 = -(cz * Z.e0), g1 = -(cz * Z.e2);
 #pragma unroll
-  for (int b = 0; b < 3; ++b) acc[b] = __ffma2_rn(gx0, fz[b], acc[b]);
-  const float2 gz0 = Lanes2::neg(__fmul2_rn(cz, e0)), gz1 = Lanes2::neg(__fmul2_rn(cz, e2));
-  acc[3] = __ffma2_rn(gz0, fx0, acc[3]);
-  acc[4] = __ffma2_rn(gz1, fx0, acc[4]);
-  acc[5] = __ffma2_rn(gz0, fx1, acc[5]);
-  acc[6] = __ffma2_rn(gz1, fx1, acc[6]);
-  const float2 hx0 = __fmul2_rn(cy, fx0), hx1 = __fmul2_rn(cy, fx1);
-  const float2 kx1 = __fmul2_rn(__fmul2_rn(cy, dx), make_float2(1.f / 12.f, 1.f / 12.f)), kx0 = Lanes2::neg(kx1);
+  for (int c = 0; c < 3; ++c) {
+    const T wy = ky * ez[c], wx = kx * ez[c];
+    acc[c * 2 + 0] = fma(gx, fma(fy0, fz[c], -wy), acc[c * 2 + 0]);  // Jx(1/2, b, c)
+    acc[c * 2 + 1] = fma(gx, fma(fy1, fz[c], wy), acc[c * 2 + 1]);
+    acc[6 + c * 2 + 0] = fma(gy, fma(fx0, fz[c], -wx), acc[6 + c * 2 + 0]);  // Jy(a, 1/2, c)
+    acc[6 + c * 2 + 1] = fma(gy, fma(fx1, fz[c], wx), acc[6 + c * 2 + 1]);
+  }
+  const T w = kx * dy;
+  const T t[4] = {fma(fx0, fy0, w), fma(fx1, fy0, -w), fma(fx0, fy1, -w), fma(fx1, fy1, w)};
 #pragma unroll
-  for (int b = 0; b < 3; ++b) {
-    acc[7 + 2 * b] = __ffma2_rn(hx0, fz[b], __ffma2_rn(kx0, dS[b], acc[7 + 2 * b]));
-    acc[8 + 2 * b] = __ffma2_rn(hx1, fz[b], __ffma2_rn(kx1, dS[b], acc[8 + 2 * b]));
+  for (int i = 0; i < 4; ++i) {  // Jz(a, b, c + 1/2), i = b * 2 + a
+    acc[12 + 2 * i] = fma(g0, t[i], acc[12 + 2 * i]);
+    acc[13 + 2 * i] = fma(g1, t[i], acc[13 + 2 * i]);
   }
 }
-// A particle of a pair outside the register window: its full window, into shared memory.
+// A particle outside the register window: its full window, into shared memory.
 template <typename T>
 __device__ __noinline__ void deposit2_far(T* sj, int lx, int lz, T ox, T oz, T dx, T dz, T cx, T cy, T cz) {
   const EsirDir<T> X = esir_dir(ox, dx), Z = esir_dir(oz, dz);
   deposit2_smem<T, 2>(sj, lx + X.a + 1, lz + Z.a + 1, X, Z, cx, cy, cz);
+}
+template <typename T>
+__device__ __noinline__ void deposit3_far(T* sj, int lx, int ly, int lz, T ox, T oy, T oz, T dx, T dy, T dz, T cx, T cy,
+                                          T cz) {
+  const EsirDir<T> X = esir_dir(ox, dx), Y = esir_dir(oy, dy), Z = esir_dir(oz, dz);
+  deposit3_smem<T, 3>(sj, lx + X.a + 1, ly + Y.a + 1, lz + Z.a + 1, X, Y, Z, cx, cy, cz);
 }
 
 // One direction of a cubic Esirkepov move: S0 + dS / 2 and the shape change dS on the nodes -1 .. 3 of
@@ -1239,6 +1232,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
 
   T kin = T(0);
   int npush = 0;
+  // current per particle of the uniform weight and unit W (2D Jy: and unit v_y)
+  const T cwx = r.wconst * r.jfx, cwy = r.wconst * (NDIM == 3 ? r.jfy : r.jfy2d), cwz = r.wconst * r.jfz;
 
   // Items of this warp: (cell group, pack round). The packs of the next item are copied into the
   // warp's shared-memory stage with cp.async while the current item is computed.
@@ -1394,8 +1389,10 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           const float2 ign = WIN ? make_float2(fine_rsqrt(gp.x), fine_rsqrt(gp.y))
                                  : make_float2(fast_rsqrt(gp.x), fast_rsqrt(gp.y));
           const float2 g1 = fma2(gp, ign, one2);  // gamma + 1; gamma - 1 = u^2 / (gamma + 1)
-          kin = fmaf(wa, fast_div(u2.x, g1.x), kin);
-          kin = fmaf(wb, fast_div(u2.y, g1.y), kin);
+          if (r.kin) {
+            kin = fmaf(wa, fast_div(u2.x, g1.x), kin);
+            kin = fmaf(wb, fast_div(u2.y, g1.y), kin);
+          }
           npush += (va ? 1 : 0) + (vb ? 1 : 0);
           const float2 vy2 = mul2(uy2, ign);
           const float2 ddx2 = mul2(dtdx2, mul2(ux2, ign)), ddz2 = mul2(dtdz2, mul2(Uz, ign));
@@ -1425,7 +1422,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
                                                        cubic_dir<Lanes2, float, true>(o_z, d_z, Z.up, Z.c), mul2(qr, jx2),
                                                        mul2(mul2(qr, vyp), jy2), mul2(qr, jz2));
           else
-            deposit2_pair<NVP>(acc2, o_x, d_x, X, o_z, d_z, Z, mul2(qr, jx2), mul2(mul2(qr, vyp), jy2), mul2(qr, jz2));
+            deposit2_lin<Lanes2, float, NVP>(acc2, o_x, d_x, X.am, LinearZ<Lanes2, float>(o_z, d_z, Z.am, Z.c, Z.up),
+                                             mul2(qr, jx2), mul2(mul2(qr, vyp), jy2), mul2(qr, jz2));
           if (!rega && va) {
             if constexpr (ORDER == 3)
               deposit_general<float, 2>(sj, lx, 0, lz, oxa, 0.f, oza, dxa, 0.f, dza, qw.x * r.jfx, qw.x * vya * r.jfy2d,
@@ -1531,7 +1529,6 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
         int s;
         const bool valid = slot_of(k, s);
         const SpeciesBuf<T> pout = s ? r.out[1] : r.out[0];
-        const T qs = s ? T(1) : T(-1);
         int dkey = -1 - lane;  // unique per lane when there is no particle
         bool leave = false;
         T nox = T(0), noy = T(0), noz = T(0), ux = T(0), uy = T(0), uz = T(0);
@@ -1563,80 +1560,78 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
             for (int c = 0; c < 6; ++c)
               F[c] = gather_comp<T, NDIM, SCHEME>(sg + c * S::GN, c, lx, ly, lz, dwx, dwy, dwz);
           }
-          // relativistic Boris, momenta relative to the drift u0 z_hat
-          const T h = qs * r.hq;
-          const T mx = ux + h * F[0], my = uy + h * F[1], mz = uz + h * F[2];
+          // relativistic Boris, momenta relative to the drift u0 z_hat (FP64: every operation here counts, its
+          // pipe bounds this kernel)
+          const T h = s ? r.hq : -r.hq;
+          const T mx = fma(h, F[0], ux), my = fma(h, F[1], uy), mz = fma(h, F[2], uz);
           const T Mz = r.u0 + mz;
-          const T mm = T(1) + mx * mx + my * my + Mz * Mz;
-          const T ig = WIN ? fine_rsqrt(mm) : fast_rsqrt(mm);
-          const T tx = h * F[3] * ig, ty = h * F[4] * ig, tz = h * F[5] * ig;
-          const T sf = fast_div(T(2), T(1) + tx * tx + ty * ty + tz * tz);
+          const T mm = fma(Mz, Mz, fma(my, my, fma(mx, mx, T(1))));
+          const T hig = h * (WIN ? fine_rsqrt(mm) : fast_rsqrt(mm));
+          const T tx = hig * F[3], ty = hig * F[4], tz = hig * F[5];
+          const T sf = two_over(fma(tz, tz, fma(ty, ty, fma(tx, tx, T(1)))));
           const T sx = sf * tx, sy = sf * ty, sz = sf * tz;
-          const T qx = mx + (my * tz - Mz * ty);
-          const T qy = my + (Mz * tx - mx * tz);
-          const T qz = Mz + (mx * ty - my * tx);
-          ux = mx + (qy * sz - qz * sy) + h * F[0];
-          uy = my + (qz * sx - qx * sz) + h * F[1];
-          uz = mz + (qx * sy - qy * sx) + h * F[2];
+          const T qx = fma(my, tz, fma(-Mz, ty, mx));
+          const T qy = fma(Mz, tx, fma(-mx, tz, my));
+          const T qz = fma(mx, ty, fma(-my, tx, Mz));
+          ux = fma(qy, sz, fma(-qz, sy, fma(h, F[0], mx)));
+          uy = fma(qz, sx, fma(-qx, sz, fma(h, F[1], my)));
+          uz = fma(qx, sy, fma(-qy, sx, fma(h, F[2], mz)));
           const T Uz = r.u0 + uz;
-          const T u2 = ux * ux + uy * uy + Uz * Uz;
-          const T ign = WIN ? fine_rsqrt(T(1) + u2) : fast_rsqrt(T(1) + u2);
-          T vx = ux * ign, vy = uy * ign;
-          const T vz = Uz * ign;
-          kin += w * fast_div(u2, (T(1) + u2) * ign + T(1));  // gamma - 1 = u^2 / (gamma + 1)
+          const T u2 = fma(Uz, Uz, fma(uy, uy, ux * ux)), gp = T(1) + u2;
+          const T ign = WIN ? fine_rsqrt(gp) : fast_rsqrt(gp);
+          T vy = uy * ign;
+          if (r.kin) kin = fma(w, fast_div(u2, fma(gp, ign, T(1))), kin);  // gamma - 1 = u^2 / (gamma + 1)
           ++npush;
           // move (cell-relative displacement in grid units)
-          T ddx = r.dtdx * vx, ddy = NDIM == 3 ? r.dtdy * vy : T(0), ddz = r.dtdz * vz;
+          T ddx = r.dtdx * (ux * ign), ddy = NDIM == 3 ? r.dtdy * vy : T(0), ddz = r.dtdz * (Uz * ign);
           if (!(abs_lt_one(ddx) && abs_lt_one(ddy) && abs_lt_one(ddz))) {
             flag_error(r.err, ERR_NONFINITE);
             ddx = ddy = ddz = T(0);
             ux = uy = uz = T(0);
             vy = T(0);
           }
-          const EsirDir<T> ex_ = esir_dir(o_x, ddx);
-          const EsirDir<T> ez_ = esir_dir(o_z, ddz);
-          EsirDir<T> ey_;
-          if (NDIM == 3) ey_ = esir_dir(o_y, ddy);
-          else { ey_.a = 0; ey_.shift = 0; ey_.off = T(0); }
+          const Move1<T> X(o_x, ddx), Y(o_y, ddy), Z(o_z, ddz);
           // Esirkepov deposit: summed in registers when the window fits RegLayout (no step back across
-          // a face and no transverse crossing), else straight to shared memory
-          const T qw = qs * w;
-          const bool own = reg_window<T, NDIM>(ex_, NDIM == 3 ? ey_ : ex_, ez_);
+          // a face and no transverse crossing; zero coefficients otherwise), else straight to shared memory
+          const bool own = !(X.down || X.up || Z.down || (NDIM == 3 && (Y.down || Y.up)));
+          T cx = has_w ? w * r.jfx : cwx, cz = has_w ? w * r.jfz : cwz;
+          T cy = NDIM == 3 ? (has_w ? w * r.jfy : cwy) : (has_w ? w * r.jfy2d : cwy) * vy;
+          cx = s ? cx : -cx;
+          cy = s ? cy : -cy;
+          cz = s ? cz : -cz;
+          const T rx = own ? cx : T(0), ry = own ? cy : T(0), rz = own ? cz : T(0);
           if constexpr (LATE) {  // summed after the item's push, from the particle's stage slot
             const_cast<T*>(stq)[4 * k + 3] = ddx;
             st2(const_cast<T*>(str) + 2 * k, ddy, ddz);
-            const_cast<T*>(stw)[k] = own ? qw : T(0);
-            if (!own)
-              deposit_general<T, 3>(sj, lx, ly, lz, o_x, o_y, o_z, ddx, ddy, ddz, qw * r.jfx, qw * r.jfy, qw * r.jfz);
+            const_cast<T*>(stw)[k] = own ? (s ? w : -w) : T(0);
+            if (!own) deposit_general<T, 3>(sj, lx, ly, lz, o_x, o_y, o_z, ddx, ddy, ddz, cx, cy, cz);
           } else if constexpr (ORDER == 3) {
-            const T cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vy * r.jfy2d;
-            if (own)
-              deposit2_cubic<Lanes1<T>, T, NVP, T>(acc, cubic_dir<Lanes1<T>, T, false>(o_x, ddx, false, T(0)),
-                                                   cubic_dir<Lanes1<T>, T, true>(o_z, ddz, !is_zero(ez_.dS[2]), ez_.off),
-                                                   cx, cy, cz);
-            else deposit_general<T, 2>(sj, lx, 0, lz, o_x, T(0), o_z, ddx, T(0), ddz, cx, cy, cz);
-          } else if (NDIM == 2) {
-            const T cx = qw * r.jfx, cz = qw * r.jfz, cy = qw * vy * r.jfy2d;
-            if (own) deposit2_reg<T, NVP>(acc, ex_, ez_, cx, cy, cz);
-            else deposit2_smem<T, NDIM>(sj, lx + ex_.a + 1, lz + ez_.a + 1, ex_, ez_, cx, cy, cz);
+            deposit2_cubic<Lanes1<T>, T, NVP, T>(acc, cubic_dir<Lanes1<T>, T, false>(o_x, ddx, false, T(0)),
+                                                 cubic_dir<Lanes1<T>, T, true>(o_z, ddz, Z.up, Z.c), rx, ry, rz);
+            if (!own) deposit_general<T, 2>(sj, lx, 0, lz, o_x, T(0), o_z, ddx, T(0), ddz, cx, cy, cz);
           } else {
-            const T cx = qw * r.jfx, cy = qw * r.jfy, cz = qw * r.jfz;
-            if (own) deposit3_reg<T, NVP>(acc, ex_, ey_, ez_, cx, cy, cz);
-            else deposit3_smem<T, NDIM>(sj, lx + ex_.a + 1, ly + ey_.a + 1, lz + ez_.a + 1, ex_, ey_, ez_, cx, cy, cz);
+            const LinearZ<Lanes1<T>, T> LZ(o_z, ddz, Z.am, Z.c, Z.up);
+            if constexpr (NDIM == 2) {
+              deposit2_lin<Lanes1<T>, T, NVP>(acc, o_x, ddx, X.am, LZ, rx, ry, rz);
+              if (!own) deposit2_far(sj, lx, lz, o_x, o_z, ddx, ddz, cx, cy, cz);
+            } else {
+              deposit3_lin<T, NVP>(acc, o_x, ddx, o_y, ddy, LZ, rx, ry, rz);
+              if (!own) deposit3_far(sj, lx, ly, lz, o_x, o_y, o_z, ddx, ddy, ddz, cx, cy, cz);
+            }
           }
           // new cell and offsets
-          nox = ex_.off;
-          noy = NDIM == 3 ? ey_.off : T(0);
-          noz = ez_.off;
-          const int nlx = lx + ex_.shift, nly = NDIM == 3 ? ly + ey_.shift : 0, nlz = lz + ez_.shift;
+          nox = X.off;
+          noy = NDIM == 3 ? Y.off : T(0);
+          noz = Z.off;
+          const int nlx = lx + X.sh, nly = NDIM == 3 ? ly + Y.sh : 0, nlz = lz + Z.sh;
           if (nlx >= 0 && nlx < wx && nly >= 0 && nly < wy && nlz >= 0 && nlz < wz) {
             dkey = ((nlz * TY + nly) * TX + nlx) * 2 + s;  // stays in this tile
           } else {
             leave = true;  // global destination, as cell * 2 + species
             // one cell across a face: the index stays within [-1, n] (cells < 2^30: int keys)
-            const int ni = wrap_near_p(gi + ex_.shift, r.nx);
-            const int nj = NDIM == 3 ? wrap_near_p(gj + ey_.shift, r.ny) : 0;
-            const int nk = wrap_near_p(gk + ez_.shift, r.nz);
+            const int ni = wrap_near_p(gi + X.sh, r.nx);
+            const int nj = NDIM == 3 ? wrap_near_p(gj + Y.sh, r.ny) : 0;
+            const int nk = wrap_near_p(gk + Z.sh, r.nz);
             dkey = ((nk * r.ny + nj) * r.nx + ni) * 2 + s;
           }
         }
