@@ -985,7 +985,7 @@ __device__ __noinline__ void deposit_general(T* sj, int lx, int ly, int lz, T ox
   }
   // window node 0 (two below the cell) is current-tile index (lx, ly, lz)
   T* w0 = sj + (lz * S::JY + (NDIM == 3 ? ly : 0)) * S::JX + lx;
-  if (NDIM == 2) {
+  if constexpr (NDIM == 2) {
 #pragma unroll 1
     for (int b = 0; b < NW; ++b) {
       T px = T(0), pz = T(0);
@@ -1002,27 +1002,27 @@ __device__ __noinline__ void deposit_general(T* sj, int lx, int ly, int lz, T ox
         if (vy != T(0)) atomicAdd(w0 + S::JN + b * S::JX + a, vy);
       }
     }
-    return;
-  }
+  } else {
 #pragma unroll 1
-  for (int t2 = 0; t2 < NW; ++t2)
+    for (int t2 = 0; t2 < NW; ++t2)
 #pragma unroll 1
-    for (int t1 = 0; t1 < NW; ++t1) {
-      const T gx = Ty[t1] * Tz[t2] + ey[t1] * ez[t2] * T(1.0 / 12.0);  // Jx: (y, z) = (t1, t2)
-      const T gy = Tx[t1] * Tz[t2] + ex[t1] * ez[t2] * T(1.0 / 12.0);  // Jy: (x, z) = (t1, t2)
-      const T gz = Tx[t1] * Ty[t2] + ex[t1] * ey[t2] * T(1.0 / 12.0);  // Jz: (x, y) = (t1, t2)
-      T px = T(0), py = T(0), pz = T(0);
+      for (int t1 = 0; t1 < NW; ++t1) {
+        const T gx = Ty[t1] * Tz[t2] + ey[t1] * ez[t2] * T(1.0 / 12.0);  // Jx: (y, z) = (t1, t2)
+        const T gy = Tx[t1] * Tz[t2] + ex[t1] * ez[t2] * T(1.0 / 12.0);  // Jy: (x, z) = (t1, t2)
+        const T gz = Tx[t1] * Ty[t2] + ex[t1] * ey[t2] * T(1.0 / 12.0);  // Jz: (x, y) = (t1, t2)
+        T px = T(0), py = T(0), pz = T(0);
 #pragma unroll 1
-      for (int a = 0; a < NW - 1; ++a) {
-        px += ex[a];
-        py += ey[a];
-        pz += ez[a];
-        const T vx = cx * px * gx, vy = cy * py * gy, vz = cz * pz * gz;
-        if (vx != T(0)) atomicAdd(w0 + (t2 * S::JY + t1) * S::JX + a, vx);
-        if (vy != T(0)) atomicAdd(w0 + S::JN + (t2 * S::JY + a) * S::JX + t1, vy);
-        if (vz != T(0)) atomicAdd(w0 + 2 * S::JN + (a * S::JY + t2) * S::JX + t1, vz);
+        for (int a = 0; a < NW - 1; ++a) {
+          px += ex[a];
+          py += ey[a];
+          pz += ez[a];
+          const T vx = cx * px * gx, vy = cy * py * gy, vz = cz * pz * gz;
+          if (vx != T(0)) atomicAdd(w0 + (t2 * S::JY + t1) * S::JX + a, vx);
+          if (vy != T(0)) atomicAdd(w0 + S::JN + (t2 * S::JY + a) * S::JX + t1, vy);
+          if (vz != T(0)) atomicAdd(w0 + 2 * S::JN + (a * S::JY + t2) * S::JX + t1, vz);
+        }
       }
-    }
+  }
 }
 
 // 3D cubic deposit of one item and one component (0 Jx, 1 Jy, 2 Jz). The window of all components has 184
@@ -1139,31 +1139,34 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
 
   // 1. field copies of the tile and its halo into shared memory (periodic wrap); zero the current
   const bool near_ok = r.nx >= S::GX && r.nz >= S::GZ && (NDIM == 2 || r.ny >= S::GY);
-  for (int e = tid; e < 6 * S::GN; e += PUSH_THREADS) {
-    int c = e / S::GN, rem = e - c * S::GN;
-    int lz = rem / (S::GX * S::GY);
-    int ly = (rem / S::GX) % S::GY;
-    int lx = rem % S::GX;
-    // tile + halo lies within one period of the grid when the grid is at least as wide
-    int gx = near_ok ? wrap_near_p(X0 - S::H + lx, r.nx) : wrapi(X0 - S::H + lx, r.nx);
-    int gy = NDIM == 3 ? (near_ok ? wrap_near_p(Y0 - S::H + ly, r.ny) : wrapi(Y0 - S::H + ly, r.ny)) : 0;
-    int gz = near_ok ? wrap_near_p(Z0 - S::H + lz, r.nz) : wrapi(Z0 - S::H + lz, r.nz);
-    const T* src = r.g[0];
-    switch (c) {  // constant-indexed parameter reads (no local copy of r.g)
-      case 1: src = r.g[1]; break;
-      case 2: src = r.g[2]; break;
-      case 3: src = r.g[3]; break;
-      case 4: src = r.g[4]; break;
-      case 5: src = r.g[5]; break;
-      default: break;
-    }
-    copy1_async(sg + e, src + (long long)gz * nxy + (long long)gy * r.nx + gx);
+  // global index of node (lx, ly, lz) of a tile region that starts H nodes below the tile (cells < 2^30);
+  // it lies within one period of the grid when the grid is at least as wide as the region
+  auto node_at = [&](int lx, int ly, int lz) -> int {
+    const int gx = X0 - S::H + lx, gy = Y0 - S::H + ly, gz = Z0 - S::H + lz;
+    const int kx = near_ok ? wrap_near_p(gx, r.nx) : wrapi(gx, r.nx);
+    const int ky = NDIM == 3 ? (near_ok ? wrap_near_p(gy, r.ny) : wrapi(gy, r.ny)) : 0;
+    const int kz = near_ok ? wrap_near_p(gz, r.nz) : wrapi(gz, r.nz);
+    return (kz * r.ny + ky) * r.nx + kx;
+  };
+  // the planes this tile uses (wz of TZ), one index computation per node for all components: a step of
+  // an empty 512x1024 FP32 grid, which is these prologues and epilogues alone, took 47 us with one per
+  // component and node
+  const int gn = S::GX * S::GY * (wz + 2 * S::H), jn = S::JX * S::JY * (wz + 2 * S::H + 1);
+  const int ncl = TX * TY * wz;
+  const int ngrp = (ncl + CPW - 1) / CPW;  // cell groups of the tile
+  for (int e = tid; e < gn; e += PUSH_THREADS) {
+    const int o = node_at(e % S::GX, (e / S::GX) % S::GY, e / (S::GX * S::GY));
+#pragma unroll
+    for (int c = 0; c < 6; ++c) copy1_async(sg + c * S::GN + e, r.g[c] + o);
   }
-  for (int e = tid; e < 3 * S::JN; e += PUSH_THREADS) sj[e] = T(0);
+  for (int e = tid; e < jn; e += PUSH_THREADS) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sj[c * S::JN + e] = T(0);
+  }
   // 2. particle counts of the tile's cells, copied in the same asynchronous batch as the fields (one
   // global round trip for both); then clamped, and the input counts zeroed (they are the next
   // step's output counts). Each thread reads back only the counts it copied itself.
-  for (int cl = tid; cl < NCL; cl += PUSH_THREADS) {
+  for (int cl = tid; cl < ngrp * CPW; cl += PUSH_THREADS) {
     const int lx = cl % TX, ly = (cl / TX) % TY, lz = cl / (TX * TY);
     if (lx < wx && ly < wy && lz < wz) {
       const long long cell = (long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx;
@@ -1210,7 +1213,7 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   static_assert(NCL / CPW >= NWARP, "every warp needs a first cell group");
   cp_async_commit();
   cp_async_wait_all();
-  for (int cl = tid; cl < NCL; cl += PUSH_THREADS) {
+  for (int cl = tid; cl < ncl; cl += PUSH_THREADS) {
     const int lx = cl % TX, ly = (cl / TX) % TY, lz = cl / (TX * TY);
     if (lx < wx && ly < wy && lz < wz) {
       const long long cell = (long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx;
@@ -1237,7 +1240,6 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
 
   // Items of this warp: (cell group, pack round). The packs of the next item are copied into the
   // warp's shared-memory stage with cp.async while the current item is computed.
-  constexpr int NGRP = NCL / CPW;
   auto group_iters = [&](int g) -> int {
     const int c = g * CPW + lane / LPC;
     const int nq = ((sn[c] + 3) >> 2) + ((sn[NCL + c] + 3) >> 2);
@@ -1257,36 +1259,38 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     return __shfl_sync(0xffffffffu, v, 0);
   };
   int g = warp, it = 0;
-  int giters = g < NGRP ? group_iters(g) : 0;
-  while (g < NGRP && giters == 0) {
+  int giters = g < ngrp ? group_iters(g) : 0;
+  while (g < ngrp && giters == 0) {
     g = take_group();
-    giters = g < NGRP ? group_iters(g) : 0;
+    giters = g < ngrp ? group_iters(g) : 0;
   }
   int stage = 0;
-  if (g < NGRP) issue(g, 0, 0, g == warp);  // the first group's first item was copied speculatively
+  if (g < ngrp) issue(g, 0, 0, g == warp);  // the first group's first item was copied speculatively
   cp_async_commit();
   // the register sums; a linear paired push keeps one half per particle of the pair until the group's end
   constexpr bool ACC2 = PushPaired<T, NDIM>::value && ORDER == 1;
   T acc[NVP];
   float2 acc2[ACC2 ? NVP : 1];
   GalCache<T, NDIM> gc;  // Galerkin nodes of the lane's cell, loaded once per cell group
-  while (g < NGRP) {
+  while (g < ngrp) {
     // prefetch the next item
     int ng = g, nit = it + 1, niters = giters;
     if (nit >= giters) {
       nit = 0;
       do {
         ng = take_group();
-        niters = ng < NGRP ? group_iters(ng) : 0;
-      } while (ng < NGRP && niters == 0);
+        niters = ng < ngrp ? group_iters(ng) : 0;
+      } while (ng < ngrp && niters == 0);
     }
-    if (ng < NGRP) issue(ng, nit, stage ^ 1, false);
+    if (ng < ngrp) issue(ng, nit, stage ^ 1, false);
     cp_async_commit();
     cp_async_wait_1();
     __syncwarp();
 
     const int cl = g * CPW + lane / LPC;
-    const int lx = cl % TX, ly = (cl / TX) % TY, lz = cl / (TX * TY);
+    // (an empty cell past the tile's last plane, in the last group, stands in that plane: its nodes are
+    // staged, so that the lanes without a particle compute with finite fields)
+    const int lx = cl % TX, ly = (cl / TX) % TY, lz = min(cl / (TX * TY), wz - 1);
     const int gi = X0 + lx, gj = Y0 + ly, gk = Z0 + lz;
     const int n0 = sn[cl], n1 = sn[NCL + cl];
     const int nq0 = (n0 + 3) >> 2, nq = nq0 + ((n1 + 3) >> 2);
@@ -1793,7 +1797,7 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
 
   // 5. output counts of the tile's cells (leavers from other tiles are added by k_migrate); a count
   // past the capacity (particles sent on through the leaver list) is stored as the capacity
-  for (int cl = tid; cl < NCL; cl += PUSH_THREADS) {
+  for (int cl = tid; cl < ncl; cl += PUSH_THREADS) {
     const int lx = cl % TX, ly = (cl / TX) % TY, lz = cl / (TX * TY);
     if (lx < wx && ly < wy && lz < wz) {
       const long long cell = (long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx;
@@ -1803,31 +1807,30 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   }
 
   // 6. flush the tile's current to global memory
-  for (int e = tid; e < 3 * S::JN; e += PUSH_THREADS) {
-    T v = sj[e];
-    if (v == T(0)) continue;
-    int c = e / S::JN, rem = e - c * S::JN;
-    int lz = rem / (S::JX * S::JY);
-    int ly = (rem / S::JX) % S::JY;
-    int lx = rem % S::JX;
-    int gx = near_ok ? wrap_near_p(X0 - S::H + lx, r.nx) : wrapi(X0 - S::H + lx, r.nx);
-    int gy = NDIM == 3 ? (near_ok ? wrap_near_p(Y0 - S::H + ly, r.ny) : wrapi(Y0 - S::H + ly, r.ny)) : 0;
-    int gz = near_ok ? wrap_near_p(Z0 - S::H + lz, r.nz) : wrapi(Z0 - S::H + lz, r.nz);
-    atomicAdd(r.j[c] + (long long)gz * nxy + (long long)gy * r.nx + gx, v);
+  for (int e = tid; e < jn; e += PUSH_THREADS) {
+    const T v0 = sj[e], v1 = sj[S::JN + e], v2 = sj[2 * S::JN + e];
+    if (v0 == T(0) && v1 == T(0) && v2 == T(0)) continue;
+    const int o = node_at(e % S::JX, (e / S::JX) % S::JY, e / (S::JX * S::JY));
+    if (v0 != T(0)) atomicAdd(r.j[0] + o, v0);
+    if (v1 != T(0)) atomicAdd(r.j[1] + o, v1);
+    if (v2 != T(0)) atomicAdd(r.j[2] + o, v2);
   }
 
   // 7. kinetic energy and particle count of this step: per-thread partial sums in the working
-  // precision, FP64 across the block and the grid
+  // precision, FP32 pairs (FP64: FP64) across the warp, FP64 across the block and the grid
   if (r.kin) {
-    double kd = (double)kin;
-    int nd = npush;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      kd += __shfl_xor_sync(0xffffffffu, kd, o);
-      nd += __shfl_xor_sync(0xffffffffu, nd, o);
-    }
     __shared__ double skin[NWARP];
     __shared__ int swcnt[NWARP];
+    double kd;
+    if constexpr (sizeof(T) == 4) {
+      const FPair t = warp_sum_pair(FPair{kin, 0.f});
+      kd = lane == 0 ? (double)t.s + (double)t.c : 0.0;
+    } else {
+      kd = kin;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) kd += __shfl_xor_sync(0xffffffffu, kd, o);
+    }
+    const int nd = __reduce_add_sync(0xffffffffu, npush);
     if (lane == 0) {
       skin[warp] = kd;
       swcnt[warp] = nd;
