@@ -154,7 +154,7 @@ struct PTile<T, 2> {
 };
 template <>
 struct PTile<float, 3> {
-  static constexpr int TX = 2, TY = 2, TZ = 128;
+  static constexpr int TX = 2, TY = 2, TZ = 64;
 };
 template <>
 struct PTile<double, 3> {

@@ -57,7 +57,7 @@ __device__ __forceinline__ void gweights(T o, int st, int ord, int& first, T (&w
 // per species 115 -> 30 us; momentum-conserving linear on 301x517 287 -> 169 us; cubic 3D on 44x36x70
 // with 8 per species 2062 -> 265 us.
 template <typename T, int NDIM, int ORDER, int SCHEME, int LPC>
-__global__ void __launch_bounds__(PushThreads<T, NDIM, ORDER>::value, PushMinBlocks<T, NDIM>::value)
+__global__ void __launch_bounds__(PushThreads<T, NDIM, ORDER>::value, PushMinBlocks<T, NDIM, ORDER>::value)
     k_push_ho(const __grid_constant__ RunDev<T> r) {
   pdl_wait();
   push_tile<T, NDIM, SCHEME, LPC, ORDER>(r, blockIdx.x);

@@ -13,7 +13,7 @@ namespace picgb {
 template <typename T, int NDIM, int ORDER = 1>
 struct PushThreads {
   static constexpr int value = ORDER == 3 ? (NDIM == 3 ? (sizeof(T) == 4 ? 384 : 192) : (sizeof(T) == 4 ? 192 : 256))
-                                          : (NDIM == 3 && sizeof(T) == 4) ? 384 : 256;
+                                          : (NDIM == 3 && sizeof(T) == 4) ? 192 : 256;
 };
 
 // The tile's compile-time extents by shape order.
@@ -74,7 +74,8 @@ struct PushSmem {
   static constexpr int JN = JX * JY * JZ;
   // particles leaving the tile, buffered per block: [7][LVB] values (ox oy oz dux duy duz w), LVB
   // keys, LVB ids and the buffer's counter; written to the global leaver list once per tile
-  static constexpr int LVB = (NDIM == 3 && sizeof(T) == 8) ? 128 : 512;  // 3D FP64: within 227 KB
+  // (3D: within the shared memory of one block per SM in FP64, of two in FP32)
+  static constexpr int LVB = NDIM == 2 || ORDER == 3 && sizeof(T) == 4 ? 512 : sizeof(T) == 8 ? 128 : 256;
   static constexpr size_t lv_bytes() { return (size_t)LVB * (7 * sizeof(T) + 2 * sizeof(int)) + 16; }
   static constexpr size_t bytes() {
     return sizeof(T) * (6 * GN * GCOPY + 3 * JN) + sizeof(int) * (4 * NCL) + 16 +
@@ -527,9 +528,9 @@ struct PushPlan {
 };
 
 // Resident blocks per SM the push kernel is compiled for (register budget): FP32 2D fits two.
-template <typename T, int NDIM>
+template <typename T, int NDIM, int ORDER = 1>
 struct PushMinBlocks {
-  static constexpr int value = (sizeof(T) == 4 && NDIM == 2) ? 2 : 1;
+  static constexpr int value = sizeof(T) == 4 && !(NDIM == 3 && ORDER == 3) ? 2 : 1;
 };
 
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
