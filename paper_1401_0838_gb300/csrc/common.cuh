@@ -142,33 +142,36 @@ __device__ __forceinline__ FPair warp_sum_pair(FPair v) {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Particle tile of the linear push (cells per direction, the shared-memory tiles' size). A run's
-// tiles are at most this (push_tiles); the launchers check it. Tall and narrow, along the drift:
-// few particles leave a tile through a z face per step, and a warp's cell group spans several z
-// rows, so a particle crossing into the next z cell mostly lands in a cell of its own group (one
-// slot reservation for both). 3D FP64 keeps a cube: its shared-memory tiles are twice as large.
+// tiles are at most this (push_tiles); the launchers check it. Longest along the drift, where the particles
+// cross faces: few leave a tile through a z face per step, and a warp's cell group spans several z rows,
+// so a particle crossing into the next z cell mostly lands in a cell of its own group (one slot
+// reservation for both). But not too narrow: the halo of a narrow tile is staged and flushed in short
+// rows, which cost the shared-memory pipe one cache line each. Push + migrate per step at 512x1024 FP32,
+// 16 per species: 8x32 308 us, 4x64 312 us, 16x16 311 us; 3D 64x64x256, 8 per species: 4x4x16 542 us,
+// 4x2x32 544 us, 8x2x16 555 us, 2x2x64 605 us. 3D FP64 keeps a cube: its shared-memory tiles are twice
+// as large.
 template <typename T, int NDIM>
 struct PTile;
 template <typename T>
 struct PTile<T, 2> {
-  static constexpr int TX = 4, TY = 1, TZ = 64;
+  static constexpr int TX = 8, TY = 1, TZ = 32;
 };
 template <>
 struct PTile<float, 3> {
-  static constexpr int TX = 2, TY = 2, TZ = 64;
+  static constexpr int TX = 4, TY = 4, TZ = 16;
 };
 template <>
 struct PTile<double, 3> {
   static constexpr int TX = 8, TY = 8, TZ = 8;
 };
 
-// Particle tile of the cubic push (k_push_ho): as PTile in 2D; in 3D the two-node halo makes narrow
-// tiles mostly halo (a 2x2x128 tile would stage 9 nodes a cell), so 4x4 columns, as tall as shared memory
-// allows.
+// Particle tile of the cubic push (k_push_ho): as PTile in 2D; in 3D the two-node halo asks for wider
+// tiles, so 4x4 columns, as tall as shared memory allows.
 template <typename T, int NDIM>
 struct HoTile;
 template <typename T>
 struct HoTile<T, 2> {
-  static constexpr int TX = 4, TY = 1, TZ = 64;
+  static constexpr int TX = 8, TY = 1, TZ = 32;
 };
 template <>
 struct HoTile<float, 3> {

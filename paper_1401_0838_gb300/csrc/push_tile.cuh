@@ -75,7 +75,7 @@ struct PushSmem {
   // particles leaving the tile, buffered per block: [7][LVB] values (ox oy oz dux duy duz w), LVB
   // keys, LVB ids and the buffer's counter; written to the global leaver list once per tile
   // (3D: within the shared memory of one block per SM in FP64, of two in FP32)
-  static constexpr int LVB = NDIM == 2 || ORDER == 3 && sizeof(T) == 4 ? 512 : sizeof(T) == 8 ? 128 : 256;
+  static constexpr int LVB = NDIM == 3 && sizeof(T) == 8 ? 128 : 512;
   static constexpr size_t lv_bytes() { return (size_t)LVB * (7 * sizeof(T) + 2 * sizeof(int)) + 16; }
   static constexpr size_t bytes() {
     return sizeof(T) * (6 * GN * GCOPY + 3 * JN) + sizeof(int) * (4 * NCL) + 16 +
