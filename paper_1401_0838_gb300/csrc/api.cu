@@ -2,6 +2,7 @@
 // diagnostics, batched runs and the adjoint's checkpoint / recompute schedule. All arithmetic of
 // the step and of its adjoint runs in the CUDA kernels of k_fields.cu, k_particles.cu and
 // k_adjoint.cu; this file only allocates, marshals and orders launches on one stream.
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 #include <math.h>
@@ -57,7 +58,6 @@ struct pic_handle {
   double* d_red_yee = nullptr;  // block partials of the energies recorded by the Yee launch
   double* d_rho = nullptr;      // Gauss-law diagnostic: rho and F rho (FP64), then its scratch
   double* d_gauss = nullptr;
-  long long* d_offs = nullptr;
   long long* d_bsum = nullptr;
   long long* d_total = nullptr;
   // import / export staging (device)
@@ -616,6 +616,47 @@ FlatDev<T> stage_view(pic_handle* h, long long n) {
   return f;
 }
 
+// Whether n elements of a caller's array can be read or written by a kernel of this handle: device memory
+// of the current device, aligned to the element size es, inside one allocation. Anything else (host
+// memory, another device, a length past the allocation) goes through the staging arrays and
+// cudaMemcpyAsync, which reports what it cannot copy.
+bool kernel_reachable(const void* p, long long n, size_t es) {
+  static const PFN_cuMemGetAddressRange_v3020 range = [] {
+    void* q = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &q, 3020, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess)
+      q = nullptr;
+    (void)cudaGetLastError();
+    return (PFN_cuMemGetAddressRange_v3020)q;
+  }();
+  if (!range || reinterpret_cast<uintptr_t>(p) % es != 0) return false;
+  cudaPointerAttributes a;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  if (a.type != cudaMemoryTypeDevice || a.device != dev) return false;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (range(&base, &size, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+  return (size_t)((CUdeviceptr)p - base) + (size_t)n * es <= size;
+}
+
+// The caller's particle arrays as the import and export kernels take them, when every one that is given
+// is device memory they can reach (one pass over the particles less than through the staging arrays).
+template <typename T>
+bool caller_view(pic_handle* h, const pic_state* s, long long n, FlatDev<T>* f) {
+  if (s->where != PIC_DEVICE) return false;
+  const void* arr[10] = {s->cell, s->species, s->id, s->ox, s->oy, s->oz, s->dux, s->duy, s->duz, s->w};
+  for (int q = 0; q < 10; ++q)
+    if (arr[q] && !(q == 4 && h->cfg.ndim != 3) && !kernel_reachable(arr[q], n, q < 3 ? 4 : sizeof(T))) return false;
+  *f = FlatDev<T>{n, s->cell, s->species, (T*)s->ox, (T*)s->oy, (T*)s->oz, (T*)s->dux, (T*)s->duy, (T*)s->duz,
+                  (T*)s->w, s->id};
+  return true;
+}
+
 template <typename T>
 int set_state_t(pic_handle* h, const pic_state* s) {
   cudaStream_t st = h->stream;
@@ -644,33 +685,40 @@ int set_state_t(pic_handle* h, const pic_state* s) {
   if (!s->cell || !s->species || !s->ox || !s->oz || !s->dux || !s->duy || !s->duz ||
       (h->cfg.ndim == 3 && !s->oy))
     return fail(h, PIC_E_ARG, "missing particle array");
-  int rc = ensure_stage(h, n);
-  if (rc) return rc;
-  FlatDev<T> f = stage_view<T>(h, n);
-  CK(cudaMemcpyAsync(f.cell, s->cell, 4 * (size_t)n, k, st), "copy cell");
-  CK(cudaMemcpyAsync(f.species, s->species, 4 * (size_t)n, k, st), "copy species");
-  CK(cudaMemcpyAsync(f.ox, s->ox, sizeof(T) * n, k, st), "copy ox");
-  if (h->cfg.ndim == 3) CK(cudaMemcpyAsync(f.oy, s->oy, sizeof(T) * n, k, st), "copy oy");
-  else f.oy = nullptr;
-  CK(cudaMemcpyAsync(f.oz, s->oz, sizeof(T) * n, k, st), "copy oz");
-  CK(cudaMemcpyAsync(f.dux, s->dux, sizeof(T) * n, k, st), "copy dux");
-  CK(cudaMemcpyAsync(f.duy, s->duy, sizeof(T) * n, k, st), "copy duy");
-  CK(cudaMemcpyAsync(f.duz, s->duz, sizeof(T) * n, k, st), "copy duz");
-  if (s->w && h->has_w) CK(cudaMemcpyAsync(f.w, s->w, sizeof(T) * n, k, st), "copy w");
-  else f.w = nullptr;
-  if (s->id && h->has_id) CK(cudaMemcpyAsync(f.id, s->id, 4 * (size_t)n, k, st), "copy id");
-  else f.id = nullptr;
+  FlatDev<T> f;
+  if (caller_view<T>(h, s, n, &f)) {  // device arrays are read by the import itself
+    if (h->cfg.ndim != 3) f.oy = nullptr;
+    if (!h->has_w) f.w = nullptr;
+    if (!h->has_id) f.id = nullptr;
+  } else {
+    int rc = ensure_stage(h, n);
+    if (rc) return rc;
+    f = stage_view<T>(h, n);
+    CK(cudaMemcpyAsync(f.cell, s->cell, 4 * (size_t)n, k, st), "copy cell");
+    CK(cudaMemcpyAsync(f.species, s->species, 4 * (size_t)n, k, st), "copy species");
+    CK(cudaMemcpyAsync(f.ox, s->ox, sizeof(T) * n, k, st), "copy ox");
+    if (h->cfg.ndim == 3) CK(cudaMemcpyAsync(f.oy, s->oy, sizeof(T) * n, k, st), "copy oy");
+    else f.oy = nullptr;
+    CK(cudaMemcpyAsync(f.oz, s->oz, sizeof(T) * n, k, st), "copy oz");
+    CK(cudaMemcpyAsync(f.dux, s->dux, sizeof(T) * n, k, st), "copy dux");
+    CK(cudaMemcpyAsync(f.duy, s->duy, sizeof(T) * n, k, st), "copy duy");
+    CK(cudaMemcpyAsync(f.duz, s->duz, sizeof(T) * n, k, st), "copy duz");
+    if (s->w && h->has_w) CK(cudaMemcpyAsync(f.w, s->w, sizeof(T) * n, k, st), "copy w");
+    else f.w = nullptr;
+    if (s->id && h->has_id) CK(cudaMemcpyAsync(f.id, s->id, 4 * (size_t)n, k, st), "copy id");
+    else f.id = nullptr;
+  }
   RunDev<T> r = make_run<T>(h, 0);
   CK(launch(h, PIC_K_OTHER, [&] { return launch_import<T>(r, f, st); }), "import");
   return PIC_OK;
 }
 
-// Particles per species in the bins of the current buffers (the spill list not included).
+// Particles per species in the bins of the current buffers (the spill list not included), and their
+// prefix over the cells for an export.
 int count_bins(pic_handle* h, long long out[2]) {
-  for (int s = 0; s < 2; ++s) {
-    CK(launch_count_prefix(h->cnt[s][h->parity], h->ncell, h->cap, h->d_offs, h->d_bsum, h->d_total + s, h->stream),
-       "count prefix");
-  }
+  CK(launch_count_prefix(h->cnt[0][h->parity], h->cnt[1][h->parity], h->ncell, h->cap, h->d_bsum, h->d_total,
+                         h->stream),
+     "count prefix");
   CK(cudaMemcpyAsync(out, h->d_total, 2 * sizeof(long long), cudaMemcpyDeviceToHost, h->stream), "read counts");
   CK(cudaStreamSynchronize(h->stream), "synchronize");
   return PIC_OK;
@@ -716,14 +764,9 @@ int settle(pic_handle* h) {
   if (!h->has_w) f.w = nullptr;
   if (!h->has_id) f.id = nullptr;
   RunDev<T> r = make_run<T>(h, h->parity);
-  long long base = 0;
-  for (int sp = 0; sp < 2; ++sp) {
-    CK(launch_count_prefix(h->cnt[sp][h->parity], h->ncell, h->cap, h->d_offs, h->d_bsum, h->d_total, st),
-       "count prefix");
-    CK(launch(h, PIC_K_OTHER, [&] { return launch_export<T>(r, sp, h->d_offs, base, f, st); }), "export");
-    base += cnts[sp];
-  }
-  CK(launch(h, PIC_K_OTHER, [&] { return launch_spill_export<T>(r, nsp, base, f, st); }), "spill export");
+  CK(launch(h, PIC_K_OTHER, [&] { return launch_export<T>(r, h->d_bsum, h->d_total, f, st); }), "export");
+  CK(launch(h, PIC_K_OTHER, [&] { return launch_spill_export<T>(r, nsp, cnts[0] + cnts[1], f, st); }),
+     "spill export");
   CK(cudaStreamSynchronize(st), "synchronize");
   // new bins for both buffers and species; the old ones are freed only once all are in place
   const pic_config& c = h->cfg;
@@ -829,12 +872,11 @@ int get_state_t(pic_handle* h, pic_state* s) {
     if (dst[q]) CK(cudaMemcpyAsync(dst[q], h->f[q], fb, k, st), "copy field out");
   s->u_drift = h->u0;
   long long cnts[2];
-  rc = count_particles<T>(h, cnts);
+  rc = count_bins(h, cnts);  // synchronises
   if (rc) return rc;
   const long long n = cnts[0] + cnts[1];
   if (!s->cell && !s->species && !s->ox && !s->oy && !s->oz && !s->dux && !s->duy && !s->duz && !s->w && !s->id) {
     s->np = n;  // fields only
-    CK(cudaStreamSynchronize(st), "synchronize");
     return check_err(h);
   }
   if (s->np < n) {
@@ -843,18 +885,17 @@ int get_state_t(pic_handle* h, pic_state* s) {
   }
   s->np = n;
   if (n == 0) return PIC_OK;
-  rc = ensure_stage(h, n);
-  if (rc) return rc;
-  FlatDev<T> f = stage_view<T>(h, n);
+  FlatDev<T> f;
+  const bool direct = caller_view<T>(h, s, n, &f);  // device arrays are written by the export itself
+  if (!direct) {
+    rc = ensure_stage(h, n);
+    if (rc) return rc;
+    f = stage_view<T>(h, n);
+  }
   if (h->cfg.ndim != 3) f.oy = nullptr;
   RunDev<T> r = make_run<T>(h, h->parity);
-  long long base = 0;
-  for (int sp = 0; sp < 2; ++sp) {
-    CK(launch_count_prefix(h->cnt[sp][h->parity], h->ncell, h->cap, h->d_offs, h->d_bsum, h->d_total, st),
-       "count prefix");
-    CK(launch(h, PIC_K_OTHER, [&] { return launch_export<T>(r, sp, h->d_offs, base, f, st); }), "export");
-    base += cnts[sp];
-  }
+  CK(launch(h, PIC_K_OTHER, [&] { return launch_export<T>(r, h->d_bsum, h->d_total, f, st); }), "export");
+  if (direct) return check_err(h);  // synchronises
   if (s->cell) CK(cudaMemcpyAsync(s->cell, f.cell, 4 * (size_t)n, k, st), "copy cell out");
   if (s->species) CK(cudaMemcpyAsync(s->species, f.species, 4 * (size_t)n, k, st), "copy species out");
   if (s->ox) CK(cudaMemcpyAsync(s->ox, f.ox, sizeof(T) * n, k, st), "copy ox out");
@@ -865,8 +906,7 @@ int get_state_t(pic_handle* h, pic_state* s) {
   if (s->duz) CK(cudaMemcpyAsync(s->duz, f.duz, sizeof(T) * n, k, st), "copy duz out");
   if (s->w) CK(cudaMemcpyAsync(s->w, f.w, sizeof(T) * n, k, st), "copy w out");
   if (s->id) CK(cudaMemcpyAsync(s->id, f.id, 4 * (size_t)n, k, st), "copy id out");
-  CK(cudaStreamSynchronize(st), "synchronize");
-  return check_err(h);
+  return check_err(h);  // synchronises
 }
 
 template <typename T>
@@ -1036,8 +1076,7 @@ int pic_create(const pic_config* cfg_in, pic_handle** out) {
   if (ok) ok = cudaMemset(h->d_red, 0, field_energy_scratch_bytes()) == cudaSuccess;
   if (ok) ok = (h->d_red_yee = (double*)dalloc(h, yee_energy_scratch_bytes(c.ndim, c.nx, c.ny, c.nz, h->nsm))) != nullptr;
   if (ok) ok = cudaMemset(h->d_red_yee, 0, yee_energy_scratch_bytes(c.ndim, c.nx, c.ny, c.nz, h->nsm)) == cudaSuccess;
-  if (ok) ok = (h->d_offs = (long long*)dalloc(h, sizeof(long long) * h->ncell)) != nullptr;
-  if (ok) ok = (h->d_bsum = (long long*)dalloc(h, sizeof(long long) * (count_prefix_blocks(h->ncell) + 1))) != nullptr;
+  if (ok) ok = (h->d_bsum = (long long*)dalloc(h, 2 * sizeof(long long) * (count_prefix_blocks(h->ncell) + 1))) != nullptr;
   if (ok) ok = (h->d_total = (long long*)dalloc(h, 4 * sizeof(long long))) != nullptr;
   h->hist_cap = c.diag_capacity > 0 ? c.diag_capacity : 4096;
   if (ok) ok = (h->d_hist = (double*)dalloc(h, 8 * sizeof(double) * (size_t)h->hist_cap)) != nullptr;

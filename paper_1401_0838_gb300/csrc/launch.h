@@ -127,9 +127,11 @@ cudaError_t launch_spill_export(const RunDev<T>& r, long long n, long long base,
 // *out = max(*out, max over cells of c0, c1)
 cudaError_t launch_max_count(const int* c0, const int* c1, long long ncell, int* out, cudaStream_t st);
 template <typename T>
-cudaError_t launch_export(const RunDev<T>& r, int s, const long long* offs, long long base, const FlatDev<T>& f,
+cudaError_t launch_export(const RunDev<T>& r, const long long* bsum, const long long* total, const FlatDev<T>& f,
                           cudaStream_t st);
-cudaError_t launch_count_prefix(const int* cnt, long long ncell, int cap, long long* offs, long long* bsum,
+// particles of the bins (counts clamped to cap): per species, the number before each block of
+// count_prefix_blocks(ncell) blocks of cells into bsum[2][blocks], the totals into total[2]
+cudaError_t launch_count_prefix(const int* c0, const int* c1, long long ncell, int cap, long long* bsum,
                                 long long* total, cudaStream_t st);
 long long count_prefix_blocks(long long ncell);
 
