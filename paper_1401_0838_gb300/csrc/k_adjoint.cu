@@ -14,6 +14,7 @@
 // (symmetric taps), the last fused with the coefficient gradient in k_adj_psi.
 #include <climits>
 
+#include "fastmath.cuh"
 #include "launch.h"
 
 namespace picgb {
@@ -100,41 +101,27 @@ __device__ __constant__ int kStagX[6] = {1, 0, 0, 0, 1, 1};
 __device__ __constant__ int kStagZ[6] = {0, 0, 1, 1, 1, 0};
 
 // Gather weights along one direction at cell-relative offset o in [0, 1): S1 on two nodes
-// (weights 1-f, f; derivatives -1, +1 in o) or S0 on one node (derivative 0).
+// (weights 1-f, f; derivatives -1, +1 in o).
 template <typename T>
 struct Gw {
   int i0, i1;  // node indices (periodic)
-  int fl;      // first node relative to the start cell
   T w0, w1;
-  bool two;
 };
 
 // Periodic index of i in [-n, 2n).
 __device__ __forceinline__ int wrap1(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
-// nodes[k] = periodic index of start cell + k - 1, k = 0..3
+// nodes[k] = periodic index of start cell + k - 1, k = 0..3; st: half-staggered nodes
 template <typename T>
-__device__ __forceinline__ Gw<T> gweights(T o, int st, int order, const int nodes[4]) {
+__device__ __forceinline__ Gw<T> gweights(T o, int st, const int nodes[4]) {
   Gw<T> g;
-  if (order == 1) {
-    const T xs = st ? o - T(0.5) : o;
-    const int fl = xs < T(0) ? -1 : 0;
-    const T fr = xs - T(fl);
-    g.i0 = fl < 0 ? nodes[0] : nodes[1];
-    g.i1 = fl < 0 ? nodes[1] : nodes[2];
-    g.fl = fl;
-    g.w0 = T(1) - fr;
-    g.w1 = fr;
-    g.two = true;
-  } else {
-    const T xs = st ? o : o + T(0.5);  // the box of the node floor(x - st/2 + 1/2)
-    const int fl = xs >= T(1) ? 1 : 0;
-    g.i0 = g.i1 = fl ? nodes[2] : nodes[1];
-    g.fl = fl;
-    g.w0 = T(1);
-    g.w1 = T(0);
-    g.two = false;
-  }
+  const T xs = st ? o - T(0.5) : o;
+  const int fl = xs < T(0) ? -1 : 0;
+  const T fr = xs - T(fl);
+  g.i0 = fl < 0 ? nodes[0] : nodes[1];
+  g.i1 = fl < 0 ? nodes[1] : nodes[2];
+  g.w0 = T(1) - fr;
+  g.w1 = fr;
   return g;
 }
 
@@ -187,98 +174,36 @@ __device__ __forceinline__ void atomic_add(T* p, T v) {
 constexpr int ADJ_THREADS = 128;
 
 // Inclusive sum of v over the run of consecutive lanes that hold the same key (the run starts at
-// lane `start`); the last lane of a run ends with the run's total. All 32 lanes take part.
+// lane `start`); the last lane of a run ends with the run's total. All 32 lanes take part; `longest`: the
+// warp's longest run (uniform).
 template <typename T>
-__device__ __forceinline__ T run_sum(T v, int start, int lane) {
+__device__ __forceinline__ T run_sum(T v, int start, int lane, int longest) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
+    if (o >= longest) break;
     const T t = __shfl_up_sync(0xffffffffu, v, o);
     if (lane - o >= start) v += t;
   }
   return v;
 }
 
-template <typename T, int SCHEME>
-__global__ void __launch_bounds__(ADJ_THREADS) k_adj_particles(const __grid_constant__ AdjPartArgs<T> a) {
-  // Consecutive ids start close together (the beam keeps its lattice order), so neighbouring lanes
-  // mostly add into the same nodes of the copies' adjoint: each node's contributions are summed over
-  // the run of lanes that share it, and the run's last lane adds the total to global memory.
-  const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const int nx = a.nx, nz = a.nz;
-  bool active = p < a.n;
-  int cell = 0, s = 0;
-  if (active) {
-    cell = a.cell[p];
-    s = a.species[p];
-    if (cell < 0 || cell >= nx * nz || (s != 0 && s != 1)) {  // a particle the recomputed step lost
-      flag_error(a.err, ERR_IDS);
-      active = false;
-      cell = 0;
-      s = 0;
-    }
-  }
-  const int ck = cell / nx, ci = cell - ck * nx;
-  int ix[4], iz[4];  // periodic node indices of the start cell - 1 .. + 2
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    ix[q] = wrap1(ci + q - 1, nx);
-    iz[q] = wrap1(ck + q - 1, nz);
-  }
-  T lF[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-  T ox = T(0), oz = T(0);
-  if (active) {
-  ox = a.ox[p];
-  oz = a.oz[p];
-  const T ux0 = a.dux[p], uy0 = a.duy[p], uz0 = a.duz[p];
-  const T w = a.w ? a.w[p] : a.wconst;
-  const T qs = s ? T(1) : T(-1);
+// Gradient of lambda_J . J, the Esirkepov current of one particle against the adjoint of J, in its
+// offsets, displacements and v_y.
+template <typename T>
+struct DepGrad {
+  T ox, dx, oz, dz, vy;
+};
 
-  // 1. gather at x^n (recomputed) with the derivatives of each component in ox and oz
-  T F[6], dFx[6], dFz[6];
-  Gw<T> gx[6], gz[6];
-#pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    const int sx = kStagX[c], sz = kStagZ[c];
-    gx[c] = gweights(ox, sx, SCHEME == 0 ? 1 - sx : 1, ix);
-    gz[c] = gweights(oz, sz, SCHEME == 0 ? 1 - sz : 1, iz);
-    const T* G0 = a.g[c] + gz[c].i0 * nx;  // 32-bit offsets: the launcher caps the cell count
-    const T* G1 = a.g[c] + gz[c].i1 * nx;
-    const T g00 = G0[gx[c].i0], g01 = G0[gx[c].i1], g10 = G1[gx[c].i0], g11 = G1[gx[c].i1];
-    const T zx0 = gz[c].w0 * gx[c].w0, zx1 = gz[c].w0 * gx[c].w1, zx2 = gz[c].w1 * gx[c].w0, zx3 = gz[c].w1 * gx[c].w1;
-    F[c] = zx0 * g00 + zx1 * g01 + zx2 * g10 + zx3 * g11;
-    dFx[c] = gx[c].two ? gz[c].w0 * (g01 - g00) + gz[c].w1 * (g11 - g10) : T(0);
-    dFz[c] = gz[c].two ? gx[c].w0 * (g10 - g00) + gx[c].w1 * (g11 - g01) : T(0);
-  }
-
-  // 2. Boris u^{n-1/2} -> u^{n+1/2} (recomputed; momenta relative to the drift u0 z_hat)
-  const T h = qs * a.hq;
-  const T mx = ux0 + h * F[0], my = uy0 + h * F[1], mz = uz0 + h * F[2];
-  const T Mz = a.u0 + mz;
-  const T gm = sqrt(T(1) + mx * mx + my * my + Mz * Mz);
-  const T igm = T(1) / gm;
-  const T tx = h * F[3] * igm, ty = h * F[4] * igm, tz = h * F[5] * igm;
-  const T tt = tx * tx + ty * ty + tz * tz;
-  const T den = T(1) + tt;
-  const T iden = T(1) / den;
-  const T sx = T(2) * tx * iden, sy = T(2) * ty * iden, sz = T(2) * tz * iden;
-  const T px = mx + (my * tz - Mz * ty), py = my + (Mz * tx - mx * tz), pz = Mz + (mx * ty - my * tx);
-  const T ux = mx + (py * sz - pz * sy) + h * F[0];
-  const T uy = my + (pz * sx - px * sz) + h * F[1];
-  const T uz = mz + (px * sy - py * sx) + h * F[2];
-  const T Uz = a.u0 + uz;
-  const T ux2 = ux * ux, uy2 = uy * uy, uz2 = Uz * Uz;
-  const T gam = sqrt(T(1) + ux2 + uy2 + uz2);
-  const T ig = T(1) / gam;
-  const T vx = ux * ig, vy = uy * ig, vz = Uz * ig;
-  const T ddx = a.dtdx * vx, ddz = a.dtdz * vz;
-
-  // 3. Esirkepov transpose: lambda_J . J as a function of (ox, ddx, oz, ddz, vy)
+// Any move of less than a cell: the window nodes -1 .. 2 of the start cell.
+template <typename T>
+__device__ __noinline__ DepGrad<T> deposit_grad_any(const AdjPartArgs<T>& a, int ix0, int ix1, int ix2, int ix3, int iz0,
+                                                    int iz1, int iz2, int iz3, T ox, T ddx, T oz, T ddz, T vy, T cx,
+                                                    T cz, T cyc) {
+  const int ix[4] = {ix0, ix1, ix2, ix3}, iz[4] = {iz0, iz1, iz2, iz3}, nx = a.nx;
+  DepGrad<T> g = {T(0), T(0), T(0), T(0), T(0)};
   Win<T> wx, wz;
   shape_win(ox, ddx, wx);
   shape_win(oz, ddz, wz);
-  const T qw = qs * w;
-  const T cx = qw * a.jfx, cz = qw * a.jfz, cyc = qw * a.jfy2d;
   T gS0x[4] = {}, gdSx[4] = {}, gS0z[4] = {}, gdSz[4] = {};
   T Tx[4], Tz[4];
 #pragma unroll
@@ -325,35 +250,180 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_particles(const __grid_cons
       Db[b] += l * wx.dS[q];
     }
   }
-  T gcy = T(0);
   const T lvy = cyc * vy, k12 = T(1.0 / 12.0);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    gcy += Tx[q] * Aq[q] + k12 * wx.dS[q] * Bq[q];
+    g.vy += Tx[q] * Aq[q] + k12 * wx.dS[q] * Bq[q];
     gS0x[q] += lvy * Aq[q];
     gdSx[q] += lvy * (T(0.5) * Aq[q] + k12 * Bq[q]);
     gS0z[q] += lvy * Cb[q];
     gdSz[q] += lvy * (T(0.5) * Cb[q] + k12 * Db[q]);
   }
-  gcy *= cyc;
-  T lox_dep = T(0), lddx = T(0), loz_dep = T(0), lddz = T(0);
+  g.vy *= cyc;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     gS0x[q] += gTx[q];
     gdSx[q] += T(0.5) * gTx[q];
     gS0z[q] += gTz[q];
     gdSz[q] += T(0.5) * gTz[q];
-    lox_dep += gS0x[q] * wx.dS0o[q] + gdSx[q] * wx.dSo[q];
-    lddx += gdSx[q] * wx.dSd[q];
-    loz_dep += gS0z[q] * wz.dS0o[q] + gdSz[q] * wz.dSo[q];
-    lddz += gdSz[q] * wz.dSd[q];
+    g.ox += gS0x[q] * wx.dS0o[q] + gdSx[q] * wx.dSo[q];
+    g.dx += gdSx[q] * wx.dSd[q];
+    g.oz += gS0z[q] * wz.dS0o[q] + gdSz[q] * wz.dSo[q];
+    g.dz += gdSz[q] * wz.dSd[q];
   }
+  return g;
+}
+
+// A move that stays in its cell along x and stays or steps up along z (`up`): the window nodes 0-1 and
+// 0-2. With x: T = (1 - o - d/2, o + d/2), dS = (-d, d), and z: e0 = 1 - o or d (up or not), e2 = c or 0,
+// e1 = e0 - e2, T = (1 - o - e0/2, o + e1/2, e2/2), dS = (-e0, e1, e2) (the deposit's form in the push),
+// the currents are Jx(b) = -cx d Tz_b, Jz(a, 0) = -cz e0 Tx_a, Jz(a, 1) = -cz e2 Tx_a and Jy(a, b) = cy
+// (Tx_a Tz_b + dSx_a dSz_b / 12); 13 values of lambda_J instead of the general window's 40.
+template <typename T>
+__device__ __forceinline__ DepGrad<T> deposit_grad_near(const AdjPartArgs<T>& a, int x0, int x1, int r0, int r1, int r2,
+                                                        T ox, T d, T oz, T ddz, bool up, T vy, T cx, T cz, T cyc) {
+  const T am = T(1) - oz, c = ddz - am, half = T(0.5), k12 = T(1.0 / 12.0);
+  const T e0 = up ? am : ddz, e2 = up ? c : T(0), e1 = e0 - e2;
+  const T tx0 = fma(-half, d, T(1) - ox), tx1 = fma(half, d, ox);
+  const T tz[3] = {fma(-half, e0, am), fma(half, e1, oz), half * e2};
+  const T ds[3] = {-e0, e1, e2};
+  const int row[3] = {r0, r1, r2};
+  const T lvy = cyc * vy, k = lvy * d * k12, cxd = -cx * d;
+  T sx = T(0), A = T(0), B = T(0), t0 = T(0), t1 = T(0), gt[3], gd[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    const T lx = a.lj[0][row[b] + x0], l0 = a.lj[1][row[b] + x0], l1 = a.lj[1][row[b] + x1];
+    const T sb = fma(tx1, l1, tx0 * l0), q = l1 - l0;
+    sx = fma(lx, tz[b], sx);
+    A = fma(sb, tz[b], A);
+    B = fma(q, ds[b], B);
+    t0 = fma(l0, tz[b], t0);
+    t1 = fma(l1, tz[b], t1);
+    gt[b] = fma(cxd, lx, lvy * sb);
+    gd[b] = k * q;
+  }
+  const T z00 = a.lj[2][r0 + x0], z01 = a.lj[2][r1 + x0], z10 = a.lj[2][r0 + x1], z11 = a.lj[2][r1 + x1];
+  const T dt = fma(lvy, t1 - t0, -cz * fma(e0, z10 - z00, e2 * (z11 - z01)));  // gTx1 - gTx0
+  const T g1 = fma(half, gt[1], gd[1]);
+  const T ge0 = fma(-half, gt[0], -gd[0]) + g1 - cz * fma(tx1, z10, tx0 * z00);
+  const T ge2 = fma(half, gt[2], gd[2]) - g1 - cz * fma(tx1, z11, tx0 * z01);
+  DepGrad<T> g;
+  g.vy = cyc * fma(d * k12, B, A);
+  g.ox = dt;
+  g.dx = fma(half, dt, fma(lvy * k12, B, -cx * sx));
+  g.oz = gt[1] - gt[0] + (up ? ge2 - ge0 : T(0));
+  g.dz = up ? ge2 : ge0;
+  return g;
+}
+
+template <typename T, int SCHEME>
+__global__ void __launch_bounds__(ADJ_THREADS, sizeof(T) == 4 ? 4 : 2) k_adj_particles(const __grid_constant__ AdjPartArgs<T> a) {
+  // Consecutive ids start close together (the beam keeps its lattice order), so neighbouring lanes
+  // mostly add into the same nodes of the copies' adjoint: each node's contributions are summed over
+  // the run of lanes that share it, and the run's last lane adds the total to global memory.
+  const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int nx = a.nx, nz = a.nz;
+  bool active = p < a.n;
+  int cell = 0, s = 0;
+  if (active) {
+    cell = a.cell[p];
+    s = a.species[p];
+    if (cell < 0 || cell >= nx * nz || (s != 0 && s != 1)) {  // a particle the recomputed step lost
+      flag_error(a.err, ERR_IDS);
+      active = false;
+      cell = 0;
+      s = 0;
+    }
+  }
+  const int ck = cell / nx, ci = cell - ck * nx;
+  int ix[4], iz[4];  // periodic node indices of the start cell - 1 .. + 2
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    ix[q] = wrap1(ci + q - 1, nx);
+    iz[q] = wrap1(ck + q - 1, nz);
+  }
+  T lF[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+  T ox = T(0), oz = T(0);
+  if (active) {
+  ox = a.ox[p];
+  oz = a.oz[p];
+  const T ux0 = a.dux[p], uy0 = a.duy[p], uz0 = a.duz[p];
+  const T w = a.w ? a.w[p] : a.wconst;
+  const T qs = s ? T(1) : T(-1);
+
+  // 1. gather at x^n (recomputed) with the derivatives of each component in ox and oz
+  T F[6], dFx[6], dFz[6];
+  if constexpr (SCHEME == 0) {  // order 0 along each half-staggered direction: the cell's own nodes
+    const int r0 = iz[1] * nx, r1 = iz[2] * nx, x0 = ix[1], x1 = ix[2];
+    auto along = [&](const T* G, int n0, int n1, T o, T& d) {  // linear between two nodes
+      const T v0 = G[n0];
+      d = G[n1] - v0;
+      return fma(o, d, v0);
+    };
+    F[0] = along(a.g[0], r0 + x0, r1 + x0, oz, dFz[0]);
+    F[2] = along(a.g[2], r0 + x0, r0 + x1, ox, dFx[2]);
+    F[3] = along(a.g[3], r0 + x0, r0 + x1, ox, dFx[3]);
+    F[4] = a.g[4][r0 + x0];
+    F[5] = along(a.g[5], r0 + x0, r1 + x0, oz, dFz[5]);
+    T d0, d1;
+    const T y0 = along(a.g[1], r0 + x0, r0 + x1, ox, d0), y1 = along(a.g[1], r1 + x0, r1 + x1, ox, d1);
+    dFz[1] = y1 - y0;
+    dFx[1] = fma(oz, d1 - d0, d0);
+    F[1] = fma(oz, dFz[1], y0);
+    dFx[0] = dFx[4] = dFx[5] = dFz[2] = dFz[3] = dFz[4] = T(0);
+  } else {
+    Gw<T> gx[6], gz[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const int sx = kStagX[c], sz = kStagZ[c];
+      gx[c] = gweights(ox, sx, ix);
+      gz[c] = gweights(oz, sz, iz);
+      const T* G0 = a.g[c] + gz[c].i0 * nx;  // 32-bit offsets: the launcher caps the cell count
+      const T* G1 = a.g[c] + gz[c].i1 * nx;
+      const T g00 = G0[gx[c].i0], g01 = G0[gx[c].i1], g10 = G1[gx[c].i0], g11 = G1[gx[c].i1];
+      const T zx0 = gz[c].w0 * gx[c].w0, zx1 = gz[c].w0 * gx[c].w1, zx2 = gz[c].w1 * gx[c].w0,
+              zx3 = gz[c].w1 * gx[c].w1;
+      F[c] = zx0 * g00 + zx1 * g01 + zx2 * g10 + zx3 * g11;
+      dFx[c] = gz[c].w0 * (g01 - g00) + gz[c].w1 * (g11 - g10);
+      dFz[c] = gx[c].w0 * (g10 - g00) + gx[c].w1 * (g11 - g01);
+    }
+  }
+
+  // 2. Boris u^{n-1/2} -> u^{n+1/2} (recomputed; momenta relative to the drift u0 z_hat)
+  const T h = qs * a.hq;
+  const T mx = ux0 + h * F[0], my = uy0 + h * F[1], mz = uz0 + h * F[2];
+  const T Mz = a.u0 + mz;
+  const T igm = fine_rsqrt(T(1) + mx * mx + my * my + Mz * Mz);
+  const T tx = h * F[3] * igm, ty = h * F[4] * igm, tz = h * F[5] * igm;
+  const T tt = tx * tx + ty * ty + tz * tz;
+  const T den = T(1) + tt;
+  const T iden = fine_recip(den);
+  const T sx = T(2) * tx * iden, sy = T(2) * ty * iden, sz = T(2) * tz * iden;
+  const T px = mx + (my * tz - Mz * ty), py = my + (Mz * tx - mx * tz), pz = Mz + (mx * ty - my * tx);
+  const T ux = mx + (py * sz - pz * sy) + h * F[0];
+  const T uy = my + (pz * sx - px * sz) + h * F[1];
+  const T uz = mz + (px * sy - py * sx) + h * F[2];
+  const T Uz = a.u0 + uz;
+  const T ux2 = ux * ux, uy2 = uy * uy, uz2 = Uz * Uz;
+  const T ig = fine_rsqrt(T(1) + ux2 + uy2 + uz2);
+  const T vx = ux * ig, vy = uy * ig, vz = Uz * ig;
+  const T ddx = a.dtdx * vx, ddz = a.dtdz * vz;
+
+  // 3. Esirkepov transpose
+  const T qw = qs * w;
+  const T cx = qw * a.jfx, cz = qw * a.jfz, cyc = qw * a.jfy2d;
+  const T x1 = ox + ddx, z1 = oz + ddz;
+  const bool near_win = !(x1 < T(0) || (x1 >= T(1) && ddx - (T(1) - ox) > T(0)) || z1 < T(0));
+  const DepGrad<T> dg =
+      near_win ? deposit_grad_near(a, ix[1], ix[2], iz[1] * nx, iz[2] * nx, iz[3] * nx, ox, ddx, oz, ddz,
+                                   z1 >= T(1) && ddz - (T(1) - oz) > T(0), vy, cx, cz, cyc)
+               : deposit_grad_any(a, ix[0], ix[1], ix[2], ix[3], iz[0], iz[1], iz[2], iz[3], ox, ddx, oz, ddz, vy, cx, cz,
+                                  cyc);
 
   // 4. move transpose: x^{n+1} = x^n + d, d = (dt/dx) u / gamma
   const T lx1 = a.lox[p], lz1 = a.loz[p];
-  lddx += lx1;
-  lddz += lz1;
-  const T gxv = lddx * a.dtdx, gyv = gcy, gzv = lddz * a.dtdz;  // adjoints of vx, vy, vz
+  const T gxv = (dg.dx + lx1) * a.dtdx, gyv = dg.vy, gzv = (dg.dz + lz1) * a.dtdz;  // adjoints of vx, vy, vz
   // d(u_i/gamma)/du_j = (delta_ij (1 + |u|^2) - u_i u_j) / gamma^3, with 1 + |u|^2 - u_i^2 summed
   // from the other components (no cancellation at large gamma)
   const T ig3 = ig * ig * ig;
@@ -399,7 +469,7 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_particles(const __grid_cons
   a.luz[p] = lmz;
 
   // 6. gather transpose: the weights' dependence on x^n here, the copies' adjoint below
-  T lox = lx1 + lox_dep, loz = lz1 + loz_dep;
+  T lox = lx1 + dg.ox, loz = lz1 + dg.oz;
   const T lFv[6] = {lE[0], lE[1], lE[2], lB[0], lB[1], lB[2]};
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
@@ -412,33 +482,51 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_particles(const __grid_cons
   }  // active
   // adjoint of the copies: lambda_F times the gather weights, summed over runs of lanes that share
   // the component's base node (inactive lanes carry zeros under keys of their own)
-#pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    const int sx = kStagX[c], sz = kStagZ[c];
-    const Gw<T> wx = gweights(ox, sx, SCHEME == 0 ? 1 - sx : 1, ix);
-    const Gw<T> wz = gweights(oz, sz, SCHEME == 0 ? 1 - sz : 1, iz);
-    const int key = active ? wz.i0 * nx + wx.i0 : -1 - lane;
+  int start = 0, longest = 0;
+  bool tail = false;
+  auto runs_of = [&](int key) {
     const int prev = __shfl_up_sync(0xffffffffu, key, 1);
     const int next = __shfl_down_sync(0xffffffffu, key, 1);
     const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || prev != key);
-    const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-    const bool tail = active && (lane == 31 || next != key);
+    start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+    tail = active && (lane == 31 || next != key);
+    longest = __reduce_max_sync(0xffffffffu, lane - start + 1);
+  };
+  auto add = [&](T* node, T v) {
+    const T t = run_sum(v, start, lane, longest);
+    if (tail) atomic_add(node, t);
+  };
+  if constexpr (SCHEME == 0) {  // every component's base node is the cell's: one set of runs
+    runs_of(active ? cell : -1 - lane);
+    const int n00 = iz[1] * nx + ix[1], n10 = iz[1] * nx + ix[2], n01 = iz[2] * nx + ix[1], n11 = iz[2] * nx + ix[2];
+    const T px = T(1) - ox, pz = T(1) - oz;
+    add(a.lg[0] + n00, lF[0] * pz);
+    add(a.lg[0] + n01, lF[0] * oz);
+    add(a.lg[1] + n00, lF[1] * pz * px);
+    add(a.lg[1] + n10, lF[1] * pz * ox);
+    add(a.lg[1] + n01, lF[1] * oz * px);
+    add(a.lg[1] + n11, lF[1] * oz * ox);
+    add(a.lg[2] + n00, lF[2] * px);
+    add(a.lg[2] + n10, lF[2] * ox);
+    add(a.lg[3] + n00, lF[3] * px);
+    add(a.lg[3] + n10, lF[3] * ox);
+    add(a.lg[4] + n00, lF[4]);
+    add(a.lg[5] + n00, lF[5] * pz);
+    add(a.lg[5] + n01, lF[5] * oz);
+  } else {
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const int sx = kStagX[c], sz = kStagZ[c];
+    const Gw<T> wx = gweights(ox, sx, ix);
+    const Gw<T> wz = gweights(oz, sz, iz);
+    runs_of(active ? wz.i0 * nx + wx.i0 : -1 - lane);
     T* LG = a.lg[c];
     const T v = lF[c];
-    const T s00 = run_sum(v * wz.w0 * wx.w0, start, lane);
-    if (tail) atomic_add(LG + wz.i0 * nx + wx.i0, s00);
-    if (wx.two) {  // the same for every lane (the order depends on the component only)
-      const T s01 = run_sum(v * wz.w0 * wx.w1, start, lane);
-      if (tail) atomic_add(LG + wz.i0 * nx + wx.i1, s01);
-    }
-    if (wz.two) {
-      const T s10 = run_sum(v * wz.w1 * wx.w0, start, lane);
-      if (tail) atomic_add(LG + wz.i1 * nx + wx.i0, s10);
-      if (wx.two) {
-        const T s11 = run_sum(v * wz.w1 * wx.w1, start, lane);
-        if (tail) atomic_add(LG + wz.i1 * nx + wx.i1, s11);
-      }
-    }
+    add(LG + wz.i0 * nx + wx.i0, v * wz.w0 * wx.w0);
+    add(LG + wz.i0 * nx + wx.i1, v * wz.w0 * wx.w1);
+    add(LG + wz.i1 * nx + wx.i0, v * wz.w1 * wx.w0);
+    add(LG + wz.i1 * nx + wx.i1, v * wz.w1 * wx.w1);
+  }
   }
 }
 
@@ -458,9 +546,37 @@ template cudaError_t launch_adj_particles<double>(const AdjPartArgs<double>&, in
 //   lf_q += Psi_q(D_z) y_q          (y = F_filter applied to the adjoint of the copies)
 //   dots[n] += f_q . D_z^n y_q      (n = 0..4; Psi_E rows for q < 2, Psi_B rows for q >= 2)
 // since G_q = Psi_q(D_z) F_filter f_q with Psi_q = sum_n a_n D^n, every operator symmetric.
-// Block partial sums in FP64, one atomic per block and coefficient.
+// Block partial sums in FP64.
 // ---------------------------------------------------------------------------------------------
-constexpr int PSI_BLOCKS = 304;  // blocks per component (grid-stride), partial sums per block
+// Blocks per component (grid-stride), partial sums per block. Few, because the block reductions and the
+// final sum over the partials cost more than the passes over the cells (with 304 blocks and FP64 products
+// 45 + 13 us on 256x512 cells).
+constexpr int PSI_BLOCKS = 76;
+
+// A sum of products per thread: FP32 as a pair (the product exact in two floats, added by TwoSum), because
+// the FP64 pipe would bound this kernel; FP64 in FP64.
+template <typename T>
+struct PsiSum;
+template <>
+struct PsiSum<float> {
+  FPair p;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float x = a * b;
+    p = pair_add(p, FPair{x, fmaf(a, b, -x)});
+  }
+  __device__ __forceinline__ void warp_sum() { p = warp_sum_pair(p); }
+  __device__ __forceinline__ double get() const { return (double)p.s + (double)p.c; }
+};
+template <>
+struct PsiSum<double> {
+  double p;
+  __device__ __forceinline__ void add(double a, double b) { p = fma(a, b, p); }
+  __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+  }
+  __device__ __forceinline__ double get() const { return p; }
+};
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_adj_psi(const __grid_constant__ AdjPsiArgs<T> a) {
@@ -476,7 +592,7 @@ __global__ void __launch_bounds__(256) k_adj_psi(const __grid_constant__ AdjPsiA
 #pragma unroll
     for (int n = 0; n < 5; ++n) dp[n][m] = a.dpow[n][m];
   }
-  double dn[5] = {0, 0, 0, 0, 0};
+  PsiSum<T> dn[5] = {};
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < a.ncell;
        c += (long long)gridDim.x * blockDim.x) {
     const long long k = c / a.nxy, base = c - k * a.nxy;
@@ -492,28 +608,26 @@ __global__ void __launch_bounds__(256) k_adj_psi(const __grid_constant__ AdjPsiA
 #pragma unroll
     for (int m = 0; m < 9; ++m) psi += taps[m] * y[m];
     L[c] += psi;
-    const double f = (double)Fq[c];
+    const T f = Fq[c];
 #pragma unroll
     for (int n = 0; n < 5; ++n) {
       T v = T(0);
 #pragma unroll
       for (int m = 0; m < 9; ++m) v += dp[n][m] * y[m];
-      dn[n] += f * (double)v;
+      dn[n].add(f, v);
     }
   }
-  __shared__ double red[5][8];
+  __shared__ PsiSum<T> red[5][8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
   for (int n = 0; n < 5; ++n) {
-    double v = dn[n];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[n][wid] = v;
+    dn[n].warp_sum();
+    if (lane == 0) red[n][wid] = dn[n];
   }
   __syncthreads();
   if (threadIdx.x < 5) {
     double t = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[threadIdx.x][w];
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[threadIdx.x][w].get();
     a.partial[((long long)q * gridDim.x + blockIdx.x) * 5 + threadIdx.x] = t;
   }
 }

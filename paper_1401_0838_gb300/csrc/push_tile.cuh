@@ -1091,14 +1091,6 @@ __device__ __forceinline__ void deposit3_cubic(const T* stq, const T* str, const
   }
 }
 
-// Reciprocal square root of the window gathers' push: FP32 refined by one Newton step (as accurate as
-// the quotient 1 / sqrt), FP64 as fast_rsqrt.
-__device__ __forceinline__ double fine_rsqrt(double x) { return fast_rsqrt(x); }
-__device__ __forceinline__ float fine_rsqrt(float x) {
-  const float y = rsqrtf(x);
-  return fmaf(fmaf(-0.5f * x * y, y, 0.5f), y, y);
-}
-
 template <typename T, int NDIM, int SCHEME, int LPC, int ORDER = 1>
 __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   constexpr bool WIN = ORDER == 3 || SCHEME == 2;    // the gather reads the cell's window of nodes
