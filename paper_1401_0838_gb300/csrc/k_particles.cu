@@ -166,9 +166,13 @@ static void tile_of(int ndim, int te[3]) {
 
 void push_tiles(int ndim, int es, bool ho, int nx, int ny, int nz, int spread, int nt[3], int te[3]) {
   const int n[3] = {nx, ndim == 3 ? ny : 1, nz};
-  if (es == 4) ho ? tile_of<HoTile, float>(ndim, te) : tile_of<PTile, float>(ndim, te);
-  else ho ? tile_of<HoTile, double>(ndim, te) : tile_of<PTile, double>(ndim, te);
-  auto count = [&]() {
+  int full[3];
+  if (es == 4) ho ? tile_of<HoTile, float>(ndim, full) : tile_of<PTile, float>(ndim, full);
+  else ho ? tile_of<HoTile, double>(ndim, full) : tile_of<PTile, double>(ndim, full);
+  auto set = [&](int ex, int ey, int ez) {
+    te[0] = ex;
+    te[1] = ey;
+    te[2] = ez;
     long long t = 1;
     for (int d = 0; d < 3; ++d) {
       nt[d] = (n[d] + te[d] - 1) / te[d];
@@ -176,15 +180,31 @@ void push_tiles(int ndim, int es, bool ho, int nx, int ny, int nz, int spread, i
     }
     return t;
   };
-  long long tiles = count();
-  while (spread > 0 && 2 * tiles <= spread) {
-    int d = -1;  // the longest extent above 4 that still splits the grid further
-    for (int k = 0; k < 3; ++k)
-      if (te[k] > 4 && n[k] > te[k] / 2 && (d < 0 || te[k] > te[d])) d = k;
-    if (d < 0) break;
-    te[d] /= 2;
-    tiles = count();
-  }
+  set(full[0], full[1], full[2]);
+  if (spread <= 0) return;
+  // the resident blocks, and a tile's fixed cost (prologue and epilogue) in cells
+  const bool two = es == 4 && !(ndim == 3 && ho);
+  const long long slots = (long long)spread * (two ? 2 : 1);
+  const int fixed = es == 4 ? 40 : 6;
+  auto cost_of = [&](long long tiles) {
+    return (double)((tiles + slots - 1) / slots) * ((double)te[0] * te[1] * te[2] + fixed);
+  };
+  const long long all = set(full[0], full[1], full[2]);
+  if (two && all > slots) return;  // several waves of block pairs: the partner of a late block speeds it up
+  double best = 0.97 * cost_of(all);  // full tiles unless others gain 3 %
+  int b[3] = {full[0], full[1], full[2]};
+  for (int ex = full[0]; ex >= 4 || ex == full[0]; ex /= 2)
+    for (int ey = full[1]; ey >= 4 || ey == full[1]; ey /= 2)
+      for (int ez = full[2]; ez >= 4 || ez == full[2]; --ez) {
+        const double cost = cost_of(set(ex, ey, ez));
+        if (cost < best * (1 - 1e-9)) {
+          best = cost;
+          b[0] = ex;
+          b[1] = ey;
+          b[2] = ez;
+        }
+      }
+  set(b[0], b[1], b[2]);
 }
 
 // ---------------------------------------------------------------------------------------------
