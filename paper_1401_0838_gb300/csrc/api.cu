@@ -496,6 +496,7 @@ int step_once(pic_handle* h) {
       ia.lam_im[q] = h->inv_li[q];
     }
     ia.scale = h->inv_scale;
+    ia.nsm = h->nsm;
     psi_stencil(h->pe, ia.pe_taps);
     CK(launch(h, PIC_K_COPIES, [&] { return launch_inverse_psi_z<T>(ia, st); }), "inverse Psi_B");
   }

@@ -5,6 +5,8 @@
 #include "common.cuh"
 #include "launch.h"
 
+#include <algorithm>
+#include <cmath>
 #include <mutex>
 #include <unordered_map>
 
@@ -1338,114 +1340,234 @@ __global__ void k_inverse_psi_z(InvPsiArgs<T> a) {
   for (int k = 0; k < nz; ++k) f[k * nxy + l] = (T)(a.scale * w[k * nxy + l].x);
 }
 
-// The same operator with one warp per z-line and the line in shared memory (FP64 complex, one
-// padding slot per 32 elements against bank conflicts). Each periodic first-order recursion
-// y_k = x_k + lam y_(k-1) is a blocked scan: every lane runs it over its own chunk of L = ceil(nz/32)
-// elements from zero, the 32 chunk maps y -> lam^len y + e are composed around the ring by a cyclic
-// doubling scan (Y_j = A_j Y_j + B_j after the full window, so Y_j = B_j / (1 - lam^nz)), and each
-// lane adds lam^(i+1) times the previous chunk's end value to its elements.
-constexpr int IPZ_LINES = 8;  // z-lines (warps) per block
+// The same operator with one warp per z-line and the line in shared memory. The recursions are real and of
+// second order: two factors (1 - lam1 S)(1 - lam2 S), a conjugate pair or two real ones, are y_k = x_k + a
+// y_(k-1) - b y_(k-2) with a = lam1 + lam2, b = lam1 lam2, two FMAs an element where the complex first-order
+// recursions took sixteen. What bounds this kernel is the FP64 pipe (a warp's instruction holds its
+// scheduler's for 64 cycles), so everything that does not depend on the data comes in ready: with the state
+// (y_k, y_(k-1)) and M its step matrix, a lane runs its chunk of L elements from zero, a scan over the lanes
+// applies M^(L 2^q), and every lane runs its chunk again from its own start. The scan runs around the
+// period and stops once the matrix of its window is below 1e-20, a share of the state that no rounding
+// sees; on lines too short for that it runs over the whole line, and the periodic start state is
+// (I - M^nz)^-1 times the last lane's. Psi_E(D_z) is applied on the way out (all of it commutes).
+// A launch on 128x128 cells 75 -> 16 us, on 512x1024 160 -> 71 us; the pass of 100 steps around it 12.5 -> 6.6 ms.
+struct InvSection {
+  double a, b;
+  double m[5][4];   // M^(L 2^q)
+  double mp[5][4];  // M^((2^q - 1) L + r), r = the last chunk's length
+  double c[4];      // (I - M^nz)^-1
+  int around;       // steps of the scan around the period, 0: the line is too short for it
+};
+struct InvLines {
+  int nsec, L, nl;  // sections, elements per lane, lanes in use
+  unsigned over_l;  // 2^32 / L for an even L: the chunks lie L + 1 apart, so that they spread over the banks; 0: odd
+  InvSection s[2];
+};
 
-__device__ __forceinline__ double2 c_mul(double2 a, double2 b) {
-  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+__device__ __forceinline__ double2 m_apply(const double (&m)[4], double2 v) {
+  return make_double2(fma(m[0], v.x, m[1] * v.y), fma(m[2], v.x, m[3] * v.y));
 }
-__device__ __forceinline__ double2 c_fma(double2 a, double2 b, double2 c) {  // a b + c
-  return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
+__device__ __forceinline__ double2 m_apply_add(const double (&m)[4], double2 v, double2 t) {
+  return make_double2(fma(m[0], v.x, fma(m[1], v.y, t.x)), fma(m[2], v.x, fma(m[3], v.y, t.y)));
 }
-__device__ __forceinline__ double2 c_shfl(double2 v, int src) {
+__device__ __forceinline__ double2 d2_shfl(double2 v, int src) {
   return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
-__device__ __forceinline__ int ipz_pad(int k) { return k + (k >> 5); }
 
-__device__ __forceinline__ void periodic_recursion(double2* w, int nz, double2 lam, bool rev, int lane) {
-  const int L = (nz + 31) >> 5;
-  const int k0 = min(lane * L, nz), k1 = min(k0 + L, nz);
-  // 1. the chunk's recursion from zero; mu = lam^len
-  double2 y = make_double2(0.0, 0.0), mu = make_double2(1.0, 0.0);
-  for (int k = k0; k < k1; ++k) {
-    double2& v = w[ipz_pad(rev ? nz - 1 - k : k)];
-    y = c_fma(lam, y, v);
-    v = y;
-    mu = c_mul(mu, lam);
+// One periodic recursion over the line's chunks w[chunk * LP + i]: upwards, or (rev) downwards, where lane 0
+// takes the last chunk, which may be short.
+template <bool REV>
+__device__ __forceinline__ void periodic_section(double* w, const InvSection& sc, int nz, int L, int LP, int nl,
+                                                 int lane) {
+  const bool on = lane < nl;
+  const int chunk = REV ? nl - 1 - lane : lane;
+  const int len = on ? min(L, nz - chunk * L) : 0;
+  double* v = w + chunk * LP;
+  double2 B = make_double2(0.0, 0.0);
+  for (int i = 0; i < len; ++i) {
+    const double y = fma(sc.a, B.x, fma(-sc.b, B.y, v[REV ? len - 1 - i : i]));
+    B.y = B.x;
+    B.x = y;
   }
-  // 2. cyclic composition of the chunk maps: Y_j = A Y_(j - window) + B
-  double2 A = mu, B = y;
+  double2 y;
+  if (sc.around > 0) {
+    for (int q = 0; q < sc.around; ++q) {
+      const int src = lane - (1 << q);
+      const double2 t = d2_shfl(B, (src < 0 ? src + nl : src) & 31);
+      // the window of 2^q chunks that ends here holds the short one
+      const bool partial = REV ? lane < (1 << q) : (lane == nl - 1 || lane < (1 << q) - 1);
+      double m[4];
 #pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const double2 Ap = c_shfl(A, (lane - s) & 31), Bp = c_shfl(B, (lane - s) & 31);
-    B = c_fma(A, Bp, B);
-    A = c_mul(A, Ap);
+      for (int e = 0; e < 4; ++e) m[e] = partial ? sc.mp[q][e] : sc.m[q][e];
+      B = m_apply_add(m, t, B);
+    }
+    y = d2_shfl(B, lane == 0 ? nl - 1 : lane - 1);
+  } else {
+    const bool partial = !REV && lane == nl - 1;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      const double2 t = d2_shfl(B, (lane - (1 << q)) & 31);
+      double m[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) m[e] = partial ? sc.mp[q][e] : sc.m[q][e];
+      if (lane >= (1 << q)) B = m_apply_add(m, t, B);
+    }
+    y = m_apply(sc.c, d2_shfl(B, nl - 1));  // the periodic start state
+    const double2 before = d2_shfl(B, (lane - 1) & 31);
+    if (REV && lane > 0) y = m_apply(sc.mp[0], y);
+    const int hops = REV ? lane - 1 : lane;  // full chunks between the start and this one
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+      if (hops > 0 && (hops >> q & 1)) y = m_apply(sc.m[q], y);
+    if (lane > 0) {
+      y.x += before.x;
+      y.y += before.y;
+    }
   }
-  const double dr = 1.0 - A.x, di = -A.y, dd = dr * dr + di * di;
-  const double2 Y = make_double2((B.x * dr + B.y * di) / dd, (B.y * dr - B.x * di) / dd);
-  // 3. the previous chunk's end value carried into this chunk
-  const double2 cin = c_shfl(Y, (lane - 1) & 31);
-  double2 p = lam;
-  for (int k = k0; k < k1; ++k) {
-    double2& v = w[ipz_pad(rev ? nz - 1 - k : k)];
-    v = c_fma(p, cin, v);
-    p = c_mul(p, lam);
+  for (int i = 0; i < len; ++i) {
+    double& x = v[REV ? len - 1 - i : i];
+    const double t = fma(sc.a, y.x, fma(-sc.b, y.y, x));
+    y.y = y.x;
+    y.x = t;
+    x = t;
   }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(32 * IPZ_LINES) k_inverse_psi_lines(const __grid_constant__ InvPsiArgs<T> a) {
+__global__ void __launch_bounds__(256) k_inverse_psi_lines(const __grid_constant__ InvPsiArgs<T> a,
+                                                           const __grid_constant__ InvLines s) {
   extern __shared__ __align__(16) unsigned char ipz_raw[];
-  const int nz = a.nz, lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-  const int stride = ipz_pad(nz - 1) + 1;  // padded line length
-  double2* lines = reinterpret_cast<double2*>(ipz_raw);
+  const int nz = a.nz, lane = threadIdx.x & 31, wl = threadIdx.x >> 5, lines = blockDim.x >> 5;
+  const int L = s.L, LP = L | 1, stride = s.nl * LP;
+  double* w = reinterpret_cast<double*>(ipz_raw);
   T* f = blockIdx.y == 0 ? a.f[0] : a.f[1];
-  const long long l0 = (long long)blockIdx.x * IPZ_LINES;
-  const int nl = (int)min((long long)IPZ_LINES, a.nxy - l0);
-  // load the block's lines (consecutive l for each k: 8 values side by side) into the imaginary
-  // slots, which the Psi_E pass reads while it writes the real slots
-  for (int e = threadIdx.x; e < nz * IPZ_LINES; e += blockDim.x) {
-    const int k = e / IPZ_LINES, li = e % IPZ_LINES;
-    if (li < nl) lines[li * stride + ipz_pad(k)] = make_double2(0.0, (double)f[k * a.nxy + l0 + li]);
-  }
+  const long long l0 = (long long)blockIdx.x * lines;
+  const int nline = (int)min((long long)lines, a.nxy - l0);
+  // lines is a power of two: a thread keeps its line and takes every 32nd element of it
+  const int li = threadIdx.x & (lines - 1), k0 = threadIdx.x / lines;
+  double* wk = w + li * stride;
+  T* fk = f + l0 + li;
+  if (li < nline)
+    for (int k = k0; k < nz; k += 32) wk[k + __umulhi(k, s.over_l)] = (double)fk[k * a.nxy];
   __syncthreads();
-  if (wl < nl) {
-    double2* w = lines + wl * stride;
-    for (int k = lane; k < nz; k += 32) {  // Psi_E(D_z), 9 taps, periodic, FP64
+  if (wl < nline)
+    for (int i = 0; i < s.nsec; ++i) {
+      periodic_section<false>(w + wl * stride, s.s[i], nz, L, LP, s.nl, lane);  // causal
+      __syncwarp();
+      periodic_section<true>(w + wl * stride, s.s[i], nz, L, LP, s.nl, lane);  // anticausal
+      __syncwarp();
+    }
+  __syncthreads();
+  if (li < nline)
+    for (int k = k0; k < nz; k += 32) {
       double acc = 0.0;
 #pragma unroll
-      for (int m = 0; m < 9; ++m) acc += a.pe_taps[m] * w[ipz_pad(wrapi(k + m - 4, nz))].y;
-      w[ipz_pad(k)].x = acc;
+      for (int m = 0; m < 9; ++m) {  // Psi_E(D_z), periodic
+        int kk = k + m - 4;
+        kk = kk < 0 ? kk + nz : (kk >= nz ? kk - nz : kk);
+        if (kk < 0 || kk >= nz) kk = wrapi(kk, nz);  // lines shorter than 4 cells
+        acc = fma(a.pe_taps[m], wk[kk + __umulhi(kk, s.over_l)], acc);
+      }
+      fk[k * a.nxy] = (T)(a.scale * acc);
     }
-    __syncwarp();
-    for (int k = lane; k < nz; k += 32) w[ipz_pad(k)].y = 0.0;
-    __syncwarp();
-    for (int i = 0; i < a.nf; ++i) {
-      const double2 lam = make_double2(a.lam_re[i], a.lam_im[i]);
-      periodic_recursion(w, nz, lam, false, lane);  // causal
-      __syncwarp();
-      periodic_recursion(w, nz, lam, true, lane);   // anticausal
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < nz * IPZ_LINES; e += blockDim.x) {
-    const int k = e / IPZ_LINES, li = e % IPZ_LINES;
-    if (li < nl) f[k * a.nxy + l0 + li] = (T)(a.scale * lines[li * stride + ipz_pad(k)].x);
-  }
 }
 
-size_t inverse_psi_lines_smem(int nz) {
-  return sizeof(double2) * (size_t)IPZ_LINES * (size_t)((nz - 1) + ((nz - 1) >> 5) + 1);
+// The real second-order sections of the factors and their matrices. Returns false when the factors do
+// not pair up (they are the roots of a real polynomial, so they do).
+static bool inverse_sections(const double* lam_re, const double* lam_im, int nf, int nz, InvLines* out) {
+  double re[4];
+  int nr = 0, up = 0, down = 0;
+  out->nsec = 0;
+  out->L = (nz + 31) / 32;
+  out->nl = (nz + out->L - 1) / out->L;
+  out->over_l = out->L % 2 ? 0u : (unsigned)((0x100000000ull + out->L - 1) / out->L);
+  auto add = [&](double a, double b) {
+    if (out->nsec == 2) return false;
+    out->s[out->nsec].a = a;
+    out->s[out->nsec].b = b;
+    ++out->nsec;
+    return true;
+  };
+  for (int i = 0; i < nf; ++i) {
+    const double mag2 = lam_re[i] * lam_re[i] + lam_im[i] * lam_im[i];
+    if (lam_im[i] * lam_im[i] <= 1e-24 * mag2) {
+      re[nr++] = lam_re[i];
+    } else if (lam_im[i] > 0) {
+      ++up;
+      if (!add(2.0 * lam_re[i], mag2)) return false;
+    } else {
+      ++down;
+    }
+  }
+  if (up != down) return false;
+  for (int i = 0; i < nr; i += 2) {
+    const double l2 = i + 1 < nr ? re[i + 1] : 0.0;
+    if (!add(re[i] + l2, re[i] * l2)) return false;
+  }
+  struct Mat {
+    double v[4];
+  };
+  auto mul = [](const Mat& x, const Mat& y) {
+    return Mat{{x.v[0] * y.v[0] + x.v[1] * y.v[2], x.v[0] * y.v[1] + x.v[1] * y.v[3],
+                x.v[2] * y.v[0] + x.v[3] * y.v[2], x.v[2] * y.v[1] + x.v[3] * y.v[3]}};
+  };
+  for (int i = 0; i < out->nsec; ++i) {
+    InvSection& sc = out->s[i];
+    auto power = [&](long long n) {
+      Mat r{{1, 0, 0, 1}}, x{{sc.a, -sc.b, 1, 0}};
+      for (; n > 0; n >>= 1, x = mul(x, x))
+        if (n & 1) r = mul(r, x);
+      return r;
+    };
+    const int L = out->L, rest = nz - (out->nl - 1) * L;
+    for (int q = 0; q < 5; ++q) {
+      const Mat m = power((long long)L << q), mp = power((((long long)1 << q) - 1) * L + rest);
+      for (int e = 0; e < 4; ++e) {
+        sc.m[q][e] = m.v[e];
+        sc.mp[q][e] = mp.v[e];
+      }
+    }
+    sc.around = 0;
+    for (int q = 1; q <= 5 && 1 << q <= out->nl && sc.around == 0; ++q) {
+      const Mat m = power((((long long)1 << q) - 1) * L + rest);
+      double big = 0.0;
+      for (int e = 0; e < 4; ++e) big = std::max(big, std::fabs(m.v[e]));
+      if (big < 1e-20) sc.around = q;
+    }
+    const Mat z = power(nz);
+    const double p = 1.0 - z.v[0], q = -z.v[1], r = -z.v[2], t = 1.0 - z.v[3], det = p * t - q * r;
+    sc.c[0] = t / det;
+    sc.c[1] = -q / det;
+    sc.c[2] = -r / det;
+    sc.c[3] = p / det;
+  }
+  return true;
 }
 
 template <typename T>
 cudaError_t launch_inverse_psi_z(const InvPsiArgs<T>& a, cudaStream_t st) {
   if (a.nxy <= 0 || a.nz <= 0) return cudaSuccess;
-  const size_t sm = inverse_psi_lines_smem(a.nz);
-  if (sm <= 200 * 1024) {  // lines up to about 1500 cells: the warp-per-line kernel
-    cudaError_t e = ensure_dynamic_smem((const void*)k_inverse_psi_lines<T>, sm);
+  InvLines s;
+  const size_t line = sizeof(double) * (size_t)(((a.nz + 31) / 32 | 1) * 32);
+  if (line <= 200 * 1024 && inverse_sections(a.lam_re, a.lam_im, a.nf, a.nz, &s)) {
+    // lines per block, a warp each: an SM takes four at once, one per scheduler; the fewest such turns on
+    // the busiest SM, and the larger block among equals (its loads are wider)
+    const long long sms = a.nsm > 0 ? a.nsm : 152;
+    int lines = 1;
+    long long best = -1;
+    for (int q = 8; q >= 1; q /= 2) {
+      const long long per_sm = (2 * ((a.nxy + q - 1) / q) + sms - 1) / sms * q, turns = (per_sm + 3) / 4;
+      if (q * line <= 200 * 1024 && (best < 0 || turns < best)) {
+        best = turns;
+        lines = q;
+      }
+    }
+    cudaError_t e = ensure_dynamic_smem((const void*)k_inverse_psi_lines<T>, lines * line);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)((a.nxy + IPZ_LINES - 1) / IPZ_LINES), 2);
-    k_inverse_psi_lines<T><<<grid, 32 * IPZ_LINES, sm, st>>>(a);
+    k_inverse_psi_lines<T><<<dim3((unsigned)((a.nxy + lines - 1) / lines), 2), 32 * lines, lines * line, st>>>(a, s);
     return cudaGetLastError();
   }
-  dim3 grid((unsigned)((a.nxy + 63) / 64), 2);  // longer lines: one thread per line in global memory
+  dim3 grid((unsigned)((a.nxy + 63) / 64), 2);  // lines past shared memory: one thread per line in global memory
   k_inverse_psi_z<T><<<grid, 64, 0, st>>>(a);
   return cudaGetLastError();
 }

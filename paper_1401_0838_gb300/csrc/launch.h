@@ -209,7 +209,8 @@ struct InvPsiArgs {
   int nf;  // factors (the degree of Psi_B)
   double lam_re[4], lam_im[4];
   double scale;
-  double pe_taps[9];  // Psi_E(D_z), applied first
+  double pe_taps[9];  // Psi_E(D_z)
+  int nsm;            // SMs to spread the lines over
 };
 template <typename T>
 cudaError_t launch_inverse_psi_z(const InvPsiArgs<T>& a, cudaStream_t st);
