@@ -17,8 +17,9 @@ constexpr int GR_BLOCKS = 4 * 152;
 
 // Weights of the nodes base, base + 1, ... for offset o in [0, 1) inside the cell: order 1 on the
 // cell's two nodes (base = cell), order 3 the cubic B-spline on four nodes (base = cell - 1).
-__device__ __forceinline__ void node_weights(int order, double o, double (&w)[4]) {
-  if (order == 3) {
+template <int ORDER>
+__device__ __forceinline__ void node_weights(double o, double (&w)[ORDER + 1]) {
+  if constexpr (ORDER == 3) {
     const double p = 1.0 - o;
     w[0] = p * p * p / 6.0;
     w[1] = (4.0 - 6.0 * o * o + 3.0 * o * o * o) / 6.0;
@@ -27,8 +28,6 @@ __device__ __forceinline__ void node_weights(int order, double o, double (&w)[4]
   } else {
     w[0] = 1.0 - o;
     w[1] = o;
-    w[2] = 0.0;
-    w[3] = 0.0;
   }
 }
 
@@ -37,47 +36,95 @@ __device__ __forceinline__ int wrap_any(int g, int n) {
   return g < 0 ? g + n : g;
 }
 
-// rho += q w S(x - x_node) / dV for every particle: one warp per cell, lanes over its slots.
-template <typename T>
-__global__ void __launch_bounds__(RHO_THREADS) k_rho(const __grid_constant__ RunDev<T> r, int order, double inv_dv,
+// rho += q w S(x - x_node) / dV for every particle. lpc lanes per cell, a power of two: one where the cells
+// alone fill the GPU, so that every lane of an FP64 instruction works (that pipe bounds this kernel: a
+// warp per cell left half to three quarters of the lanes idle). A lane sums its particles' weights in
+// registers, the cell's lanes add up, and one lane adds each node once instead of once per particle:
+// 331 -> 95 us on 301 x 517 cells of 2 x 8 particles.
+template <typename T, int NDIM, int ORDER>
+__global__ void __launch_bounds__(RHO_THREADS) k_rho(const __grid_constant__ RunDev<T> r, int lpc, double inv_dv,
                                                      double* __restrict__ rho) {
-  const int lane = threadIdx.x & 31;
-  const long long warps = (long long)gridDim.x * (RHO_THREADS / 32);
-  const long long nxy = (long long)r.nx * r.ny;
-  const int nn = order == 3 ? 4 : 2, lo = order == 3 ? -1 : 0;
-  for (long long cell = blockIdx.x * (long long)(RHO_THREADS / 32) + (threadIdx.x >> 5); cell < r.ncell;
-       cell += warps) {
-    const int i = (int)(cell % r.nx), j = (int)((cell / r.nx) % r.ny), k = (int)(cell / nxy);
+  constexpr int NN = ORDER + 1, NY = NDIM == 3 ? NN : 1, LO = ORDER == 3 ? -1 : 0;
+  const int sub = threadIdx.x & (lpc - 1);
+  const long long step = (long long)gridDim.x * RHO_THREADS / lpc;
+  // every lane of a warp runs the same trips: the lanes past the last cell take part in the sums with nothing
+  for (long long c0 = ((long long)blockIdx.x * RHO_THREADS + (threadIdx.x & ~31)) / lpc; c0 < r.ncell; c0 += step) {
+    const long long cell = c0 + (threadIdx.x & 31) / lpc;
+    const bool on = cell < r.ncell;
+    double acc[NN * NY * NN] = {};
+#pragma unroll 1
     for (int s = 0; s < 2; ++s) {
       const SpeciesBuf<T>& b = s ? r.in[1] : r.in[0];
-      const int n = min(b.cnt[cell], r.cap);
-      const double q = s ? 1.0 : -1.0;
-      for (int slot = lane; slot < n; slot += 32) {
+      const int n = on ? min(b.cnt[cell], r.cap) : 0;
+      const double q = s ? inv_dv : -inv_dv;
+      for (int slot = sub; slot < n; slot += lpc) {
         const long long o = cell * r.cap + slot;
-        const double qw = q * (b.w ? (double)b.w[o] : (double)r.wconst) * inv_dv;
-        double wx[4], wy[4] = {1.0, 0.0, 0.0, 0.0}, wz[4];
-        const PartVals<T> v = part_get(b, r.ndim, o);
-        node_weights(order, (double)v.ox, wx);
-        if (r.ndim == 3) node_weights(order, (double)v.oy, wy);
-        node_weights(order, (double)v.oz, wz);
-        const int ny_n = r.ndim == 3 ? nn : 1;
-        for (int c = 0; c < nn; ++c) {
-          const long long kz = wrap_any(k + lo + c, r.nz);
-          for (int bb = 0; bb < ny_n; ++bb) {
-            const long long jy = r.ndim == 3 ? wrap_any(j + lo + bb, r.ny) : 0;
-            const double wyz = qw * wy[bb] * wz[c];
-            for (int a = 0; a < nn; ++a)
-              atomicAdd(rho + (kz * r.ny + jy) * r.nx + wrap_any(i + lo + a, r.nx), wyz * wx[a]);
+        const double qw = q * (b.w ? (double)b.w[o] : (double)r.wconst);
+        double wx[NN], wy[NN], wz[NN];
+        const PartVals<T> v = part_get(b, NDIM, o);
+        node_weights<ORDER>((double)v.ox, wx);
+        if constexpr (NDIM == 3) node_weights<ORDER>((double)v.oy, wy);
+        node_weights<ORDER>((double)v.oz, wz);
+#pragma unroll
+        for (int c = 0; c < NN; ++c)
+#pragma unroll
+          for (int bb = 0; bb < NY; ++bb) {
+            const double wyz = NDIM == 3 ? qw * wy[bb] * wz[c] : qw * wz[c];
+#pragma unroll
+            for (int a = 0; a < NN; ++a) acc[(c * NY + bb) * NN + a] = fma(wyz, wx[a], acc[(c * NY + bb) * NN + a]);
           }
+      }
+    }
+    for (int d = lpc >> 1; d > 0; d >>= 1)
+#pragma unroll
+      for (int e = 0; e < NN * NY * NN; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], d);
+    if (!on || sub != 0) continue;
+    const int ci = (int)cell, i = ci % r.nx, j = ci / r.nx % r.ny, k = ci / r.nx / r.ny;
+#pragma unroll
+    for (int c = 0; c < NN; ++c) {
+      const long long kz = wrap_any(k + LO + c, r.nz);
+#pragma unroll
+      for (int bb = 0; bb < NY; ++bb) {
+        const long long jy = NDIM == 3 ? wrap_any(j + LO + bb, r.ny) : 0;
+#pragma unroll
+        for (int a = 0; a < NN; ++a) {
+          const double v = acc[(c * NY + bb) * NN + a];
+          if (v != 0.0) atomicAdd(rho + (kz * r.ny + jy) * r.nx + wrap_any(i + LO + a, r.nx), v);
         }
       }
     }
   }
 }
 
+// (max, sum, max) of the block's values, in thread 0.
+__device__ __forceinline__ void block_max_sum_max(double& m0, double& s, double& m1) {
+  __shared__ double red[3][GR_THREADS / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    m0 = fmax(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    m1 = fmax(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+  }
+  __syncthreads();  // the sums of an earlier call are read
+  if (lane == 0) {
+    red[0][w] = m0;
+    red[1][w] = s;
+    red[2][w] = m1;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int q = 1; q < GR_THREADS / 32; ++q) {
+      m0 = fmax(m0, red[0][q]);
+      s += red[1][q];
+      m1 = fmax(m1, red[2][q]);
+    }
+}
+
 // Node residual res = div E - rho_f (FP64 from the stored precision). Per thread: max |res|, sum
 // res^2, max |rho_f|; per block: tree into scratch[3 * block + r]; the last block to finish combines
-// the partials in a fixed order and writes out = (max |res|, rms res, max |rho_f|).
+// the partials in a fixed order (all its threads: one thread's walk over 608 blocks took 120 of 129 us)
+// and writes out = (max |res|, rms res, max |rho_f|).
 template <typename T>
 __global__ void __launch_bounds__(GR_THREADS) k_gauss_residual(const T* __restrict__ ex, const T* __restrict__ ey,
                                                                const T* __restrict__ ez,
@@ -98,50 +145,30 @@ __global__ void __launch_bounds__(GR_THREADS) k_gauss_residual(const T* __restri
     ssq += res * res;
     mrho = fmax(mrho, fabs(rhof[c]));
   }
-  __shared__ double red[3][GR_THREADS / 32];
   __shared__ bool last;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    mres = fmax(mres, __shfl_xor_sync(0xffffffffu, mres, o));
-    ssq += __shfl_xor_sync(0xffffffffu, ssq, o);
-    mrho = fmax(mrho, __shfl_xor_sync(0xffffffffu, mrho, o));
-  }
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) {
-    red[0][w] = mres;
-    red[1][w] = ssq;
-    red[2][w] = mrho;
-  }
-  __syncthreads();
+  block_max_sum_max(mres, ssq, mrho);
   if (threadIdx.x == 0) {
-    double a = 0.0, s = 0.0, m = 0.0;
-    for (int q = 0; q < GR_THREADS / 32; ++q) {
-      a = fmax(a, red[0][q]);
-      s += red[1][q];
-      m = fmax(m, red[2][q]);
-    }
-    scratch[3 * blockIdx.x + 0] = a;
-    scratch[3 * blockIdx.x + 1] = s;
-    scratch[3 * blockIdx.x + 2] = m;
-  }
-  __threadfence();
-  __syncthreads();
-  unsigned* done = reinterpret_cast<unsigned*>(scratch + 3 * GR_BLOCKS);
-  if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (last && threadIdx.x == 0) {
+    scratch[3 * blockIdx.x + 0] = mres;
+    scratch[3 * blockIdx.x + 1] = ssq;
+    scratch[3 * blockIdx.x + 2] = mrho;
     __threadfence();
-    const volatile double* v = scratch;
-    double a = 0.0, s = 0.0, m = 0.0;
-    for (unsigned q = 0; q < gridDim.x; ++q) {
-      a = fmax(a, v[3 * q + 0]);
-      s += v[3 * q + 1];
-      m = fmax(m, v[3 * q + 2]);
-    }
-    out[0] = a;
-    out[1] = sqrt(s / (double)n);
-    out[2] = m;
-    *done = 0u;
+    last = atomicAdd(reinterpret_cast<unsigned*>(scratch + 3 * GR_BLOCKS), 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  mres = ssq = mrho = 0.0;
+  for (unsigned q = threadIdx.x; q < gridDim.x; q += GR_THREADS) {
+    mres = fmax(mres, __ldcg(scratch + 3 * q + 0));
+    ssq += __ldcg(scratch + 3 * q + 1);
+    mrho = fmax(mrho, __ldcg(scratch + 3 * q + 2));
+  }
+  block_max_sum_max(mres, ssq, mrho);
+  if (threadIdx.x == 0) {
+    out[0] = mres;
+    out[1] = sqrt(ssq / (double)n);
+    out[2] = mrho;
+    *reinterpret_cast<unsigned*>(scratch + 3 * GR_BLOCKS) = 0u;
   }
 }
 
@@ -149,9 +176,18 @@ size_t gauss_scratch_bytes() { return sizeof(double) * (3 * GR_BLOCKS + 2); }
 
 template <typename T>
 cudaError_t launch_rho(const RunDev<T>& r, int order, double inv_dv, double* rho, cudaStream_t st) {
-  const long long want = (r.ncell + RHO_THREADS / 32 - 1) / (RHO_THREADS / 32);
+  int lpc = 1;  // lanes per cell: until the cells fill the 152 SMs with 16 warps each, or a warp has one cell
+  while (lpc < 32 && r.ncell * lpc < 152ll * 512) lpc *= 2;
+  const long long want = (r.ncell * lpc + RHO_THREADS - 1) / RHO_THREADS;
   const int blocks = (int)(want < 8 * 152 ? (want < 1 ? 1 : want) : 8 * 152);
-  k_rho<T><<<blocks, RHO_THREADS, 0, st>>>(r, order, inv_dv, rho);
+  if (r.ndim == 3 && order == 3)
+    k_rho<T, 3, 3><<<blocks, RHO_THREADS, 0, st>>>(r, lpc, inv_dv, rho);
+  else if (r.ndim == 3)
+    k_rho<T, 3, 1><<<blocks, RHO_THREADS, 0, st>>>(r, lpc, inv_dv, rho);
+  else if (order == 3)
+    k_rho<T, 2, 3><<<blocks, RHO_THREADS, 0, st>>>(r, lpc, inv_dv, rho);
+  else
+    k_rho<T, 2, 1><<<blocks, RHO_THREADS, 0, st>>>(r, lpc, inv_dv, rho);
   return cudaGetLastError();
 }
 
