@@ -645,17 +645,42 @@ bool kernel_reachable(const void* p, long long n, size_t es) {
   return (size_t)((CUdeviceptr)p - base) + (size_t)n * es <= size;
 }
 
+bool overlap(const void* a, long long na, const void* b, long long nb) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + (uintptr_t)nb && y < x + (uintptr_t)na;
+}
+
 // The caller's particle arrays as the import and export kernels take them, when every one that is given
-// is device memory they can reach (one pass over the particles less than through the staging arrays).
+// is device memory they can reach (one pass over the particles less than through the staging arrays). An
+// array given twice goes through the staging arrays, where the copies keep their order.
 template <typename T>
 bool caller_view(pic_handle* h, const pic_state* s, long long n, FlatDev<T>* f) {
   if (s->where != PIC_DEVICE) return false;
   const void* arr[10] = {s->cell, s->species, s->id, s->ox, s->oy, s->oz, s->dux, s->duy, s->duz, s->w};
   for (int q = 0; q < 10; ++q)
     if (arr[q] && !(q == 4 && h->cfg.ndim != 3) && !kernel_reachable(arr[q], n, q < 3 ? 4 : sizeof(T))) return false;
+  for (int q = 1; q < 10; ++q)
+    for (int p = 0; p < q; ++p)
+      if (arr[p] && arr[q] && overlap(arr[p], n * (long long)(p < 3 ? 4 : sizeof(T)), arr[q], n * (long long)(q < 3 ? 4 : sizeof(T))))
+        return false;
   *f = FlatDev<T>{n, s->cell, s->species, (T*)s->ox, (T*)s->oy, (T*)s->oz, (T*)s->dux, (T*)s->duy, (T*)s->duz,
                   (T*)s->w, s->id};
   return true;
+}
+
+cudaError_t flush(pic_handle* h, BulkArgs* b) {
+  if (b->n == 0) return cudaSuccess;
+  const cudaError_t e = launch(h, PIC_K_OTHER, [&] { return launch_bulk(*b, h->stream); });
+  b->n = 0;
+  return e;
+}
+
+// Empties the bins of both buffers and the leaver and spill lists.
+void clear_counters(pic_handle* h, BulkArgs* b) {
+  for (int sp = 0; sp < 2; ++sp)
+    for (int q = 0; q < 2; ++q) b->add(h->cnt[sp][q], nullptr, (long long)sizeof(int) * h->ncell);
+  b->add(h->d_lv_count, nullptr, 2 * sizeof(int));
+  b->add(h->d_sp_count, nullptr, 2 * sizeof(int));
 }
 
 template <typename T>
@@ -665,16 +690,19 @@ int set_state_t(pic_handle* h, const pic_state* s) {
   const cudaMemcpyKind k = s->where == PIC_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   const size_t fb = (size_t)h->ncell * sizeof(T);
   void* const src[6] = {s->ex, s->ey, s->ez, s->bx, s->by, s->bz};
-  for (int q = 0; q < 6; ++q)
-    if (src[q]) CK(cudaMemcpyAsync(h->f[q], src[q], fb, k, st), "copy field in");
+  BulkArgs bulk;
+  for (int q = 0; q < 6; ++q) {
+    if (!src[q]) continue;
+    if (s->where == PIC_DEVICE && kernel_reachable(src[q], h->ncell, sizeof(T)))
+      bulk.add(h->f[q], src[q], (long long)fb);
+    else
+      CK(cudaMemcpyAsync(h->f[q], src[q], fb, k, st), "copy field in");
+  }
   const long long n = s->np;
+  if (n >= 0) clear_counters(h, &bulk);  // particles: clear bins, leaver and spill counters, stage, bin
+  CK(flush(h, &bulk), "copy fields in");
   if (n == -1) return PIC_OK;  // fields only: particles untouched
   if (n < 0) return fail(h, PIC_E_ARG, "negative particle count");
-  // particles: clear bins, leaver and spill counters, stage, bin
-  for (int sp = 0; sp < 2; ++sp)
-    for (int b = 0; b < 2; ++b) CK(cudaMemsetAsync(h->cnt[sp][b], 0, sizeof(int) * h->ncell, st), "clear counts");
-  CK(cudaMemsetAsync(h->d_lv_count, 0, 2 * sizeof(int), st), "clear leaver counters");
-  CK(cudaMemsetAsync(h->d_sp_count, 0, 2 * sizeof(int), st), "clear spill counters");
   h->parity = 0;
   h->sp_pending = false;
   if (n == 0) return PIC_OK;
@@ -869,8 +897,20 @@ int get_state_t(pic_handle* h, pic_state* s) {
   const cudaMemcpyKind k = s->where == PIC_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   const size_t fb = (size_t)h->ncell * sizeof(T);
   void* const dst[6] = {s->ex, s->ey, s->ez, s->bx, s->by, s->bz};
-  for (int q = 0; q < 6; ++q)
-    if (dst[q]) CK(cudaMemcpyAsync(dst[q], h->f[q], fb, k, st), "copy field out");
+  BulkArgs bulk;
+  for (int q = 0; q < 6; ++q) {
+    if (!dst[q]) continue;
+    for (int p = 0; p < bulk.n; ++p)
+      if (overlap(bulk.dst[p], (long long)fb, dst[q], (long long)fb)) {  // one buffer twice: the later field stays
+        CK(flush(h, &bulk), "copy fields out");
+        break;
+      }
+    if (s->where == PIC_DEVICE && kernel_reachable(dst[q], h->ncell, sizeof(T)))
+      bulk.add(dst[q], h->f[q], (long long)fb);
+    else
+      CK(cudaMemcpyAsync(dst[q], h->f[q], fb, k, st), "copy field out");  // host memory, another device
+  }
+  CK(flush(h, &bulk), "copy fields out");
   s->u_drift = h->u0;
   long long cnts[2];
   rc = count_bins(h, cnts);  // synchronises
@@ -2118,13 +2158,15 @@ int adj_save(pic_handle* h, void* const* fields, const pic_handle::Flat& flat, b
   if (rc0) return rc0;
   cudaStream_t st = h->stream;
   const size_t fb = (size_t)h->ncell * sizeof(T);
-  for (int q = 0; q < 6; ++q)
-    if (fields) CK(cudaMemcpyAsync(fields[q], h->f[q], fb, cudaMemcpyDeviceToDevice, st), "save fields");
+  BulkArgs bulk;
+  if (fields)
+    for (int q = 0; q < 6; ++q) bulk.add(fields[q], h->f[q], (long long)fb);
   unsigned long long* seen = nullptr;
   if (check_ids) {
     seen = h->adj.seen;
-    CK(cudaMemsetAsync(seen, 0, 8 * (size_t)(h->adj.np / 64 + 1), st), "clear id bitmap");
+    bulk.add(seen, nullptr, 8 * (h->adj.np / 64 + 1));
   }
+  CK(flush(h, &bulk), "save fields");
   RunDev<T> r = make_run<T>(h, h->parity);
   FlatDev<T> f = flat_view<T>(flat, h->adj.np);
   CK(launch(h, PIC_K_OTHER, [&] { return launch_tape<T>(r, f, seen, st); }), "tape");
@@ -2138,12 +2180,10 @@ int adj_restore(pic_handle* h, int j) {
   cudaStream_t st = h->stream;
   const size_t fb = (size_t)h->ncell * sizeof(T);
   drop_graph(h);
-  for (int q = 0; q < 6; ++q)
-    CK(cudaMemcpyAsync(h->f[q], A.ck_f[(size_t)j * 6 + q], fb, cudaMemcpyDeviceToDevice, st), "restore fields");
-  for (int sp = 0; sp < 2; ++sp)
-    for (int b = 0; b < 2; ++b) CK(cudaMemsetAsync(h->cnt[sp][b], 0, sizeof(int) * h->ncell, st), "clear counts");
-  CK(cudaMemsetAsync(h->d_lv_count, 0, 2 * sizeof(int), st), "clear leaver counters");
-  CK(cudaMemsetAsync(h->d_sp_count, 0, 2 * sizeof(int), st), "clear spill counters");
+  BulkArgs bulk;
+  for (int q = 0; q < 6; ++q) bulk.add(h->f[q], A.ck_f[(size_t)j * 6 + q], (long long)fb);
+  clear_counters(h, &bulk);
+  CK(flush(h, &bulk), "restore fields");
   h->parity = 0;
   h->sp_pending = false;
   RunDev<T> r = make_run<T>(h, 0);
@@ -2211,7 +2251,9 @@ int adj_step(pic_handle* h, int s) {
   for (int q = 0; q < 3; ++q) ca.zero[q] = nullptr;
   CK(launch(h, PIC_K_COPIES, [&] { return launch_sep<T>(ca, st); }), "adjoint: copies");
   // particles
-  for (int q = 0; q < 6; ++q) CK(cudaMemsetAsync(A.lg[q], 0, fb, st), "zero copy adjoint");
+  BulkArgs bulk;
+  for (int q = 0; q < 6; ++q) bulk.add(A.lg[q], nullptr, (long long)fb);
+  CK(flush(h, &bulk), "zero copy adjoint");
   const pic_handle::Flat& tp = A.tape_p[s];
   AdjPartArgs<T> pa;
   pa.n = A.np;

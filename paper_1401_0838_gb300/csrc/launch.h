@@ -191,6 +191,21 @@ cudaError_t launch_kinetic(const RunDev<T>& r, double* out, cudaStream_t st);
 // Gauss-law residual (k_gauss.cu): rho += q w S / dV from the particle bins of r.in (shape order 1 or
 // 3, FP64 atomics; rho zeroed by the caller), and (max |div E - rhof|, rms, max |rhof|) into out[0..2]
 // (scratch of gauss_scratch_bytes, zeroed once).
+// Up to 12 copies (or clears, where src is null) of device memory in one launch: addresses and lengths are
+// multiples of 4 bytes, nothing overlaps.
+struct BulkArgs {
+  int n = 0;
+  void* dst[12];
+  const void* src[12];
+  long long bytes[12];
+  void add(void* d, const void* s, long long b) {
+    dst[n] = d;
+    src[n] = s;
+    bytes[n++] = b;
+  }
+};
+cudaError_t launch_bulk(const BulkArgs& a, cudaStream_t st);
+
 template <typename T>
 cudaError_t launch_rho(const RunDev<T>& r, int order, double inv_dv, double* rho, cudaStream_t st);
 template <typename T>

@@ -83,3 +83,34 @@ def test_state_through_device_arrays(ndim, nx, ny, nz, precision, shift):
         assert e["np"] == n
     finally:
         P.pic_destroy(h)
+
+
+# field arrays at every alignment the copy kernel distinguishes (16 bytes, the element, less: the plain copies),
+# lengths with and without a remainder of its 16-byte units, one and many blocks; one array given for several fields
+@pytest.mark.parametrize("precision", [1, 0])
+@pytest.mark.parametrize("nx,nz", [(3, 5), (7, 9), (64, 64), (301, 517)])
+@pytest.mark.parametrize("shift", [0, 8, 4, 2])
+def test_fields_through_device_arrays(nx, nz, precision, shift):
+    import torch
+
+    cfg = make_cfg(nx=nx, nz=nz, precision=precision, ppc=1, init_beam=0)
+    T = np.float32 if precision == 0 else np.float64
+    names = ("ex", "ey", "ez", "bx", "by", "bz")
+    rng = np.random.default_rng(4)
+    f = {n: rng.normal(size=nx * nz).astype(T) for n in names}
+    dev = {n: _on_device(f[n], shift) for n in names}
+    out = {n: _on_device(np.zeros_like(f[n]), shift) for n in names}
+    h = P.pic_create(cfg)
+    try:
+        P.pic_set_state(h, _state(P.PIC_DEVICE, dev, -1, shift))
+        P.pic_get_state(h, _state(P.PIC_DEVICE, out, 0, shift))
+        for n in names:
+            raw = out[n].cpu().numpy()
+            assert raw[shift:shift + f[n].nbytes].tobytes() == f[n].tobytes(), n
+            assert not raw[:shift].any() and not raw[shift + f[n].nbytes:].any(), n
+        one = _on_device(np.zeros_like(f["ex"]), shift)
+        P.pic_get_state(h, _state(P.PIC_DEVICE, {n: one for n in names}, 0, shift))
+        torch.cuda.synchronize()
+        assert one.cpu().numpy()[shift:shift + f["bz"].nbytes].tobytes() == f["bz"].tobytes()  # the last one stays
+    finally:
+        P.pic_destroy(h)
