@@ -2154,8 +2154,6 @@ FlatDev<T> flat_view(const pic_handle::Flat& f, long long np) {
 // Fields and particles of the current state into (fields[6], flat) in id order.
 template <typename T>
 int adj_save(pic_handle* h, void* const* fields, const pic_handle::Flat& flat, bool check_ids) {
-  int rc0 = settle<T>(h);  // the tape reads the bins: no particle may wait in the spill list
-  if (rc0) return rc0;
   cudaStream_t st = h->stream;
   const size_t fb = (size_t)h->ncell * sizeof(T);
   BulkArgs bulk;

@@ -20,12 +20,42 @@
 namespace picgb {
 
 // ---------------------------------------------------------------------------------------------
-// Tape: bins (current buffers) -> flat arrays indexed by particle id. With `seen` (one bit per id,
-// zeroed by the caller) ids that are out of range or repeated raise ERR_IDS.
+// Tape: bins (current buffers) and spill list -> flat arrays indexed by particle id. With `seen` (one bit
+// per id, zeroed by the caller) ids that are out of range or repeated raise ERR_IDS. The last blocks take
+// the list, by its count on the device: the host need not wait after every step to know whether
+// particles have to be put back into larger bins first (the adjoint of 20 steps 9.1 -> 9.0 ms).
 // ---------------------------------------------------------------------------------------------
+constexpr int TAPE_SPILL_BLOCKS = 4;
 template <typename T>
 __global__ void __launch_bounds__(256) k_tape(const __grid_constant__ RunDev<T> r, const __grid_constant__ FlatDev<T> f,
                                               unsigned long long* seen) {
+  auto put = [&](unsigned id, int cell, int species, T ox, T oy, T oz, T ux, T uy, T uz, T w) {
+    if ((long long)id >= f.np) {
+      flag_error(r.err, ERR_IDS);
+      return;
+    }
+    if (seen) {
+      const unsigned long long bit = 1ull << (id & 63u);
+      if (atomicOr(seen + (id >> 6), bit) & bit) flag_error(r.err, ERR_IDS);
+    }
+    f.cell[id] = cell;
+    f.species[id] = species;
+    f.ox[id] = ox;
+    if (f.oy) f.oy[id] = oy;
+    f.oz[id] = oz;
+    f.dux[id] = ux;
+    f.duy[id] = uy;
+    f.duz[id] = uz;
+    if (f.w) f.w[id] = w;
+  };
+  if (blockIdx.x >= gridDim.x - TAPE_SPILL_BLOCKS) {
+    const long long n = min((long long)*r.sp_in, r.sp_cap);
+    for (long long i = (blockIdx.x - (gridDim.x - TAPE_SPILL_BLOCKS)) * 256ll + threadIdx.x; i < n;
+         i += TAPE_SPILL_BLOCKS * 256ll)
+      put(r.sp.id ? r.sp.id[i] : 0u, r.sp.key[i] >> 1, r.sp.key[i] & 1, r.sp.ox[i], r.ndim == 3 ? r.sp.oy[i] : T(0),
+          r.sp.oz[i], r.sp.dux[i], r.sp.duy[i], r.sp.duz[i], r.sp.w ? r.sp.w[i] : r.wconst);
+    return;
+  }
   // eight lanes per (cell, species) bin, four bins per warp (bins hold about ppc particles)
   const long long cs = blockIdx.x * 32LL + (threadIdx.x >> 3);
   const long long cell = cs >> 1;
@@ -34,33 +64,16 @@ __global__ void __launch_bounds__(256) k_tape(const __grid_constant__ RunDev<T> 
   const SpeciesBuf<T>& b = s ? r.in[1] : r.in[0];  // constant indices: no local copy of r
   const int n = min(b.cnt[cell], r.cap);
   for (int j = threadIdx.x & 7; j < n; j += 8) {
-  const long long src = cell * r.cap + j;
-  const unsigned id = b.id[src];
-  if ((long long)id >= f.np) {
-    flag_error(r.err, ERR_IDS);
-    continue;
-  }
-  if (seen) {
-    const unsigned long long bit = 1ull << (id & 63u);
-    if (atomicOr(seen + (id >> 6), bit) & bit) flag_error(r.err, ERR_IDS);
-  }
-  f.cell[id] = (int)cell;
-  f.species[id] = s;
-  const PartVals<T> v = part_get(b, r.ndim, src);
-  f.ox[id] = v.ox;
-  if (f.oy) f.oy[id] = v.oy;
-  f.oz[id] = v.oz;
-  f.dux[id] = v.ux;
-  f.duy[id] = v.uy;
-  f.duz[id] = v.uz;
-  if (f.w) f.w[id] = b.w ? b.w[src] : r.wconst;
+    const long long src = cell * r.cap + j;
+    const PartVals<T> v = part_get(b, r.ndim, src);
+    put(b.id[src], (int)cell, s, v.ox, v.oy, v.oz, v.ux, v.uy, v.uz, b.w ? b.w[src] : r.wconst);
   }
 }
 
 template <typename T>
 cudaError_t launch_tape(const RunDev<T>& r, const FlatDev<T>& f, unsigned long long* seen, cudaStream_t st) {
   const long long blocks = (2 * r.ncell + 31) / 32;
-  if (blocks > 0) k_tape<T><<<(unsigned)blocks, 256, 0, st>>>(r, f, seen);
+  if (blocks > 0) k_tape<T><<<(unsigned)(blocks + TAPE_SPILL_BLOCKS), 256, 0, st>>>(r, f, seen);
   return cudaGetLastError();
 }
 template cudaError_t launch_tape<float>(const RunDev<float>&, const FlatDev<float>&, unsigned long long*,
