@@ -275,46 +275,86 @@ struct SepGeom {
   static constexpr size_t SMEM_BYTES = 128 + STAGE_BYTES + (NDIM == 3 ? sizeof(T) * (size_t)CZ * CY * PX : 0);
 };
 
-// Overwrite the staged elements that lie outside the grid (a TMA box reads them as zero) with their
-// periodic images: columns, rows and (3D) planes past either end, within the first UX x UY x UZ elements,
-// which are what the tile's passes read (a small grid's tiles are smaller than the box; replacing all of
-// the box's outside, up to its whole width, took 20 us of the 28 us Yee launch on 64x128 cells). PX, LY:
-// the box's row and plane lengths. The grid is at least as wide as the staged region in every direction,
-// so every index is within one period of the grid. Elements on two edges are written twice, with the
-// same value.
-template <typename T, int NDIM, int NT>
-__device__ __forceinline__ void patch_wrapped(T* s0, const T* __restrict__ src, int xs, int ys, int zs, int PX, int LY,
-                                              int UX, int UY, int UZ, int nx, int ny, int nz) {
-  const WrapOnce w;
-  const int xlo = max(0, -xs), xhi = max(0, xs + UX - nx);
-  const int ylo = NDIM == 3 ? max(0, -ys) : 0, yhi = NDIM == 3 ? max(0, ys + UY - ny) : 0;
-  const int zlo = max(0, -zs), zhi = max(0, zs + UZ - nz);
-  if (!(xlo | xhi | ylo | yhi | zlo | zhi)) return;
-  const long long nxy = (long long)nx * ny;
-  auto fix = [&](int lx, int ly, int lz) {
-    const int gx = w(xs + lx, nx), gy = NDIM == 3 ? w(ys + ly, ny) : 0, gz = w(zs + lz, nz);
-    s0[(lz * LY + ly) * PX + lx] = src[gz * nxy + (long long)gy * nx + gx];
-  };
-  const int nxe = xlo + xhi;  // outside columns, every row
-  for (int i = threadIdx.x; i < nxe * UY * UZ; i += NT) {
-    const int c = i % nxe, row = i / nxe;
-    fix(c < xlo ? c : UX - xhi + (c - xlo), row % UY, row / UY);
+// The staged elements that lie outside the grid (a TMA box reads them as zero) get their periodic images:
+// columns, rows and (3D) planes past either end, within the first UX x UY x UZ elements, which are what
+// the tile's passes read (a small grid's tiles are smaller than the box). NA arrays of one geometry, PX and
+// LY the box's row and plane lengths, (xs, ys, zs) its origin. The grid is at least as wide as the staged
+// region in every direction, so every index is within one period of the grid. Elements on two edges are
+// written twice, with the same value.
+// These are the tile's only loads that wait on global memory one by one, so a thread reads its first
+// element of every array before the wait for the boxes (fetch) and writes it after (store): one latency, and
+// that beside the boxes', where a loop per array and direction took up to 18 on the edge tiles that decide
+// when a one-wave launch ends. The step on 64x128 FP64 cells 68 -> 61 us, on 128x128 FP32 with CK 64 -> 58
+// us, on 512x1024 FP32 7 us less.
+template <typename T, int NDIM, int NT, int NA>
+struct EdgeValues {
+  int xs, ys, zs, PX, LY, UX, UY, UZ, nx, ny, nz;
+  int xlo, ylo, zlo, nxe, nye, nze, nxp, nzp, total;
+  int l = 0;
+  T v[NA];
+  __device__ __forceinline__ EdgeValues(int xs_, int ys_, int zs_, int px, int ly, int ux, int uy, int uz, int nx_,
+                                        int ny_, int nz_)
+      : xs(xs_), ys(ys_), zs(zs_), PX(px), LY(ly), UX(ux), UY(uy), UZ(uz), nx(nx_), ny(ny_), nz(nz_) {
+    xlo = max(0, -xs);
+    ylo = NDIM == 3 ? max(0, -ys) : 0;
+    zlo = max(0, -zs);
+    nxe = xlo + max(0, xs + UX - nx);
+    nye = NDIM == 3 ? ylo + max(0, ys + UY - ny) : 0;
+    nze = zlo + max(0, zs + UZ - nz);
+    nxp = nxe * UY * UZ;  // outside columns, every row; then outside rows, then (3D) outside planes
+    nzp = nze * UY * UX;
+    total = nxp + nzp + nye * UZ * UX;
   }
-  const int nze = zlo + zhi;  // outside rows, every column
-  for (int i = threadIdx.x; i < nze * UY * UX; i += NT) {
-    const int lx = i % UX, r = i / UX;
-    const int zr = r / UY;
-    fix(lx, r % UY, zr < zlo ? zr : UZ - zhi + (zr - zlo));
+  // Index in the box and in the grid (cells < 2^30) of element i of the outside ones.
+  __device__ __forceinline__ int locate(int i, int& o) const {
+    int lx, ly, lz;
+    if (i < nxp) {
+      const int r = i / nxe, c = i - r * nxe;
+      lx = c < xlo ? c : UX - nxe + c;
+      ly = r % UY;
+      lz = r / UY;
+    } else {
+      const bool z = i < nxp + nzp;
+      i -= z ? nxp : nxp + nzp;
+      const int r = i / UX;
+      lx = i - r * UX;
+      if (NDIM == 2 || z) {
+        const int zr = r / UY;
+        ly = r - zr * UY;
+        lz = zr < zlo ? zr : UZ - nze + zr;
+      } else {
+        const int yr = r % nye;
+        lz = r / nye;
+        ly = yr < ylo ? yr : UY - nye + yr;
+      }
+    }
+    const WrapOnce w;
+    o = (w(zs + lz, nz) * ny + (NDIM == 3 ? w(ys + ly, ny) : 0)) * nx + w(xs + lx, nx);
+    return (lz * LY + ly) * PX + lx;
   }
-  if constexpr (NDIM == 3) {
-    const int nye = ylo + yhi;  // outside y planes
-    for (int i = threadIdx.x; i < nye * UZ * UX; i += NT) {
-      const int lx = i % UX, r = i / UX;
-      const int yr = r % nye, lz = r / nye;
-      fix(lx, yr < ylo ? yr : UY - yhi + (yr - ylo), lz);
+  template <class Src>
+  __device__ __forceinline__ void fetch(Src src) {
+    if ((int)threadIdx.x >= total) return;
+    int o;
+    l = locate(threadIdx.x, o);
+#pragma unroll
+    for (int c = 0; c < NA; ++c) v[c] = src(c)[o];
+  }
+  // array c of the staged region starts at s + c * pitch
+  template <class Src>
+  __device__ __forceinline__ void store(T* s, int pitch, Src src) {
+    for (int i = threadIdx.x; i < total; i += NT) {
+      if (i != (int)threadIdx.x) {
+        int o;
+        l = locate(i, o);
+#pragma unroll
+        for (int c = 0; c < NA; ++c) v[c] = src(c)[o];
+      }
+#pragma unroll
+      for (int c = 0; c < NA; ++c) s[c * pitch + l] = v[c];
     }
   }
-}
+};
 
 template <typename T, int NDIM, int HZ, int HX>
 __device__ __forceinline__ void sep_tile(const SepArgs<T>& a, const int tile, const int comp, const int ntx,
@@ -363,6 +403,9 @@ __device__ __forceinline__ void sep_tile(const SepArgs<T>& a, const int tile, co
       if (NDIM == 2) tma_load_2d(s0, &a.tm[comp], xs, zs0, &mbar);
       else tma_load_3d(s0, &a.tm[comp], xs, ys, zs0, &mbar);
     }
+    EdgeValues<T, NDIM, SEP_THREADS, 1> edge(xs, ys, zs0, PX, LY, C0 + ncx, ncy, rows_staged, a.nx, a.ny, a.nz);
+    const auto edge_src = [&](int) { return src; };
+    edge.fetch(edge_src);
     __syncthreads();  // the barrier is initialised before anyone polls it
     const bool ok = __syncthreads_and(mbar_wait(&mbar, 0, TMA_WAIT_POLLS));
     if (!ok) {  // give up: record it, let the copy land (bounded), and leave the tile
@@ -370,7 +413,7 @@ __device__ __forceinline__ void sep_tile(const SepArgs<T>& a, const int tile, co
       mbar_wait(&mbar, 0, TMA_WAIT_POLLS);
       return;
     }
-    patch_wrapped<T, NDIM, SEP_THREADS>(s0, src, xs, ys, zs0, PX, LY, C0 + ncx, ncy, rows_staged, a.nx, a.ny, a.nz);
+    edge.store(s0, 0, edge_src);
   } else {
     auto stage = [&](auto wrap) {  // the rows and columns the passes read
       for (int row = ty; row < rows_staged * LY; row += TYN) {
@@ -911,6 +954,9 @@ __device__ __forceinline__ void yee_tile(const YeeArgs<T>& a, const int tile, co
         else tma_load_3d(sm + c * LN, &a.tm[c], xs, ys, zs, &mbar);
       }
     }
+    EdgeValues<T, NDIM, YEE_THREADS, 9> edge(xs, ys, zs, LX, LY, G::XAL + wx + 2, NDIM == 3 ? wy + 3 : 1, wz + HL + 2, a.nx,
+                                             a.ny, a.nz);
+    edge.fetch(gsrc);
     __syncthreads();  // the barrier is initialised before anyone polls it
     const bool ok = __syncthreads_and(mbar_wait(&mbar, 0, TMA_WAIT_POLLS));
     if (!ok) {  // give up: record it, let the copies land (bounded), and leave the tile unchanged
@@ -919,9 +965,7 @@ __device__ __forceinline__ void yee_tile(const YeeArgs<T>& a, const int tile, co
       if (DIAG) energy_finish(0.0, 0.0, 0.0, escratch, gridDim.x, nullptr, *hc);
       return;
     }
-    for (int c = 0; c < 9; ++c)
-      patch_wrapped<T, NDIM, YEE_THREADS>(sm + c * LN, gsrc(c), xs, ys, zs, LX, LY, G::XAL + wx + 2, NDIM == 3 ? wy + 3 : 1,
-                                          wz + HL + 2, a.nx, a.ny, a.nz);
+    edge.store(sm, LN, gsrc);
   } else {
     auto stage = [&](auto wrap) {
       // the region the phases read: columns [0, XAL + wx + 2), y rows [0, wy + 3), z rows [0, wz + HL + 2)
