@@ -270,6 +270,9 @@ struct SepGeom {
   static constexpr int HY = NDIM == 3 ? HX : 0;
   static constexpr int XA = SepPitch<T, HX>::XA;
   static constexpr int PX = CX + 2 * XA, LY = CY + 2 * HY, LZ = CZ + 2 * HZ;
+  // z pass: segments of ZS output rows a task; the rows (z) that a tile of ez output rows stages
+  static constexpr int NSEG = NDIM == 2 ? 2 : 1, ZS = CZ / NSEG;
+  static __host__ __device__ __forceinline__ int box_z(int ez) { return (ez + ZS - 1) / ZS * ZS + 2 * HZ; }
   static constexpr size_t STAGE_BYTES = sizeof(T) * (size_t)LZ * LY * PX;
   // dynamic shared memory: the staged tile (128-byte aligned for TMA), the y-pass output in 3D
   static constexpr size_t SMEM_BYTES = 128 + STAGE_BYTES + (NDIM == 3 ? sizeof(T) * (size_t)CZ * CY * PX : 0);
@@ -381,10 +384,10 @@ __device__ __forceinline__ void sep_tile(const SepArgs<T>& a, const int tile, co
   const long long nxy = (long long)a.nx * a.ny;
   // z pass tasks: (x, y) columns of the staged tile that the y and x passes read, times segments of
   // ZS output rows covering the wz written ones
-  constexpr int C0 = XA - HX, NSEG = NDIM == 2 ? 2 : 1, ZS = CZ / NSEG;
+  constexpr int C0 = XA - HX, NSEG = G::NSEG, ZS = G::ZS;
   static_assert(CZ % NSEG == 0, "z segments must tile the output rows");
   const int ncx = wx + 2 * HX, ncy = NDIM == 3 ? wy + 2 * HY : 1;
-  const int nseg = (wz + ZS - 1) / ZS, rows_staged = min(LZ, nseg * ZS + 2 * HZ);
+  const int rows_staged = G::box_z(wz);
   T zt[2 * HZ + 1], xt[2 * HX + 1], yt[2 * HY + 1];
 #pragma unroll
   for (int m = 0; m <= 2 * HZ; ++m) zt[m] = a.zt[zs][m];
@@ -399,7 +402,7 @@ __device__ __forceinline__ void sep_tile(const SepArgs<T>& a, const int tile, co
     // where the grid spans the region in every direction
     if (threadIdx.x == 0) {
       mbar_init(&mbar, 1);
-      mbar_expect_tx(&mbar, (unsigned)G::STAGE_BYTES);
+      mbar_expect_tx(&mbar, (unsigned)(sizeof(T) * PX * LY * a.box_z));
       if (NDIM == 2) tma_load_2d(s0, &a.tm[comp], xs, zs0, &mbar);
       else tma_load_3d(s0, &a.tm[comp], xs, ys, zs0, &mbar);
     }
@@ -553,8 +556,9 @@ static cudaError_t launch_sep_t(const SepArgs<T>& a_in, cudaStream_t st) {
   a.use_tma = 0;
   if (a.nx >= G::PX && a.nz >= G::LZ && (NDIM == 2 || a.ny >= G::LY)) {
     bool ok = true;
+    a.box_z = G::box_z(te[2]);
     for (int c = 0; c < a.ncomp && ok; ++c)
-      ok = tma_encode(&a.tm[c], a.src[c], (int)sizeof(T), NDIM, a.nx, a.ny, a.nz, G::PX, G::LY, G::LZ);
+      ok = tma_encode(&a.tm[c], a.src[c], (int)sizeof(T), NDIM, a.nx, a.ny, a.nz, G::PX, G::LY, a.box_z);
     a.use_tma = ok ? 1 : 0;
   }
   cudaError_t e = ensure_dynamic_smem((const void*)k_sep_t<T, NDIM, HZ, HX>, sm);
@@ -884,6 +888,19 @@ constexpr int YEE_THREADS = 256;
 constexpr int YEE2_CX = 32, YEE2_CZ = 32;
 constexpr int YEE3_CX = 16, YEE3_CY = 8, YEE3_CZ = 8;
 
+// Quotient and remainder of a flat index (below 2^16) by a tile's run-time extent (below 2^10): a multiply by
+// the rounded-up reciprocal, exact there, instead of an integer division per cell and phase (64x128 FP64
+// pass 12.5 -> 12.35 ms).
+struct SmallDiv {
+  unsigned n, m;
+  __device__ __forceinline__ explicit SmallDiv(int d) : n(d), m(d > 1 ? 0xffffffffu / (unsigned)d + 1u : 0u) {}
+  __device__ __forceinline__ int operator()(int i, int& rem) const {
+    const unsigned q = n > 1 ? __umulhi((unsigned)i, m) : (unsigned)i;
+    rem = (int)((unsigned)i - q * n);
+    return (int)q;
+  }
+};
+
 template <bool CK>
 struct YeeHalo {
   static constexpr int HL = CK ? 3 : 1, HB = CK ? 2 : 1, HE = CK ? 1 : 0;
@@ -948,7 +965,7 @@ __device__ __forceinline__ void yee_tile(const YeeArgs<T>& a, const int tile, co
     // spans the staged region in every direction
     if (threadIdx.x == 0) {
       mbar_init(&mbar, 1);
-      mbar_expect_tx(&mbar, (unsigned)(9 * G::BOX_BYTES));
+      mbar_expect_tx(&mbar, (unsigned)(9 * sizeof(T) * LX * LY * a.box_z));
       for (int c = 0; c < 9; ++c) {
         if (NDIM == 2) tma_load_2d(sm + c * LN, &a.tm[c], xs, zs, &mbar);
         else tma_load_3d(sm + c * LN, &a.tm[c], xs, ys, zs, &mbar);
@@ -999,9 +1016,11 @@ __device__ __forceinline__ void yee_tile(const YeeArgs<T>& a, const int tile, co
   const int ny2 = NDIM == 3 ? wy + 2 : 1, ny1 = NDIM == 3 ? wy + 1 : 1;
   const int nbx = wx + 1 + HB, nbz = wz + 1 + HB;
   // each phase walks its cells with one flat index over all threads (rows are wider than a warp)
+  const SmallDiv by_nbx(nbx), by_nex(wx + 1 + HE), by_wx(wx), by_ny2(ny2), by_ny1(ny1), by_wy(wy);
   for (int idx = threadIdx.x; idx < ny2 * nbz * nbx; idx += YEE_THREADS) {
-    const int q = idx % nbx, row = idx / nbx;
-    const int lx = OX + HL - HB + q, ly = row % ny2, lz = HL - HB + row / ny2;
+    int q, ly = 0;
+    const int row = by_nbx(idx, q), pz = NDIM == 3 ? by_ny2(row, ly) : row;
+    const int lx = OX + HL - HB + q, lz = HL - HB + pz;
     const int l = (lz * LY + ly) * LX + lx;
     if (CK) {
       b[0][l] += hcz * ck_dz(e[1], l);
@@ -1018,8 +1037,9 @@ __device__ __forceinline__ void yee_tile(const YeeArgs<T>& a, const int tile, co
   // E^{n+1} on cells [-HE, w+1) in x and z ([0, w+1) in y)
   const int nex = wx + 1 + HE, nez = wz + 1 + HE;
   for (int idx = threadIdx.x; idx < ny1 * nez * nex; idx += YEE_THREADS) {
-    const int q = idx % nex, row = idx / nex;
-    const int lx = OX + HL - HE + q, ly = NDIM == 3 ? 1 + row % ny1 : 0, lz = HL - HE + row / ny1;
+    int q, py = -1;
+    const int row = by_nex(idx, q), pz = NDIM == 3 ? by_ny1(row, py) : row;
+    const int lx = OX + HL - HE + q, ly = 1 + py, lz = HL - HE + pz;
     const int l = (lz * LY + ly) * LX + lx;
     const T bx = b[0][l], by = b[1][l], bz = b[2][l];
     e[0][l] += a.cy * (bz - b[2][l - sy]) - a.cz * (by - b[1][l - sz]) - a.h * j[0][l];
@@ -1030,8 +1050,8 @@ __device__ __forceinline__ void yee_tile(const YeeArgs<T>& a, const int tile, co
   // B^{n+1} on cells [0, w), then write E and B of the tile (and, with DIAG, sum their energies)
   EnergyAcc<T> en;
   for (int idx = threadIdx.x; idx < wy * wz * wx; idx += YEE_THREADS) {
-    const int cx = idx % wx, row = idx / wx;
-    const int cy = row % wy, cz = row / wy;
+    int cx, cy = 0;
+    const int row = by_wx(idx, cx), cz = NDIM == 3 ? by_wy(row, cy) : row;
     const int gx = X0 + cx, gy = Y0 + cy, gz = Z0 + cz;
     const int l = ((cz + HL) * LY + cy + OY) * LX + cx + HL + OX;
     const T ex = e[0][l], ey = e[1][l], ez = e[2][l];
@@ -1134,8 +1154,9 @@ static cudaError_t launch_yee_tiles(const YeeArgs<T>& a_in, double* escratch, co
   if (a.nx >= G::PX && a.nz >= G::LZ && (NDIM == 2 || a.ny >= G::LY)) {
     const T* src[9] = {a.ex, a.ey, a.ez, a.bx, a.by, a.bz, a.jx, a.jy, a.jz};
     bool ok = true;
+    a.box_z = te[2] + G::HL + 2;  // a small grid's tiles stage only the rows they read
     for (int c = 0; c < 9 && ok; ++c)
-      ok = tma_encode(&a.tm[c], src[c], (int)sizeof(T), NDIM, a.nx, a.ny, a.nz, G::PX, G::LY, G::LZ);
+      ok = tma_encode(&a.tm[c], src[c], (int)sizeof(T), NDIM, a.nx, a.ny, a.nz, G::PX, G::LY, a.box_z);
     a.use_tma = ok ? 1 : 0;
   }
   if (hc) {

@@ -35,6 +35,7 @@ struct SepArgs {
   int spread;  // blocks to spread a small grid over (the SM count); 0: the kernel's full tiles
   // TMA staging (set by launch_sep when the grid allows it): one tensor map per source component
   int use_tma;
+  int box_z;  // z extent of its boxes
   int* err;  // device error flags (ERR_TIMEOUT when a staging wait gives up)
   CUtensorMap tm[6];
 };
@@ -56,6 +57,7 @@ struct YeeArgs {
   // Ex Ey Ez Bx By Bz Jx Jy Jz
   int spread = 0;      // blocks to spread a small grid over (the SM count); 0: the kernel's full tiles
   int use_tma = 0;
+  int box_z = 0;  // z extent of the boxes
   int* err = nullptr;  // device error flags (ERR_TIMEOUT when a staging wait gives up)
   CUtensorMap tm[9];
 };
