@@ -7,7 +7,7 @@
 
 namespace picgb {
 
-// Threads per push block: 8 warps; the 3D FP32 kernel, one block per SM, takes 12 warps. Cubic shapes
+// Threads per push block: 8 warps; the 3D FP32 kernel 6, so that two blocks fit an SM. Cubic shapes
 // (ORDER 3): the 51 register sums of the 2D window leave 168 registers a thread, two blocks of 6 warps
 // in FP32; 3D FP64 6 warps (their stages have to fit in shared memory).
 template <typename T, int NDIM, int ORDER = 1>
@@ -263,8 +263,8 @@ struct DepLayout<3> {
 // neighbour cell index in [-1, n]).
 __device__ __forceinline__ int wrap_near_p(int g, int n) { return g < 0 ? g + n : (g >= n ? g - n : g); }
 
-// FP32 uses the hardware reciprocal square root and fast division (relative error ~1e-7, inside
-// the 1e-5 per-step bar); FP64 keeps IEEE division and square root.
+// Reciprocals and square roots: FP32 the hardware's estimates (relative error ~1e-7, inside the 1e-5
+// per-step bar), FP64 one third-order step from them (fastmath.cuh).
 
 // Galerkin gather (order 0 along each half-staggered direction, order 1 elsewhere): the nodes are
 // the same for every particle of a cell, so they are read once per lane and each component is an
@@ -1468,25 +1468,26 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           bb = __shfl_sync(0xffffffffu, bb, ldb) + __popc(pb & lt);
           const bool fa = sta && ba >= r.cap, fb = stb && bb >= r.cap;  // full bins: on to k_migrate
           // leavers: the tile's shared buffer (one reservation for the pair), then the global list
-          // for full bins and once the shared buffer is full
-          const unsigned lma = __ballot_sync(0xffffffffu, lva), lmb = __ballot_sync(0xffffffffu, lvb);
+          // for full bins and once the shared buffer is full. Most rounds have neither: one vote
           int lsa = 0, lsb = 0;
-          if (lma | lmb) {
+          long long goa = 0, gob = 0;
+          bool ga = false, gb = false;
+          if (__any_sync(0xffffffffu, lva || lvb || fa || fb)) {
+            const unsigned lma = __ballot_sync(0xffffffffu, lva), lmb = __ballot_sync(0xffffffffu, lvb);
             int b0 = 0;
             if (lane == 0) b0 = atomicAdd(lvn, __popc(lma) + __popc(lmb));
             b0 = __shfl_sync(0xffffffffu, b0, 0);
             lsa = b0 + __popc(lma & lt);
             lsb = b0 + __popc(lma) + __popc(lmb & lt);
-          }
-          const bool ga = fa || (lva && lsa >= S::LVB), gb = fb || (lvb && lsb >= S::LVB);
-          const unsigned gma = __ballot_sync(0xffffffffu, ga), gmb = __ballot_sync(0xffffffffu, gb);
-          long long goa = 0, gob = 0;
-          if (gma | gmb) {
-            int b0 = 0;
-            if (lane == 0) b0 = atomicAdd(r.lv_count, __popc(gma) + __popc(gmb));
-            b0 = __shfl_sync(0xffffffffu, b0, 0);
-            goa = (long long)b0 + __popc(gma & lt);
-            gob = (long long)b0 + __popc(gma) + __popc(gmb & lt);
+            ga = fa || (lva && lsa >= S::LVB);
+            gb = fb || (lvb && lsb >= S::LVB);
+            const unsigned gma = __ballot_sync(0xffffffffu, ga), gmb = __ballot_sync(0xffffffffu, gb);
+            if (gma | gmb) {
+              if (lane == 0) b0 = atomicAdd(r.lv_count, __popc(gma) + __popc(gmb));
+              b0 = __shfl_sync(0xffffffffu, b0, 0);
+              goa = (long long)b0 + __popc(gma & lt);
+              gob = (long long)b0 + __popc(gma) + __popc(gmb & lt);
+            }
           }
           const int gcell = gk * r.nx + gi;  // cells < 2^30
           auto place = [&](bool st, bool full, bool lv, bool g, int dk, int jo, int ls, long long go, float nox,
@@ -1651,33 +1652,34 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
         // a full destination bin: the particle goes through the global leaver list instead, and
         // k_migrate spills it when the bin is still full there (nothing is dropped)
         const bool full = stay && base + rank >= r.cap;
-        const unsigned fmask = __ballot_sync(0xffffffffu, full);
-        long long fglob = 0;
-        if (fmask) {
-          const int fl = __ffs(fmask) - 1;
-          int fb = 0;
-          if (lane == fl) fb = atomicAdd(r.lv_count, __popc(fmask));
-          fb = __shfl_sync(0xffffffffu, fb, fl);
-          fglob = (long long)fb + __popc(fmask & ((1u << lane) - 1u));
-        }
-        // leavers: a slot in the tile's shared-memory buffer (one shared atomic per warp), or, once
-        // the buffer is full, straight in the global list
-        const unsigned lmask = __ballot_sync(0xffffffffu, valid && leave);
+        long long fglob = 0, lglob = 0;
         int lslot = 0;
-        long long lglob = 0;
-        if (lmask) {
-          const int lleader = __ffs(lmask) - 1;
-          int b = 0;
-          if (lane == lleader) b = atomicAdd(lvn, __popc(lmask));
-          b = __shfl_sync(0xffffffffu, b, lleader);
-          lslot = b + __popc(lmask & ((1u << lane) - 1u));
-          const unsigned gmask = __ballot_sync(0xffffffffu, valid && leave && lslot >= S::LVB);
-          if (gmask) {
-            const int gl = __ffs(gmask) - 1;
-            int gb = 0;
-            if (lane == gl) gb = atomicAdd(r.lv_count, __popc(gmask));
-            gb = __shfl_sync(0xffffffffu, gb, gl);
-            lglob = (long long)gb + __popc(gmask & ((1u << lane) - 1u));
+        if (__any_sync(0xffffffffu, full || (valid && leave))) {  // most rounds: neither
+          const unsigned fmask = __ballot_sync(0xffffffffu, full);
+          if (fmask) {
+            const int fl = __ffs(fmask) - 1;
+            int fb = 0;
+            if (lane == fl) fb = atomicAdd(r.lv_count, __popc(fmask));
+            fb = __shfl_sync(0xffffffffu, fb, fl);
+            fglob = (long long)fb + __popc(fmask & ((1u << lane) - 1u));
+          }
+          // leavers: a slot in the tile's shared-memory buffer (one shared atomic per warp), or, once
+          // the buffer is full, straight in the global list
+          const unsigned lmask = __ballot_sync(0xffffffffu, valid && leave);
+          if (lmask) {
+            const int lleader = __ffs(lmask) - 1;
+            int b = 0;
+            if (lane == lleader) b = atomicAdd(lvn, __popc(lmask));
+            b = __shfl_sync(0xffffffffu, b, lleader);
+            lslot = b + __popc(lmask & ((1u << lane) - 1u));
+            const unsigned gmask = __ballot_sync(0xffffffffu, valid && leave && lslot >= S::LVB);
+            if (gmask) {
+              const int gl = __ffs(gmask) - 1;
+              int gb = 0;
+              if (lane == gl) gb = atomicAdd(r.lv_count, __popc(gmask));
+              gb = __shfl_sync(0xffffffffu, gb, gl);
+              lglob = (long long)gb + __popc(gmask & ((1u << lane) - 1u));
+            }
           }
         }
         if (stay) {
