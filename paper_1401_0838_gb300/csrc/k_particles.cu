@@ -183,14 +183,14 @@ void push_tiles(int ndim, int es, bool ho, int nx, int ny, int nz, int spread, i
   set(full[0], full[1], full[2]);
   if (spread <= 0) return;
   // the resident blocks, and a tile's fixed cost (prologue and epilogue) in cells
-  const bool two = es == 4 && !(ndim == 3 && ho);
-  const long long slots = (long long)spread * (two ? 2 : 1);
+  const int per_sm = es == 8 ? 1 : (ndim == 2 ? 2 : (ho ? 1 : 3));
+  const long long slots = (long long)spread * per_sm;
   const int fixed = es == 4 ? 40 : 6;
   auto cost_of = [&](long long tiles) {
     return (double)((tiles + slots - 1) / slots) * ((double)te[0] * te[1] * te[2] + fixed);
   };
   const long long all = set(full[0], full[1], full[2]);
-  if (two && all > slots) return;  // several waves of block pairs: the partner of a late block speeds it up
+  if (per_sm > 1 && all > slots) return;  // several waves: the partners of a late block speed it up
   double best = 0.97 * cost_of(all);  // full tiles unless others gain 3 %
   int b[3] = {full[0], full[1], full[2]};
   for (int ex = full[0]; ex >= 4 || ex == full[0]; ex /= 2)

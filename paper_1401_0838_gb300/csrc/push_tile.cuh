@@ -7,13 +7,15 @@
 
 namespace picgb {
 
-// Threads per push block: 8 warps; the 3D FP32 kernel 6, so that two blocks fit an SM. Cubic shapes
+// Threads per push block: 8 warps; the 3D FP32 kernel 4, so that three blocks fit an SM at 168 registers: the
+// 16 cell groups of a tile are four rounds of them, and one block's prologue and epilogue run beside the
+// others' particles (128x128x512 pass 21.15 -> 20.2 ms against two blocks of 6 warps). Cubic shapes
 // (ORDER 3): the 51 register sums of the 2D window leave 168 registers a thread, two blocks of 6 warps
 // in FP32; 3D FP64 6 warps (their stages have to fit in shared memory).
 template <typename T, int NDIM, int ORDER = 1>
 struct PushThreads {
   static constexpr int value = ORDER == 3 ? (NDIM == 3 ? (sizeof(T) == 4 ? 384 : 192) : (sizeof(T) == 4 ? 192 : 256))
-                                          : (NDIM == 3 && sizeof(T) == 4) ? 192 : 256;
+                                          : (NDIM == 3 && sizeof(T) == 4) ? 128 : 256;
 };
 
 // The tile's compile-time extents by shape order.
@@ -74,8 +76,8 @@ struct PushSmem {
   static constexpr int JN = JX * JY * JZ;
   // particles leaving the tile, buffered per block: [7][LVB] values (ox oy oz dux duy duz w), LVB
   // keys, LVB ids and the buffer's counter; written to the global leaver list once per tile
-  // (3D: within the shared memory of one block per SM in FP64, of two in FP32)
-  static constexpr int LVB = NDIM == 3 && sizeof(T) == 8 ? 128 : 512;
+  // (3D: within the shared memory of one block per SM in FP64, of three in FP32)
+  static constexpr int LVB = NDIM == 3 ? (sizeof(T) == 8 ? 128 : 256) : 512;
   static constexpr size_t lv_bytes() { return (size_t)LVB * (7 * sizeof(T) + 2 * sizeof(int)) + 16; }
   static constexpr size_t bytes() {
     return sizeof(T) * (6 * GN * GCOPY + 3 * JN) + sizeof(int) * (4 * NCL) + 16 +
@@ -527,10 +529,10 @@ struct PushPlan {
   static __device__ __forceinline__ int first_window(int c) { return LPC == 4 ? (c >> 1) + (c & 1) : c; }
 };
 
-// Resident blocks per SM the push kernel is compiled for (register budget): FP32 2D fits two.
+// Resident blocks per SM the push kernel is compiled for (register budget).
 template <typename T, int NDIM, int ORDER = 1>
 struct PushMinBlocks {
-  static constexpr int value = sizeof(T) == 4 && !(NDIM == 3 && ORDER == 3) ? 2 : 1;
+  static constexpr int value = sizeof(T) == 8 || (NDIM == 3 && ORDER == 3) ? 1 : (NDIM == 3 ? 3 : 2);
 };
 
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
