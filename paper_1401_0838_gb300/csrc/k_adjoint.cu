@@ -559,37 +559,15 @@ template cudaError_t launch_adj_particles<double>(const AdjPartArgs<double>&, in
 //   lf_q += Psi_q(D_z) y_q          (y = F_filter applied to the adjoint of the copies)
 //   dots[n] += f_q . D_z^n y_q      (n = 0..4; Psi_E rows for q < 2, Psi_B rows for q >= 2)
 // since G_q = Psi_q(D_z) F_filter f_q with Psi_q = sum_n a_n D^n, every operator symmetric.
-// Block partial sums in FP64.
+// The products and their sums are FP64 in both precisions: an adjoint value scales with the caller's
+// upstream gradient, so a product leaves FP32's range (and the error term of an FP32 pair sooner) while
+// both factors are well inside it. That costs the adjoint of 20 steps on 256x512 cells 0.2 of 8.5 ms
+// against sums in FP32 pairs.
 // ---------------------------------------------------------------------------------------------
 // Blocks per component (grid-stride), partial sums per block. Few, because the block reductions and the
-// final sum over the partials cost more than the passes over the cells (with 304 blocks and FP64 products
-// 45 + 13 us on 256x512 cells).
+// final sum over the partials cost more than the passes over the cells (with 304 blocks 45 + 13 us on
+// 256x512 cells).
 constexpr int PSI_BLOCKS = 76;
-
-// A sum of products per thread: FP32 as a pair (the product exact in two floats, added by TwoSum), because
-// the FP64 pipe would bound this kernel; FP64 in FP64.
-template <typename T>
-struct PsiSum;
-template <>
-struct PsiSum<float> {
-  FPair p;
-  __device__ __forceinline__ void add(float a, float b) {
-    const float x = a * b;
-    p = pair_add(p, FPair{x, fmaf(a, b, -x)});
-  }
-  __device__ __forceinline__ void warp_sum() { p = warp_sum_pair(p); }
-  __device__ __forceinline__ double get() const { return (double)p.s + (double)p.c; }
-};
-template <>
-struct PsiSum<double> {
-  double p;
-  __device__ __forceinline__ void add(double a, double b) { p = fma(a, b, p); }
-  __device__ __forceinline__ void warp_sum() {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
-  }
-  __device__ __forceinline__ double get() const { return p; }
-};
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_adj_psi(const __grid_constant__ AdjPsiArgs<T> a) {
@@ -605,7 +583,7 @@ __global__ void __launch_bounds__(256) k_adj_psi(const __grid_constant__ AdjPsiA
 #pragma unroll
     for (int n = 0; n < 5; ++n) dp[n][m] = a.dpow[n][m];
   }
-  PsiSum<T> dn[5] = {};
+  double dn[5] = {0, 0, 0, 0, 0};
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < a.ncell;
        c += (long long)gridDim.x * blockDim.x) {
     const long long k = c / a.nxy, base = c - k * a.nxy;
@@ -621,26 +599,27 @@ __global__ void __launch_bounds__(256) k_adj_psi(const __grid_constant__ AdjPsiA
 #pragma unroll
     for (int m = 0; m < 9; ++m) psi += taps[m] * y[m];
     L[c] += psi;
-    const T f = Fq[c];
+    const double f = (double)Fq[c];
 #pragma unroll
     for (int n = 0; n < 5; ++n) {
       T v = T(0);
 #pragma unroll
       for (int m = 0; m < 9; ++m) v += dp[n][m] * y[m];
-      dn[n].add(f, v);
+      dn[n] = fma(f, (double)v, dn[n]);
     }
   }
-  __shared__ PsiSum<T> red[5][8];
+  __shared__ double red[5][8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
   for (int n = 0; n < 5; ++n) {
-    dn[n].warp_sum();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dn[n] += __shfl_xor_sync(0xffffffffu, dn[n], o);
     if (lane == 0) red[n][wid] = dn[n];
   }
   __syncthreads();
   if (threadIdx.x < 5) {
     double t = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[threadIdx.x][w].get();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[threadIdx.x][w];
     a.partial[((long long)q * gridDim.x + blockIdx.x) * 5 + threadIdx.x] = t;
   }
 }
