@@ -1832,19 +1832,13 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   }
 
   // 7. kinetic energy and particle count of this step: per-thread partial sums in the working
-  // precision, FP32 pairs (FP64: FP64) across the warp, FP64 across the block and the grid
+  // precision, FP64 across the warp, the block and the grid
   if (r.kin) {
     __shared__ double skin[NWARP];
     __shared__ int swcnt[NWARP];
-    double kd;
-    if constexpr (sizeof(T) == 4) {
-      const FPair t = warp_sum_pair(FPair{kin, 0.f});
-      kd = lane == 0 ? (double)t.s + (double)t.c : 0.0;
-    } else {
-      kd = kin;
+    double kd = (double)kin;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) kd += __shfl_xor_sync(0xffffffffu, kd, o);
-    }
+    for (int o = 16; o > 0; o >>= 1) kd += __shfl_xor_sync(0xffffffffu, kd, o);
     const int nd = __reduce_add_sync(0xffffffffu, npush);
     if (lane == 0) {
       skin[warp] = kd;
