@@ -1379,7 +1379,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           float2 t2 = fma2(tx, tx, one2);
           t2 = fma2(ty, ty, t2);
           t2 = fma2(tz, tz, t2);
-          const float2 sf = make_float2(fast_div(2.f, t2.x), fast_div(2.f, t2.y));
+          const float2 sf = WIN ? make_float2(fine_two_over(t2.x), fine_two_over(t2.y))
+                                : make_float2(two_over(t2.x), two_over(t2.y));
           const float2 sx = mul2(sf, tx), sy = mul2(sf, ty), sz = mul2(sf, tz);
           const float2 qx = fma2(my, tz, fma2(neg2(Mz), ty, mx));
           const float2 qy = fma2(Mz, tx, fma2(neg2(mx), tz, my));
@@ -1394,10 +1395,10 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           const float2 gp = add2(one2, u2);
           const float2 ign = WIN ? make_float2(fine_rsqrt(gp.x), fine_rsqrt(gp.y))
                                  : make_float2(fast_rsqrt(gp.x), fast_rsqrt(gp.y));
-          const float2 g1 = fma2(gp, ign, one2);  // gamma + 1; gamma - 1 = u^2 / (gamma + 1)
           if (r.kin) {
-            kin = fmaf(wa, fast_div(u2.x, g1.x), kin);
-            kin = fmaf(wb, fast_div(u2.y, g1.y), kin);
+            const float2 g1 = fma2(gp, ign, one2);  // gamma + 1; gamma - 1 = u^2 / (gamma + 1)
+            kin = fmaf(wa, WIN ? fine_kinetic(u2.x, gp.x, ign.x) : fast_div(u2.x, g1.x), kin);
+            kin = fmaf(wb, WIN ? fine_kinetic(u2.y, gp.y, ign.y) : fast_div(u2.y, g1.y), kin);
           }
           const float2 vy2 = mul2(uy2, ign);
           const float2 ddx2 = mul2(dtdx2, mul2(ux2, ign)), ddz2 = mul2(dtdz2, mul2(Uz, ign));
@@ -1586,7 +1587,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           const T mm = fma(Mz, Mz, fma(my, my, fma(mx, mx, T(1))));
           const T hig = h * (WIN ? fine_rsqrt(mm) : fast_rsqrt(mm));
           const T tx = hig * F[3], ty = hig * F[4], tz = hig * F[5];
-          const T sf = two_over(fma(tz, tz, fma(ty, ty, fma(tx, tx, T(1)))));
+          const T tt = fma(tz, tz, fma(ty, ty, fma(tx, tx, T(1))));
+          const T sf = WIN ? fine_two_over(tt) : two_over(tt);
           const T sx = sf * tx, sy = sf * ty, sz = sf * tz;
           const T qx = fma(my, tz, fma(-Mz, ty, mx));
           const T qy = fma(Mz, tx, fma(-mx, tz, my));
@@ -1598,7 +1600,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           const T u2 = fma(Uz, Uz, fma(uy, uy, ux * ux)), gp = T(1) + u2;
           const T ign = WIN ? fine_rsqrt(gp) : fast_rsqrt(gp);
           T vy = uy * ign;
-          if (r.kin) kin = fma(w, fast_div(u2, fma(gp, ign, T(1))), kin);  // gamma - 1 = u^2 / (gamma + 1)
+          if (r.kin)  // gamma - 1 = u^2 / (gamma + 1)
+            kin = fma(w, WIN ? fine_kinetic(u2, gp, ign) : fast_div(u2, fma(gp, ign, T(1))), kin);
           if (LATE) ++npush;
           // move (cell-relative displacement in grid units)
           T ddx = r.dtdx * (ux * ign), ddy = NDIM == 3 ? r.dtdy * vy : T(0), ddz = r.dtdz * (Uz * ign);

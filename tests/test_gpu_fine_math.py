@@ -1,0 +1,119 @@
+"""The roots and quotients of csrc/fastmath.cuh that stand for IEEE expressions (fine_*, and the FP64 steps under them)
+against exactly rounded references: an error no larger than that of the expression they stand for, every FP32
+significand and FP64 samples, and the values past the FP32 estimates' range. A small kernel that includes the header is
+built here with nvcc and run through ctypes."""
+import ctypes
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1401_0838_gb300 import build as B
+
+pytestmark = pytest.mark.gpu
+
+SRC = r"""
+#include <cuda_runtime.h>
+#include "fastmath.cuh"
+using namespace picgb;
+
+template <typename T>
+__global__ void k_fine(const T* x, const T* u2, T* o, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const T v = x[i], q = u2[i], gp = T(1) + q, ign = fine_rsqrt(gp);
+  T* r = o + 8 * (size_t)i;
+  r[0] = fine_rsqrt(v);
+  r[1] = T(1) / sqrt(v);
+  r[2] = fine_recip(v);
+  r[3] = T(1) / v;
+  r[4] = fine_two_over(v);
+  r[5] = T(2) / v;
+  r[6] = fine_kinetic(q, gp, ign);
+  r[7] = q / (sqrt(T(1) + q) + T(1));
+}
+
+template <typename T>
+static int run(const T* x, const T* u2, T* out, int n) {
+  T *dx = nullptr, *du = nullptr, *dout = nullptr;
+  const size_t b = sizeof(T) * (size_t)n;
+  int rc = cudaMalloc(&dx, b) || cudaMalloc(&du, b) || cudaMalloc(&dout, 8 * b);
+  if (!rc) rc = cudaMemcpy(dx, x, b, cudaMemcpyHostToDevice) || cudaMemcpy(du, u2, b, cudaMemcpyHostToDevice);
+  if (!rc) {
+    k_fine<T><<<(n + 255) / 256, 256>>>(dx, du, dout, n);
+    rc = cudaGetLastError() != cudaSuccess || cudaMemcpy(out, dout, 8 * b, cudaMemcpyDeviceToHost) != cudaSuccess;
+  }
+  cudaFree(dx);
+  cudaFree(du);
+  cudaFree(dout);
+  return rc;
+}
+extern "C" int run_f(const float* x, const float* u, float* o, int n) { return run(x, u, o, n); }
+extern "C" int run_d(const double* x, const double* u, double* o, int n) { return run(x, u, o, n); }
+"""
+
+
+@pytest.fixture(scope="module")
+def fine(tmp_path_factory):
+    d = tmp_path_factory.mktemp("fine")
+    src, so = d / "fine.cu", d / "libfine.so"
+    src.write_text(SRC)
+    r = subprocess.run([B.nvcc(), "-shared", "-Xcompiler", "-fPIC", "-O3", "-std=c++17", *B.ARCH, "-I", B.CSRC, "-o",
+                        str(so), str(src), "-lcudart"], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    lib = ctypes.CDLL(str(so))
+
+    def call(x, u2):
+        out = np.empty((len(x), 8), x.dtype)
+        f = lib.run_f if x.dtype == np.float32 else lib.run_d
+        assert f(*(ctypes.c_void_p(a.ctypes.data) for a in (x, u2, out)), ctypes.c_int(len(x))) == 0
+        return out
+
+    return call
+
+
+def _ulps(got, exact):
+    """Error of got in units of its own type's spacing at the exact value (which has more bits)."""
+    return np.abs(got.astype(exact.dtype) - exact) / np.spacing(np.abs(exact).astype(got.dtype)).astype(exact.dtype)
+
+
+def _check(r, x, u2, wide):
+    X, U = x.astype(wide), u2.astype(wide)
+    one = wide(1)
+    exact = [one / np.sqrt(X), one / X, wide(2) / X, U / (np.sqrt(one + U) + one)]
+    for k, e in enumerate(exact):
+        fine, ieee = _ulps(r[:, 2 * k], e).max(), _ulps(r[:, 2 * k + 1], e).max()
+        assert fine <= ieee * (1 + 1e-9), (k, fine, ieee)
+
+
+def test_fp32_every_significand(fine):
+    m = np.arange(1 << 23, dtype=np.uint32)
+    rng = np.random.default_rng(1)
+    for e in (0, 1):  # the root's two exponent classes
+        x = (m + np.uint32((127 + e) << 23)).view(np.float32)
+        u2 = (10.0 ** rng.uniform(-12, 10, len(m))).astype(np.float32)
+        _check(fine(x, u2), x, u2, np.float64)
+
+
+def test_fp64_samples(fine):
+    rng = np.random.default_rng(2)
+    n = 1 << 20
+    x = np.ldexp(rng.uniform(1, 2, n), rng.integers(0, 60, n))
+    u2 = 10.0 ** rng.uniform(-16, 12, n)
+    r = fine(x, u2)
+    if np.finfo(np.longdouble).nmant < 63:
+        pytest.skip("no wider type for the reference")
+    _check(r, x, u2, np.longdouble)
+
+
+@pytest.mark.parametrize("T", [np.float32, np.float64])
+def test_range(fine, T):
+    # past 2^126 (the FP32 reciprocal estimate's end) and, in FP64, past FP32's largest value; infinities and NaN
+    x = np.array([2.0 ** 120, 2.0 ** 125, 2.0 ** 126, 1.5 * 2.0 ** 126, 2.0 ** 127, 3.4e38] +
+                 ([1e40, 1e80, 1e300] if T is np.float64 else []) + [np.inf, np.nan], dtype=T)
+    u2 = np.where(np.isfinite(x), x, T(1)).astype(T) if T is np.float64 else np.ones(len(x), T)
+    r = fine(x, u2)
+    for k in range(4):
+        a, b = r[:, 2 * k], r[:, 2 * k + 1]
+        ok = (a == b) | (np.isnan(a) & np.isnan(b)) | (np.abs(a - b) <= 2 * np.spacing(np.abs(b)))
+        assert ok.all(), (k, x[~ok], a[~ok], b[~ok])

@@ -1,4 +1,5 @@
-"""Single steps at the ends of the number range."""
+"""Single steps at the ends of the number range: recorded kinetic energies past FP32's range, rotations by fields so
+strong that 1 + t^2 nears it, momenta whose square leaves it."""
 import numpy as np
 import pytest
 
@@ -6,6 +7,8 @@ from tests._pic import P, make_cfg
 
 pytestmark = pytest.mark.gpu
 FN = ("ex", "ey", "ez", "bx", "by", "bz")
+# the pushes that read a window of nodes: cubic shapes, and the momentum-conserving gather
+WINDOW = [(2, 3, 0), (2, 3, 1), (2, 3, 2), (2, 1, 2), (3, 3, 0), (3, 3, 1), (3, 3, 2), (3, 1, 2)]
 
 
 def _handle(ndim, precision, order=1, scheme=0, cells=None, species=None, mom=None, fields=None, sigma=0.0, w=None,
@@ -30,6 +33,16 @@ def _handle(ndim, precision, order=1, scheme=0, cells=None, species=None, mom=No
     return h, cfg, T
 
 
+def _momenta(h, n, T):
+    out = {k: np.zeros(n, T) for k in ("dux", "duy", "duz", "oz")}
+    out.update({k: np.zeros(n, np.int32) for k in ("cell", "species")}, id=np.zeros(n, np.uint32))
+    s = P.make_state(P.PIC_HOST, None, out)
+    s.np = n
+    P.pic_get_state(h, s)
+    order = np.argsort(out["id"])
+    return {k: v[order] for k, v in out.items()}
+
+
 @pytest.mark.parametrize("ndim,order,scheme", [(2, 1, 0), (2, 3, 0), (3, 1, 0), (3, 3, 0)])
 def test_kinetic_record_past_fp32(ndim, order, scheme):
     # a thread's sum stays below 3.4e38, a warp's does not; the record is FP64 from there on. An electron and a
@@ -47,3 +60,42 @@ def test_kinetic_record_past_fp32(ndim, order, scheme):
     want = len(cell) * float(T(w)) * 129.0
     assert want > 3.4e38 * 8
     assert abs(e["k"] - want) <= 1e-5 * want, e
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("ndim,order,scheme", WINDOW)
+def test_rotation_by_a_very_strong_field(ndim, order, scheme, precision):
+    # t = dt/2 B / gamma with t^2 past the FP32 estimates' range (a reciprocal of more than 2^126): the rotation
+    # about B tends to half a turn, u perpendicular to B changes sign
+    t = 1.25e19 if precision == 0 else 1e25
+    cells, species = [5 * 24 + 7] * 2, [0, 1]
+    h, cfg, T = _handle(ndim, precision, order, scheme, cells, species, (3.0, 0.25, 0.0), {"by": t * 130.0 / 0.25})
+    u0 = float(T(np.sqrt(130.0 ** 2 - 1)))
+    try:
+        P.pic_step(h, 1)
+        P.pic_sync(h)
+        m = _momenta(h, 2, T)
+    finally:
+        P.pic_destroy(h)
+    tol = 1e-5 if precision == 0 else 1e-10
+    assert np.abs(m["duz"] + u0 + u0).max() <= tol * u0, m  # u_z = u0 + duz -> -u0
+    assert np.abs(m["dux"] + 3.0).max() <= tol * u0, m
+    assert np.abs(m["duy"] - 0.25).max() <= tol * u0, m
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("ndim,order,scheme", WINDOW)
+def test_momenta_past_fp32_squares(ndim, order, scheme, precision):
+    # FP64: u = 1e25 moves at the speed of light. FP32: u^2 is infinite and the velocity comes out zero, which is no
+    # error of the step
+    h, cfg, T = _handle(ndim, precision, order, scheme, [5 * 24 + 7] * 2, [0, 1], (0.0, 0.0, 1e25))
+    try:
+        P.pic_step(h, 1)
+        P.pic_sync(h)
+        m = _momenta(h, 2, T)
+    finally:
+        P.pic_destroy(h)
+    assert (m["duz"] == T(1e25)).all(), m
+    k = m["cell"] // (24 * (10 if ndim == 3 else 1))
+    z0 = 5 // (10 if ndim == 3 else 1)
+    assert np.abs(k + m["oz"] - (z0 + (1.0 if precision else 0.5))).max() <= 1e-12, m
