@@ -1284,13 +1284,17 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     cp_async_wait_1();
     __syncwarp();
 
-    const int cl = g * CPW + lane / LPC;
-    // (an empty cell past the tile's last plane, in the last group, stands in that plane: its nodes are
-    // staged, so that the lanes without a particle compute with finite fields)
-    const int lx = cl % TX, ly = (cl / TX) % TY, lz = min(cl / (TX * TY), wz - 1);
-    const int gi = X0 + lx, gj = Y0 + ly, gk = Z0 + lz;
+    int cl = g * CPW + lane / LPC;
     const int n0 = sn[cl], n1 = sn[NCL + cl];
     const int nq0 = (n0 + 3) >> 2, nq = nq0 + ((n1 + 3) >> 2);
+    // the lanes of an empty cell stand in a cell that holds particles: a pair's empty slots go through the
+    // arithmetic, and an empty cell's fields may be anything (not finite, or past the tile's last plane not staged)
+    if constexpr (PushPaired<T, NDIM>::value) {
+      const unsigned live = __ballot_sync(0xffffffffu, nq > 0);
+      if (nq == 0) cl = g * CPW + (__ffs(live) - 1) / LPC;
+    }
+    const int lx = cl % TX, ly = (cl / TX) % TY, lz = min(cl / (TX * TY), wz - 1);
+    const int gi = X0 + lx, gj = Y0 + ly, gk = Z0 + lz;
     const int okey = ((lz + 1) * S::JY + (NDIM == 3 ? ly + 1 : 0)) * S::JX + lx + 1;  // cell-origin window
     if (it == 0) {
       if (SCHEME == 0 && !WIN) gc.load(sg, lx, ly, lz);

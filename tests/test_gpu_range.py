@@ -1,5 +1,6 @@
-"""Single steps at the ends of the number range: recorded kinetic energies past FP32's range, rotations by fields so
-strong that 1 + t^2 nears it, momenta whose square leaves it."""
+"""Single steps at the ends of the number range: recorded kinetic energies past FP32's range, rotations by
+fields so strong that (1 + t^2) nears it, momenta whose square leaves it, and fields that are not finite where no
+particle is."""
 import numpy as np
 import pytest
 
@@ -99,3 +100,31 @@ def test_momenta_past_fp32_squares(ndim, order, scheme, precision):
     k = m["cell"] // (24 * (10 if ndim == 3 else 1))
     z0 = 5 // (10 if ndim == 3 else 1)
     assert np.abs(k + m["oz"] - (z0 + (1.0 if precision else 0.5))).max() <= 1e-12, m
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("ndim,order,scheme", WINDOW + [(2, 1, 0), (2, 1, 1), (3, 1, 0)])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_bad_fields_without_particles(ndim, order, scheme, precision, bad):
+    # particles in cells x = 0 of some rows, a bad value seven cells on in the same rows, filters off: no particle
+    # reads it, and the cells beside it, which share the particles' warps, are empty
+    nx, ny, nz = 24, 10 if ndim == 3 else 1, 32
+    rows = np.arange(ny * nz) * nx
+    cells, species = np.tile(rows, 2), np.repeat([0, 1], len(rows))
+    f = np.zeros((nz, ny, nx))
+    f[:, :, 7] = bad
+    want, got = [], None
+    for fields in ({}, {"ex": f, "ez": f, "by": f}):
+        h, cfg, T = _handle(ndim, precision, order, scheme, cells, species, (0.1, 0.2, 0.3), fields, targets=0)
+        try:
+            P.pic_step(h, 1)
+            P.pic_sync(h)
+            m = _momenta(h, len(cells), T)
+            m["k"] = P.pic_energy_history(h, 4)[-1]["k"]
+            want.append(m)
+        finally:
+            P.pic_destroy(h)
+    a, b = want
+    for k in ("dux", "duy", "duz", "oz", "cell"):
+        np.testing.assert_array_equal(a[k], b[k])
+    assert abs(a["k"] - b["k"]) <= 1e-6 * abs(a["k"])
