@@ -186,24 +186,23 @@ void push_tiles(int ndim, int es, bool ho, int nx, int ny, int nz, int spread, i
   const int per_sm = es == 8 ? 1 : (ndim == 2 ? 2 : (ho ? 1 : 3));
   const long long slots = (long long)spread * per_sm;
   const int fixed = es == 4 ? 40 : 6;
+  // a warp's cell group takes whole rows of the full tile's width, so narrower tiles only leave lanes idle
   auto cost_of = [&](long long tiles) {
-    return (double)((tiles + slots - 1) / slots) * ((double)te[0] * te[1] * te[2] + fixed);
+    return (double)((tiles + slots - 1) / slots) * ((double)full[0] * te[1] * te[2] + fixed);
   };
   const long long all = set(full[0], full[1], full[2]);
   if (per_sm > 1 && all > slots) return;  // several waves: the partners of a late block speed it up
   double best = 0.97 * cost_of(all);  // full tiles unless others gain 3 %
   int b[3] = {full[0], full[1], full[2]};
-  for (int ex = full[0]; ex >= 4 || ex == full[0]; ex /= 2)
-    for (int ey = full[1]; ey >= 4 || ey == full[1]; ey /= 2)
-      for (int ez = full[2]; ez >= 4 || ez == full[2]; --ez) {
-        const double cost = cost_of(set(ex, ey, ez));
-        if (cost < best * (1 - 1e-9)) {
-          best = cost;
-          b[0] = ex;
-          b[1] = ey;
-          b[2] = ez;
-        }
+  for (int ey = full[1]; ey >= 4 || ey == full[1]; ey /= 2)
+    for (int ez = full[2]; ez >= 4 || ez == full[2]; --ez) {
+      const double cost = cost_of(set(full[0], ey, ez));
+      if (cost < best * (1 - 1e-9)) {
+        best = cost;
+        b[1] = ey;
+        b[2] = ez;
       }
+    }
   set(b[0], b[1], b[2]);
 }
 

@@ -87,8 +87,9 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 }
 
 // Particle tiles of a grid. spread = 0: the push kernel's tile (PTile, or HoTile for cubic shapes) for
-// the precision (es bytes per value). spread = the number of SMs: the extents, at most that tile's and not
-// below 4 cells, whose tiles fill the resident blocks (per SM two in FP32, three in 3D, one in FP64 and for cubic 3D)
+// the precision (es bytes per value). spread = the number of SMs: the extents along y and z, at most that tile's
+// and not below 4 cells (its width is kept, since a warp takes whole
+// rows of it: on 44^3 FP64 cells 4x4x4 tiles took 1350 us, 8x4x5 973), whose tiles fill the resident blocks (per SM two in FP32, three in 3D, one in FP64 and for cubic 3D)
 // in the fewest cells, counting a tile's fixed cost as 40 cells in FP32 and 6 in FP64 (measured on empty
 // grids: 6 us of the 44 us a wave of full tiles takes at 16 FP32 particles per cell and species, 6 of
 // 360 us in FP64): push on 128x256 with 8 FP32 particles 26 -> 20 us, 256x512 FP64 1216 -> 1088 us, cubic
