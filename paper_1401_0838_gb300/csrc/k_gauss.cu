@@ -40,58 +40,98 @@ __device__ __forceinline__ int wrap_any(int g, int n) {
 // alone fill the GPU, so that every lane of an FP64 instruction works (that pipe bounds this kernel: a
 // warp per cell left half to three quarters of the lanes idle). A lane sums its particles' weights in
 // registers, the cell's lanes add up, and one lane adds each node once instead of once per particle:
-// 331 -> 95 us on 301 x 517 cells of 2 x 8 particles.
+// 331 -> 95 us on 301 x 517 cells of 2 x 8 particles. Cells that hold far more particles than their
+// neighbours (bunches) would keep a warp on one lane: past a limit the whole warp takes a cell's
+// particles together, RHOB.
 template <typename T, int NDIM, int ORDER>
 __global__ void __launch_bounds__(RHO_THREADS) k_rho(const __grid_constant__ RunDev<T> r, int lpc, double inv_dv,
                                                      double* __restrict__ rho) {
   constexpr int NN = ORDER + 1, NY = NDIM == 3 ? NN : 1, LO = ORDER == 3 ? -1 : 0;
-  const int sub = threadIdx.x & (lpc - 1);
+  const int lane = threadIdx.x & 31;
   const long long step = (long long)gridDim.x * RHO_THREADS / lpc;
   // every lane of a warp runs the same trips: the lanes past the last cell take part in the sums with nothing
   for (long long c0 = ((long long)blockIdx.x * RHO_THREADS + (threadIdx.x & ~31)) / lpc; c0 < r.ncell; c0 += step) {
-    const long long cell = c0 + (threadIdx.x & 31) / lpc;
-    const bool on = cell < r.ncell;
-    double acc[NN * NY * NN] = {};
-#pragma unroll 1
-    for (int s = 0; s < 2; ++s) {
-      const SpeciesBuf<T>& b = s ? r.in[1] : r.in[0];
-      const int n = on ? min(b.cnt[cell], r.cap) : 0;
-      const double q = s ? inv_dv : -inv_dv;
-      for (int slot = sub; slot < n; slot += lpc) {
-        const long long o = cell * r.cap + slot;
-        const double qw = q * (b.w ? (double)b.w[o] : (double)r.wconst);
-        double wx[NN], wy[NN], wz[NN];
-        const PartVals<T> v = part_get(b, NDIM, o);
-        node_weights<ORDER>((double)v.ox, wx);
-        if constexpr (NDIM == 3) node_weights<ORDER>((double)v.oy, wy);
-        node_weights<ORDER>((double)v.oz, wz);
-#pragma unroll
-        for (int c = 0; c < NN; ++c)
-#pragma unroll
-          for (int bb = 0; bb < NY; ++bb) {
-            const double wyz = NDIM == 3 ? qw * wy[bb] * wz[c] : qw * wz[c];
-#pragma unroll
-            for (int a = 0; a < NN; ++a) acc[(c * NY + bb) * NN + a] = fma(wyz, wx[a], acc[(c * NY + bb) * NN + a]);
-          }
-      }
-    }
-    for (int d = lpc >> 1; d > 0; d >>= 1)
-#pragma unroll
-      for (int e = 0; e < NN * NY * NN; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], d);
-    if (!on || sub != 0) continue;
-    const int ci = (int)cell, i = ci % r.nx, j = ci / r.nx % r.ny, k = ci / r.nx / r.ny;
-#pragma unroll
-    for (int c = 0; c < NN; ++c) {
-      const long long kz = wrap_any(k + LO + c, r.nz);
-#pragma unroll
-      for (int bb = 0; bb < NY; ++bb) {
-        const long long jy = NDIM == 3 ? wrap_any(j + LO + bb, r.ny) : 0;
-#pragma unroll
-        for (int a = 0; a < NN; ++a) {
-          const double v = acc[(c * NY + bb) * NN + a];
-          if (v != 0.0) atomicAdd(rho + (kz * r.ny + jy) * r.nx + wrap_any(i + LO + a, r.nx), v);
+    const long long own = c0 + lane / lpc;
+    const bool in = own < r.ncell;
+    const int own0 = in ? min(r.in[0].cnt[own], r.cap) : 0, own1 = in ? min(r.in[1].cnt[own], r.cap) : 0;
+    // slots per species that the cell's own lanes take: all, or what leaves clearly fewer rounds of the warp (a
+    // round of the lanes' own cells, or 32 slots of a crowded one, which also costs two for its sums)
+    const int most = __reduce_max_sync(0xffffffffu, max(own0, own1));
+    int limit = most;
+    unsigned more = 0;
+    if (lpc < 32 && most > 16 * lpc) {
+      int best = 3 * ((most + lpc - 1) / lpc) / 2;  // a quarter less than all of them
+      for (int l = 8 * lpc; l < most; l *= 2) {
+        const int x = max(own0 - l, 0), y = max(own1 - l, 0);
+        const int extra = lane % lpc == 0 && (x | y) != 0 ? (x + 31) / 32 + (y + 31) / 32 + 2 : 0;
+        const int rounds = 2 * (l / lpc) + __reduce_add_sync(0xffffffffu, extra);
+        if (rounds < best) {
+          best = rounds;
+          limit = l;
         }
       }
+      more = __ballot_sync(0xffffffffu, lane % lpc == 0 && max(own0, own1) > limit);
+    }
+    int lanes = lpc, first = 0;
+    bool on = in;
+    long long cell = own;
+    int n0 = min(own0, limit), n1 = min(own1, limit);
+    for (;;) {
+      const int sub = lane & (lanes - 1);
+      double acc[NN * NY * NN] = {};
+#pragma unroll 1
+      for (int s = 0; s < 2; ++s) {
+        const SpeciesBuf<T>& b = s ? r.in[1] : r.in[0];
+        const int n = s ? n1 : n0;
+        const double q = s ? inv_dv : -inv_dv;
+        for (int slot = first + sub; slot < n; slot += lanes) {
+          const long long o = cell * r.cap + slot;
+          const double qw = q * (b.w ? (double)b.w[o] : (double)r.wconst);
+          double wx[NN], wy[NN], wz[NN];
+          const PartVals<T> v = part_get(b, NDIM, o);
+          node_weights<ORDER>((double)v.ox, wx);
+          if constexpr (NDIM == 3) node_weights<ORDER>((double)v.oy, wy);
+          node_weights<ORDER>((double)v.oz, wz);
+#pragma unroll
+          for (int c = 0; c < NN; ++c)
+#pragma unroll
+            for (int bb = 0; bb < NY; ++bb) {
+              const double wyz = NDIM == 3 ? qw * wy[bb] * wz[c] : qw * wz[c];
+#pragma unroll
+              for (int a = 0; a < NN; ++a) acc[(c * NY + bb) * NN + a] = fma(wyz, wx[a], acc[(c * NY + bb) * NN + a]);
+            }
+        }
+      }
+      int d = lanes >> 1;
+      while (d >= most && d > 0) d >>= 1;  // the lanes past the fullest cell's slots hold nothing
+      for (; d > 0; d >>= 1)
+#pragma unroll
+        for (int e = 0; e < NN * NY * NN; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], d);
+      if (on && sub == 0) {
+        const int ci = (int)cell, i = ci % r.nx, j = ci / r.nx % r.ny, k = ci / r.nx / r.ny;
+#pragma unroll
+        for (int c = 0; c < NN; ++c) {
+          const long long kz = wrap_any(k + LO + c, r.nz);
+#pragma unroll
+          for (int bb = 0; bb < NY; ++bb) {
+            const long long jy = NDIM == 3 ? wrap_any(j + LO + bb, r.ny) : 0;
+#pragma unroll
+            for (int a = 0; a < NN; ++a) {
+              const double v = acc[(c * NY + bb) * NN + a];
+              if (v != 0.0) atomicAdd(rho + (kz * r.ny + jy) * r.nx + wrap_any(i + LO + a, r.nx), v);
+            }
+          }
+        }
+      }
+      if (more == 0) break;
+      const int src = __ffs(more) - 1;  // the next crowded cell, past its lanes' share
+      more &= more - 1;
+      lanes = 32;
+      first = limit;
+      on = true;
+      cell = c0 + src / lpc;
+      n0 = __shfl_sync(0xffffffffu, own0, src);
+      n1 = __shfl_sync(0xffffffffu, own1, src);
     }
   }
 }
@@ -176,8 +216,10 @@ size_t gauss_scratch_bytes() { return sizeof(double) * (3 * GR_BLOCKS + 2); }
 
 template <typename T>
 cudaError_t launch_rho(const RunDev<T>& r, int order, double inv_dv, double* rho, cudaStream_t st) {
-  int lpc = 1;  // lanes per cell: until the cells fill the 152 SMs with 16 warps each, or a warp has one cell
-  while (lpc < 32 && r.ncell * lpc < 152ll * 512) lpc *= 2;
+  // lanes per cell: until the cells give each of the 152 SMs four warps, one per scheduler, or a warp has one
+  // cell. The residual on 64x64 cubic cells of 2 x 8 takes 123 us (with 8 warps per SM 140, with 16 191)
+  int lpc = 1;
+  while (lpc < 32 && r.ncell * lpc < 152ll * 128) lpc *= 2;
   const long long want = (r.ncell * lpc + RHO_THREADS - 1) / RHO_THREADS;
   const int blocks = (int)(want < 8 * 152 ? (want < 1 ? 1 : want) : 8 * 152);
   if (r.ndim == 3 && order == 3)

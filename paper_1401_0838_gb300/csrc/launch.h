@@ -87,14 +87,15 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 }
 
 // Particle tiles of a grid. spread = 0: the push kernel's tile (PTile, or HoTile for cubic shapes) for
-// the precision (es bytes per value). spread = the number of SMs: the extents along y and z, at most that tile's
-// and not below 4 cells (its width is kept, since a warp takes whole
-// rows of it: on 44^3 FP64 cells 4x4x4 tiles took 1350 us, 8x4x5 973), whose tiles fill the resident blocks (per SM two in FP32, three in 3D, one in FP64 and for cubic 3D)
-// in the fewest cells, counting a tile's fixed cost as 40 cells in FP32 and 6 in FP64 (measured on empty
-// grids: 6 us of the 44 us a wave of full tiles takes at 16 FP32 particles per cell and species, 6 of
-// 360 us in FP64): push on 128x256 with 8 FP32 particles 26 -> 20 us, 256x512 FP64 1216 -> 1088 us, cubic
-// 3D 44x36x70 230 -> 177 us. Several waves of more than one block per SM keep full tiles (301x517: 61 us against 67
-// on the extents the count of waves would choose). te: cells per tile and direction.
+// the precision (es bytes per value). spread = the number of SMs: the extents along y and z, at most that
+// tile's and not below 4 cells, whose tiles fill the resident blocks (per SM two in FP32, three in 3D, one
+// in FP64 and for cubic 3D) in the fewest rows of cells, counting a tile's fixed cost as 40 cells in FP32
+// and 6 in FP64 (measured on empty grids: 6 us of the 44 us a wave of full tiles takes at 16 FP32
+// particles per cell and species, 6 of 360 us in FP64): push on 128x256 with 8 FP32 particles 26 -> 20 us,
+// 256x512 FP64 1216 -> 1088 us, cubic 3D 44x36x70 230 -> 177 us. The width stays, because a warp takes whole
+// rows of it (a step on 44^3 FP64 cells: 4x4x4 tiles 1350 us, 8x4x5 973). Several waves of more than one
+// block per SM keep full tiles (301x517: 61 us against 67 on the extents the count of waves would
+// choose). te: cells per tile and direction.
 void push_tiles(int ndim, int es, bool ho, int nx, int ny, int nz, int spread, int nt[3], int te[3]);
 
 // Raise a kernel's dynamic shared memory limit to `bytes` (once per kernel and size).

@@ -1,0 +1,69 @@
+"""Diagnostics on a state whose particles crowd into a few cells (an instability bunches the beam): right, and not at the
+mercy of a few lanes that walk a crowded cell alone."""
+import time
+
+import numpy as np
+import pytest
+
+import synth
+from tests._pic import P, Pair, make_cfg
+from tests.test_gpu_gauss import _oracle_residual
+
+pytestmark = pytest.mark.gpu
+
+
+def _clumped(ndim, nx, ny, nz, crowd, seed=5):
+    """One particle per cell, and `crowd` more in each of five cells."""
+    n = nx * ny * nz
+    p = synth.random_particles(ndim, nx, ny, nz, n + 5 * crowd, seed=seed)
+    rng = np.random.default_rng(seed)
+    cell = np.concatenate([np.arange(n), np.repeat(rng.integers(0, n, 5), crowd)])
+    for k, v, m in (("x", cell % nx, nx), ("y", cell // nx % ny, ny), ("z", cell // (nx * ny), nz)):
+        if k != "y" or ndim == 3:
+            p[k] = v + rng.uniform(0, 0.999, len(cell))
+    return p
+
+
+# at one lane per cell (the larger grids) and at several: the crowded cells of a warp are taken by all its lanes
+@pytest.mark.parametrize("precision", [1, 0])
+@pytest.mark.parametrize("ndim,order", [(2, 1), (2, 3), (3, 1), (3, 3)])
+@pytest.mark.parametrize("large", [0, 1])
+@pytest.mark.parametrize("crowd", [33, 700])
+def test_charge_density_of_clumps(precision, ndim, order, large, crowd):
+    nx, ny, nz = [[(37, 1, 41), (281, 1, 277)], [(11, 9, 13), (44, 43, 42)]][ndim - 2][large]
+    cfg = make_cfg(ndim=ndim, nx=nx, ny=ny, nz=nz, dt=0.4, precision=precision, order=order, cap=8 if crowd < 100 else 800)
+    pair = Pair(cfg, part=_clumped(ndim, nx, ny, nz, crowd))
+    try:
+        got, want = P.pic_charge_residual(pair.h), _oracle_residual(pair, cfg)
+    finally:
+        pair.close()
+    # a node sums up to 8 crowd FP64 terms on either side
+    for name, w in zip(("max", "rms", "rho_max"), want):
+        assert abs(got[name] - w) <= 1e-11 * want[0], (name, got, want)
+
+
+def _best(f, n=7):
+    t = []
+    for _ in range(n):
+        t0 = time.perf_counter()
+        f()
+        t.append(time.perf_counter() - t0)
+    return min(t)
+
+
+def test_charge_density_time_of_clumps():
+    # what 4000 particles more in each of five cells cost on 281 x 277 cells, where a cell has one lane, against 24 x 32
+    # cells, where it has 32: the same rounds of 32 lanes, not 4000 of one lane (up to 30 times that)
+    extra = []
+    for nx, nz in ((24, 32), (281, 277)):
+        t = []
+        for crowd in (0, 4000):
+            cfg = make_cfg(nx=nx, nz=nz, precision=0, order=3, cap=4096)
+            pair = Pair(cfg, part=_clumped(2, nx, 1, nz, crowd))
+            try:
+                P.pic_charge_residual(pair.h)
+                t.append(_best(lambda: P.pic_charge_residual(pair.h)))
+            finally:
+                pair.close()
+        extra.append(t[1] - t[0])
+    assert extra[1] <= 2 * extra[0] + 50e-6, extra
