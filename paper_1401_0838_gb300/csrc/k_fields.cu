@@ -1271,7 +1271,7 @@ size_t field_energy_scratch_bytes() { return sizeof(double) * (3 * FE_BLOCKS + 2
 // comes from two Newton steps on k (k + 2) = u^2 from an FP32 estimate (relative error 1e-7, then 1e-14,
 // then rounding; no cancellation at small u) instead of an FP64 square root and quotient, and eight lanes
 // share a bin of a cell (a warp per cell left half of them idle at 16 particles, and the pipe issues whole
-// warps). 16.8M FP32 particles: 1.7 ms before.
+// warps), but what a bin holds past its neighbours the whole warp takes. 16.8M FP32 particles: 1.7 ms before.
 __device__ __forceinline__ double kinetic_of(double u2) {
   const float a = (float)u2, g = sqrtf(1.f + a);
   if (!(a < 1e30f)) return u2 / (sqrt(1.0 + u2) + 1.0);  // past the FP32 estimate's range, or not a number
@@ -1285,16 +1285,38 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_kinetic(const __grid_constant__ RunDev<T> r, double* out) {
   double acc = 0;
   const long long bins = 2 * r.ncell;
-  for (long long cs = blockIdx.x * 32ll + (threadIdx.x >> 3); cs < bins; cs += gridDim.x * 32ll) {
-    const long long c = cs >> 1;
+  const int lane = threadIdx.x & 31;
+  auto add = [&](long long cs, int j0, int step, int n) {
     const SpeciesBuf<T>& b = cs & 1 ? r.in[1] : r.in[0];  // constant indices: no local copy of r
-    const int n = min(b.cnt[c], r.cap);
-    for (int j = threadIdx.x & 7; j < n; j += 8) {
-      const long long o = c * r.cap + j;
+    for (int j = j0; j < n; j += step) {
+      const long long o = (cs >> 1) * r.cap + j;
       const PartVals<T> v = part_get(b, r.ndim, o);
       const double ux = v.ux, uy = v.uy, uz = (double)r.u0 + (double)v.uz;
       const double k = kinetic_of(fma(uz, uz, fma(uy, uy, ux * ux)));
       acc = b.w ? fma((double)b.w[o], k, acc) : acc + k;
+    }
+  };
+  for (long long cs0 = blockIdx.x * 32ll + (threadIdx.x >> 5) * 4; cs0 < bins; cs0 += gridDim.x * 32ll) {
+    const long long cs = cs0 + (lane >> 3);
+    const int n = cs < bins ? min((cs & 1 ? r.in[1] : r.in[0]).cnt[cs >> 1], r.cap) : 0;
+    // slots that a bin's own lanes take: all, or what leaves clearly fewer rounds of the warp
+    const int most = __reduce_max_sync(0xffffffffu, n);
+    int limit = most;
+    if (most > 128) {
+      int best = 3 * (most / 8) / 4;
+      for (int l = 64; l < most; l *= 2) {
+        const int rounds = l / 8 + __reduce_add_sync(0xffffffffu, (lane & 7) == 0 ? (max(n - l, 0) + 31) / 32 : 0);
+        if (rounds < best) {
+          best = rounds;
+          limit = l;
+        }
+      }
+    }
+    add(cs, lane & 7, 8, min(n, limit));
+    unsigned more = __ballot_sync(0xffffffffu, (lane & 7) == 0 && n > limit);
+    for (; more != 0; more &= more - 1) {
+      const int src = __ffs(more) - 1;
+      add(cs0 + (src >> 3), limit + lane, 32, __shfl_sync(0xffffffffu, n, src));
     }
   }
   if (!r.in[0].w) acc *= (double)r.wconst;

@@ -67,3 +67,40 @@ def test_charge_density_time_of_clumps():
                 pair.close()
         extra.append(t[1] - t[0])
     assert extra[1] <= 2 * extra[0] + 50e-6, extra
+
+
+@pytest.mark.parametrize("precision", [1, 0])
+@pytest.mark.parametrize("ndim", [2, 3])
+@pytest.mark.parametrize("crowd", [33, 700])
+def test_kinetic_energy_of_clumps(precision, ndim, crowd):
+    nx, ny, nz = (37, 1, 41) if ndim == 2 else (11, 9, 13)
+    cfg = make_cfg(ndim=ndim, nx=nx, ny=ny, nz=nz, dt=0.4, precision=precision, cap=8 if crowd < 100 else 800)
+    part = _clumped(ndim, nx, ny, nz, crowd)
+    pair = Pair(cfg, part=part)
+    try:
+        e = P.pic_energy(pair.h)
+        u2 = (pair.o.part["ux"] ** 2 + pair.o.part["uy"] ** 2 + pair.o.part["uz"] ** 2)
+        want = np.sum(pair.o.part["w"] * (u2 / (1 + np.sqrt(1 + u2))))
+    finally:
+        pair.close()
+    # FP32: the drift and the weight are rounded to it
+    assert abs(e["k"] - want) <= (1e-12 if precision else 1e-6) * want
+    assert e["np"] == len(part["x"])
+
+
+def test_kinetic_energy_time_of_clumps():
+    # 200,000 particles in one bin against the same number in the four bins (two cells, two species) that a warp takes:
+    # its 32 lanes share them either way, where eight lanes would walk the one bin four times as long
+    t = []
+    for cells in (1, 2):
+        n = 200000
+        part = synth.clustered_particles(2, 12, 1, 12, n, seed=4, corner=(4, 0, 5), size=1)
+        part["q"] = np.where(np.arange(n) % cells == 0, 1.0, -1.0)
+        part["x"] = 4 + part["x"] % 1.0 + np.arange(n) // cells % cells
+        pair = Pair(make_cfg(nx=12, nz=12, precision=0, cap=n // cells ** 2), part=part)
+        try:
+            P.pic_energy(pair.h)
+            t.append(_best(lambda: P.pic_energy(pair.h)))
+        finally:
+            pair.close()
+    assert t[0] <= 2 * t[1], t
