@@ -1028,6 +1028,51 @@ __device__ __noinline__ void deposit_general(T* sj, int lx, int ly, int lz, T ox
   }
 }
 
+// The same in 2D for the n particles that an item of the paired push has queued (`far`: their slots in the
+// stage, which holds offsets, displacements, v_y and charge), eight lanes per particle: lane a forms the
+// shapes of window node a of both directions, and the lanes add a row of nodes at a time, to addresses of
+// their own. Few particles of a beam come here, but every eighth of a hot load: 2.1M of u_th = 1 at gamma
+// = 3 on 256x512 cells, a step 998 us with deposit_general called by the lane or two of a round that have one
+// (646 us when a warp took a cell), 419 us so.
+template <int LPC>
+__device__ __noinline__ void deposit_queue(float* sj, const float* sq, const float* sr, const float* sw,
+                                           const unsigned char* far, int n, int cell0, float jfx, float jfy, float jfz) {
+  using S = PushSmem<float, 2, 3, true>;
+  const int lane = threadIdx.x & 31, a = lane & 7;
+#pragma unroll 1
+  for (int f0 = 0; f0 < n; f0 += 4) {
+    const bool on = f0 + (lane >> 3) < n && a < 6;
+    const int e = far[min(f0 + (lane >> 3), n - 1)], cl = cell0 + e / (4 * LPC);
+    float q[4];
+    ld4(sq + 4 * e, q);
+    const float w = on ? sw[e] : 0.f, node = (float)(a - 2);
+    const float ex = on ? shape_change(3, node - q[0], q[2]) : 0.f, ez = on ? shape_change(3, node - q[1], q[3]) : 0.f;
+    const float Tx = on ? bspl(3, node - q[0]) + 0.5f * ex : 0.f, Tz = on ? bspl(3, node - q[1]) + 0.5f * ez : 0.f;
+    float px = ex, pz = ez;  // running sums; the last closes to zero
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      const float tx = __shfl_up_sync(0xffffffffu, px, o, 8), tz = __shfl_up_sync(0xffffffffu, pz, o, 8);
+      if (a >= o) {
+        px += tx;
+        pz += tz;
+      }
+    }
+    if (a >= 5) px = pz = 0.f;
+    const float vx = w * jfx * px, vz = w * jfz * Tx, cy = w * sr[e] * jfy, vy = cy * Tx, ky = cy * ex * (1.f / 12.f);
+    // window node 0 (two below the cell) is current-tile index of the cell itself
+    float* j = sj + (cl / S::TX) * S::JX + cl % S::TX + a;
+#pragma unroll
+    for (int b = 0; b < 6; ++b) {
+      const float Tb = __shfl_sync(0xffffffffu, Tz, b, 8), eb = __shfl_sync(0xffffffffu, ez, b, 8);
+      const float pb = __shfl_sync(0xffffffffu, pz, b, 8);
+      const float v0 = vx * Tb, v1 = fmaf(vy, Tb, ky * eb), v2 = vz * pb;
+      if (v0 != 0.f) atomicAdd(j + b * S::JX, v0);
+      if (v1 != 0.f) atomicAdd(j + S::JN + b * S::JX, v1);
+      if (v2 != 0.f) atomicAdd(j + 2 * S::JN + b * S::JX, v2);
+    }
+  }
+}
+
 // 3D cubic deposit of one item and one component (0 Jx, 1 Jy, 2 Jz). The window of all components has 184
 // sums, more than a thread can hold beside the push, so the push leaves each particle's offsets,
 // displacements and charge (zero: nothing to add) in its stage slot and the three components are summed
@@ -1097,6 +1142,7 @@ template <typename T, int NDIM, int SCHEME, int LPC, int ORDER = 1>
 __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   constexpr bool WIN = ORDER == 3 || SCHEME == 2;    // the gather reads the cell's window of nodes
   constexpr bool LATE = NDIM == 3 && ORDER == 3;     // the deposit follows the push of each item
+  constexpr bool QUEUE = PushPaired<T, NDIM>::value && ORDER == 3;  // so do the far deposits
   using S = PushSmem<T, NDIM, ORDER, WIN>;
   using PL = PushPlan<NDIM, LPC, ORDER>;
   constexpr int TX = S::TX, TY = S::TY, NCL = S::NCL;
@@ -1224,6 +1270,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   // cell groups after each warp's first one are handed out in the order warps ask for them, so
   // warps whose groups hold more packs do fewer groups
   __shared__ int s_next_group;
+  // per warp: the slots of the present item whose deposit leaves the register window
+  __shared__ unsigned char s_far[QUEUE ? NWARP : 1][QUEUE ? 128 : 1];
   if (tid == 0) {
     *lvn = 0;
     s_next_group = PUSH_THREADS / 32;
@@ -1324,6 +1372,7 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
       s = k >= k1 ? 1 : 0;
       return k < (s ? end1 : end0);
     };
+    int nfar = 0;
 #pragma unroll 1
     for (int rnd = 0; rnd < nrnd; ++rnd) {
       if constexpr (PushPaired<T, NDIM>::value) {
@@ -1434,17 +1483,26 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           else
             deposit2_lin<Lanes2, float, NVP>(acc2, o_x, d_x, X.am, LinearZ<Lanes2, float>(o_z, d_z, Z.am, Z.c, Z.up),
                                              mul2(qr, jx2), mul2(mul2(qr, vyp), jy2), mul2(qr, jz2));
-          if (!rega && va) {
-            if constexpr (ORDER == 3)
-              deposit_general<float, 2>(sj, lx, 0, lz, oxa, 0.f, oza, dxa, 0.f, dza, qw.x * r.jfx, qw.x * vya * r.jfy2d,
-                                        qw.x * r.jfz);
-            else deposit2_far(sj, lx, lz, oxa, oza, dxa, dza, qw.x * r.jfx, qw.x * vya * r.jfy2d, qw.x * r.jfz);
-          }
-          if (!regb && vb) {
-            if constexpr (ORDER == 3)
-              deposit_general<float, 2>(sj, lx, 0, lz, oxb, 0.f, ozb, dxb, 0.f, dzb, qw.y * r.jfx, qw.y * vyb * r.jfy2d,
-                                        qw.y * r.jfz);
-            else deposit2_far(sj, lx, lz, oxb, ozb, dxb, dzb, qw.y * r.jfx, qw.y * vyb * r.jfy2d, qw.y * r.jfz);
+          if constexpr (QUEUE) {
+            if (__any_sync(0xffffffffu, (!rega && va) || (!regb && vb))) {
+              // into the stage: displacements, v_y and charge of the slot
+              auto queue = [&](bool far, int k, float dx, float dz, float vy, float w) {
+                const unsigned m = __ballot_sync(0xffffffffu, far);
+                if (far) {
+                  const_cast<float*>(stq)[4 * k + 2] = dx;
+                  const_cast<float*>(stq)[4 * k + 3] = dz;
+                  const_cast<float*>(str)[k] = vy;
+                  const_cast<float*>(stw)[k] = w;
+                  s_far[warp][nfar + __popc(m & lt)] = (unsigned char)((lane - sl) * 4 + k);
+                }
+                nfar += __popc(m);
+              };
+              queue(!rega && va, ka, dxa, dza, vya, qw.x);
+              queue(!regb && vb, kb, dxb, dzb, vyb, qw.y);
+            }
+          } else {
+            if (!rega && va) deposit2_far(sj, lx, lz, oxa, oza, dxa, dza, qw.x * r.jfx, qw.x * vya * r.jfy2d, qw.x * r.jfz);
+            if (!regb && vb) deposit2_far(sj, lx, lz, oxb, ozb, dxb, dzb, qw.y * r.jfx, qw.y * vyb * r.jfy2d, qw.y * r.jfz);
           }
           // destinations: a cell of this tile (key (cell * 2 + species) in the tile) or, leaving
           // the tile, the global cell (key global cell * 2 + species)
@@ -1751,6 +1809,13 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           }
         }
       }
+      }
+    }
+    if constexpr (QUEUE) {
+      if (nfar > 0) {
+        __syncwarp();
+        deposit_queue<LPC>(sj, SG::q(stg, stage, 0), SG::r(stg, stage, 0), SG::w(stg, stage, 0), s_far[warp], nfar, g * CPW,
+                           r.jfx, r.jfy2d, r.jfz);
       }
     }
     if constexpr (LATE) {
