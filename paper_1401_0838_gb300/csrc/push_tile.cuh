@@ -529,6 +529,17 @@ struct PushPlan {
   static __device__ __forceinline__ int first_window(int c) { return LPC == 4 ? (c >> 1) + (c & 1) : c; }
 };
 
+// Crowded cells. A cell with many more packs than its group's others would keep its warp on its LPC lanes, so
+// the group leaves it out and the warp then takes it by itself, its packs spread over all lanes (an item is
+// 32 of them). Eight cells of 1500 more particles per species: momentum-conserving 128x256 FP32 495 -> 98 us a
+// step, FP64 3.5 -> 0.59 ms, cubic FP64 7.6 -> 1.26 ms, 3D 24^3 FP32 1359 -> 138 us; even cells are up to 0.4 %
+// slower. Not the cubic FP32 push in 2D, whose registers are full (512x1024 pass 6.22 -> 6.33 ms).
+template <typename T, int NDIM, int ORDER, bool WIN>
+struct PushCrowd {
+  static constexpr bool value = WIN ? NDIM == 2 && (ORDER == 1 || sizeof(T) == 8)
+                                    : NDIM == 3 && sizeof(T) == 4;
+};
+
 // Resident blocks per SM the push kernel is compiled for (register budget).
 template <typename T, int NDIM, int ORDER = 1>
 struct PushMinBlocks {
@@ -1143,6 +1154,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   constexpr bool WIN = ORDER == 3 || SCHEME == 2;    // the gather reads the cell's window of nodes
   constexpr bool LATE = NDIM == 3 && ORDER == 3;     // the deposit follows the push of each item
   constexpr bool QUEUE = PushPaired<T, NDIM>::value && ORDER == 3;  // so do the far deposits
+  constexpr bool CROWD = PushCrowd<T, NDIM, ORDER, WIN>::value;     // crowded cells apart from their group
+  static_assert(!(QUEUE && CROWD), "the queue's cells are the group's");
   using S = PushSmem<T, NDIM, ORDER, WIN>;
   using PL = PushPlan<NDIM, LPC, ORDER>;
   constexpr int TX = S::TX, TY = S::TY, NCL = S::NCL;
@@ -1285,17 +1298,37 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
 
   // Items of this warp: (cell group, pack round). The packs of the next item are copied into the
   // warp's shared-memory stage with cp.async while the current item is computed.
-  auto group_iters = [&](int g) -> int {
+  // A job is the cells of a group, or (CROWD) one crowded cell of it, whose place in the group is `one` (else
+  // -1); crowd: the lanes of the group's crowded cells.
+  auto group_iters = [&](int g, unsigned& crowd) -> int {
     const int c = g * CPW + lane / LPC;
     const int nq = ((sn[c] + 3) >> 2) + ((sn[NCL + c] + 3) >> 2);
+    crowd = 0;
+    if constexpr (CROWD) {
+      const int most = __reduce_max_sync(0xffffffffu, nq);
+      if (most > 8 * LPC) {  // twice the group's mean and eight items more
+        const int mean = __reduce_add_sync(0xffffffffu, nq) >> 5;
+        crowd = __ballot_sync(0xffffffffu, nq > 2 * mean + 8 * LPC);
+        return __reduce_max_sync(0xffffffffu, crowd >> lane & 1u ? 0 : (nq + LPC - 1) / LPC);
+      }
+      return (most + LPC - 1) / LPC;
+    }
     return __reduce_max_sync(0xffffffffu, (nq + LPC - 1) / LPC);
   };
-  auto issue = [&](int g, int it, int stage, bool fix) {
-    const int c = g * CPW + lane / LPC;
-    const int n0 = sn[c], n1 = sn[NCL + c];
+  // The lane's cell and the counts that the job takes of it; returns which LPC packs of it are the lane's.
+  auto lane_cell = [&](int g, int it, int one, unsigned crowd, int& c, int& n0, int& n1) -> int {
+    c = g * CPW + (one >= 0 ? one : lane / LPC);
+    n0 = sn[c];
+    n1 = sn[NCL + c];
+    if (CROWD && one < 0 && crowd >> lane & 1u) n0 = n1 = 0;
+    return one >= 0 ? it * CPW + lane / LPC : it;
+  };
+  auto issue = [&](int g, int it, int one, unsigned crowd, int stage, bool fix) {
+    int c, n0, n1;
+    const int itl = lane_cell(g, it, one, crowd, c, n0, n1);
     const int nq0 = (n0 + 3) >> 2, nq = nq0 + ((n1 + 3) >> 2);
     const int lx = c % TX, ly = (c / TX) % TY, lz = c / (TX * TY);
-    copy_item(((long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx) * r.cap, it, nq0, nq, stage, fix);
+    copy_item(((long long)(Z0 + lz) * nxy + (long long)(Y0 + ly) * r.nx + X0 + lx) * r.cap, itl, nq0, nq, stage, fix);
   };
 
   auto take_group = [&]() -> int {
@@ -1303,14 +1336,31 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     if (lane == 0) v = atomicAdd(&s_next_group, 1);
     return __shfl_sync(0xffffffffu, v, 0);
   };
-  int g = warp, it = 0;
-  int giters = g < ngrp ? group_iters(g) : 0;
-  while (g < ngrp && giters == 0) {
-    g = take_group();
-    giters = g < ngrp ? group_iters(g) : 0;
-  }
+  int g = warp, it = 0, one = -1, giters = 0;
+  unsigned crowd = 0, left = 0;  // the group's crowded cells: their lanes, and those still to be taken (a lane each)
+  const unsigned heads = CROWD ? __ballot_sync(0xffffffffu, sl == 0) : 0u;
+  // The next job after group g's: its next crowded cell, or another group's cells.
+  auto next_job = [&](int& g, int& one, int& giters, unsigned& crowd, unsigned& left, bool first) {
+    for (;;) {
+      if (CROWD && left != 0) {
+        one = (__ffs(left) - 1) / LPC;
+        left &= left - 1;
+        const int c = g * CPW + one;
+        giters = (((sn[c] + 3) >> 2) + ((sn[NCL + c] + 3) >> 2) + 31) >> 5;
+        return;
+      }
+      if (!first) g = take_group();
+      first = false;
+      one = -1;
+      giters = g < ngrp ? group_iters(g, crowd) : 0;
+      if (CROWD) left = g < ngrp ? crowd & heads : 0u;
+      if (g >= ngrp || giters > 0) return;
+    }
+  };
+  next_job(g, one, giters, crowd, left, true);
   int stage = 0;
-  if (g < ngrp) issue(g, 0, 0, g == warp);  // the first group's first item was copied speculatively
+  // the first group's first item was copied speculatively
+  if (g < ngrp) issue(g, 0, one, crowd, 0, g == warp && one < 0);
   cp_async_commit();
   // the register sums; a linear paired push keeps one half per particle of the pair until the group's end
   constexpr bool ACC2 = PushPaired<T, NDIM>::value && ORDER == 1;
@@ -1319,21 +1369,19 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   GalCache<T, NDIM> gc;  // Galerkin nodes of the lane's cell, loaded once per cell group
   while (g < ngrp) {
     // prefetch the next item
-    int ng = g, nit = it + 1, niters = giters;
+    int ng = g, nit = it + 1, niters = giters, none = one;
+    unsigned ncrowd = crowd;
     if (nit >= giters) {
       nit = 0;
-      do {
-        ng = take_group();
-        niters = ng < ngrp ? group_iters(ng) : 0;
-      } while (ng < ngrp && niters == 0);
+      next_job(ng, none, niters, ncrowd, left, false);
     }
-    if (ng < ngrp) issue(ng, nit, stage ^ 1, false);
+    if (ng < ngrp) issue(ng, nit, none, ncrowd, stage ^ 1, false);
     cp_async_commit();
     cp_async_wait_1();
     __syncwarp();
 
-    int cl = g * CPW + lane / LPC;
-    const int n0 = sn[cl], n1 = sn[NCL + cl];
+    int cl, n0, n1;
+    const int itl = lane_cell(g, it, one, crowd, cl, n0, n1);
     const int nq0 = (n0 + 3) >> 2, nq = nq0 + ((n1 + 3) >> 2);
     // the lanes of an empty cell stand in a cell that holds particles: a pair's empty slots go through the
     // arithmetic, and an empty cell's fields may be anything (not finite, or past the tile's last plane not staged)
@@ -1353,7 +1401,7 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     }
     // rounds of this item: up to the last slot in use of the fullest cell
     constexpr int NR = PushRounds<T, NDIM>::value, U = 4 / NR;
-    int nk = 4 * (nq - it * LPC);  // slots of the cell's packs from this item on, then the last pack's empty ones
+    int nk = 4 * (nq - itl * LPC);  // slots of the cell's packs from this item on, then the last pack's empty ones
     if (nk > 0 && nk <= 4 * LPC) nk -= 4 * (nq > nq0 ? nq - nq0 : nq0) - (nq > nq0 ? n1 : n0);
     const int nrnd = min(NR, (__reduce_max_sync(0xffffffffu, nk) + U * LPC - 1) / (U * LPC));
     const int win0 = U == 2 || nrnd == NR ? PL::first_window(lane / LPC) : 0;
@@ -1362,10 +1410,10 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     const T* stw = SG::w(stg, stage, lane - sl);
     const unsigned* sti = SG::id(stg, stage, lane - sl);
     // whether slot k of the cell's 4 LPC holds a particle, and its species
-    const int k1 = 4 * (nq0 - it * LPC), end0 = n0 - 4 * it * LPC, end1 = n1 + k1;
+    const int k1 = 4 * (nq0 - itl * LPC), end0 = n0 - 4 * itl * LPC, end1 = n1 + k1;
     auto slot_of = [&](int k, int& s) -> bool {
       if constexpr (LATE) {  // the cubic 3D push is 2 % slower with the shorter form
-        const int q = it * LPC + (k >> 2);
+        const int q = itl * LPC + (k >> 2);
         s = q >= nq0 ? 1 : 0;
         return q < nq && (s ? n1 + 4 * nq0 : n0) > 4 * q + (k & 3);
       }
@@ -1854,6 +1902,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     __syncwarp();  // the stage just read is refilled by the next iteration's prefetch
     g = ng;
     it = nit;
+    one = none;
+    crowd = ncrowd;
     giters = niters;
     stage ^= 1;
   }

@@ -1,4 +1,4 @@
-"""Diagnostics on a state whose particles crowd into a few cells (an instability bunches the beam): right, and not at the
+"""Steps and diagnostics of a state whose particles crowd into a few cells (an instability bunches the beam): right, and not at the
 mercy of a few lanes that walk a crowded cell alone."""
 import time
 
@@ -8,6 +8,7 @@ import pytest
 import synth
 from tests._pic import P, Pair, make_cfg
 from tests.test_gpu_gauss import _oracle_residual
+from tests.test_gpu_parity import TOL, _coeffs, _compare
 
 pytestmark = pytest.mark.gpu
 
@@ -104,3 +105,61 @@ def test_kinetic_energy_time_of_clumps():
         finally:
             pair.close()
     assert t[0] <= 2 * t[1], t
+
+
+# pushes that give a crowded cell a warp of its own (PushCrowd), and others; a crowded cell among cells of one particle, several in one group, fewer and more than an item of 128 slots
+STEPS = [(2, 1, 2), (2, 3, 0), (2, 3, 1), (2, 3, 2), (2, 1, 0), (3, 1, 0), (3, 1, 1), (3, 1, 2), (3, 3, 0)]
+
+
+@pytest.mark.parametrize("precision", [1, 0])
+@pytest.mark.parametrize("ndim,order,scheme", STEPS)
+@pytest.mark.parametrize("crowd", [60, 150, 400])
+@pytest.mark.parametrize("sigma", [0.0, 2.0])
+def test_step_of_clumps(precision, ndim, order, scheme, crowd, sigma):
+    nx, ny, nz = (19, 1, 37) if ndim == 2 else (11, 7, 13)
+    cfg = make_cfg(ndim=ndim, nx=nx, ny=ny, nz=nz, dt=0.5, scheme=scheme, precision=precision, ppc=4, order=order, cap=512,
+                   sigma_perp=sigma)
+    n = nx * ny * nz
+    part = synth.random_particles(ndim, nx, ny, nz, n + 8 * crowd, seed=5, weight=1e-3, per_particle_weight=sigma > 0)
+    rng = np.random.default_rng(6)
+    base = rng.integers(0, n - 8, 3)  # single cells, and runs of neighbours
+    cell = np.concatenate([np.arange(n), np.repeat(np.concatenate([base, base[0] + np.arange(1, 6)]), crowd)])
+    for k, v in (("x", cell % nx), ("y", cell // nx % ny), ("z", cell // (nx * ny))):
+        if k != "y" or ndim == 3:
+            part[k] = v + rng.uniform(0, 0.999, len(cell))
+    pair = Pair(cfg, psi=_coeffs(scheme, 0.5), fields=synth.random_fields((nz, ny, nx), seed=3, scale=2e-2, smooth=1),
+                part=part)
+    try:
+        pair.step(2)
+        _compare(pair, TOL[precision])
+    finally:
+        pair.close()
+
+
+@pytest.mark.parametrize("ndim,order,scheme,precision", [(2, 1, 2, 0), (2, 1, 2, 1), (2, 3, 0, 1), (3, 1, 0, 0), (3, 1, 1, 0)])
+def test_step_time_of_clumps(ndim, order, scheme, precision):
+    # 6000 particles in one cell against the same in the 8 (3D: 16) cells of its warp's group: the warp's 32 lanes take
+    # them either way, where the cell's 4 (2) lanes would be 8 (16) times as long
+    nx, ny, nz = (64, 1, 64) if ndim == 2 else (16, 16, 16)
+    t = []
+    for size in (1, 8 if ndim == 2 else 4):
+        n = 6000
+        rng = np.random.default_rng(2)
+        part = synth.random_particles(ndim, nx, ny, nz, n, seed=3, weight=1e-6)
+        i = np.arange(n)
+        part["x"] = 8 + i % size + rng.uniform(0, 0.999, n)
+        part["y"] = (8 + i // size % size + rng.uniform(0, 0.999, n)) if ndim == 3 else np.zeros(n)
+        part["z"] = 20.0 % nz + rng.uniform(0, 0.999, n)
+        best = []
+        for _ in range(3):
+            pair = Pair(make_cfg(ndim=ndim, nx=nx, ny=ny, nz=nz, dt=0.5, scheme=scheme, order=order, precision=precision,
+                                 ppc=4, cap=4096), part=part)
+            try:
+                P.pic_enable_timing(pair.h)
+                P.pic_step(pair.h, 1)
+                P.pic_sync(pair.h)
+                best.append(P.pic_kernel_times(pair.h)["push"][0])
+            finally:
+                pair.close()
+        t.append(min(best))
+    assert t[0] <= 3 * t[1], t
