@@ -49,7 +49,8 @@ struct pic_handle {
   long long sp_cap = 0;
   int* d_maxc = nullptr;        // scratch of the bin growth (largest count)
   unsigned long long* d_sp_total = nullptr;  // insertions that found their bin full, since creation
-  int* h_sp_mirror = nullptr;   // pinned copy of the waiting count, written after each pic_step
+  int* h_sp_mirror = nullptr;   // pinned copy of the waiting count, written after each pic_step; 8 bytes on, one of
+                                // d_sp_total, written by the adjoint
   cudaEvent_t ev_sp = nullptr;  // completion of that copy
   bool sp_pending = false;
   int grow_gen = 0;             // reallocations of bins or lists (batched runs re-upload their tables)
@@ -118,6 +119,8 @@ struct pic_handle {
     double* dots = nullptr;     // 10 coefficient-gradient accumulators
     double* partial = nullptr;  // block partial sums of the coefficient gradient
     unsigned long long* seen = nullptr;
+    bool noted = false;              // a copy of d_sp_total is on its way
+    unsigned long long spilled = 0;  // d_sp_total when the bins last had their size checked
     std::vector<void*> mem;
   } adj;
   bool no_diag = false;  // the adjoint's recomputed steps record no diagnostics
@@ -753,6 +756,32 @@ int count_bins(pic_handle* h, long long out[2]) {
   return PIC_OK;
 }
 
+// New bins of nc slots per cell and species in both buffers; their contents are lost. The old ones are freed
+// only once all are in place: a failed allocation keeps them.
+bool resize_bins(pic_handle* h, long long nc) {
+  const size_t slots = (size_t)h->ncell * (size_t)nc;
+  void* np_[2][2][4] = {};
+  bool ok = true;
+  for (int sp = 0; sp < 2 && ok; ++sp)
+    for (int b = 0; b < 2 && ok; ++b)
+      for (int a = 0; a < 4 && ok; ++a) {
+        if (!h->parr[sp][b][a]) continue;  // arrays the run does not carry
+        ok = (np_[sp][b][a] = dalloc(h, slots * slot_bytes(h, a))) != nullptr;
+      }
+  for (int sp = 0; sp < 2; ++sp)
+    for (int b = 0; b < 2; ++b)
+      for (int a = 0; a < 4; ++a) {
+        if (!h->parr[sp][b][a]) continue;
+        dfree(h, ok ? h->parr[sp][b][a] : np_[sp][b][a]);
+        if (ok) h->parr[sp][b][a] = np_[sp][b][a];
+      }
+  if (!ok) return false;
+  h->cap = (int)nc;
+  drop_graph(h);
+  h->grow_gen++;
+  return true;
+}
+
 // Empty the spill list into larger bins. Particles whose bin was full wait in the spill list (the
 // step pushes them from there, so nothing is lost); here, at a synchronising call, every particle
 // (bins and list) is exported to the staging arrays, the bins of both buffers are reallocated with
@@ -797,32 +826,7 @@ int settle(pic_handle* h) {
   CK(launch(h, PIC_K_OTHER, [&] { return launch_spill_export<T>(r, nsp, cnts[0] + cnts[1], f, st); }),
      "spill export");
   CK(cudaStreamSynchronize(st), "synchronize");
-  // new bins for both buffers and species; the old ones are freed only once all are in place
-  const pic_config& c = h->cfg;
-  const size_t slots = (size_t)h->ncell * (size_t)nc;
-  void* np_[2][2][4] = {};
-  bool ok = true;
-  for (int sp = 0; sp < 2 && ok; ++sp)
-    for (int b = 0; b < 2 && ok; ++b)
-      for (int a = 0; a < 4 && ok; ++a) {
-        if (!h->parr[sp][b][a]) continue;  // arrays the run does not carry
-        ok = (np_[sp][b][a] = dalloc(h, slots * slot_bytes(h, a))) != nullptr;
-      }
-  if (!ok) {
-    for (int sp = 0; sp < 2; ++sp)
-      for (int b = 0; b < 2; ++b)
-        for (int a = 0; a < 4; ++a) dfree(h, np_[sp][b][a]);
-    return fail(h, PIC_E_OOM, "particle bin growth: allocation failed");
-  }
-  for (int sp = 0; sp < 2; ++sp)
-    for (int b = 0; b < 2; ++b)
-      for (int a = 0; a < 4; ++a)
-        if (h->parr[sp][b][a]) {
-          dfree(h, h->parr[sp][b][a]);
-          h->parr[sp][b][a] = np_[sp][b][a];
-        }
-  (void)c;
-  h->cap = (int)nc;
+  if (!resize_bins(h, nc)) return fail(h, PIC_E_OOM, "particle bin growth: allocation failed");
   for (int sp = 0; sp < 2; ++sp)
     for (int b = 0; b < 2; ++b) CK(cudaMemsetAsync(h->cnt[sp][b], 0, sizeof(int) * h->ncell, st), "clear counts");
   CK(cudaMemsetAsync(h->d_sp_count, 0, 2 * sizeof(int), st), "clear spill counters");
@@ -830,8 +834,6 @@ int settle(pic_handle* h) {
   RunDev<T> r2 = make_run<T>(h, h->parity);
   CK(launch(h, PIC_K_OTHER, [&] { return launch_import<T>(r2, f, st); }), "re-bin");
   CK(cudaStreamSynchronize(st), "synchronize");
-  drop_graph(h);
-  h->grow_gen++;
   return PIC_OK;
 }
 
@@ -2190,6 +2192,31 @@ int adj_restore(pic_handle* h, int j) {
   return PIC_OK;
 }
 
+// The backward pass restores every segment into the bins there are and does not stop for particles that wait in
+// the spill list. Where some did in an earlier segment (or backward pass), as far as that is known without a
+// wait, the bins grow by half before the next is restored; without the memory the list goes on holding them.
+// 1M particles that focus into every fifth column and part again, 96 FP32 steps: backward 43.9 -> 27.1 ms.
+unsigned long long* spill_total_mirror(pic_handle* h) {
+  return reinterpret_cast<unsigned long long*>(h->h_sp_mirror + 2);
+}
+void adj_note(pic_handle* h) {
+  h->adj.noted = cudaMemcpyAsync(spill_total_mirror(h), h->d_sp_total, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                 h->stream) == cudaSuccess &&
+                 cudaEventRecord(h->ev_sp, h->stream) == cudaSuccess;
+}
+void adj_room(pic_handle* h) {
+  auto& A = h->adj;
+  if (!A.noted) return;
+  if (cudaEventQuery(h->ev_sp) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return;
+  }
+  A.noted = false;
+  const long long align = (long long)(64 / h->es), nc = (h->cap + h->cap / 2 + align - 1) / align * align;
+  if (*spill_total_mirror(h) > A.spilled && nc <= (1 << 24) && !resize_bins(h, nc)) (void)cudaGetLastError();
+  A.spilled = *spill_total_mirror(h);
+}
+
 template <typename T>
 void put_taps(T* dst, const double* src, int n, double scale = 1.0) {
   for (int i = 0; i < n; ++i) dst[i] = (T)(src[i] * scale);
@@ -2342,6 +2369,8 @@ int adjoint_forward_t(pic_handle* h, int nsteps, int every, double* w_perp) {
   A.nseg = nseg;
   A.np = np;
   for (int j = 0; j < nseg; ++j) {
+    // room for the particles that wait: the recomputed steps, which do not stop for it, start from these bins
+    if (j > 0 && (rc = settle<T>(h))) return rc;
     rc = adj_save<T>(h, &A.ck_f[(size_t)j * 6], A.ck_p[j], j == 0);
     if (rc) return rc;
     const int len = nsteps - j * every < every ? nsteps - j * every : every;
@@ -2350,9 +2379,12 @@ int adjoint_forward_t(pic_handle* h, int nsteps, int every, double* w_perp) {
   }
   rc = adj_save<T>(h, &A.ck_f[(size_t)nseg * 6], A.ck_p[nseg], nseg == 0);
   if (rc) return rc;
+  adj_note(h);
   pic_energy_t e;
   rc = energy_t<T>(h, &e);  // synchronises and reads the device error flag (ids, overflow)
   if (rc) return rc;
+  A.spilled = *spill_total_mirror(h);
+  A.noted = false;
   if (e.np != np) return fail(h, PIC_E_STATE, "particles were lost during the recorded run");
   *w_perp = e.w_perp;
   A.final_step = h->nstep;
@@ -2387,11 +2419,13 @@ int adjoint_backward_t(pic_handle* h, double dw, double grad_psi_e[5], double gr
   int rc = PIC_OK;
   for (int j = A.nseg - 1; j >= 0 && rc == PIC_OK; --j) {
     const int len = A.nsteps - j * A.every < A.every ? A.nsteps - j * A.every : A.every;
+    adj_room(h);
     rc = adj_restore<T>(h, j);
     for (int s = 0; s < len && rc == PIC_OK; ++s) {
       rc = adj_save<T>(h, &A.tape_f[(size_t)s * 6], A.tape_p[s], false);
       if (rc == PIC_OK && s + 1 < len) rc = step_once<T>(h);
     }
+    adj_note(h);
     for (int s = len - 1; s >= 0 && rc == PIC_OK; --s) rc = adj_step<T>(h, s);
   }
   h->no_diag = false;
