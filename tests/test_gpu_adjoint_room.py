@@ -44,3 +44,29 @@ def test_bins_grow(precision, every):
         assert P.pic_num_particles(h) == len(part["cell"])
     finally:
         P.pic_destroy(h)
+
+
+@pytest.mark.parametrize("precision", [1, 0])
+@pytest.mark.parametrize("every", [1, 3, 12])
+def test_gradient_with_waiting_particles(precision, every):
+    # the tape takes the particles that wait from the spill list: the same gradient as with room for all of them
+    nx, nz, steps = 25, 24, 12
+    T = np.float64 if precision else np.float32
+    rng = np.random.default_rng(2)
+    fields = {n: (2e-2 * rng.standard_normal((nz, 1, nx))).astype(T) for n in ("ex", "ey", "ez", "bx", "by", "bz")}
+    part, out = _focus(nx, nz, 8, T, steps), []
+    for cap in (16, 128):
+        h = P.pic_create(make_cfg(nx=nx, nz=nz, dt=0.5, gamma=1.0, precision=precision, ppc=8, cap=cap))
+        try:
+            P.pic_set_correction_stencil(h, *P.pic_compute_correction_coeffs(0, 0.5))
+            P.pic_set_state(h, P.make_state(P.PIC_HOST, fields, part))
+            w = P.pic_adjoint_forward(h, steps, every)
+            out.append(np.concatenate([[w], *P.pic_adjoint_backward(h, 1.0)]))
+            assert (P.pic_bin_stats(h)[1] > 0) == (cap == 16)
+            assert P.pic_num_particles(h) == len(part["cell"])
+        finally:
+            P.pic_destroy(h)
+    a, b = out
+    # the same sums in another order, through 12 steps
+    assert np.abs(a[1:] - b[1:]).max() <= (1e-11 if precision else 1e-3) * np.abs(b[1:]).max()
+    assert abs(a[0] - b[0]) <= (1e-11 if precision else 1e-4) * abs(b[0])
