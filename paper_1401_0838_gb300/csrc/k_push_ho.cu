@@ -130,7 +130,7 @@ __device__ __noinline__ T gather_global(const T* g, const RunDev<T>& r, int orde
 template <typename T, int NDIM>
 __device__ __forceinline__ void push_spill_body(const RunDev<T>& r, int order, int scheme, int bid, int nblk) {
   constexpr int NWMAX = 6;
-  const int NW = order == 3 ? 6 : 4, K0 = order == 3 ? -2 : -1;  // deposit window (as HoGeom)
+  const int NW = order == 3 ? 6 : 4, K0 = order == 3 ? -2 : -1;  // deposit window (as deposit_general's, esir_dir's)
   const int tid = threadIdx.x;
   if (bid == 0 && tid == 0) *r.sp_out = 0;  // this step's k_migrate spills into a fresh list
   const long long n = min((long long)*r.sp_in, r.sp_cap);

@@ -192,9 +192,6 @@ cudaError_t launch_yee_fused(const YeeArgs<T>& a, int ndim, cudaStream_t st, dou
 template <typename T>
 cudaError_t launch_kinetic(const RunDev<T>& r, double* out, cudaStream_t st);
 
-// Gauss-law residual (k_gauss.cu): rho += q w S / dV from the particle bins of r.in (shape order 1 or
-// 3, FP64 atomics; rho zeroed by the caller), and (max |div E - rhof|, rms, max |rhof|) into out[0..2]
-// (scratch of gauss_scratch_bytes, zeroed once).
 // Up to 12 copies (or clears, where src is null) of device memory in one launch: addresses and lengths are
 // multiples of 4 bytes, nothing overlaps.
 struct BulkArgs {
@@ -210,6 +207,9 @@ struct BulkArgs {
 };
 cudaError_t launch_bulk(const BulkArgs& a, cudaStream_t st);
 
+// Gauss-law residual (k_gauss.cu): rho += q w S / dV from the particle bins of r.in (shape order 1 or
+// 3, FP64 atomics; rho zeroed by the caller), and (max |div E - rhof|, rms, max |rhof|) into out[0..2]
+// (scratch of gauss_scratch_bytes, zeroed once).
 template <typename T>
 cudaError_t launch_rho(const RunDev<T>& r, int order, double inv_dv, double* rho, cudaStream_t st);
 template <typename T>

@@ -197,11 +197,6 @@ __device__ __forceinline__ bool ge_one(T x) {  // x >= 1
   else return x >= T(1);
 }
 template <typename T>
-__device__ __forceinline__ bool is_zero(T x) {  // x == 0 (either sign)
-  if constexpr (sizeof(T) == 8) return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) == 0;
-  else return x == T(0);
-}
-template <typename T>
 __device__ __forceinline__ bool abs_lt_one(T x) {  // -1 < x < 1; false for a NaN or an infinity
   if constexpr (sizeof(T) == 8) return (__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll) < 0x3FF0000000000000ll;
   else return x > T(-1) && x < T(1);
