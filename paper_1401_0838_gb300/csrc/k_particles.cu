@@ -186,7 +186,7 @@ void push_tiles(int ndim, int es, bool ho, int nx, int ny, int nz, int spread, i
   const int per_sm = es == 8 ? 1 : (ndim == 2 ? 2 : (ho ? 1 : 3));
   const long long slots = (long long)spread * per_sm;
   const int fixed = es == 4 ? 40 : 6;
-  // a warp's cell group takes whole rows of the full tile's width, so narrower tiles only leave lanes idle
+  // a warp's cell group takes whole rows of the full tile's width, however narrow the tile is
   auto cost_of = [&](long long tiles) {
     return (double)((tiles + slots - 1) / slots) * ((double)full[0] * te[1] * te[2] + fixed);
   };
@@ -203,6 +203,8 @@ void push_tiles(int ndim, int es, bool ho, int nx, int ny, int nz, int spread, i
         b[2] = ez;
       }
     }
+  // half the width where the tiles still fill one wave: the same rows, on twice as many SMs
+  if (full[0] >= 8 && set(full[0] / 2, b[1], b[2]) <= slots) return;
   set(b[0], b[1], b[2]);
 }
 
