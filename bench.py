@@ -187,11 +187,12 @@ def parse_clock_samples(text: str) -> dict:
 def profiled_traffic(prof=None, src=None):
     """DRAM bytes per launch of the push kernel from the committed ncu summary, if that summary was
     taken on the current kernel source (else None). src: a file or a list of files, hashed as one
-    byte string in order (the push: its kernel file, the header that fixes its tile shape, the tile's work)."""
+    byte string in order (the push: its kernel file, the header that fixes its tile shape, the tile's work, its
+    roots and quotients)."""
     import hashlib
     prof = prof or os.path.join(ROOT, "profiles", "k_push_2d_512x1024_fp32.md")
     csrc = os.path.join(ROOT, "paper_1401_0838_gb300", "csrc")
-    src = src or [os.path.join(csrc, f) for f in ("k_particles.cu", "common.cuh", "push_tile.cuh")]
+    src = src or [os.path.join(csrc, f) for f in ("k_particles.cu", "common.cuh", "push_tile.cuh", "fastmath.cuh")]
     files = [src] if isinstance(src, str) else list(src)
     try:
         text = open(prof).read()

@@ -94,10 +94,9 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 // particles per cell and species, 6 of 360 us in FP64): push on 128x256 with 8 FP32 particles 26 -> 20 us,
 // 256x512 FP64 1216 -> 1088 us, cubic 3D 44x36x70 230 -> 177 us. The width stays, because a warp takes whole
 // rows of it (a step on 44^3 FP64 cells: 4x4x4 tiles 1350 us, 8x4x5 973), unless tiles of half of it all
-// run at once (hot 16^3 FP64: 4x4x4 tiles 213 us, 8x4x4
-// 235). Several waves of more than one
-// block per SM keep full tiles (301x517: 61 us against 67 on the extents the count of waves would
-// choose). te: cells per tile and direction.
+// run at once (hot 16^3 FP64: 4x4x4 tiles 213 us, 8x4x4 235). Several waves of more than one block per SM
+// keep full tiles (301x517: 61 us against 67 on the extents the count of waves would choose). te: cells
+// per tile and direction.
 void push_tiles(int ndim, int es, bool ho, int nx, int ny, int nz, int spread, int nt[3], int te[3]);
 
 // Raise a kernel's dynamic shared memory limit to `bytes` (once per kernel and size).

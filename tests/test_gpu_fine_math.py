@@ -117,3 +117,23 @@ def test_range(fine, T):
         a, b = r[:, 2 * k], r[:, 2 * k + 1]
         ok = (a == b) | (np.isnan(a) & np.isnan(b)) | (np.abs(a - b) <= 2 * np.spacing(np.abs(b)))
         assert ok.all(), (k, x[~ok], a[~ok], b[~ok])
+
+
+def test_kinetic_energy_over_momenta():
+    # pic_energy's gamma - 1, from FP32 estimates refined in FP64, one particle at a time: no cancellation at small u,
+    # the IEEE expression past the estimates' range
+    from tests._pic import P, make_cfg, uniform_weight
+
+    cfg = make_cfg(nx=8, nz=8, gamma=1.0, precision=1, ppc=1)
+    h = P.pic_create(cfg)
+    try:
+        for u in [0.0, 1e-30, 1e-12, 1e-6, 1e-3, 0.1, 0.5, 1.0, 2.7, 130.0, 1e4, 1e9, 3e14, 1e16, 1e40, 1e150]:
+            part = {"cell": np.zeros(1, np.int32), "species": np.zeros(1, np.int32), "id": np.zeros(1, np.uint32), "oy": None,
+                    "w": None, "dux": np.full(1, u), "duy": np.zeros(1), "duz": np.zeros(1), "ox": np.full(1, 0.5),
+                    "oz": np.full(1, 0.5)}
+            P.pic_set_state(h, P.make_state(P.PIC_HOST, None, part))
+            U = np.longdouble(u) ** 2
+            want = np.longdouble(uniform_weight(cfg)) * (U / (np.sqrt(1 + U) + 1))
+            assert abs(np.longdouble(P.pic_energy(h)["k"]) - want) <= 2.0 ** -50 * want, u
+    finally:
+        P.pic_destroy(h)
