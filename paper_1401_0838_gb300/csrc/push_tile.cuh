@@ -1469,14 +1469,12 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           float2 m2 = fma2(mx, mx, one2);
           m2 = fma2(my, my, m2);
           m2 = fma2(Mz, Mz, m2);
-          const float2 hig = mul2(hh, WIN ? make_float2(fine_rsqrt(m2.x), fine_rsqrt(m2.y))
-                                       : make_float2(fast_rsqrt(m2.x), fast_rsqrt(m2.y)));
+          const float2 hig = mul2(hh, WIN ? fine_rsqrt(m2) : make_float2(fast_rsqrt(m2.x), fast_rsqrt(m2.y)));
           const float2 tx = mul2(hig, Bx), ty = mul2(hig, By), tz = mul2(hig, Bz);
           float2 t2 = fma2(tx, tx, one2);
           t2 = fma2(ty, ty, t2);
           t2 = fma2(tz, tz, t2);
-          const float2 sf = WIN ? make_float2(fine_two_over(t2.x), fine_two_over(t2.y))
-                                : make_float2(two_over(t2.x), two_over(t2.y));
+          const float2 sf = WIN ? fine_two_over(t2) : make_float2(two_over(t2.x), two_over(t2.y));
           const float2 sx = mul2(sf, tx), sy = mul2(sf, ty), sz = mul2(sf, tz);
           const float2 qx = fma2(my, tz, fma2(neg2(Mz), ty, mx));
           const float2 qy = fma2(Mz, tx, fma2(neg2(mx), tz, my));
@@ -1489,12 +1487,12 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
           u2 = fma2(uy2, uy2, u2);
           u2 = fma2(Uz, Uz, u2);
           const float2 gp = add2(one2, u2);
-          const float2 ign = WIN ? make_float2(fine_rsqrt(gp.x), fine_rsqrt(gp.y))
-                                 : make_float2(fast_rsqrt(gp.x), fast_rsqrt(gp.y));
-          if (r.kin) {
-            const float2 g1 = fma2(gp, ign, one2);  // gamma + 1; gamma - 1 = u^2 / (gamma + 1)
-            kin = fmaf(wa, WIN ? fine_kinetic(u2.x, gp.x, ign.x) : fast_div(u2.x, g1.x), kin);
-            kin = fmaf(wb, WIN ? fine_kinetic(u2.y, gp.y, ign.y) : fast_div(u2.y, g1.y), kin);
+          const float2 ign = WIN ? fine_rsqrt(gp) : make_float2(fast_rsqrt(gp.x), fast_rsqrt(gp.y));
+          if (r.kin) {  // gamma - 1 = u^2 / (gamma + 1)
+            const float2 g1 = fma2(gp, ign, one2);
+            const float2 k = WIN ? fine_kinetic(u2, gp, ign) : make_float2(fast_div(u2.x, g1.x), fast_div(u2.y, g1.y));
+            kin = fmaf(wa, k.x, kin);
+            kin = fmaf(wb, k.y, kin);
           }
           const float2 vy2 = mul2(uy2, ign);
           const float2 ddx2 = mul2(dtdx2, mul2(ux2, ign)), ddz2 = mul2(dtdz2, mul2(Uz, ign));

@@ -48,6 +48,34 @@ static int run(const T* x, const T* u2, T* out, int n) {
   cudaFree(dout);
   return rc;
 }
+// 1 where a pair's values differ from the single ones
+__global__ void k_pairs(const float* x, const float* u2, float* o, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int j = (i * 7 + 1) % n;
+  const float2 v = make_float2(x[i], x[j]), q = make_float2(u2[i], u2[j]), gp = make_float2(1.f + q.x, 1.f + q.y);
+  const float2 ign = fine_rsqrt(gp), r = fine_rsqrt(v), t = fine_two_over(v), k = fine_kinetic(q, gp, ign);
+  auto same = [](float a, float b) { return __float_as_int(a) == __float_as_int(b) || (a != a && b != b); };
+  auto one = [&](float a, float b, float g, float vr, float vt, float vk, float vi) {
+    const float gi = fine_rsqrt(g);
+    return same(fine_rsqrt(a), vr) && same(fine_two_over(a), vt) && same(fine_kinetic(b, g, gi), vk) && same(gi, vi);
+  };
+  o[i] = one(v.x, q.x, gp.x, r.x, t.x, k.x, ign.x) && one(v.y, q.y, gp.y, r.y, t.y, k.y, ign.y) ? 0.f : 1.f;
+}
+extern "C" int run_pairs(const float* x, const float* u2, float* out, int n) {
+  float *dx = nullptr, *du = nullptr, *dout = nullptr;
+  const size_t b = sizeof(float) * (size_t)n;
+  int rc = cudaMalloc(&dx, b) || cudaMalloc(&du, b) || cudaMalloc(&dout, b);
+  if (!rc) rc = cudaMemcpy(dx, x, b, cudaMemcpyHostToDevice) || cudaMemcpy(du, u2, b, cudaMemcpyHostToDevice);
+  if (!rc) {
+    k_pairs<<<(n + 255) / 256, 256>>>(dx, du, dout, n);
+    rc = cudaGetLastError() != cudaSuccess || cudaMemcpy(out, dout, b, cudaMemcpyDeviceToHost) != cudaSuccess;
+  }
+  cudaFree(dx);
+  cudaFree(du);
+  cudaFree(dout);
+  return rc;
+}
 extern "C" int run_f(const float* x, const float* u, float* o, int n) { return run(x, u, o, n); }
 extern "C" int run_d(const double* x, const double* u, double* o, int n) { return run(x, u, o, n); }
 """
@@ -69,6 +97,7 @@ def fine(tmp_path_factory):
         assert f(*(ctypes.c_void_p(a.ctypes.data) for a in (x, u2, out)), ctypes.c_int(len(x))) == 0
         return out
 
+    call.lib = lib
     return call
 
 
@@ -104,6 +133,17 @@ def test_fp64_samples(fine):
     if np.finfo(np.longdouble).nmant < 63:
         pytest.skip("no wider type for the reference")
     _check(r, x, u2, np.longdouble)
+
+
+def test_pairs_equal_single_values(fine):
+    rng = np.random.default_rng(3)
+    n = 1 << 20
+    x = np.ldexp(rng.uniform(1, 2, n), rng.integers(0, 128, n)).astype(np.float32)
+    x[:4] = [np.inf, np.nan, 2.0 ** 126, 1.0]
+    u2 = (10.0 ** rng.uniform(-12, 30, n)).astype(np.float32)
+    out = np.empty(n, np.float32)
+    assert fine.lib.run_pairs(*(ctypes.c_void_p(a.ctypes.data) for a in (x, u2, out)), ctypes.c_int(n)) == 0
+    assert not out.any(), x[out != 0][:5]
 
 
 @pytest.mark.parametrize("T", [np.float32, np.float64])
