@@ -42,7 +42,8 @@ __device__ __forceinline__ int wrap_any(int g, int n) {
 // registers, the cell's lanes add up, and one lane adds each node once instead of once per particle:
 // 331 -> 95 us on 301 x 517 cells of 2 x 8 particles. Cells that hold far more particles than their
 // neighbours (bunches) would keep a warp on one lane: past a limit the whole warp takes a cell's
-// particles together, RHOB.
+// particles together (3000 more in each of eight cells of 300 x 300, cubic: the residual in 0.7 ms, 12 ms
+// on the cells' own lanes).
 template <typename T, int NDIM, int ORDER>
 __global__ void __launch_bounds__(RHO_THREADS) k_rho(const __grid_constant__ RunDev<T> r, int lpc, double inv_dv,
                                                      double* __restrict__ rho) {
