@@ -526,13 +526,13 @@ struct PushPlan {
 
 // Crowded cells. A cell with many more packs than its group's others would keep its warp on its LPC lanes, so
 // the group leaves it out and the warp then takes it by itself, its packs spread over all lanes (an item is
-// 32 of them). Eight cells of 1500 more particles per species: momentum-conserving 128x256 FP32 495 -> 98 us a
-// step, FP64 3.5 -> 0.59 ms, cubic FP64 7.6 -> 1.26 ms, 3D 24^3 FP32 1359 -> 138 us; even cells are up to 0.4 %
-// slower. Not the cubic FP32 push in 2D, whose registers are full (512x1024 pass 6.22 -> 6.33 ms).
+// 32 of them). A step with 1500 more particles per species in eight cells: momentum-conserving 128x256 FP32
+// 495 -> 98 us, FP64 3.5 -> 0.59 ms, cubic FP64 7.6 -> 1.26 ms, 3D 24^3 FP32 1359 -> 138 us; 20,000 in one
+// cell, cubic FP32 8.3 -> 0.97 ms (6.3 when a cell had a warp). Even cells pay 0.4 % of the 3D pass, 1.4 %
+// of the cubic FP32 one (6.18 -> 6.27 ms on 512x1024).
 template <typename T, int NDIM, int ORDER, bool WIN>
 struct PushCrowd {
-  static constexpr bool value = WIN ? NDIM == 2 && (ORDER == 1 || sizeof(T) == 8)
-                                    : NDIM == 3 && sizeof(T) == 4;
+  static constexpr bool value = WIN ? NDIM == 2 : NDIM == 3 && sizeof(T) == 4;
 };
 
 // Resident blocks per SM the push kernel is compiled for (register budget).
@@ -1040,15 +1040,15 @@ __device__ __noinline__ void deposit_general(T* sj, int lx, int ly, int lz, T ox
 // their own. Few particles of a beam come here, but every eighth of a hot load: 2.1M of u_th = 1 at gamma
 // = 3 on 256x512 cells, a step 998 us with deposit_general called by the lane or two of a round that have one
 // (646 us when a warp took a cell), 419 us so.
-template <int LPC>
-__device__ __noinline__ void deposit_queue(float* sj, const float* sq, const float* sr, const float* sw,
-                                           const unsigned char* far, int n, int cell0, float jfx, float jfy, float jfz) {
+inline __device__ __noinline__ void deposit_queue(float* sj, const float* sq, const float* sr, const float* sw,
+                                                  const unsigned char* far, int n, int cell0, int per_cell, float jfx,
+                                                  float jfy, float jfz) {
   using S = PushSmem<float, 2, 3, true>;
   const int lane = threadIdx.x & 31, a = lane & 7;
 #pragma unroll 1
   for (int f0 = 0; f0 < n; f0 += 4) {
     const bool on = f0 + (lane >> 3) < n && a < 6;
-    const int e = far[min(f0 + (lane >> 3), n - 1)], cl = cell0 + e / (4 * LPC);
+    const int e = far[min(f0 + (lane >> 3), n - 1)], cl = cell0 + e / per_cell;
     float q[4];
     ld4(sq + 4 * e, q);
     const float w = on ? sw[e] : 0.f, node = (float)(a - 2);
@@ -1150,7 +1150,6 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
   constexpr bool LATE = NDIM == 3 && ORDER == 3;     // the deposit follows the push of each item
   constexpr bool QUEUE = PushPaired<T, NDIM>::value && ORDER == 3;  // so do the far deposits
   constexpr bool CROWD = PushCrowd<T, NDIM, ORDER, WIN>::value;     // crowded cells apart from their group
-  static_assert(!(QUEUE && CROWD), "the queue's cells are the group's");
   using S = PushSmem<T, NDIM, ORDER, WIN>;
   using PL = PushPlan<NDIM, LPC, ORDER>;
   constexpr int TX = S::TX, TY = S::TY, NCL = S::NCL;
@@ -1855,8 +1854,8 @@ __device__ __forceinline__ void push_tile(const RunDev<T>& r, const int tile) {
     if constexpr (QUEUE) {
       if (nfar > 0) {
         __syncwarp();
-        deposit_queue<LPC>(sj, SG::q(stg, stage, 0), SG::r(stg, stage, 0), SG::w(stg, stage, 0), s_far[warp], nfar, g * CPW,
-                           r.jfx, r.jfy2d, r.jfz);
+        deposit_queue(sj, SG::q(stg, stage, 0), SG::r(stg, stage, 0), SG::w(stg, stage, 0), s_far[warp], nfar,
+                      g * CPW + max(one, 0), one < 0 ? 4 * LPC : 128, r.jfx, r.jfy2d, r.jfz);
       }
     }
     if constexpr (LATE) {

@@ -136,7 +136,8 @@ def test_step_of_clumps(precision, ndim, order, scheme, crowd, sigma):
         pair.close()
 
 
-@pytest.mark.parametrize("ndim,order,scheme,precision", [(2, 1, 2, 0), (2, 1, 2, 1), (2, 3, 0, 1), (3, 1, 0, 0), (3, 1, 1, 0)])
+@pytest.mark.parametrize("ndim,order,scheme,precision", [(2, 1, 2, 0), (2, 1, 2, 1), (2, 3, 0, 0), (2, 3, 2, 0), (2, 3, 0, 1),
+                                                         (3, 1, 0, 0), (3, 1, 1, 0)])
 def test_step_time_of_clumps(ndim, order, scheme, precision):
     # 6000 particles in one cell against the same in the 8 (3D: 16) cells of its warp's group: the warp's 32 lanes take
     # them either way, where the cell's 4 (2) lanes would be 8 (16) times as long
